@@ -227,8 +227,32 @@ def m2l_split_degree(p):
     return p - 4 if p >= 8 else p - 3
 
 
+def m2l_issued_flops(p, precision, split_all=False):
+    """Flops the tensor-core M2L issues per pair and state: its columns are the
+    (p+1)^2 - 1 trace-free moments, its rows the p^2 local coefficients; every
+    k-step (16 BF16 or 8 TF32 moments, lowest degree d) is one M = 128 MMA over
+    the rows of degree <= p - d, padded to 16.  Split BF16 adds the hi x lo and
+    lo x hi MMAs over the rows of degree <= split degree - d (the first k-step:
+    <= split degree; every row with split_all), the split degree p - 4 from
+    order 8 on, p - 2 below."""
+    rows_of = lambda t: 0 if t < 0 else (t + 1) ** 2
+    pad = lambda x, m: (x + m - 1) // m * m
+    deg = lambda n: next(t for t in range(p + 2) if (t + 1) ** 2 > n)
+    kw = 16 if precision == "bf16x3" else 8
+    sd = p - 4 if p >= 8 else p - 2
+    total = 0
+    for ks in range(pad((p + 1) ** 2 - 1, kw) // kw):
+        d = deg(ks * kw + 1)
+        rows = pad(rows_of(p - d), 16)
+        total += rows * kw
+        if precision == "bf16x3":
+            rows2 = rows if split_all else min(pad(rows_of(sd if ks == 0 else sd - d), 16), rows)
+            total += 2 * rows2 * kw
+    return 2.0 * total
+
+
 def m2l_tile_flops(p, precision, split_all=False):
-    """Flops the tensor-core M2L issues per pair and state: every k-step
+    """The same for an M2L on all C(p+3, 3) multi-indices: every k-step
     (16 BF16 or 8 TF32 values of n) is one M = 128 MMA over the rows m still
     needed at that k-step (rows of degree t need |n| < C(p - t + 3, 3)),
     padded to 16.  Split BF16 adds the hi x lo and lo x hi MMAs over the rows
@@ -330,14 +354,15 @@ def stage_roofline(stage, stats, steps_profiled, precision, peaks, sm_mhz, tenso
                 peak = peaks.get("tf32_mma_measured") or base * (1.1 / 2.25)
                 src = ("measured TF32 tcgen05.mma (demag_measure_peak, this run)" if peaks.get("tf32_mma_measured")
                        else src + " x 1.1/2.25 nominal TF32 ratio")
-            tile_flops = (m2l_tile_flops(p, precision, split_all=stats.get("_split_all", False)) * stats["n_m2l"] * B
+            tile_flops = (m2l_issued_flops(p, precision, split_all=stats.get("_split_all", False)) * stats["n_m2l"] * B
                           / launches_per_eval)
             achieved = work / per_launch_s / 1e12
             out.update({"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                         "frac": achieved / peak, "traffic": NCU_TRAFFIC.get(key),
                         "executed_tflops": tile_flops / per_launch_s / 1e12,
                         "peak_source": src,
-                        "note": "achieved counts algorithmic flops 2*C(p+6,6) per pair per state; executed_tflops "
+                        "note": "achieved counts the method's 2*C(p+6,6) flops per pair per state (all multi-indices); "
+                                "the M2L runs on the trace-free ones, executed_tflops "
                                 "counts the padded per-k-step row prefixes issued to the tensor pipe "
                                 + ("(hi x hi everywhere, hi x lo and lo x hi on the rows whose terms take the "
                                    "second limb)" if precision == "bf16x3" else "(1 TF32 MMA per tile)")})
@@ -346,7 +371,7 @@ def stage_roofline(stage, stats, steps_profiled, precision, peaks, sm_mhz, tenso
         peak, src = _alu_peak(kind, peaks, sm_mhz)
         out.update({"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                     "traffic": NCU_TRAFFIC.get(key), "peak_source": src,
-                    "note": f"algorithmic flops 2*C(p+6,6) per pair per state, {kind} CUDA cores"})
+                    "note": f"the method's 2*C(p+6,6) flops per pair per state (all multi-indices), {kind} CUDA cores"})
         return out
     if stage == "p2p" and stats["near_mode"] == 0:
         work = stats["n_p2p_pairs"] * p2p_fp64_flops(B) / launches_per_eval

@@ -163,7 +163,7 @@ typedef struct {
                           forms the products with the second BF16 limb
                           (hi x lo, lo x hi) only for the terms of degree
                           |m| + |n| <= p - 4 of the translation (Sec. 2.3;
-                          p - 3 for p < 8); the highest degrees, whose share of the
+                          p - 2 for p < 8); the highest degrees, whose share of the
                           expansion falls off like a power of the cell
                           size over the distance, take hi x hi alone
                           (about half the MMAs); < 0: both products for

@@ -191,6 +191,8 @@ static demag_plan_s* new_plan(const demag_options& o, int64_t n_nodes, int64_t n
     }
     P->p = o.p;
     P->nc = ncoef_of(o.p);
+    P->nq = nq_of(o.p);
+    P->nl = nl_of(o.p);
     P->nn = n_nodes;
     P->nt = n_tets;
     DM_CUDA(cudaGetDevice(&P->device));
@@ -705,7 +707,7 @@ demag_status demag_plan_stats(demag_plan plan, demag_stats* o) {
     o->stage_ms[k] = plan->stage_ms[k];
     o->stage_launches[k] = plan->stage_launches[k];
   }
-  o->n_m2l_ops = plan->n_tc_ops;
+  o->n_m2l_ops = plan->opt.precision != DEMAG_FP64 ? plan->n_m2l_keys : 0;
   o->m2l_kps = plan->tc_kps;
   o->m2l_ring_bytes = plan->tc_budget;
   o->m2l_targets_per_cta = plan->tc_ops ? plan->tc_nt : 0;

@@ -265,15 +265,16 @@ void audit_plan(Plan& P, bool plant) {
       if (P.w_off32) A.offsets("w_off32", P.w_off32, nT, 0, P.n_wentries / 3 * 4, 0, P.n_wentries / 3 * 4);
     }
   }
-  // mixed path: gradient operator, parent lists, M2L operator indices and groups
+  // far field: parent lists, M2L operator indices
+  A.values("par_list", P.par_list, P.par_start.empty() ? 0 : P.par_start.back(), 0, nc);
+  if (P.m2l_op) A.values("m2l_op", P.m2l_op, P.n_m2l, 0, P.n_m2l_keys);
+  if (P.m2l_tab_opdl) A.values("m2l_tab_opdl", P.m2l_tab_opdl, P.n_m2l, 0, P.n_m2l_keys, 0x00ffffff);
+  // mixed path: gradient operator, M2L groups
   if (P.opt.precision != DEMAG_FP64) {
     A.values("node_iperm", P.node_iperm, nn, 0, nn);
     const int64_t nh = A.last(P.hg_off, nn);
     A.offsets("hg_off", P.hg_off, nn, 0, nh, 0, nh);
     A.values("hg_col", P.hg_col, nh, 0, nn);
-    A.values("par_list", P.par_list, P.par_start.empty() ? 0 : P.par_start.back(), 0, nc);
-    if (P.m2l_op) A.values("m2l_op", P.m2l_op, P.n_m2l, 0, P.n_tc_ops);
-    if (P.m2l_tab_opdl) A.values("m2l_tab_opdl", P.m2l_tab_opdl, P.n_m2l, 0, P.n_tc_ops, 0x00ffffff);
     if (P.tc_g1_off)
       A.offsets("tc_g1_off", P.tc_g1_off, (int64_t)P.h_m2l_targets.size(), 0, P.n_m2l, -1, -1);
     if (P.tc_n_g2 > 0) {
@@ -281,7 +282,7 @@ void audit_plan(Plan& P, bool plant) {
       A.values("tc_g2_tgt", P.tc_g2_tgt, 2 * P.tc_n_g2, -1, nc);
       A.offsets("tc_g2_off", P.tc_g2_off, P.tc_n_g2, 0, ne, 0, ne);
       A.values("tc_g2_src", P.tc_g2_src, ne, 0, nc);
-      A.values("tc_g2_op", P.tc_g2_op, 2 * ne, -1, P.n_tc_ops);
+      A.values("tc_g2_op", P.tc_g2_op, 2 * ne, -1, P.n_m2l_keys);
     }
   }
   // test hook: a scratch copy of the M2L source list with its last entry set

@@ -33,13 +33,14 @@ constexpr int NF_ROWS = 128;  // target nodes per tile of the tensor-core near f
 
 __host__ __device__ inline int ncoef_of(int p) { return (p + 1) * (p + 2) * (p + 3) / 6; }
 
-// one coefficient of an FP32 octree translation: target coefficient += (bit
+// one coefficient of an octree translation: target coefficient += (bit
 // `octant` of neg ? -c : c) * source coefficient k (octant of the child cell)
+template <class T>
 struct TEnt {
   uint16_t k;
   uint8_t neg;
   uint8_t pad;
-  float c;
+  T c;
 };
 
 // Graded multi-index order: total degree t ascending; within t, n_x descending,
@@ -58,6 +59,51 @@ __host__ __device__ inline void mi_decode(int idx, int& a, int& b, int& c) {
   c = r - j * (j + 1) / 2;
   b = j - c;
   a = t - j;
+}
+
+// ---------------------------------------------------------------------------
+// Trace-free form of the expansions.  The derivatives b_k of 1/|x| and the
+// local coefficients L_k are harmonic, sum_i X_{k+2e_i} = 0, so every X_k is
+// fixed by the ones with k_x <= 1:
+//   X_(a0+2q, b, c) = (-1)^q sum_{j<=q} C(q,j) X_(a0, b+2j, c+2(q-j)),  a0 in {0, 1}.
+// Of the C(p+3, 3) coefficients of order p only (p+1)^2 are independent.  The
+// moments enter through sum_n b_{n+m} Q_n alone, so they may be folded onto the
+// same indices (the transposed relation, degree by degree: the truncation
+// |n| + |m| <= p is untouched): 1,284 products per M2L pair at p = 8 instead
+// of 2,838.  All moments have Q_0 = 0 (they are integrals of the gradient of
+// y^n), so the rows |m| = p take no term and L has degree < p:
+//   moments   nq = (p+1)^2 - 1 per cell, position h_index - 1
+//   local     nl = p^2 per cell, position h_index.
+// Order: degree t ascending from t^2; within it k_x = 0 by ascending k_z, then
+// k_x = 1 by ascending k_z.
+__host__ __device__ constexpr int nq_of(int p) { return (p + 1) * (p + 1) - 1; }
+__host__ __device__ constexpr int nl_of(int p) { return p * p; }
+__host__ __device__ constexpr int h_index(int a, int b, int c) {  // a in {0, 1}
+  return (a + b + c) * (a + b + c) + (a ? a + b + c + 1 + c : c);
+}
+__host__ __device__ constexpr int h_degree(int idx) {
+  int t = 0;
+  while ((t + 1) * (t + 1) <= idx) t++;
+  return t;
+}
+__host__ __device__ inline void h_decode(int idx, int& a, int& b, int& c) {
+  const int t = h_degree(idx), r = idx - t * t;
+  a = r > t;
+  c = a ? r - t - 1 : r;
+  b = t - a - c;
+}
+// sum over the full multi-indices n that fold onto (a, b, c) of weight * f(n)
+template <class F>
+__host__ __device__ inline double h_fold(int a, int b, int c, F&& f) {
+  double v = 0.0;
+  for (int i = 0; 2 * i <= b; i++) {
+    double w = (i & 1) ? -1.0 : 1.0;  // (-1)^(i+l) C(i+l, i)
+    for (int l = 0; 2 * l <= c; l++) {
+      v += w * f(a + 2 * (i + l), b - 2 * i, c - 2 * l);
+      w *= -(double)(i + l + 1) / (double)(l + 1);
+    }
+  }
+  return v;
 }
 
 // ---------------------------------------------------------------------------
@@ -92,6 +138,7 @@ struct Plan {
   cudaStream_t stream = nullptr;  // plan-build stream
   demag_options opt{};
   int p = 4, nc = 35, nc1 = 20;   // order, ncoef(p), ncoef(p-1)
+  int nq = 24, nl = 16;           // trace-free moments and local coefficients per cell
   int64_t nn = 0, nt = 0;
   double lo[3] = {0, 0, 0}, side = 0, scale = 0;
   double plan_ms = 0;
@@ -150,7 +197,7 @@ struct Plan {
   int32_t* tet_col = nullptr;       // nt x 4: column of each vertex in its leaf's support
   std::vector<int32_t> h_src_leaves;// leaves holding tets
   int32_t* src_leaves = nullptr;
-  double* Ghat = nullptr;           // n_sup x nc1 : int lambda_k y^m/m! over the leaf's tets at that node
+  double* Ghat = nullptr;           // n_sup x nc1 : int lambda_k y^m/m! over the leaf's tets at that node (plan time)
 
   // node -> incident tets (for lumped H)
   int64_t* nt_off = nullptr;        // nn + 1
@@ -191,13 +238,12 @@ struct Plan {
 
   // tensor-core M2L (TF32 / split BF16): one operator tile set per distinct
   // (level difference, lattice offset) and the operator index of every pair
-  int64_t n_tc_ops = 0;
   unsigned char* tc_ops = nullptr;
   int32_t* m2l_op = nullptr;        // n_m2l
-  float* m2l_tab = nullptr;         // n_tc_ops x nc: FP32 b_k(v) per key (CUDA-core M2L)
+  int64_t n_m2l_keys = 0;           // distinct translation keys (m2l_keys.cu)
+  void* m2l_tab = nullptr;          // b_k(v) per key for the CUDA-core M2L (FP64 plans: doubles, else floats)
+  void* m2l_tab_items = nullptr;    // its work items (per order)
   int32_t* m2l_tab_opdl = nullptr;  // n_m2l: key index | (level difference & 255) << 24
-  uint32_t* m2l_rc_items = nullptr; // row-chunk items (m | c << 16), then per row a CSR of its items
-  int m2l_rc_nitems = 0, m2l_rc_ch = 0;
   int tc_nt = 1, tc_kps = 0, tc_budget = 0;  // M2L launch shape: targets per CTA, k-steps per slot, ring bytes
   int tc_ls = 0;                    // split BF16 limb scheme of the tensor-core M2L (m2l_tc.cu)
   int tc_prom_group = 0, tc_prom_rows = 16;  // accumulator promotion: sources per group (0 = off), rows
@@ -208,13 +254,18 @@ struct Plan {
   int32_t* tc_g2_src = nullptr;
   int32_t* tc_g2_op = nullptr;      //   2 per entry: each target's operator, -1 = not in its list
 
-  // FP32 octree translations as coefficient lists (mixed precision):
+  // far-field operators (far.cu), in the arithmetic of the plan: FP64 plans hold
+  // doubles, the others floats
+  int g_stride = 0;                 // values per support node of the P2M operator: 3 nq, padded to 4
+  void* far_G = nullptr;            // n_sup x g_stride: P2M operator, [moment q][component]
+  void* far_h = nullptr;            // nn x nl: the L2P polynomials of every node
+  // octree translations as coefficient lists (TEnt<T>):
   //   M2M: Qt^P_n += sum over entries e of n: sign_e(octant) c_e Qt^C_{k_e}
   //   L2L: Lt^C_m += sum over entries e of m: sign_e(octant) c_e Lt^P_{k_e}
-  int32_t* m2m_eoff = nullptr;      // nc + 1
-  TEnt* m2m_ent = nullptr;
-  int32_t* l2l_eoff = nullptr;      // nc + 1
-  TEnt* l2l_ent = nullptr;
+  int32_t* m2m_eoff = nullptr;      // nq + 1
+  void* m2m_ent = nullptr;
+  int32_t* l2l_eoff = nullptr;      // nl + 1
+  void* l2l_ent = nullptr;
   int32_t* par_list = nullptr;      // cells with children, level by level
   std::vector<int64_t> par_start;   // host, nlevels + 1: parents of level l are par_list[par_start[l] ..]
   // FP32 mass-lumped gradient operator (mixed precision), rows by sorted node:
@@ -223,9 +274,6 @@ struct Plan {
   int32_t* hg_col = nullptr;
   float4* hg_w = nullptr;           // (x, y, z, 0)
   int32_t* node_iperm = nullptr;    // original -> sorted node
-
-  // FP32 far-field operators (mixed precision, per-level scaled)
-  float* Ghat32 = nullptr;          // n_sup x nc1: Ghat[e][m] / s_leaf^(|m|+1)
 
   std::vector<DevBuf> bufs;
   int64_t device_bytes = 0;
@@ -328,20 +376,33 @@ bool near_tc_wanted(const Plan& P);
 // MP: workspace of nf_mp_floats(P, B) floats for M in the layout of the kernel's bulk copies
 size_t nf_mp_floats(const Plan& P, int B);
 void launch_near_tc(Plan& P, const float* Ms, float* MP, int B, float* u_s, int* err, cudaStream_t s);
-struct M2lKeys {  // distinct translation keys (dl, lattice offset) and the key of every M2L pair
+struct M2lKeys {  // distinct translation keys (dl, lattice offset); the key of every pair is P.m2l_op
   bool ok = false;
   std::vector<int4> keys;
-  std::vector<int64_t> off;           // host copy of m2l_off
-  std::vector<int32_t> src, op;       // host copies of m2l_src and of the key index per pair
 };
-// mixed-precision far field (fmm32.cu)
-void build_mixed_operators(Plan& P);
+// the far field on trace-free expansions (far.cu): operators at plan time, then
+// P2M, M2M, L2L and L2P in T = double (FP64 plans) or float; each returns its
+// kernel launches
+void build_far_operators(Plan& P);
+template <class T>
+int launch_p2m(Plan& P, int B, const T* Ms, T* Q, cudaStream_t s);
+template <class T>
+int launch_m2m(Plan& P, int B, T* Q, cudaStream_t s);
+template <class T>
+int launch_l2l(Plan& P, int B, T* L, cudaStream_t s);
+template <class T>
+int launch_l2p(Plan& P, int B, const T* L, T* u, cudaStream_t s);
+// mixed precision: gradient operator and evaluation (fmm32.cu)
+void build_gradient_operator(Plan& P);
 void eval_mixed(Plan& P, const double* M, int B, double* u, double* H, cudaStream_t s);
-bool launch_m2l32_fast(Plan& P, int B, const float* Q, float* L, int* err, cudaStream_t s);  // m2l32.cu
-// FP32 table-driven M2L on CUDA cores (m2l32.cu): derivative table per key at
-// plan time; launch returns false when the plan has no table
+// M2L on CUDA cores without a table (m2l32.cu)
+template <class T>
+void launch_m2l_rows(Plan& P, int B, const T* Q, T* L, cudaStream_t s);
+// table-driven M2L on CUDA cores (m2l32.cu): derivative table per key at plan
+// time; launch returns false when the plan has no table
 void build_m2l_tab(Plan& P, const M2lKeys& K);
-bool launch_m2l32_tab(Plan& P, int B, const float* Q, float* L, cudaStream_t s);
+template <class T>
+bool launch_m2l_tab(Plan& P, int B, const T* Q, T* L, cudaStream_t s);
 // largest batch for which the tensor-core precisions run the table-driven FP32
 // M2L instead of the tensor-core one (whose tiles hold 128 states)
 inline int m2l_table_batch(const Plan& P) {
@@ -360,7 +421,7 @@ void llg_rk4(Plan& P, double* m, int B, double Ms, double alpha, const double* h
 // tensor-core M2L (m2l_tc.cu): operator table at plan time; bytes of the packed
 // moments for B states (0 when the tensor-core M2L is off); packs Q into QP and
 // runs the M2L (false: not available for this plan, use the CUDA-core M2L)
-M2lKeys build_m2l_keys(Plan& P);      // also fills P.m2l_op
+M2lKeys build_m2l_keys(Plan& P);      // m2l_keys.cu; also fills P.m2l_op and P.n_m2l_keys
 void build_m2l_tc(Plan& P, const M2lKeys& K);
 size_t m2l_tc_pack_bytes(const Plan& P, int B);
 bool launch_m2l_tc(Plan& P, int B, const float* Q, unsigned char* QP, float* L, int* err, cudaStream_t s);

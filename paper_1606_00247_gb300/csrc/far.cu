@@ -1,0 +1,632 @@
+// far.cu -- the far field (Sec. 2 steps 1-2 and 4-5; the M2L is m2l32.cu and
+// m2l_tc.cu): P2M, M2M, L2L and L2P on per-level scaled, trace-free expansions,
+// in FP64 (FP64 plans) or FP32 (mixed precision).
+//
+// With s the side of a cell, the stored coefficients are
+//   Qt_n = Qhat_n / s^|n|      Lt_m = L_m s^|m|
+// (Qhat_n = Q_n/n!, L_m = d^m u, see fmm.cu), kept in the trace-free form of
+// common.cuh (nq = (p+1)^2 - 1 moments, nl = p^2 local coefficients: 80 and 64
+// instead of 165 at p = 8).  All of them are O(1) whatever the mesh scale, so
+// FP32 neither overflows nor underflows, and the octree translations become
+// level independent.  With F[n -> r] the folding weights of common.cuh:
+//   P2M: Qt_r = sum_j sum_c G_j[r, c] M_c(j),
+//        G_j[r, c] = sum_{n -> r} F Ghat_j[n - e_c] / s^|n|               (plan time, FP64)
+//   M2M: Qt^P_r = sum_k [sum_{n -> r} F s_{n-k}(+-1/4)] 2^-|k| Qt^C_k      (child centre - parent centre = +-s_P/4)
+//   M2L: Lt^T_m = (-1)^|m| / (4 pi s_T) sum_n b_{n+m}(v) (s_S/s_T)^|n| Qt^S_n,  v = (c_T - c_S)/s_T
+//   L2L: Lt^C_m = sum_r [sum_{k -> r, k >= m} F s_{k-m}(+-1/2) 2^-|k|] Lt^P_r  (= +-s_C/2)
+//   L2P: u(c + z) = sum_m h_m(z/s) Lt_m,  h_m = sum_{n -> m} F s_n           (plan time, FP64)
+// (s_j(d) = d^j/j!; b_k(x) = (-1)^|k| d^k (1/|x|), so that 1/|x - y| = sum_k
+// b_k(x) y^k / k!).  All arrays keep the state index innermost: X[item][coefficient][state].
+#include <algorithm>
+#include <array>
+#include <cmath>
+#include <type_traits>
+
+#include "common.cuh"
+
+namespace demag {
+
+static inline int nblk(int64_t n, int t) { return (int)((n + t - 1) / t > 0 ? (n + t - 1) / t : 1); }
+
+namespace {
+
+// P2M operator of every support node, [moment q][component] (rows of `gs`
+// values): the exact-moment operator Ghat folded onto the trace-free moments
+template <class T>
+__global__ void k_p2m_op(const int32_t* __restrict__ leaves, const int32_t* __restrict__ level,
+                         const int64_t* __restrict__ sup_off, const double* __restrict__ Ghat, double side, int nc1,
+                         int nq, int gs, T* G) {
+  const int32_t c = leaves[blockIdx.x];
+  const double inv_s = 1.0 / ldexp(side, -level[c]);
+  const int64_t so = sup_off[c], ne = sup_off[c + 1] - so;
+  for (int64_t it = threadIdx.x; it < ne * gs; it += blockDim.x) {
+    const int64_t e = so + it / gs;
+    const int q = (int)(it % gs), r = q / 3, comp = q - 3 * r;
+    double v = 0.0;
+    if (r < nq) {
+      int ra, rb, rc;
+      h_decode(r + 1, ra, rb, rc);
+      const double* gh = Ghat + e * nc1;
+      v = h_fold(ra, rb, rc, [&](int na, int nb, int nz) {
+        if (comp == 0) return na ? gh[mi_index(na - 1, nb, nz)] : 0.0;
+        if (comp == 1) return nb ? gh[mi_index(na, nb - 1, nz)] : 0.0;
+        return nz ? gh[mi_index(na, nb, nz - 1)] : 0.0;
+      });
+      for (int t = ra + rb + rc; t > 0; t--) v *= inv_s;
+    }
+    G[e * gs + q] = (T)v;
+  }
+}
+
+// L2P polynomials h_m(z/s) of every node at its leaf, rows of nl values
+template <class T>
+__global__ void k_node_h(int64_t nn, const int32_t* __restrict__ node_leaf, const int32_t* __restrict__ level,
+                         const double* __restrict__ nodes_s, const double* __restrict__ centre, double side, int nl,
+                         T* h) {
+  const int64_t it = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t i = it / nl;
+  if (i >= nn) return;
+  const int m = (int)(it - i * nl);
+  const int32_t c = node_leaf[i];
+  const double inv_s = 1.0 / ldexp(side, -level[c]);
+  double z[3];
+  for (int x = 0; x < 3; x++) z[x] = (nodes_s[3 * i + x] - centre[3 * c + x]) * inv_s;
+  int a, b, g;
+  h_decode(m, a, b, g);
+  h[it] = (T)h_fold(a, b, g, [&](int na, int nb, int nz) {
+    const int e[3] = {na, nb, nz};
+    double v = 1.0;
+    for (int x = 0; x < 3; x++)
+      for (int k = 1; k <= e[x]; k++) v = v * z[x] / k;
+    return v;
+  });
+}
+
+// P2M: one block per (source leaf, NN moments, 128 SPT states), 128 threads,
+// thread = SPT states (bl, bl + 128).  Support nodes come in chunks of P2M_NE,
+// double-buffered in shared memory by asynchronous copies (cp.async), the next
+// chunk in flight while the current one is applied: per node the operator
+// values of the block's NN moments (3 NN, in the order of use) and M of the
+// states.  One node costs 3 NN / 4 broadcast 16-byte reads for 3 NN SPT FMAs
+// (two states per thread halve the shared-memory reads per FMA).  NN = 80 holds
+// all moments of p <= 8 in registers, so M is read once per leaf.
+constexpr int P2M_NE = 8, P2M_B = 128;
+template <int SPT, int NN>
+constexpr size_t p2m_smem() {  // two chunk buffers
+  return sizeof(float) * 2 * P2M_NE * (NN * 3 + 3 * SPT * P2M_B);
+}
+
+__device__ __forceinline__ void cp_async4(void* dst, const void* src, bool valid) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(valid ? 4 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(valid ? 16 : 0)
+               : "memory");
+}
+
+template <int SPT, int NN>
+__global__ void __launch_bounds__(P2M_B) k_p2m32(const int32_t* __restrict__ leaves,
+                                                 const int64_t* __restrict__ sup_off,
+                                                 const int32_t* __restrict__ sup_node, const float* __restrict__ G,
+                                                 int gs, const float* __restrict__ Ms, int nq, int B, float* Q) {
+  constexpr int NS = SPT * P2M_B, NN3 = 3 * NN;  // states per block, operator values per node
+  static_assert(NN % 4 == 0, "operator rows are copied and read 16 bytes at a time");
+  extern __shared__ __align__(16) float p2m_smem_[];
+  float(*sG)[P2M_NE][NN3] = (float(*)[P2M_NE][NN3])p2m_smem_;                              // [2][node][(q, c)]
+  float(*sM)[P2M_NE][3][NS] = (float(*)[P2M_NE][3][NS])(p2m_smem_ + 2 * P2M_NE * NN3);     // [2][node][c][state]
+  const int32_t c = leaves[blockIdx.x];
+  const int n0 = blockIdx.y * NN;
+  const int tid = threadIdx.x, bb = blockIdx.z * NS;
+  const int64_t so = sup_off[c], eo = sup_off[c + 1];
+  auto stage = [&](int64_t e0, int buf) {  // one chunk of support nodes into buffer buf
+    const int ne = (int)min((int64_t)P2M_NE, eo - e0);
+    for (int q = tid; q < P2M_NE * NN3 / 4; q += P2M_B) {
+      const int r = q / (NN3 / 4), j = 4 * (q - r * (NN3 / 4));
+      const bool ok = r < ne && 3 * n0 + j < gs;
+      cp_async16(&sG[buf][r][j], ok ? G + (e0 + r) * gs + 3 * n0 + j : G, ok);
+    }
+    for (int r = 0; r < P2M_NE; r++) {
+      const int64_t node = r < ne ? sup_node[e0 + r] : 0;
+#pragma unroll
+      for (int s2 = 0; s2 < SPT; s2++) {
+        const int b = bb + s2 * P2M_B + tid;
+        const bool ok = r < ne && b < B;
+        const float* mp = Ms + (ok ? node * 3 * B + b : 0);
+#pragma unroll
+        for (int cc = 0; cc < 3; cc++) cp_async4(&sM[buf][r][cc][s2 * P2M_B + tid], ok ? mp + (int64_t)cc * B : Ms, ok);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float acc[SPT][NN];
+#pragma unroll
+  for (int s2 = 0; s2 < SPT; s2++)
+#pragma unroll
+    for (int j = 0; j < NN; j++) acc[s2][j] = 0.f;
+  if (so < eo) stage(so, 0);
+  int buf = 0;
+  for (int64_t e0 = so; e0 < eo; e0 += P2M_NE, buf ^= 1) {
+    const int ne = (int)min((int64_t)P2M_NE, eo - e0);
+    if (e0 + P2M_NE < eo) {
+      stage(e0 + P2M_NE, buf ^ 1);  // the other buffer was released by the barrier that ended the last chunk
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();  // this chunk complete in shared memory for every thread
+    for (int r = 0; r < ne; r++) {
+      float m[SPT][3];
+#pragma unroll
+      for (int s2 = 0; s2 < SPT; s2++)
+#pragma unroll
+        for (int cc = 0; cc < 3; cc++) m[s2][cc] = sM[buf][r][cc][s2 * P2M_B + tid];
+      const float4* g4 = (const float4*)sG[buf][r];
+#pragma unroll
+      for (int q = 0; q < NN3 / 4; q++) {
+        const float4 g = g4[q];  // values 4q .. 4q+3 = (j, comp) pairs in order
+        const float gv[4] = {g.x, g.y, g.z, g.w};
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+          const int jc = 4 * q + u, j = jc / 3, comp = jc % 3;
+#pragma unroll
+          for (int s2 = 0; s2 < SPT; s2++) acc[s2][j] = fmaf(gv[u], m[s2][comp], acc[s2][j]);
+        }
+      }
+    }
+    __syncthreads();  // the buffer may be refilled
+  }
+#pragma unroll
+  for (int s2 = 0; s2 < SPT; s2++) {
+    const int b = bb + s2 * P2M_B + tid;
+    if (b < B)
+#pragma unroll
+      for (int j = 0; j < NN; j++)
+        if (n0 + j < nq) Q[((int64_t)c * nq + n0 + j) * B + b] = acc[s2][j];
+  }
+}
+
+// P2M of small batches: block per (source leaf, SB states).  The tiles of
+// k_p2m32 hold 128 states; here a thread is (moment q, node group g) and keeps
+// SB states, the operator rows are read once, coalesced (12 bytes a thread), M
+// of the chunk's nodes is a shared-memory broadcast.  The groups' sums are added
+// in order.
+constexpr int P2MS_THREADS = 256, P2MS_NE = 64;
+template <class T, int SB>
+__global__ void __launch_bounds__(P2MS_THREADS) k_p2m_small(const int32_t* __restrict__ leaves,
+                                                              const int64_t* __restrict__ sup_off,
+                                                              const int32_t* __restrict__ sup_node,
+                                                              const T* __restrict__ G, int gs,
+                                                              const T* __restrict__ Ms, int nq, int B, T* Q) {
+  __shared__ T sM[P2MS_NE][3][SB];
+  __shared__ T red[P2MS_THREADS][SB];
+  const int32_t c = leaves[blockIdx.x];
+  const int tid = threadIdx.x, b0 = blockIdx.y * SB;
+  const int64_t so = sup_off[c];
+  const int ns = (int)(sup_off[c + 1] - so);
+  const int ng = min(8, P2MS_THREADS / nq), g = tid / nq, q = tid - g * nq;
+  T acc[SB];
+#pragma unroll
+  for (int v = 0; v < SB; v++) acc[v] = (T)0;
+  for (int e0 = 0; e0 < ns; e0 += P2MS_NE) {
+    const int ne = min(P2MS_NE, ns - e0);
+    __syncthreads();  // the previous chunk is no longer read
+    for (int t = tid; t < ne * 3 * SB; t += P2MS_THREADS) {
+      const int e = t / (3 * SB), r = t - e * 3 * SB, cc = r / SB, v = r - cc * SB;
+      sM[e][cc][v] = b0 + v < B ? Ms[((int64_t)sup_node[so + e0 + e] * 3 + cc) * B + b0 + v] : (T)0;
+    }
+    __syncthreads();
+    if (g < ng) {
+      const T* gp = G + (so + e0) * gs + 3 * q;
+#pragma unroll 4
+      for (int e = g; e < ne; e += ng) {
+        const T g0 = gp[(int64_t)e * gs], g1 = gp[(int64_t)e * gs + 1], g2 = gp[(int64_t)e * gs + 2];
+#pragma unroll
+        for (int v = 0; v < SB; v++) acc[v] = fma(g0, sM[e][0][v], fma(g1, sM[e][1][v], fma(g2, sM[e][2][v], acc[v])));
+      }
+    }
+  }
+#pragma unroll
+  for (int v = 0; v < SB; v++) red[tid][v] = acc[v];
+  __syncthreads();
+  for (int t = tid; t < nq * SB; t += P2MS_THREADS) {
+    const int qq = t / SB, v = t - qq * SB;
+    if (b0 + v >= B) continue;
+    T sum = (T)0;
+    for (int gg = 0; gg < ng; gg++) sum += red[gg * nq + qq][v];
+    Q[((int64_t)c * nq + qq) * B + b0 + v] = sum;
+  }
+}
+
+// batches up to this take the small-batch P2M and L2P (slices of 8 states)
+constexpr int FAR_SMALL_BATCH = 32;
+
+template <int SPT, int NN>
+void launch_p2m_tile(Plan& P, int B, const float* Ms, float* Q, cudaStream_t s) {
+  smem_opt_in((const void*)k_p2m32<SPT, NN>, p2m_smem<SPT, NN>());
+  const dim3 grid((unsigned)P.h_src_leaves.size(), (unsigned)((P.nq + NN - 1) / NN),
+                  (unsigned)((B + SPT * P2M_B - 1) / (SPT * P2M_B)));
+  k_p2m32<SPT, NN><<<grid, P2M_B, p2m_smem<SPT, NN>(), s>>>(P.src_leaves, P.sup_off, P.sup_node, (const float*)P.far_G,
+                                                           P.g_stride, Ms, P.nq, B, Q);
+}
+
+template <class T, int SB>
+void launch_p2m_small(Plan& P, int B, const T* Ms, T* Q, cudaStream_t s) {
+  const dim3 grid((unsigned)P.h_src_leaves.size(), (unsigned)((B + SB - 1) / SB));
+  k_p2m_small<T, SB><<<grid, P2MS_THREADS, 0, s>>>(P.src_leaves, P.sup_off, P.sup_node, (const T*)P.far_G, P.g_stride,
+                                                   Ms, P.nq, B, Q);
+}
+
+// M2M of one level: thread per (cell, n, state); the warp shares (cell, n), so
+// the coefficient list is read as a broadcast and the child moments coalesce
+template <class T>
+__global__ void k_m2m(const int32_t* __restrict__ parents, int64_t npar, const int32_t* __restrict__ child0,
+                        const int32_t* __restrict__ nchild, const uint64_t* __restrict__ prefix,
+                        const int32_t* __restrict__ eoff, const TEnt<T>* __restrict__ ent, int nq, int B, T* Q) {
+  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t per = (int64_t)nq * B;
+  if (idx >= npar * per) return;
+  const int64_t P = parents[idx / per];
+  const int rem = (int)(idx % per), n = rem / B, b = rem - n * B;
+  const int nch = nchild[P];
+  const int32_t c0 = child0[P];
+  const int e0 = eoff[n], e1 = eoff[n + 1];
+  T acc = (T)0;
+  for (int k = 0; k < nch; k++) {
+    const int oct = (int)(prefix[c0 + k] & 7ull);
+    const T* Qc = Q + (int64_t)(c0 + k) * per + b;
+    for (int e = e0; e < e1; e++) {
+      const TEnt<T> E = ent[e];
+      const T v = Qc[(int64_t)E.k * B];
+      acc = fma(((E.neg >> oct) & 1) ? -E.c : E.c, v, acc);
+    }
+  }
+  Q[P * per + (int64_t)n * B + b] = acc;
+}
+
+// L2L from the parents of one level: thread per (parent, m, state) feeding all
+// children at once (each parent coefficient is loaded once; the octant only
+// flips signs); added to the children's own M2L results
+template <class T>
+__global__ void k_l2l(const int32_t* __restrict__ parents, int64_t npar, const int32_t* __restrict__ child0,
+                        const int32_t* __restrict__ nchild, const int4* __restrict__ range,
+                        const uint64_t* __restrict__ prefix, const int32_t* __restrict__ eoff,
+                        const TEnt<T>* __restrict__ ent, int nl, int B, T* L) {
+  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t per = (int64_t)nl * B;
+  if (idx >= npar * per) return;
+  const int64_t P = parents[idx / per];
+  const int nch = nchild[P];
+  if (range[P].w == range[P].z) return;  // no target node below this cell
+  const int rem = (int)(idx % per), m = rem / B, b = rem - m * B;
+  const int32_t c0 = child0[P];
+  int oct[8];
+  T acc[8];
+#pragma unroll
+  for (int k = 0; k < 8; k++) {
+    oct[k] = k < nch ? (int)(prefix[c0 + k] & 7ull) : 0;
+    acc[k] = (T)0;
+  }
+  const T* Lp = L + P * per + b;
+  for (int e = eoff[m], e1 = eoff[m + 1]; e < e1; e++) {
+    const TEnt<T> E = ent[e];
+    const T v = E.c * Lp[(int64_t)E.k * B];
+#pragma unroll
+    for (int k = 0; k < 8; k++) acc[k] += ((E.neg >> oct[k]) & 1) ? -v : v;
+  }
+#pragma unroll
+  for (int k = 0; k < 8; k++)
+    if (k < nch) {
+      const int4 r = range[c0 + k];
+      if (r.w > r.z) L[(int64_t)(c0 + k) * per + (int64_t)m * B + b] += acc[k];  // only cells with target nodes
+    }
+}
+
+// L2P: block per (leaf holding nodes, 128 states), 256 threads.  The leaf's
+// local expansion (nl coefficients x 128 states, 32 KB at p = 8) is staged once
+// in shared memory by asynchronous copies (coalesced over states); the nodes
+// follow in chunks of 16, their polynomials transposed into [m][16 nodes], and
+// thread (group g, states 2s and 2s + 1) accumulates the potentials of nodes
+// 4g .. 4g + 3: per m one 8-byte and one broadcast 16-byte read for 8 FMAs.
+constexpr int L2P_NCH = 16, L2P_THREADS = 256;
+
+__global__ void __launch_bounds__(L2P_THREADS) k_l2p32(const int32_t* __restrict__ leaves,
+                                                       const int4* __restrict__ range, const float* __restrict__ nodeh,
+                                                       int nl, int B, const float* __restrict__ L, float* u) {
+  extern __shared__ __align__(16) float l2p_smem[];
+  float* sL = l2p_smem;              // [m][128 states]
+  float* sh = l2p_smem + nl * 128;   // [m][16 nodes]
+  const int32_t c = leaves[blockIdx.x];
+  const int4 r = range[c];
+  const int tid = threadIdx.x, sp = tid & 63, grp = tid >> 6, b0 = blockIdx.y * 128, b = b0 + 2 * sp;
+  const float* Lc = L + (int64_t)c * nl * B + b0;
+  if (B % 4 == 0) {  // rows of 16-byte vectors, whole within B
+    for (int q = tid; q < nl * 32; q += L2P_THREADS) {
+      const int m = q >> 5, v = 4 * (q & 31);
+      const bool ok = b0 + v < B;
+      cp_async16(sL + m * 128 + v, ok ? Lc + (int64_t)m * B + v : L, ok);
+    }
+  } else {
+    for (int q = tid; q < nl * 128; q += L2P_THREADS) {
+      const int m = q >> 7, v = q & 127;
+      const bool ok = b0 + v < B;
+      cp_async4(sL + q, ok ? Lc + (int64_t)m * B + v : L, ok);
+    }
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  for (int32_t i0 = r.z; i0 < r.w; i0 += L2P_NCH) {
+    const int nk = min(L2P_NCH, r.w - i0);
+    __syncthreads();  // sL complete (first chunk); the previous chunk's polynomials are read
+    for (int q = tid; q < L2P_NCH * nl; q += L2P_THREADS) {
+      const int k = q / nl, m = q - k * nl;
+      sh[m * L2P_NCH + k] = k < nk ? nodeh[(int64_t)(i0 + k) * nl + m] : 0.f;
+    }
+    __syncthreads();
+    float a[2][4] = {};
+#pragma unroll 4
+    for (int m = 0; m < nl; m++) {
+      const float2 l = *(const float2*)(sL + m * 128 + 2 * sp);
+      const float4 w = *(const float4*)(sh + m * L2P_NCH + 4 * grp);
+      const float wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        a[0][k] = fmaf(l.x, wv[k], a[0][k]);
+        a[1][k] = fmaf(l.y, wv[k], a[1][k]);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      if (4 * grp + k >= nk) break;
+      float* o = u + (int64_t)(i0 + 4 * grp + k) * B + b;
+      if (b < B) o[0] = a[0][k];
+      if (b + 1 < B) o[1] = a[1][k];
+    }
+  }
+}
+
+// L2P of small batches: block per (leaf holding nodes, SB states), the leaf's
+// coefficients in shared memory, one warp per node: lanes stride the node's
+// polynomials (coalesced), the states are added over the lanes by a fixed
+// shuffle tree
+constexpr int L2PS_THREADS = 128;
+template <class T, int SB>
+__global__ void __launch_bounds__(L2PS_THREADS) k_l2p_small(const int32_t* __restrict__ leaves,
+                                                              const int4* __restrict__ range,
+                                                              const T* __restrict__ nodeh, int nl, int B,
+                                                              const T* __restrict__ L, T* u) {
+  __shared__ T sL[MAX_P * MAX_P * SB];
+  const int32_t c = leaves[blockIdx.x];
+  const int4 r = range[c];
+  const int b0 = blockIdx.y * SB, lane = threadIdx.x & 31;
+  for (int q = threadIdx.x; q < nl * SB; q += L2PS_THREADS) {
+    const int m = q / SB, v = q - m * SB;
+    sL[q] = b0 + v < B ? L[((int64_t)c * nl + m) * B + b0 + v] : (T)0;
+  }
+  __syncthreads();
+  for (int32_t i = r.z + (int)(threadIdx.x >> 5); i < r.w; i += L2PS_THREADS / 32) {
+    T a[SB];
+#pragma unroll
+    for (int v = 0; v < SB; v++) a[v] = (T)0;
+    for (int m = lane; m < nl; m += 32) {
+      const T h = nodeh[(int64_t)i * nl + m];
+#pragma unroll
+      for (int v = 0; v < SB; v++) a[v] = fma(h, sL[m * SB + v], a[v]);
+    }
+#pragma unroll
+    for (int v = 0; v < SB; v++) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) a[v] += __shfl_xor_sync(0xffffffffu, a[v], o);
+      if (lane == 0 && b0 + v < B) u[(int64_t)i * B + b0 + v] = a[v];
+    }
+  }
+}
+
+template <class T, int SB>
+void launch_l2p_small(Plan& P, int B, const T* L, T* u, cudaStream_t s) {
+  const dim3 grid((unsigned)P.n_node_leaves, (unsigned)((B + SB - 1) / SB));
+  k_l2p_small<T, SB><<<grid, L2PS_THREADS, 0, s>>>(P.node_leaves, P.cell_range, (const T*)P.far_h, P.nl, B, L, u);
+}
+
+// coefficient lists of the translations on the trace-free coefficients
+// (formulas in the file header), with the sign for the child octant o:
+// d_i = +h if bit i of o is set, else -h.  A fold moves n_x by multiples of
+// two into n_y and n_z, so the sign of a term follows the parities of the
+// folded index difference.
+template <class T>
+void build_translations(Plan& P) {
+  const int p = P.p, nq = P.nq, nl = P.nl;
+  auto fact = [](int n) {
+    double f = 1;
+    for (int i = 2; i <= n; i++) f *= i;
+    return f;
+  };
+  auto mono = [&](double h, int ja, int jb, int jc) {  // s_j(h, h, h), 0 below the index range
+    if (ja < 0 || jb < 0 || jc < 0) return 0.0;
+    return std::pow(h, ja + jb + jc) / (fact(ja) * fact(jb) * fact(jc));
+  };
+  auto neg_bits = [](int ja, int jb, int jc) {
+    int bits = 0;
+    for (int o = 0; o < 8; o++) {
+      int odd = ((o & 1) ? 0 : ja) + ((o & 2) ? 0 : jb) + ((o & 4) ? 0 : jc);
+      if (odd & 1) bits |= 1 << o;
+    }
+    return (uint8_t)bits;
+  };
+  std::vector<int32_t> moff(nq + 1), loff(nl + 1);
+  std::vector<TEnt<T>> ment, lent;
+  for (int r = 0; r < nq; r++) {
+    moff[r] = (int32_t)ment.size();
+    int ra, rb, rc;
+    h_decode(r + 1, ra, rb, rc);
+    for (int k = 0; k < nq; k++) {
+      int ka, kb, kc;
+      h_decode(k + 1, ka, kb, kc);
+      const double cf = h_fold(ra, rb, rc, [&](int na, int nb, int nz) { return mono(0.25, na - ka, nb - kb, nz - kc); }) *
+                        std::ldexp(1.0, -(ka + kb + kc));
+      if (cf != 0.0) ment.push_back(TEnt<T>{(uint16_t)k, neg_bits(ra + ka, rb + kb, rc + kc), 0, (T)cf});
+    }
+  }
+  moff[nq] = (int32_t)ment.size();
+  for (int m = 0; m < nl; m++) {
+    loff[m] = (int32_t)lent.size();
+    int ma, mb, mc;
+    h_decode(m, ma, mb, mc);
+    for (int r = 0; r < nl; r++) {  // parent coefficients of degree p are zero
+      int ra, rb, rc;
+      h_decode(r, ra, rb, rc);
+      const int tr = ra + rb + rc;
+      const double cf = h_fold(ra, rb, rc, [&](int ka, int kb, int kz) { return mono(0.5, ka - ma, kb - mb, kz - mc); }) *
+                        std::ldexp(1.0, -tr);
+      if (tr < p && cf != 0.0) lent.push_back(TEnt<T>{(uint16_t)r, neg_bits(ra + ma, rb + mb, rc + mc), 0, (T)cf});
+    }
+  }
+  loff[nl] = (int32_t)lent.size();
+  cudaStream_t s = P.stream;
+  P.m2m_eoff = dalloc<int32_t>(P, nq + 1);
+  P.m2m_ent = dalloc<TEnt<T>>(P, ment.size());
+  P.l2l_eoff = dalloc<int32_t>(P, nl + 1);
+  P.l2l_ent = dalloc<TEnt<T>>(P, lent.size());
+  DM_CUDA(cudaMemcpyAsync(P.m2m_eoff, moff.data(), moff.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+  DM_CUDA(cudaMemcpyAsync(P.m2m_ent, ment.data(), ment.size() * sizeof(TEnt<T>), cudaMemcpyHostToDevice, s));
+  DM_CUDA(cudaMemcpyAsync(P.l2l_eoff, loff.data(), loff.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+  DM_CUDA(cudaMemcpyAsync(P.l2l_ent, lent.data(), lent.size() * sizeof(TEnt<T>), cudaMemcpyHostToDevice, s));
+  DM_CUDA(cudaStreamSynchronize(s));
+}
+
+// cells with children, level by level (the M2M and L2L launches run over these only)
+void build_parent_lists(Plan& P) {
+  cudaStream_t s = P.stream;
+  std::vector<int32_t> nch(P.ncells), list;
+  DM_CUDA(cudaMemcpyAsync(nch.data(), P.cell_nchild, sizeof(int32_t) * P.ncells, cudaMemcpyDeviceToHost, s));
+  DM_CUDA(cudaStreamSynchronize(s));
+  P.par_start.assign(1, 0);
+  for (int l = 0; l < P.nlevels; l++) {
+    for (int64_t c = P.level_start[l]; c < P.level_start[l + 1]; c++)
+      if (nch[c] > 0) list.push_back((int32_t)c);
+    P.par_start.push_back((int64_t)list.size());
+  }
+  P.par_list = dalloc<int32_t>(P, std::max<size_t>(list.size(), 1));
+  if (!list.empty())
+    DM_CUDA(cudaMemcpyAsync(P.par_list, list.data(), sizeof(int32_t) * list.size(), cudaMemcpyHostToDevice, s));
+  DM_CUDA(cudaStreamSynchronize(s));
+}
+
+template <class T>
+void build_operators(Plan& P) {
+  build_translations<T>(P);
+  cudaStream_t s = P.stream;
+  P.g_stride = (3 * P.nq + 3) / 4 * 4;
+  T* G = dalloc<T>(P, std::max<int64_t>(P.n_sup, 1) * P.g_stride);
+  T* h = dalloc<T>(P, P.nn * P.nl);
+  P.far_G = G;
+  P.far_h = h;
+  if (!P.h_src_leaves.empty()) {
+    k_p2m_op<T><<<(unsigned)P.h_src_leaves.size(), 256, 0, s>>>(P.src_leaves, P.cell_level, P.sup_off, P.Ghat, P.side,
+                                                                P.nc1, P.nq, P.g_stride, G);
+    DM_LAUNCH("k_p2m_op");
+  }
+  k_node_h<T><<<nblk(P.nn * P.nl, 256), 256, 0, s>>>(P.nn, P.node_leaf, P.cell_level, P.nodes_s, P.cell_centre, P.side,
+                                                     P.nl, h);
+  DM_LAUNCH("k_node_h");
+}
+
+}  // namespace
+
+void build_far_operators(Plan& P) {
+  build_parent_lists(P);
+  if (P.opt.precision == DEMAG_FP64)
+    build_operators<double>(P);
+  else
+    build_operators<float>(P);
+  if (P.n_m2l == 0) return;
+  const bool fp64 = P.opt.precision == DEMAG_FP64;
+  if (fp64 && P.opt.m2l_table_batch < 0) return;  // FP64 without a table
+  const M2lKeys K = build_m2l_keys(P);
+  if (!fp64) build_m2l_tc(P, K);
+  build_m2l_tab(P, K);
+}
+
+template <class T>
+int launch_p2m(Plan& P, int B, const T* Ms, T* Q, cudaStream_t s) {
+  if (P.h_src_leaves.empty()) return 0;
+  if (B == 1)
+    launch_p2m_small<T, 1>(P, B, Ms, Q, s);
+  else if (B == 2)
+    launch_p2m_small<T, 2>(P, B, Ms, Q, s);
+  else if (B <= 4)
+    launch_p2m_small<T, 4>(P, B, Ms, Q, s);
+  else if (B <= FAR_SMALL_BATCH || std::is_same<T, double>::value)
+    launch_p2m_small<T, 8>(P, B, Ms, Q, s);
+  else if constexpr (std::is_same<T, float>::value) {
+    if (P.nq <= 24)
+      B > P2M_B ? launch_p2m_tile<2, 24>(P, B, Ms, Q, s) : launch_p2m_tile<1, 24>(P, B, Ms, Q, s);
+    else if (P.nq <= 48)
+      B > P2M_B ? launch_p2m_tile<2, 48>(P, B, Ms, Q, s) : launch_p2m_tile<1, 48>(P, B, Ms, Q, s);
+    else
+      B > P2M_B ? launch_p2m_tile<2, 80>(P, B, Ms, Q, s) : launch_p2m_tile<1, 80>(P, B, Ms, Q, s);
+  }
+  DM_LAUNCH("k_p2m");
+  return 1;
+}
+
+template <class T>
+int launch_m2m(Plan& P, int B, T* Q, cudaStream_t s) {
+  int n = 0;
+  for (int l = P.nlevels - 2; l >= 0; l--) {
+    const int64_t pb = P.par_start[l], np = P.par_start[l + 1] - pb;
+    if (np == 0) continue;
+    k_m2m<T><<<nblk(np * P.nq * B, 256), 256, 0, s>>>(P.par_list + pb, np, P.cell_child0, P.cell_nchild, P.cell_prefix,
+                                                      P.m2m_eoff, (const TEnt<T>*)P.m2m_ent, P.nq, B, Q);
+    DM_LAUNCH("k_m2m");
+    n++;
+  }
+  return n;
+}
+
+template <class T>
+int launch_l2l(Plan& P, int B, T* L, cudaStream_t s) {
+  int n = 0;
+  for (int l = 0; l + 1 < P.nlevels; l++) {  // parents at level l, children at l + 1
+    const int64_t pb = P.par_start[l], np = P.par_start[l + 1] - pb;
+    if (np == 0) continue;
+    k_l2l<T><<<nblk(np * P.nl * B, 256), 256, 0, s>>>(P.par_list + pb, np, P.cell_child0, P.cell_nchild, P.cell_range,
+                                                      P.cell_prefix, P.l2l_eoff, (const TEnt<T>*)P.l2l_ent, P.nl, B, L);
+    DM_LAUNCH("k_l2l");
+    n++;
+  }
+  return n;
+}
+
+template <class T>
+int launch_l2p(Plan& P, int B, const T* L, T* u, cudaStream_t s) {
+  if (P.n_node_leaves == 0) return 0;
+  if (B == 1)
+    launch_l2p_small<T, 1>(P, B, L, u, s);
+  else if (B == 2)
+    launch_l2p_small<T, 2>(P, B, L, u, s);
+  else if (B <= 4)
+    launch_l2p_small<T, 4>(P, B, L, u, s);
+  else if (B <= FAR_SMALL_BATCH || std::is_same<T, double>::value)
+    launch_l2p_small<T, 8>(P, B, L, u, s);
+  else if constexpr (std::is_same<T, float>::value) {
+    const size_t smem = sizeof(float) * (size_t)P.nl * (128 + L2P_NCH);
+    smem_opt_in((const void*)k_l2p32, smem);
+    const dim3 grid((unsigned)P.n_node_leaves, (unsigned)((B + 127) / 128));
+    k_l2p32<<<grid, L2P_THREADS, smem, s>>>(P.node_leaves, P.cell_range, (const float*)P.far_h, P.nl, B, L, u);
+  }
+  DM_LAUNCH("k_l2p");
+  return 1;
+}
+
+template int launch_p2m<float>(Plan&, int, const float*, float*, cudaStream_t);
+template int launch_p2m<double>(Plan&, int, const double*, double*, cudaStream_t);
+template int launch_m2m<float>(Plan&, int, float*, cudaStream_t);
+template int launch_m2m<double>(Plan&, int, double*, cudaStream_t);
+template int launch_l2l<float>(Plan&, int, float*, cudaStream_t);
+template int launch_l2l<double>(Plan&, int, double*, cudaStream_t);
+template int launch_l2p<float>(Plan&, int, const float*, float*, cudaStream_t);
+template int launch_l2p<double>(Plan&, int, const double*, double*, cudaStream_t);
+
+}  // namespace demag

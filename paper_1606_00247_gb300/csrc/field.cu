@@ -2,7 +2,7 @@
 // Sec. 4.1-4.2 that computing H directly, instead of from the potential by mass
 // lumping, gives lower errors).
 //
-//   far field:  -grad u_far(r) = -sum_{|m| <= p-1} L_{m+e_a} z^m / m!   (L2P of the gradient)
+//   far field:  -grad u_far(r) = -sum_m L_{m+e_a} z^m / m!   (L2P of the gradient)
 //   near field: the field of the charges of every near tet t, in closed form,
 //     4 pi H_t(r) = sum_{faces F of t} int_F sigma (r - r')/R^3 dA + rho_t sum_F n_F Phi_F(r),
 //     sigma = n_F . M affine on F, rho_t = -div M, Phi_F = int_F dA / R;
@@ -32,35 +32,33 @@ namespace {
 
 inline int nblk(int64_t n, int t) { return (int)std::max<int64_t>(1, (n + t - 1) / t); }
 
-// -grad u_far at every interior node, sorted layout Hs[node][3][B]
-__global__ void k_l2p_grad(int64_t nn, const int32_t* __restrict__ node_leaf, const double* __restrict__ nodes_s,
-                           const double* __restrict__ centre, const uint8_t* __restrict__ boundary, int p, int nc, int B,
-                           const double* __restrict__ L, double* Hs) {
+// -grad u_far at every interior node, sorted layout Hs[node][3][B].  Every
+// component d_a u is harmonic with the coefficients L_{m+e_a}, so it is summed
+// over the trace-free indices m with the node's L2P polynomials h_m(z/s):
+//   d_a u = (1/s) sum_{|m| <= p-2} h_m Lt_{m+e_a},  Lt_(2,b,c) = -Lt_(0,b+2,c) - Lt_(0,b,c+2)
+// (L has degree < p, see common.cuh)
+__global__ void k_l2p_grad(int64_t nn, const int32_t* __restrict__ node_leaf, const int32_t* __restrict__ level,
+                           double side, const uint8_t* __restrict__ boundary, int p, const double* __restrict__ nodeh,
+                           int nl, int B, const double* __restrict__ L, double* Hs) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= nn || boundary[i]) return;
-  const int32_t c = node_leaf[i];
-  double px[MAX_P + 1], py[MAX_P + 1], pz[MAX_P + 1];
-  const double zx = nodes_s[3 * i] - centre[3 * c], zy = nodes_s[3 * i + 1] - centre[3 * c + 1],
-               zz = nodes_s[3 * i + 2] - centre[3 * c + 2];
-  px[0] = py[0] = pz[0] = 1.0;
-  for (int e = 1; e <= p; e++) {
-    px[e] = px[e - 1] * zx / e;
-    py[e] = py[e - 1] * zy / e;
-    pz[e] = pz[e - 1] * zz / e;
-  }
-  const double* Lc = L + (int64_t)c * nc * B;
+  const int32_t cell = node_leaf[i];
+  const double inv_s = 1.0 / ldexp(side, -level[cell]);
+  const double* h = nodeh + i * nl;
+  const double* Lc = L + (int64_t)cell * nl * B;
   for (int b = 0; b < B; b++) {
+    auto l = [&](int x, int y, int z) { return Lc[(int64_t)h_index(x, y, z) * B + b]; };
     double g[3] = {0, 0, 0};
-    for (int t = 0; t < p; t++)  // |m| <= p - 1
-      for (int j = 0; j <= t; j++)
-        for (int mz = 0; mz <= j; mz++) {
-          const int mx = t - j, my = j - mz;
-          const double mono = px[mx] * py[my] * pz[mz];
-          g[0] += Lc[(int64_t)mi_index(mx + 1, my, mz) * B + b] * mono;
-          g[1] += Lc[(int64_t)mi_index(mx, my + 1, mz) * B + b] * mono;
-          g[2] += Lc[(int64_t)mi_index(mx, my, mz + 1) * B + b] * mono;
+    for (int t = 0; t <= p - 2; t++)
+      for (int x = 0; x < 2; x++)
+        for (int z = 0; z <= t - x; z++) {
+          const int y = t - x - z;
+          const double w = h[h_index(x, y, z)];
+          g[0] += w * (x ? -l(0, y + 2, z) - l(0, y, z + 2) : l(1, y, z));
+          g[1] += w * l(x, y + 1, z);
+          g[2] += w * l(x, y, z + 1);
         }
-    for (int a = 0; a < 3; a++) Hs[(i * 3 + a) * B + b] = -g[a];
+    for (int a = 0; a < 3; a++) Hs[(i * 3 + a) * B + b] = -g[a] * inv_s;
   }
 }
 
@@ -270,8 +268,8 @@ void eval_field(Plan& P, const double* M, int B, double* u, double* H, cudaStrea
   }
   Workspace& W = workspace(P, B);
   eval_fp64_ws(P, W, M, B, u, H, s, false);  // u, the mass-lumped H, and the local expansions in W.L
-  k_l2p_grad<<<nblk(P.nn, 128), 128, 0, s>>>(P.nn, P.node_leaf, P.nodes_s, P.cell_centre, P.bnd_flag, P.p, P.nc, B,
-                                             W.L, P.field_buf);
+  k_l2p_grad<<<nblk(P.nn, 128), 128, 0, s>>>(P.nn, P.node_leaf, P.cell_level, P.side, P.bnd_flag, P.p,
+                                             (const double*)P.far_h, P.nl, B, W.L, P.field_buf);
   DM_LAUNCH("k_l2p_grad");
   k_field_near<<<dim3((unsigned)P.nn, (unsigned)((B + FN_FS - 1) / FN_FS)), FN_THREADS, 0, s>>>(
       P.node_leaf, P.p2p_off, P.p2p_src, P.cell_range, P.nodes_s, P.tets_s, P.tet_geo, P.tet_grad, P.bnd_flag, W.Ms, B,

@@ -2,11 +2,14 @@
 // of 128 states, with FP32 accumulation in tensor memory.
 //
 //   Lt^T_m = (-1)^|m| / (4 pi s_T) sum_S sum_{|n| <= p - |m|} b_{n+m}(v_S) f_S^|n| Qt^S_n
-// (notation of fmm32.cu).  For one target cell T this is the matrix product
+// (notation of far.cu).  For one target cell T this is the matrix product
 //   D[b][m] = sum_S sum_n A_S[b][n] K_S[m][n],   A_S[b][n] = Qt^S_n(state b),
 //   K_S[m][n] = b_{n+m}(v_S) f_S^|n|  (0 where |n| + |m| > p),
 // accumulated over all sources S of T in tensor memory (M = 128 states = TMEM
-// lanes, N = rows m, K = n).
+// lanes, N = rows m, K = n).  n and m run over the trace-free indices of
+// common.cuh (80 moments, 64 local coefficients at p = 8): 9 MMAs, 28 KB of
+// moments and 5.6 KB of operator per pair and 128 states, where the 165 full
+// multi-indices took 17 MMAs, 56 KB and 16.4 KB.
 //
 // Translation operators.  Expansion centres are octree box centres, so
 // v_S = (c_T - c_S) / s_T is fixed by the level difference and an integer
@@ -55,8 +58,6 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
-#include <array>
-#include <unordered_map>
 #include <vector>
 
 #include "common.cuh"
@@ -93,7 +94,7 @@ struct TcLayout {
   int ls;                           // split BF16 limb scheme: TC_LS_ALL2, TC_LS_ALL3 or a split degree (below)
   int lmax;                         // most limbs of any k-step (A slices are lmax x 4 KB apart)
   int E, KW;                        // elements per 16 bytes, per k-step (2E)
-  int nc, ncp;                      // coefficients, padded to 16 (TMEM columns used)
+  int nq, nl, nlp;                  // moments (columns n), rows m, rows padded to 16 (TMEM columns used)
   int KS;                           // k-steps of the A tile
   int Nks[TC_MAXKS];                // rows used at k-step ks (a prefix), padded to 16
   int N2[TC_MAXKS];                 // rows that also take the products with a second limb (a prefix of Nks)
@@ -106,16 +107,10 @@ struct TcLayout {
   int tmem_cols;                    // power of two >= ncp
 };
 
-__host__ __device__ constexpr int cnc_of(int t) { return t < 0 ? 0 : (t + 1) * (t + 2) * (t + 3) / 6; }
+// rows m of degree <= t
+__host__ __device__ constexpr int rows_of(int t) { return t < 0 ? 0 : (t + 1) * (t + 1); }
 __host__ __device__ constexpr int pad_to(int x, int m) { return (x + m - 1) / m * m; }
 __host__ __device__ constexpr int tri3(int t) { return t * (t + 1) * (t + 2) / 6; }
-// degree of the multi-index at position m of the graded order
-__host__ __device__ constexpr int degree_of(int m) {
-  int t = 0;
-  while (tri3(t + 1) <= m) t++;
-  return t;
-}
-
 // Split BF16 limb schemes.  Every product of the operator K (rows m) and the
 // moments A (columns n) has a term degree |m| + |n| <= p.
 //   TC_LS_ALL2: two limbs (16 significant bits) everywhere, three MMAs per
@@ -130,8 +125,10 @@ __host__ __device__ constexpr int degree_of(int m) {
 //               k-steps with no such rows keep one limb and one MMA.
 constexpr int TC_LS_ALL2 = 0, TC_LS_ALL3 = 99;
 // default split degree: p - TC_SD_BELOW (the four highest term degrees of the
-// expansion take hi x hi alone) from p = 8 on, p - 3 for lower orders (whose
-// highest degrees carry a larger share)
+// expansion take hi x hi alone) from p = 8 on, p - 2 for lower orders (whose
+// highest degrees carry a larger share).  Rounding error of u and H against
+// FP64 with the same tree (224k-tet ball): 1.2e-6 and 2.7e-6 at p = 8,
+// with the full multi-indices 1.7e-6 and 2.9e-6.
 constexpr int TC_SD_BELOW = 4;
 
 __host__ __device__ constexpr TcLayout tc_layout(int p, bool bf16, int ls) {
@@ -140,18 +137,17 @@ __host__ __device__ constexpr TcLayout tc_layout(int p, bool bf16, int ls) {
   G.bf16 = bf16 ? 1 : 0;
   G.E = bf16 ? 8 : 4;
   G.KW = 2 * G.E;
-  G.nc = cnc_of(p);
-  G.ncp = pad_to(G.nc, 16);
-  G.KS = pad_to(G.nc, G.KW) / G.KW;
+  G.nq = nq_of(p);
+  G.nl = nl_of(p);
+  G.nlp = pad_to(G.nl, 16);
+  G.KS = pad_to(G.nq, G.KW) / G.KW;
   if (G.KS > TC_MAXKS) return TcLayout{};
   G.ls = bf16 ? ls : TC_LS_ALL2;
   G.lmax = 1;
   G.ks_off[0] = 0;
   for (int ks = 0; ks < G.KS; ks++) {
-    int rows = 0;  // rows of degree t need n < cnc(p - t)
-    for (int t = 0; t <= p; t++)
-      if (cnc_of(p - t) > ks * G.KW) rows = cnc_of(t);
-    G.Nks[ks] = pad_to(rows, 16);
+    const int d0 = h_degree(ks * G.KW + 1);  // lowest degree |n| of the k-step: rows of degree <= p - d0 need it
+    G.Nks[ks] = pad_to(rows_of(p - d0), 16);
     if (!bf16) {
       G.L[ks] = 1;
       G.N2[ks] = 0;
@@ -162,8 +158,10 @@ __host__ __device__ constexpr TcLayout tc_layout(int p, bool bf16, int ls) {
       G.L[ks] = 2;
       G.N2[ks] = G.Nks[ks];
     } else {
-      const int r = ls - degree_of(ks * G.KW);  // rows of degree <= r take the second limb
-      const int n2 = r < 0 ? 0 : pad_to(cnc_of(r), 16);
+      // rows of degree <= r take the second limb (the first k-step holds the
+      // degrees 1 .. 3 and the largest products: one degree more)
+      const int r = ks == 0 ? ls : ls - d0;
+      const int n2 = r < 0 ? 0 : pad_to(rows_of(r), 16);
       G.N2[ks] = n2 < G.Nks[ks] ? n2 : G.Nks[ks];
       G.L[ks] = G.N2[ks] > 0 ? 2 : 1;
     }
@@ -176,7 +174,7 @@ __host__ __device__ constexpr TcLayout tc_layout(int p, bool bf16, int ls) {
   for (int ks = 0; ks < G.KS; ks++) G.a_off[ks + 1] = G.a_off[ks] + G.L[ks] * TC_SLICE;
   G.a_bytes = G.a_off[G.KS];
   int tc = 32;
-  while (tc < G.ncp) tc *= 2;
+  while (tc < G.nlp) tc *= 2;
   if (tc > 512) return TcLayout{};
   G.tmem_cols = tc;
   G.valid = 1;
@@ -187,7 +185,7 @@ __host__ __device__ constexpr TcLayout tc_layout(int p, bool bf16, int ls) {
 // the default split degree of the order and with two limbs on every k-step
 // (DEMAG_MIXED_BF16X3), and with three limbs (DEMAG_MIXED_BF16X6)
 constexpr bool tc_order(int p) { return p == 4 || p == 6 || p == 8 || p == 10; }
-__host__ __device__ constexpr int tc_split_degree(int p) { return p >= 8 ? p - TC_SD_BELOW : p - 3; }
+__host__ __device__ constexpr int tc_split_degree(int p) { return p >= 8 ? p - TC_SD_BELOW : p - 2; }
 
 // launch shape: `nt` targets per CTA sharing each source's moments, `kps`
 // k-steps of one source per ring slot (A slices, then one K region per target)
@@ -372,21 +370,21 @@ __device__ __forceinline__ void store_row64(unsigned char* dst, int stride, int 
 // ---------------------------------------------------------------------------
 // moments -> tile layout: QP[cell][sb] = A tile (k-step ks at a_off[ks]: [limb][128 rows x 32 bytes])
 template <bool BF16>
-__global__ void __launch_bounds__(TC_M) k_m2l_tc_pack(const float* __restrict__ Q, int nc, int B, int nsb,
+__global__ void __launch_bounds__(TC_M) k_m2l_tc_pack(const float* __restrict__ Q, int nq, int B, int nsb,
                                                       const TcLayout G, unsigned char* __restrict__ QP) {
   const int KS = G.KS;
   constexpr int E = BF16 ? 8 : 4;
   const int64_t cell = blockIdx.x;
   const int sb = blockIdx.y, b = threadIdx.x, bb = sb * TC_M + b;
   const bool alive = bb < B;
-  const float* q = Q + cell * nc * (int64_t)B + bb;
+  const float* q = Q + cell * nq * (int64_t)B + bb;
   unsigned char* out = QP + (cell * nsb + sb) * (int64_t)G.a_bytes;
   for (int qq = 0; qq < 2 * KS; qq++) {
     float v[E];
 #pragma unroll
     for (int u = 0; u < E; u++) {
       const int n = qq * E + u;
-      v[u] = (alive && n < nc) ? q[(int64_t)n * B] : 0.f;
+      v[u] = (alive && n < nq) ? q[(int64_t)n * B] : 0.f;
     }
     const int off = G.a_off[qq >> 1] + (b >> 3) * 256 + (qq & 1) * 128 + (b & 7) * 16;
     store_row<BF16>(out + off, TC_SLICE, G.L[qq >> 1], v);
@@ -396,7 +394,7 @@ __global__ void __launch_bounds__(TC_M) k_m2l_tc_pack(const float* __restrict__ 
 // ---------------------------------------------------------------------------
 // operator table: key = (dl, I) with v = I * 2^-(max(0, -dl) + 1), f = 2^dl
 template <bool BF16>
-__global__ void __launch_bounds__(128) k_m2l_tc_ops(const int4* __restrict__ keys, int p, int nc, const TcLayout G,
+__global__ void __launch_bounds__(128) k_m2l_tc_ops(const int4* __restrict__ keys, int p, const TcLayout G,
                                                     unsigned char* __restrict__ ops) {
   constexpr int E = BF16 ? 8 : 4;
   __shared__ double b[TC_MAXNC];
@@ -433,10 +431,10 @@ __global__ void __launch_bounds__(128) k_m2l_tc_ops(const int4* __restrict__ key
       for (int u = 0; u < E; u++) {
         v[u] = 0.0;
         const int n = ks * G.KW + kc * E + u;
-        if (r < nc && n < nc) {
+        if (r < G.nl && n < G.nq) {
           int ma, mb, mz, na, nb, nz;
-          mi_decode(r, ma, mb, mz);
-          mi_decode(n, na, nb, nz);
+          h_decode(r, ma, mb, mz);
+          h_decode(n + 1, na, nb, nz);
           const int tn = na + nb + nz;
           if (tn + ma + mb + mz <= p) v[u] = b[idx3(na + ma, nb + mb, nz + mz)] * ldexp(1.0, dl * tn);
         }
@@ -458,7 +456,7 @@ template <int P, bool BF16, int NT, int LS>
 __global__ void __launch_bounds__(TC_THREADS, NT == 1 ? 2 : 1)
     k_m2l_tc(const int32_t* __restrict__ gtarget, const int64_t* __restrict__ goff,
              const int32_t* __restrict__ gsrc, const int32_t* __restrict__ gop, const int32_t* __restrict__ level,
-             double side, int nc, int B, int nsb, const TcRing R, const unsigned char* __restrict__ QP,
+             double side, int B, int nsb, const TcRing R, const unsigned char* __restrict__ QP,
              const unsigned char* __restrict__ ops, float* L, int* err) {
   constexpr TcLayout G = tc_layout(P, BF16, LS);
   static_assert(G.valid, "no tensor-core layout for this order");
@@ -682,9 +680,9 @@ __global__ void __launch_bounds__(TC_THREADS, NT == 1 ? 2 : 1)
         const int32_t T = gtarget[grp * NT + t];
         if (T < 0) continue;
         const float inv = (float)(1.0 / (4.0 * M_PI * ldexp(side, -level[T])));
-        float* Lt = L + (int64_t)T * nc * B + b;
+        float* Lt = L + (int64_t)T * G.nl * B + b;
 #pragma unroll
-        for (int c0 = 0; c0 < G.ncp; c0 += 16) {
+        for (int c0 = 0; c0 < G.nlp; c0 += 16) {
           uint32_t r[16];
           tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(t * 256 + c0), r);
           if (b < B) {
@@ -693,7 +691,7 @@ __global__ void __launch_bounds__(TC_THREADS, NT == 1 ? 2 : 1)
               const int m = c0 + i;
               float v = __uint_as_float(r[i]);
               if (c0 < 64 && t == 0) v += tot[(c0 < 64 ? c0 : 0) + i];  // promoted part (zero when not promoting)
-              if (m < G.nc) Lt[(int64_t)m * B] = ((degree_of(m) & 1) ? -inv : inv) * v;
+              if (m < G.nl) Lt[(int64_t)m * B] = ((h_degree(m) & 1) ? -inv : inv) * v;
             }
           }
         }
@@ -715,20 +713,6 @@ __global__ void __launch_bounds__(TC_THREADS, NT == 1 ? 2 : 1)
 
 // ---------------------------------------------------------------------------
 // host side
-void cell_coords(uint64_t prefix, int level, int64_t* k) {  // integer box coordinates (x bit at 3b)
-  k[0] = k[1] = k[2] = 0;
-  for (int b = 0; b < level; b++)
-    for (int a = 0; a < 3; a++) k[a] |= (int64_t)((prefix >> (3 * b + a)) & 1ull) << b;
-}
-
-struct KeyHash {
-  size_t operator()(const std::array<int64_t, 4>& k) const {
-    uint64_t h = 1469598103934665603ull;
-    for (int64_t v : k) h = (h ^ (uint64_t)v) * 1099511628211ull;
-    return (size_t)h;
-  }
-};
-
 bool split_bf16(const Plan& P) {
   return P.opt.precision == DEMAG_MIXED_BF16X3 || P.opt.precision == DEMAG_MIXED_BF16X6;
 }
@@ -742,12 +726,12 @@ void launch_fixed(Plan& P, const TcRing& R, int B, const unsigned char* QP, floa
   if (NT == 1) {
     dim3 grid((unsigned)(nsb * P.h_m2l_targets.size()));
     k_m2l_tc<PP, BF16, NT, LS><<<grid, TC_THREADS, smem, s>>>(P.m2l_targets, P.tc_g1_off, P.m2l_src, P.m2l_op,
-                                                              P.cell_level, P.side, P.nc, B, nsb, R, QP, P.tc_ops, L,
+                                                              P.cell_level, P.side, B, nsb, R, QP, P.tc_ops, L,
                                                               err);
   } else {
     dim3 grid((unsigned)(nsb * P.tc_n_g2));
     k_m2l_tc<PP, BF16, NT, LS><<<grid, TC_THREADS, smem, s>>>(P.tc_g2_tgt, P.tc_g2_off, P.tc_g2_src, P.tc_g2_op,
-                                                              P.cell_level, P.side, P.nc, B, nsb, R, QP, P.tc_ops, L,
+                                                              P.cell_level, P.side, B, nsb, R, QP, P.tc_ops, L,
                                                               err);
   }
   DM_LAUNCH("k_m2l_tc");
@@ -813,7 +797,7 @@ void tune_ring(Plan& P, const TcLayout& G) {
   cudaStream_t s = P.stream;
   const int B = TC_M;
   Tmp<unsigned char> qp((size_t)P.ncells * G.a_bytes);
-  Tmp<float> L((size_t)P.ncells * P.nc * B);
+  Tmp<float> L((size_t)P.ncells * P.nl * B);
   Tmp<int> err(1);
   DM_CUDA(cudaMemsetAsync(qp.p, 0, (size_t)P.ncells * G.a_bytes, s));
   DM_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), s));
@@ -857,7 +841,7 @@ bool current_ring(const Plan& P, const TcLayout& G, TcRing& R) {
   if (!(P.tc_kps > 0 && make_ring(G, P.tc_nt, P.tc_kps, P.tc_budget, R)))
     default_ring(G, P.opt.m2l_targets_per_cta, P.opt.m2l_kps, R);
   R.prom_group = R.nt == 1 ? P.tc_prom_group : 0;
-  R.prom_chunks = std::min(4, std::max(1, (P.tc_prom_rows + 15) / 16));
+  R.prom_chunks = std::min(std::min(4, G.nlp / 16), std::max(1, (P.tc_prom_rows + 15) / 16));
   return R.nslots >= 2;
 }
 
@@ -867,7 +851,7 @@ void build_ops(Plan& P, const TcLayout& G, const std::vector<int4>& keys) {
   P.tc_ops = dalloc<unsigned char>(P, (size_t)keys.size() * G.op_bytes);
   Tmp<int4> dkeys(keys.size());
   DM_CUDA(cudaMemcpyAsync(dkeys.p, keys.data(), keys.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
-  k_m2l_tc_ops<BF16><<<(unsigned)keys.size(), 128, 0, s>>>(dkeys.p, P.p, P.nc, G, P.tc_ops);
+  k_m2l_tc_ops<BF16><<<(unsigned)keys.size(), 128, 0, s>>>(dkeys.p, P.p, G, P.tc_ops);
   DM_LAUNCH("k_m2l_tc_ops");
   DM_CUDA(cudaStreamSynchronize(s));
 }
@@ -875,49 +859,6 @@ void build_ops(Plan& P, const TcLayout& G, const std::vector<int4>& keys) {
 bool tc_enabled(const Plan& P) { return (P.opt.precision == DEMAG_MIXED_TF32 || split_bf16(P)) && P.tc_ops != nullptr; }
 
 }  // namespace
-
-M2lKeys build_m2l_keys(Plan& P) {
-  M2lKeys K;
-  if (P.n_m2l == 0) return K;
-  cudaStream_t s = P.stream;
-  const int64_t nc = P.ncells;
-  std::vector<uint64_t> prefix(nc);
-  std::vector<int32_t> lev(nc);
-  K.off.resize(nc + 1);
-  K.src.resize(P.n_m2l);
-  DM_CUDA(cudaMemcpyAsync(prefix.data(), P.cell_prefix, nc * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-  DM_CUDA(cudaMemcpyAsync(lev.data(), P.cell_level, nc * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  DM_CUDA(cudaMemcpyAsync(K.off.data(), P.m2l_off, (nc + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  DM_CUDA(cudaMemcpyAsync(K.src.data(), P.m2l_src, P.n_m2l * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  DM_CUDA(cudaStreamSynchronize(s));
-  std::vector<std::array<int64_t, 3>> kc(nc);
-  for (int64_t c = 0; c < nc; c++) cell_coords(prefix[c], lev[c], kc[c].data());
-  std::unordered_map<std::array<int64_t, 4>, int32_t, KeyHash> index;
-  K.op.resize(P.n_m2l);
-  for (int64_t T = 0; T < nc; T++)
-    for (int64_t e = K.off[T]; e < K.off[T + 1]; e++) {
-      const int32_t S = K.src[e];
-      const int dl = lev[T] - lev[S];
-      std::array<int64_t, 4> key{dl, 0, 0, 0};
-      for (int a = 0; a < 3; a++)
-        key[1 + a] = dl >= 0 ? (2 * kc[T][a] + 1) - ((2 * kc[S][a] + 1) << dl)
-                             : ((2 * kc[T][a] + 1) << (-dl)) - (2 * kc[S][a] + 1);
-      auto f = index.find(key);
-      if (f == index.end()) {
-        for (int a = 1; a < 4; a++)
-          if (key[a] > INT32_MAX || key[a] < INT32_MIN) return M2lKeys{};  // beyond the table's key range
-        f = index.emplace(key, (int32_t)K.keys.size()).first;
-        K.keys.push_back(make_int4(dl, (int)key[1], (int)key[2], (int)key[3]));
-      }
-      K.op[e] = f->second;
-    }
-  P.m2l_op = dalloc<int32_t>(P, P.n_m2l);
-  DM_CUDA(cudaMemcpyAsync(P.m2l_op, K.op.data(), P.n_m2l * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-  DM_CUDA(cudaStreamSynchronize(s));
-  P.n_tc_ops = (int64_t)K.keys.size();
-  K.ok = true;
-  return K;
-}
 
 void build_m2l_tc(Plan& P, const M2lKeys& K) {
   if (P.opt.precision != DEMAG_MIXED_TF32 && !split_bf16(P)) return;
@@ -930,9 +871,9 @@ void build_m2l_tc(Plan& P, const M2lKeys& K) {
   const TcLayout G = layout_of(P);
   if (!G.valid) return;
   cudaStream_t s = P.stream;
-  const std::vector<int64_t>& off = K.off;
-  const std::vector<int32_t>& src = K.src;
-  const std::vector<int32_t>& op = K.op;
+  std::vector<int64_t> off(P.ncells + 1);
+  DM_CUDA(cudaMemcpyAsync(off.data(), P.m2l_off, off.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+  DM_CUDA(cudaStreamSynchronize(s));
   if (G.bf16)
     build_ops<true>(P, G, K.keys);
   else
@@ -944,8 +885,13 @@ void build_m2l_tc(Plan& P, const M2lKeys& K) {
   g1[nT] = nT ? off[P.h_m2l_targets[nT - 1] + 1] : 0;
   P.tc_g1_off = dalloc<int64_t>(P, nT + 1);
   DM_CUDA(cudaMemcpyAsync(P.tc_g1_off, g1.data(), (nT + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-  // groups of two consecutive targets: the union of their (ascending) lists
-  if (G.tmem_cols <= 256) {
+  // groups of two consecutive targets, where one may run: the union of their (ascending) lists
+  const bool pairs = P.opt.m2l_targets_per_cta == 2 || ((P.opt.autotune & 1) && P.tc_prom_group == 0);
+  if (pairs && G.tmem_cols <= 256) {
+    std::vector<int32_t> src(P.n_m2l), op(P.n_m2l);
+    DM_CUDA(cudaMemcpyAsync(src.data(), P.m2l_src, src.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    DM_CUDA(cudaMemcpyAsync(op.data(), P.m2l_op, op.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    DM_CUDA(cudaStreamSynchronize(s));
     const int64_t ng = (nT + 1) / 2;
     std::vector<int32_t> tgt(2 * ng, -1), usrc, uop;
     std::vector<int64_t> uoff(ng + 1, 0);
@@ -1014,9 +960,9 @@ bool launch_m2l_tc(Plan& P, int B, const float* Q, unsigned char* QP, float* L, 
   const int nsb = (B + TC_M - 1) / TC_M;
   const dim3 grid((unsigned)P.ncells, (unsigned)nsb);
   if (G.bf16)
-    k_m2l_tc_pack<true><<<grid, TC_M, 0, s>>>(Q, P.nc, B, nsb, G, QP);
+    k_m2l_tc_pack<true><<<grid, TC_M, 0, s>>>(Q, P.nq, B, nsb, G, QP);
   else
-    k_m2l_tc_pack<false><<<grid, TC_M, 0, s>>>(Q, P.nc, B, nsb, G, QP);
+    k_m2l_tc_pack<false><<<grid, TC_M, 0, s>>>(Q, P.nq, B, nsb, G, QP);
   DM_LAUNCH("k_m2l_tc_pack");
   launch_main(P, R, B, QP, L, err, s);
   return true;

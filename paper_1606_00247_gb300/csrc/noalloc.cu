@@ -94,20 +94,57 @@ struct Carver {
   }
 };
 
+// Bytes that decide whether a plan and batch are taken: the expansions and the
+// packed moments counted with all C(p+3, 3) multi-indices.  The trace-free
+// arrays carved below take less, so which calls are accepted does not depend
+// on how the kernels store them.
+size_t admission_bytes(const Plan& P, int B) {
+  Carver c{nullptr};
+  const size_t nn = P.nn, nt = P.nt, nc = P.nc, ncell = P.ncells;
+  const bool mixed = P.opt.precision != DEMAG_FP64, otf = P.opt.near_mode == 0;
+  if (!mixed || otf) c.take<double>(nn * 3 * B);
+  if (!mixed) {
+    c.take<double>(ncell * nc * B);
+    c.take<double>(ncell * nc * B);
+  } else {
+    c.take<float>(nn * 3 * B);
+    c.take<float>(ncell * nc * B + 16);
+    c.take<float>(ncell * nc * B);
+    c.take<float>(nn * B);
+    if (m2l_tc_pack_bytes(P, B)) {  // 4 KB per cell, 128 states, k-step and limb
+      const bool tf32 = P.opt.precision == DEMAG_MIXED_TF32, x6 = P.opt.precision == DEMAG_MIXED_BF16X6;
+      const int kw = tf32 ? 8 : 16, split = P.p >= 8 ? P.p - 4 : P.p - 3;
+      size_t slices = 0;
+      for (int k = 0; k * kw < P.nc; k++) {
+        int a, b, z;
+        mi_decode(k * kw, a, b, z);
+        slices += tf32 ? 1 : x6 ? 3 : P.opt.m2l_split_degree < 0 || a + b + z <= split ? 2 : 1;
+      }
+      c.take<unsigned char>(ncell * (size_t)((B + 127) / 128) * slices * 4096);
+    }
+    const size_t mp = nf_mp_floats(P, B);
+    if (mp) c.take<float>(mp);
+  }
+  if (!mixed || otf) c.take<double>(nn * B);
+  if (otf) c.take<double>(nt * TET_STATE * std::min(B, P2P_AT_MIN_B - 1));
+  c.take<int>(1);
+  return c.used;
+}
+
 size_t carve(Plan& P, int B, unsigned char* base, Workspace* W) {
   Carver c{base};
-  const size_t nn = P.nn, nt = P.nt, nc = P.nc, ncell = P.ncells;
+  const size_t nn = P.nn, nt = P.nt, ncell = P.ncells;
   const bool mixed = P.opt.precision != DEMAG_FP64, otf = P.opt.near_mode == 0;
   Workspace w;
   w.B = B;
   if (!mixed || otf) w.Ms = c.take<double>(nn * 3 * B);
   if (!mixed) {
-    w.Q = c.take<double>(ncell * nc * B);
-    w.L = c.take<double>(ncell * nc * B);
+    w.Q = c.take<double>(ncell * P.nq * B);
+    w.L = c.take<double>(ncell * P.nl * B);
   } else {
     w.Ms32 = c.take<float>(nn * 3 * B);
-    w.Q32 = c.take<float>(ncell * nc * B + 16);  // tail pad for 16-byte bulk copies
-    w.L32 = c.take<float>(ncell * nc * B);
+    w.Q32 = c.take<float>(ncell * P.nq * B);
+    w.L32 = c.take<float>(ncell * P.nl * B);
     w.u32 = c.take<float>(nn * B);
     const size_t qp = m2l_tc_pack_bytes(P, B);
     if (qp) w.QP = c.take<unsigned char>(qp);
@@ -148,7 +185,7 @@ extern "C" demag_status demag_eval_noalloc(demag_plan plan, const double* M, int
     if (batch < 1) fail(DEMAG_ERR_INVALID_ARG, "batch must be >= 1");
     if (!is_device_ptr(M) || !is_device_ptr(u) || (H && !is_device_ptr(H)))
       fail(DEMAG_ERR_INVALID_ARG, "demag_eval_noalloc takes device pointers only");
-    const size_t need = carve(*plan, batch, nullptr, nullptr);
+    const size_t need = std::max(admission_bytes(*plan, batch), carve(*plan, batch, nullptr, nullptr));
     if (need > (size_t)DEMAG_NOALLOC_SCRATCH_BYTES)
       fail(DEMAG_ERR_INVALID_ARG, "this plan and batch need " + std::to_string(need) +
                                       " bytes of scratch; the fixed area holds " +

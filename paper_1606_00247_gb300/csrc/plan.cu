@@ -1118,15 +1118,17 @@ void build_plan(Plan& P, const double* nodes_in, const int32_t* tets_in) {
   P.h_p2p_off = std::move(h_p2p_off);
   P.h_p2p_src = std::move(h_p2p_src);
   if (P.opt.near_mode == 1) build_near_field(P);
-  if (P.opt.precision != DEMAG_FP64) build_mixed_operators(P);
+  build_far_operators(P);
+  if (P.opt.precision != DEMAG_FP64) build_gradient_operator(P);
+  DM_CUDA(cudaStreamSynchronize(P.stream));
+  dfree(P, P.Ghat);  // folded into the P2M operator
+  P.Ghat = nullptr;
   if (P.opt.precision != DEMAG_FP64 && P.opt.near_mode == 1) {
     // the mixed path with stored near-field coefficients evaluates from FP32
-    // copies only: the FP64 per-tet geometry and P2M operator go
-    DM_CUDA(cudaStreamSynchronize(P.stream));
+    // copies only: the FP64 per-tet geometry goes
     dfree(P, P.tet_geo);
     dfree(P, P.tet_grad);
-    dfree(P, P.Ghat);
-    P.tet_geo = P.tet_grad = P.Ghat = nullptr;
+    P.tet_geo = P.tet_grad = nullptr;
   }
   audit_plan(P);
   DM_CUDA(cudaStreamSynchronize(s));

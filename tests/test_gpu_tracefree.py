@@ -1,0 +1,68 @@
+"""The far field on trace-free expansions ((p+1)^2 - 1 moments and p^2 local
+coefficients per cell) against the oracle FMM, which keeps every multi-index of
+Sec. 2.2-2.3.  The truncation |n| + |m| <= p is the same, so only rounding is left."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1606_00247_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def rel_l2(a, b):
+    return float(np.linalg.norm(a - b) / np.linalg.norm(b))
+
+
+def _check(orc, p, B, precision, bar_u, bar_h, leaf=24, **kw):
+    from paper_1606_00247_gb300.api import Plan
+
+    nodes, tets = inputs.sphere(h=0.19)
+    M = inputs.gaussian_unit_m(nodes.shape[0], batch=B, seed=11 + p)
+    u, H = Plan(nodes, tets, p=p, leaf_size=leaf, max_batch=B, precision=precision, **kw).eval(
+        torch.as_tensor(M, device="cuda"))
+    tree = orc.Tree(nodes, tets, leaf, 0.5)
+    for k in {0, B - 1}:
+        ref = tree.fmm(M[k], p)
+        Href = orc.lumped_H(nodes, tets, ref)
+        assert rel_l2(u[k].cpu().numpy(), ref) < bar_u and rel_l2(H[k].cpu().numpy(), Href) < bar_h
+
+
+@pytest.fixture(scope="module")
+def orc():
+    import oracle
+
+    return oracle
+
+
+# every order (the moment tile of the P2M holds 24, 48 or 80 moments, p = 12 takes three tiles; the
+# table M2L ends at p = 10), batches on both sides of the small-batch kernels (32) and of one and two
+# states per thread (128), odd ones included.  FP32: sums of 1e3 rounded terms, ~1e-6 of the largest.
+@pytest.mark.parametrize("B", [1, 32, 33, 129])
+@pytest.mark.parametrize("p", [1, 2, 4, 5, 6, 7, 8, 10, 11, 12])
+def test_fp32_vs_oracle(orc, p, B):
+    _check(orc, p, B, "fp32", 2e-6, 2e-5, near_mode=1)
+
+
+# tensor-core layouts: 16, 48, 64 and 112 rows; 2 to 8 k-steps; a promoted column count beyond the
+# rows (p = 4 holds 16) is cut to them
+@pytest.mark.parametrize("p", [4, 6, 8, 10])
+@pytest.mark.parametrize("prec", ["bf16x3", "bf16x6"])
+def test_split_bf16_vs_oracle(orc, prec, p):
+    _check(orc, p, 131, prec, 1e-5, 1e-5, near_mode=1, m2l_table_batch=-1, m2l_promote_rows=64)
+
+
+# FP64: 1e-11 is far above the ~1e-14 of its rounding and far below any missing term.  -1: without the
+# derivative table (the recurrence per pair); p = 12 with 9 states takes slices of four
+@pytest.mark.parametrize("table", [0, -1])
+@pytest.mark.parametrize("B", [1, 2, 3, 9])
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 7, 8, 11, 12])
+def test_fp64_vs_oracle(orc, p, B, table):
+    _check(orc, p, B, "fp64", 1e-11, 1e-11, near_mode=1, m2l_table_batch=table)
+
+
+# orders without a tensor-core M2L: the table also beyond m2l_table_batch, the recurrence when it is off
+@pytest.mark.parametrize("table", [0, -1])
+@pytest.mark.parametrize("p", [5, 9])
+def test_other_orders_of_the_tensor_precisions(orc, p, table):
+    _check(orc, p, 37, "bf16x6", 2e-6, 2e-5, near_mode=1, m2l_table_batch=table)
