@@ -193,17 +193,13 @@ def live_peaks():
     return peaks
 
 
-# FP64 operations of the on-the-fly near field per (target node, source tet)
-# pair, counted from the source (p2p.cuh, p2p.cu); sqrt, log1p, divisions and
-# atan2 are not counted.
-#  batches of fewer than P2P_AT_MIN_B states, pair_contract per pair and state:
-#   12 subtractions, 4 norms (5 each), 6 edges x 4, 4 faces x (h 5, triple
-#   product 14, 3 dots 15, denominator 7, 3 edges x 14, face combination 12),
-#   M(r) 18  -> 48+24+4*95+18 = 470 per state;
-#  larger batches, pair_at once per pair (12 + 20 + 24 + 1, then 4 faces x
-#   (h 5, triple product 14, 3 dots 15, denominator 8, Om and I 2, 3 edges x 69,
-#   a 12, T 87) = 1457) and 44 per state (M(r) 18, T:J 14, M(r).a + T:J/2 7,
-#   the warp's shuffle sum 5).
+# FP64 operations of the integrated near field per (target node, source tet)
+# pair in the tet-wise form of the method (p2p.cuh: a and T of the pair once,
+# then every state): pair 1457 = 12 + 20 + 24 + 1, then 4 faces x (h 5, triple
+# product 14, 3 dots 15, denominator 8, Om and I 2, 3 edges x 69, a 12, T 87);
+# 44 per state; for one state 470 (the contracted form).  sqrt, log1p, divisions
+# and atan2 are not counted.  The kernel (p2p.cu) shares distances, logarithms
+# and solid angles between the tets of a cluster and executes fewer.
 P2P_AT_MIN_B = 2
 P2P_PAIR_FLOPS, P2P_STATE_FLOPS, P2P_PERSTATE_FLOPS = 1457, 44, 470
 

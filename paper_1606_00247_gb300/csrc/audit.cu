@@ -265,6 +265,17 @@ void audit_plan(Plan& P, bool plant) {
       if (P.w_off32) A.offsets("w_off32", P.w_off32, nT, 0, P.n_wentries / 3 * 4, 0, P.n_wentries / 3 * 4);
     }
   }
+  // integrated near field: clusters and their parts
+  if (P.n_clusters > 0) {
+    const int64_t nT = (int64_t)P.h_p2p_targets.size();
+    A.values("cl_off", P.cl_off, nc + 1, 0, P.n_clusters + 1);
+    A.values("cl_vnode", P.cl_vnode, P.n_cl_v, 0, nn);
+    A.values("cl_ftet", (const int32_t*)P.cl_ftet, 2 * P.n_cl_f, -1, nt);
+    if (P.pc_off) {
+      A.offsets("pc_off", P.pc_off, nT, 0, P.n_pc, 0, P.n_pc);
+      A.values("pc_src", P.pc_src, P.n_pc, 0, P.n_clusters);
+    }
+  }
   // far field: parent lists, M2L operator indices
   A.values("par_list", P.par_list, P.par_start.empty() ? 0 : P.par_start.back(), 0, nc);
   if (P.m2l_op) A.values("m2l_op", P.m2l_op, P.n_m2l, 0, P.n_m2l_keys);

@@ -116,11 +116,8 @@ __host__ __device__ inline double h_fold(int a, int b, int c, F&& f) {
 // faces have the fixed counter-clockwise vertex orders below.
 // ---------------------------------------------------------------------------
 constexpr int TET_GEO = 66;
-// per-tet, per-state record for the on-the-fly near field of small batches
-// (56 doubles):
-//   [0..2] M(v0)  [3..11] J = dM/dx (row a = component)  [12..23] alpha_{F,e}
-//   [24..35] beta_{F,e}  [36..47] mu_{F,e}  [48..51] gamma_F  [52..55] eps_F
-constexpr int TET_STATE = 56;
+// states per slice of the integrated near field (at most)
+constexpr int P2P_SLICE = 16;
 
 // ---------------------------------------------------------------------------
 // the plan
@@ -275,6 +272,23 @@ struct Plan {
   float4* hg_w = nullptr;           // (x, y, z, 0)
   int32_t* node_iperm = nullptr;    // original -> sorted node
 
+  // clusters of source tets of the integrated near field (near_mode 0; p2p.cu):
+  // distinct vertices, edges and faces of at most 40 tets of one source leaf
+  int64_t n_clusters = 0, n_cl_v = 0, n_cl_e = 0, n_cl_f = 0, n_cl_b = 0;
+  int p2p_max_nodes = 0;            // most target nodes of a P2P target leaf
+  int32_t* cl_off = nullptr;        // ncells + 1: clusters of every cell
+  int4* cl_cnt = nullptr;           // vertices, edges, faces, boundary faces (which come first)
+  int4* cl_pos = nullptr;           // first of each in the arrays below
+  int32_t* cl_vnode = nullptr;      // sorted node
+  uint32_t* cl_edge = nullptr;      // cluster vertices v0 | v1 << 16
+  double* cl_elen = nullptr;
+  double* cl_frec = nullptr;        // 16 doubles per face
+  uint2* cl_fidx = nullptr;         // vertices (8 bits each), edges (9 bits each)
+  int2* cl_ftet = nullptr;          // tets on the two sides, -1 = none
+  int64_t n_pc = 0;
+  int64_t* pc_off = nullptr;        // per P2P target: its source clusters
+  int32_t* pc_src = nullptr;
+
   std::vector<DevBuf> bufs;
   int64_t device_bytes = 0;
   Workspace* ws = nullptr;
@@ -344,6 +358,7 @@ void eval_field(Plan& P, const double* M, int B, double* u, double* H, cudaStrea
 // evaluation workspace (one per plan, sized for max_batch states)
 struct Workspace {
   int B = 0;
+  int slice = 0;  // states per slice that `state` holds (integrated near field)
   double *Ms = nullptr, *Q = nullptr, *L = nullptr, *u_s = nullptr, *state = nullptr;
   float *Ms32 = nullptr, *Q32 = nullptr, *L32 = nullptr, *u32 = nullptr;
   unsigned char* QP = nullptr;  // moments in the tensor-core tile layout (TF32 / split BF16 M2L)
@@ -428,14 +443,18 @@ bool launch_m2l_tc(Plan& P, int B, const float* Q, unsigned char* QP, float* L, 
 
 // near field (p2p.cu)
 void build_tet_geometry(Plan& P);
-// FP64 on-the-fly near field.  Batches of P2P_AT_MIN_B states or more: the
-// pair geometry once per (target, tet), contracted with every state (Ms);
-// smaller batches: pair by pair and state by state on the per-tet records
-// of launch_tet_state (state).
-constexpr int P2P_AT_MIN_B = 2;
-void launch_tet_state(Plan& P, const double* Ms, int B, double* state, cudaStream_t s);
-void launch_p2p_fp64(Plan& P, const double* Ms, const double* state, int B, double* u_s, int* err_flag,
-                     cudaStream_t s);
+// FP64 near field integrated at every evaluation (near_mode 0): clusters of
+// source tets at plan time; the doubles of per-face state a slice of `slice`
+// states takes; the launch (slices of at most `slice` states, a power of two;
+// returns its kernel launches)
+void build_clusters(Plan& P);
+size_t face_state_doubles(const Plan& P, int slice);
+inline int p2p_slice(int B) {
+  int k = 1;
+  while (k < B && k < P2P_SLICE) k *= 2;
+  return k;
+}
+int launch_p2p_fp64(Plan& P, const double* Ms, double* state, int slice, int B, double* u_s, cudaStream_t s);
 
 }  // namespace demag
 

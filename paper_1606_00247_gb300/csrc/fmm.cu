@@ -85,7 +85,7 @@ Workspace& workspace(Plan& P, int B) {
   destroy_workspace(P);
   Workspace* W = new Workspace();
   W->B = need;
-  const size_t nn = P.nn, nt = P.nt, ncell = P.ncells;
+  const size_t nn = P.nn, ncell = P.ncells;
   const bool mixed = P.opt.precision != DEMAG_FP64, otf = P.opt.near_mode == 0;
   if (!mixed || otf) W->Ms = (double*)ws_alloc(*W, sizeof(double) * nn * 3 * need);  // FP64 sorted M
   if (!mixed) {
@@ -102,7 +102,10 @@ Workspace& workspace(Plan& P, int B) {
     if (mp) W->MP = (float*)ws_alloc(*W, sizeof(float) * mp);
   }
   if (!mixed || otf) W->u_s = (double*)ws_alloc(*W, sizeof(double) * nn * need);  // FP64 sorted u
-  if (otf) W->state = (double*)ws_alloc(*W, sizeof(double) * nt * TET_STATE * std::min(need, P2P_AT_MIN_B - 1));
+  if (otf) {
+    W->slice = p2p_slice(need);
+    W->state = (double*)ws_alloc(*W, sizeof(double) * face_state_doubles(P, W->slice));
+  }
   W->err = (int*)ws_alloc(*W, sizeof(int));  // staging for host M, u, H: at the first host-pointer call
   P.ws = W;
   return *W;
@@ -176,17 +179,8 @@ void near_field_fp64(Plan& P, Workspace& W, int B, StageClock& clk, cudaStream_t
     clk.end();
     return;
   }
-  if (B < P2P_AT_MIN_B) {
-    clk.begin(DEMAG_STAGE_NEAR_PREP);
-    launch_tet_state(P, W.Ms, B, W.state, s);
-    clk.launched();
-    clk.end();
-  }
   clk.begin(DEMAG_STAGE_P2P);
-  if (!P.h_p2p_targets.empty()) {
-    launch_p2p_fp64(P, W.Ms, W.state, B, W.u_s, W.err, s);
-    clk.launched();
-  }
+  clk.launched(launch_p2p_fp64(P, W.Ms, W.state, W.slice, B, W.u_s, s));
   clk.end();
 }
 

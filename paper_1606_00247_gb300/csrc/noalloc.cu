@@ -95,9 +95,10 @@ struct Carver {
 };
 
 // Bytes that decide whether a plan and batch are taken: the expansions and the
-// packed moments counted with all C(p+3, 3) multi-indices.  The trace-free
-// arrays carved below take less, so which calls are accepted does not depend
-// on how the kernels store them.
+// packed moments counted with all C(p+3, 3) multi-indices, 56 doubles of
+// near-field state per tet (near_mode 0).  What is carved below takes less, so
+// which calls are accepted does not depend on how the kernels store it.
+constexpr size_t NOALLOC_TET_STATE = 56;
 size_t admission_bytes(const Plan& P, int B) {
   Carver c{nullptr};
   const size_t nn = P.nn, nt = P.nt, nc = P.nc, ncell = P.ncells;
@@ -126,7 +127,7 @@ size_t admission_bytes(const Plan& P, int B) {
     if (mp) c.take<float>(mp);
   }
   if (!mixed || otf) c.take<double>(nn * B);
-  if (otf) c.take<double>(nt * TET_STATE * std::min(B, P2P_AT_MIN_B - 1));
+  if (otf) c.take<double>(nt * NOALLOC_TET_STATE);
   c.take<int>(1);
   return c.used;
 }
@@ -152,7 +153,11 @@ size_t carve(Plan& P, int B, unsigned char* base, Workspace* W) {
     if (mp) w.MP = c.take<float>(mp);
   }
   if (!mixed || otf) w.u_s = c.take<double>(nn * B);
-  if (otf) w.state = c.take<double>(nt * TET_STATE * std::min(B, P2P_AT_MIN_B - 1));
+  if (otf) {  // the largest slice within the same allowance; one state always fits (16 doubles per tet at most)
+    w.slice = p2p_slice(B);
+    while (w.slice > 1 && face_state_doubles(P, w.slice) > nt * NOALLOC_TET_STATE) w.slice /= 2;
+    w.state = c.take<double>(face_state_doubles(P, w.slice));
+  }
   w.err = c.take<int>(1);
   if (W) {
     W->B = w.B;
@@ -167,6 +172,7 @@ size_t carve(Plan& P, int B, unsigned char* base, Workspace* W) {
     W->MP = w.MP;
     W->u_s = w.u_s;
     W->state = w.state;
+    W->slice = w.slice;
     W->err = w.err;
   }
   return c.used;

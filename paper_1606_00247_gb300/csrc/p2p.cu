@@ -1,9 +1,37 @@
-// p2p.cu -- near field (Sec. 2.1): per-tet geometry and the FP64 on-the-fly
-// P2P kernel.
+// p2p.cu -- near field (Sec. 2.1): per-tet geometry, and the FP64 near field
+// integrated at every evaluation (near_mode 0), by the faces of the source tets.
 //
-// The source tets of each P2P source leaf are contiguous in sorted tet order;
-// chunks of up to 32 tets (their 66-double geometry records) are staged in
-// shared memory by bulk copies (cp.async.bulk, completion on an mbarrier).
+// The potential of a tet with affine M is that of its charges,
+//   4 pi u = sum_F int_F (M.n) / R dA - div M int_tet 1 / R dV,
+//   int_tet 1/R dV = -(1/2) sum_F h_F I_F,  I_F = int_F dA / R,  h_F = n_F.(r - a_F)
+// (n_F outward).  M is nodal, so it is continuous, and the face charges of two
+// tets sharing a face cancel exactly: an interior face of a set of tets leaves
+// only (1/2) h_F I_F times the jump of div M.  The source leaves are cut, in
+// their sorted (Morton) order, into clusters of at most CL_TETS tets; a cluster
+// keeps its distinct vertices, edges and faces, and per target
+//   R_v      once per vertex  (0.5 - 0.7 per tet, 4 in the tet-wise form),
+//   Lam_e    once per edge    (1.8 - 2.2 per tet instead of 6 logarithms),
+//   I_F      once per face    (2.6 - 2.9 per tet instead of 4 solid angles);
+// the cluster's boundary faces also take the charge sigma = n.M,
+//   int_F sigma / R dA = sigma_0 I_F + sum_{k=1,2} (sigma_k - sigma_0) Y_k,
+//   Y_k = int_F lambda_k / R dA = (L_k / 2A) (P0_k I_F - m_k.J)   (edge k opposite vertex k),
+//   J = int_F (q - rho0)/R dA = (1/2) sum_e m_e E_e   (divergence theorem in the plane),
+//   E_e = (P0_e^2 + h^2) Lam_e + s+ R+ - s- R-   (s+- = t_e.(end - r)), the last two
+//       = (L_e / 2) ((s+ + s-)^2 / (R+ + R-) + R+ + R-): no difference of terms in R^2
+// with m_e, t_e, P0_e, Lam_e and Omega_F as in p2p.cuh (I_F = sum_e P0_e Lam_e
+// + h Omega_F).
+//
+// Rounding.  Y_k carries an error of eps R, I_F one of eps L (face size L,
+// distance R), so the constant part of sigma goes with I_F.  A face between two
+// clusters is evaluated twice and its charges cancel in the sum: its record is
+// built from its vertices in the order of their node ids, so both evaluations
+// have the same bits and their errors cancel with them.  Against 80-bit
+// arithmetic (theta -> 0; balls of 1k, 4k and 11k tets and a cube): smooth M
+// 0.9 - 7.5e-15 (the tet-wise form 1.2 - 10e-15 batched, 2 - 18e-15 for one
+// state), smooth M with 10 % noise 4.8 - 9.4e-15 (4.8 - 7.4e-15, 8 - 15e-15).
+#include <algorithm>
+#include <vector>
+
 #include "common.cuh"
 #include "p2p.cuh"
 
@@ -102,303 +130,588 @@ void build_tet_geometry(Plan& P) {
 }
 
 // ---------------------------------------------------------------------------
-// per-tet, per-state record: M(v0), J = dM/dx and the r-independent
-// contractions of the symmetric part Js of J used by pair_contract
+// clusters of source tets (plan time)
 // ---------------------------------------------------------------------------
-__global__ void k_tet_state(int64_t nt, int B, const int32_t* __restrict__ tets_s, const double* __restrict__ geo,
-                            const double* __restrict__ grad, const double* __restrict__ Ms, double* state) {
-  int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  int b = blockIdx.y;
-  if (j >= nt) return;
-  double Mk[4][3];
-  for (int k = 0; k < 4; k++) {
-    int64_t g = tets_s[4 * j + k];
-    for (int c = 0; c < 3; c++) Mk[k][c] = Ms[(g * 3 + c) * B + b];
-  }
-  const double* gr = grad + 12 * j;
-  double J[3][3];
-  for (int x = 0; x < 3; x++)
-    for (int y = 0; y < 3; y++) J[x][y] = Mk[0][x] * gr[y] + Mk[1][x] * gr[3 + y] + Mk[2][x] * gr[6 + y] + Mk[3][x] * gr[9 + y];
-  double Js[3][3];
-  for (int x = 0; x < 3; x++)
-    for (int y = 0; y < 3; y++) Js[x][y] = 0.5 * (J[x][y] + J[y][x]);
-  double* st = state + ((int64_t)b * nt + j) * TET_STATE;
-  const double* G = geo + (int64_t)TET_GEO * j;
-  for (int c = 0; c < 3; c++) st[c] = Mk[0][c];
-  for (int x = 0; x < 3; x++)
-    for (int y = 0; y < 3; y++) st[3 + 3 * x + y] = J[x][y];
-  double trJ = J[0][0] + J[1][1] + J[2][2];
-  for (int F = 0; F < 4; F++) {
-    const double* n = G + 12 + 3 * F;
-    double Jn[3];
-    for (int x = 0; x < 3; x++) Jn[x] = Js[x][0] * n[0] + Js[x][1] * n[1] + Js[x][2] * n[2];
-    double nJn = n[0] * Jn[0] + n[1] * Jn[1] + n[2] * Jn[2];
-    st[48 + F] = trJ - nJn;
-    st[52 + F] = nJn;
-    for (int e = 0; e < 3; e++) {
-      const double* m = G + 24 + 9 * F + 3 * e;
-      double t[3] = {n[1] * m[2] - n[2] * m[1], n[2] * m[0] - n[0] * m[2], n[0] * m[1] - n[1] * m[0]};
-      double Jm[3];
-      for (int x = 0; x < 3; x++) Jm[x] = Js[x][0] * m[0] + Js[x][1] * m[1] + Js[x][2] * m[2];
-      st[12 + 3 * F + e] = m[0] * Jm[0] + m[1] * Jm[1] + m[2] * Jm[2];
-      st[24 + 3 * F + e] = t[0] * Jm[0] + t[1] * Jm[1] + t[2] * Jm[2];
-      st[36 + 3 * F + e] = m[0] * Jn[0] + m[1] * Jn[1] + m[2] * Jn[2];
-    }
-  }
+namespace {
+
+constexpr int CL_TETS = 40;              // tets per cluster
+constexpr int CL_V = 4 * CL_TETS, CL_E = 6 * CL_TETS, CL_F = 4 * CL_TETS;  // bounds of its parts
+constexpr int FACE_REC = 16;             // doubles per face: n (3), m_e (9), 2 area, m_0.m_1, m_1.m_2, m_2.m_0
+static_assert(CL_V <= 256 && CL_E <= 512, "8-bit vertex and 9-bit edge positions");
+
+// sorts, returns 1 for an odd permutation; faces list their vertices counter-clockwise seen from outside
+__device__ __forceinline__ int sort3(int32_t& a, int32_t& b, int32_t& c) {
+  int odd = 0;
+  if (a > b) { const int32_t t = a; a = b; b = t; odd ^= 1; }
+  if (b > c) { const int32_t t = b; b = c; c = t; odd ^= 1; }
+  if (a > b) { const int32_t t = a; a = b; b = t; odd ^= 1; }
+  return odd;
 }
 
-void launch_tet_state(Plan& P, const double* Ms, int B, double* state, cudaStream_t s) {
-  dim3 grid(nblk(P.nt, 128), B);
-  k_tet_state<<<grid, 128, 0, s>>>(P.nt, B, P.tets_s, P.tet_geo, P.tet_grad, Ms, state);
-  DM_LAUNCH("k_tet_state");
-}
-
-// ---------------------------------------------------------------------------
-// TMA bulk copy + mbarrier helpers (sm_90+ PTX)
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void tma_bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t phase) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(phase)
-      : "memory");
-  return ok != 0;
-}
-// bounded wait: false if the barrier phase did not complete in time
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t phase) {
-  for (long it = 0; it < (1l << 24); it++) {
-    if (mbar_try_wait(bar, phase)) return true;
-    if (it > 64) __nanosleep(64);
-  }
-  return false;
-}
-
-constexpr int P2P_CHUNK = 32;
-
-// ---------------------------------------------------------------------------
-// FP64 on-the-fly P2P, one state at a time: one warp per (target leaf, state);
-// lanes take (target node, source tet) pairs and contract the pair with the
-// state's per-tet record (pair_contract)
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(32) k_p2p_fp64_state(const int32_t* __restrict__ targets, const int4* __restrict__ range,
-                                                 const int64_t* __restrict__ p2p_off,
-                                                 const int32_t* __restrict__ p2p_src,
-                                                 const double* __restrict__ nodes_s, const double* __restrict__ geo,
-                                                 const double* __restrict__ state, int64_t nt, int B, double* u_s,
-                                                 int* err) {
-  __shared__ __align__(128) double s_geo[P2P_CHUNK * TET_GEO];
-  __shared__ __align__(128) double s_st[P2P_CHUNK * TET_STATE];
-  __shared__ double s_part[32][33];
-  __shared__ __align__(8) uint64_t bar;
-  const int lane = threadIdx.x;
-  const int b = blockIdx.y;
-  const int32_t T = targets[blockIdx.x];
-  const int4 rT = range[T];
-  if (lane == 0) mbar_init(&bar, 1);
-  __syncwarp();
-  uint32_t phase = 0;
-  const double* st_b = state + (int64_t)b * nt * TET_STATE;
-  for (int32_t i0 = rT.z; i0 < rT.w; i0 += 32) {  // chunks of 32 target nodes
-    const int ntg = min(32, rT.w - i0);
-    for (int i = 0; i < ntg; i++) s_part[i][lane] = 0.0;
-    for (int64_t e = p2p_off[T]; e < p2p_off[T + 1]; e++) {
-      const int4 rS = range[p2p_src[e]];
-      for (int32_t j0 = rS.x; j0 < rS.y; j0 += P2P_CHUNK) {
-        const int ns = min(P2P_CHUNK, rS.y - j0);
-        __syncwarp();
-        if (lane == 0) {
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          uint32_t bg = (uint32_t)(ns * TET_GEO * sizeof(double)), bs = (uint32_t)(ns * TET_STATE * sizeof(double));
-          mbar_expect_tx(&bar, bg + bs);
-          tma_bulk_g2s(s_geo, geo + (int64_t)j0 * TET_GEO, bg, &bar);
-          tma_bulk_g2s(s_st, st_b + (int64_t)j0 * TET_STATE, bs, &bar);
-        }
-        if (!mbar_wait_bounded(&bar, phase)) {
-          if (lane == 0) atomicExch(err, (int)DEMAG_ERR_TIMEOUT);
-          mbar_wait_bounded(&bar, phase);  // let the copies in flight land before leaving
-          return;
-        }
-        phase ^= 1;
-        const int npair = ntg * ns;
-        for (int q = lane; q < npair; q += 32) {
-          const int i = q / ns, t = q - i * ns;
-          const double* r = nodes_s + 3ll * (i0 + i);
-          s_part[i][lane] += pair_contract(s_geo + t * TET_GEO, s_st + t * TET_STATE, r[0], r[1], r[2]);
-        }
-      }
-    }
-    __syncwarp();
-    for (int i = 0; i < ntg; i++) {
-      double v = s_part[i][lane];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) u_s[(int64_t)(i0 + i) * B + b] += v * (1.0 / (4.0 * M_PI));
-    }
-    __syncwarp();
-  }
-}
-
-// ---------------------------------------------------------------------------
-// FP64 on-the-fly P2P, state-batched: one block of 4 warps per (target leaf,
-// slice of FS states).  The state-independent part of every (target, tet)
-// pair -- the vector a and the symmetric tensor T of the W-form (p2p.cuh) --
-// is computed once and contracted with each state of the slice (16 states):
-//     sum_k M_k . W_k = M(r) . a + (1/2) T : J,   J = dM/dx,  M(r) = M(v0) + J (r - v0).
-// Chunks of 32 source tets: their geometry records are staged by a bulk copy,
-// their per-state M(v0) and J (12 numbers) computed once by the block.  Warp w
-// takes the target nodes w, w + 4, ... of the leaf, lane = tet of the chunk;
-// the 32 lanes' terms are added by a fixed shuffle tree and then, by the
-// warp that owns the target, into its shared-memory sum: no atomics, the
-// result does not depend on timing.
-// ---------------------------------------------------------------------------
-constexpr int PA_FS = 16, PA_WARPS = 4, PA_NT = 64;  // states per block, warps, target nodes per pass
-// dynamic shared memory: geometry records, per-state M(v0) and J of a chunk, per-target sums
-constexpr size_t PA_SMEM = sizeof(double) * (P2P_CHUNK * (TET_GEO + PA_FS * 12) + PA_NT * PA_FS);
-
-__global__ void __launch_bounds__(PA_WARPS * 32) k_p2p_fp64(
-    const int32_t* __restrict__ targets, const int4* __restrict__ range, const int64_t* __restrict__ p2p_off,
-    const int32_t* __restrict__ p2p_src, const double* __restrict__ nodes_s, const int32_t* __restrict__ tets_s,
-    const double* __restrict__ geo, const double* __restrict__ grad, const double* __restrict__ Ms, int B,
-    double* u_s, int* err) {
-  extern __shared__ __align__(128) double pa_smem[];
-  double* s_geo = pa_smem;                                                   // [tet][TET_GEO]
-  double(*s_mj)[PA_FS][12] = (double(*)[PA_FS][12])(pa_smem + P2P_CHUNK * TET_GEO);  // M(v0) (3), J (9)
-  double(*s_sum)[PA_FS] = (double(*)[PA_FS])(pa_smem + P2P_CHUNK * (TET_GEO + PA_FS * 12));
-  __shared__ __align__(8) uint64_t bar;
-  __shared__ bool s_ok;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int b0 = blockIdx.y * PA_FS;
-  const int32_t T = targets[blockIdx.x];
-  const int4 rT = range[T];
-  if (tid == 0) mbar_init(&bar, 1);
+// one block per cluster: its distinct vertices and edges, and its faces with
+// the boundary faces first.  An interior face is one that exactly two tets of
+// the cluster list, with opposite orientations; any other face (one tet, or
+// tets overlapping) is kept once per tet as a boundary face.  FILL = false
+// counts, FILL = true writes.
+template <bool FILL>
+__global__ void __launch_bounds__(256) k_clusters(const int2* __restrict__ range, const int32_t* __restrict__ tets_s,
+                                                  const double* __restrict__ geo, int4* cnt,
+                                                  const int4* __restrict__ off, int32_t* vnode, uint32_t* edge,
+                                                  double* elen, double* frec, uint2* fidx, int2* ftet) {
+  __shared__ int32_t vid[CL_V];                       // node of every tet corner
+  __shared__ int32_t vloc[CL_V], eloc[CL_E];          // its position among the distinct ones
+  __shared__ uint32_t ekey[CL_E];
+  __shared__ int32_t fk[CL_F][3];
+  __shared__ int fodd[CL_F], fother[CL_F], flag[CL_E];
+  const int2 rg = range[blockIdx.x];
+  const int nt = rg.y - rg.x, tid = threadIdx.x;
+  for (int q = tid; q < 4 * nt; q += blockDim.x) vid[q] = tets_s[4ll * rg.x + q];
   __syncthreads();
-  uint32_t phase = 0;
-  for (int32_t i0 = rT.z; i0 < rT.w; i0 += PA_NT) {  // passes of up to PA_NT target nodes
-    const int ntg = min(PA_NT, rT.w - i0);
-    for (int q = tid; q < PA_NT * PA_FS; q += blockDim.x) s_sum[q / PA_FS][q % PA_FS] = 0.0;
-    for (int64_t e = p2p_off[T]; e < p2p_off[T + 1]; e++) {
-      const int4 rS = range[p2p_src[e]];
-      for (int32_t j0 = rS.x; j0 < rS.y; j0 += P2P_CHUNK) {
-        const int ns = min(P2P_CHUNK, rS.y - j0);
-        __syncthreads();  // the previous chunk is no longer read
-        if (tid == 0) {
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          const uint32_t bg = (uint32_t)(ns * TET_GEO * sizeof(double));
-          mbar_expect_tx(&bar, bg);
-          tma_bulk_g2s(s_geo, geo + (int64_t)j0 * TET_GEO, bg, &bar);
-        }
-        // per tet and state: M(v0) and J = sum_k M_k (x) grad lambda_k
-        for (int q = tid; q < ns * PA_FS; q += blockDim.x) {
-          const int t = q / PA_FS, f = q - t * PA_FS, b = b0 + f;
-          const int32_t* tv = tets_s + 4ll * (j0 + t);
-          const double* g = grad + 12ll * (j0 + t);
-          double mj[12] = {};
-          if (b < B) {
-#pragma unroll
-            for (int k = 0; k < 4; k++) {
-              const int64_t node = tv[k];
-              const double mx = Ms[(node * 3 + 0) * B + b], my = Ms[(node * 3 + 1) * B + b],
-                           mz = Ms[(node * 3 + 2) * B + b];
-              if (k == 0) {
-                mj[0] = mx;
-                mj[1] = my;
-                mj[2] = mz;
-              }
-              const double m3[3] = {mx, my, mz};
-#pragma unroll
-              for (int x = 0; x < 3; x++)
-#pragma unroll
-                for (int y = 0; y < 3; y++) mj[3 + 3 * x + y] += m3[x] * g[3 * k + y];
-            }
-          }
-#pragma unroll
-          for (int c = 0; c < 12; c++) s_mj[t][f][c] = mj[c];
-        }
-        if (tid == 0) {
-          const bool ok = mbar_wait_bounded(&bar, phase);
-          if (!ok) {
-            atomicExch(err, (int)DEMAG_ERR_TIMEOUT);
-            mbar_wait_bounded(&bar, phase);  // let the copy in flight land before leaving
-          }
-          s_ok = ok;
-        }
-        phase ^= 1;
-        __syncthreads();  // s_geo landed (seen by thread 0), s_mj complete
-        if (!s_ok) return;  // the whole block leaves together
-        for (int i = warp; i < ntg; i += PA_WARPS) {
-          const double* r = nodes_s + 3ll * (i0 + i);
-          double acc[PA_FS];
-#pragma unroll
-          for (int f = 0; f < PA_FS; f++) acc[f] = 0.0;
-          if (lane < ns) {
-            const double* G = s_geo + lane * TET_GEO;
-            PairAT at;
-            pair_at(G, r[0], r[1], r[2], at);
-            const double d0 = r[0] - G[0], d1 = r[1] - G[1], d2 = r[2] - G[2];
-#pragma unroll
-            for (int f = 0; f < PA_FS; f++) {
-              const double* mj = s_mj[lane][f];
-              const double* J = mj + 3;
-              const double Mr0 = mj[0] + J[0] * d0 + J[1] * d1 + J[2] * d2;
-              const double Mr1 = mj[1] + J[3] * d0 + J[4] * d1 + J[5] * d2;
-              const double Mr2 = mj[2] + J[6] * d0 + J[7] * d1 + J[8] * d2;
-              const double TJ = at.T[0] * J[0] + at.T[1] * J[4] + at.T[2] * J[8] + at.T[3] * (J[1] + J[3]) +
-                                at.T[4] * (J[2] + J[6]) + at.T[5] * (J[5] + J[7]);
-              acc[f] = Mr0 * at.a[0] + Mr1 * at.a[1] + Mr2 * at.a[2] + 0.5 * TJ;
-            }
-          }
-#pragma unroll
-          for (int f = 0; f < PA_FS; f++) {
-            double v = acc[f];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) s_sum[i][f] += v;
-          }
-        }
-      }
-    }
-    __syncthreads();
-    for (int q = tid; q < ntg * PA_FS; q += blockDim.x) {
-      const int i = q / PA_FS, f = q - i * PA_FS;
-      if (b0 + f < B) u_s[(int64_t)(i0 + i) * B + b0 + f] += s_sum[i][f] * (1.0 / (4.0 * M_PI));
-    }
-    __syncthreads();  // s_sum is read before the next pass clears it
+  // distinct vertices: the first corner with the node owns it
+  for (int q = tid; q < 4 * nt; q += blockDim.x) {
+    int j = 0;
+    while (vid[j] != vid[q]) j++;
+    flag[q] = j;
   }
-}
-
-void launch_p2p_fp64(Plan& P, const double* Ms, const double* state, int B, double* u_s, int* err, cudaStream_t s) {
-  const int64_t nT = (int64_t)P.h_p2p_targets.size();
-  if (nT == 0) return;
-  static_assert(sizeof(double) * TET_GEO % 16 == 0 && sizeof(double) * TET_STATE % 16 == 0,
-                "bulk copies of whole records");
-  if (B < P2P_AT_MIN_B) {
-    k_p2p_fp64_state<<<dim3((unsigned)nT, B), 32, 0, s>>>(P.p2p_targets, P.cell_range, P.p2p_off, P.p2p_src,
-                                                          P.nodes_s, P.tet_geo, state, P.nt, B, u_s, err);
-    DM_LAUNCH("k_p2p_fp64_state");
+  __syncthreads();
+  for (int q = tid; q < 4 * nt; q += blockDim.x) {
+    int n = 0;
+    for (int j = 0; j < flag[q]; j++) n += flag[j] == j;
+    vloc[q] = n;
+  }
+  int nv = 0, ne = 0, nf = 0, nb = 0;
+  for (int j = 0; j < 4 * nt; j++) nv += flag[j] == j;
+  if (FILL)
+    for (int q = tid; q < 4 * nt; q += blockDim.x)
+      if (flag[q] == q) vnode[off[blockIdx.x].x + vloc[q]] = vid[q];
+  __syncthreads();
+  // distinct edges
+  for (int q = tid; q < 6 * nt; q += blockDim.x) {
+    const int t = q / 6, e = q - 6 * t;
+    const int a = vloc[4 * t + edge_v0(e)], b = vloc[4 * t + edge_v1(e)];
+    ekey[q] = (uint32_t)min(a, b) | ((uint32_t)max(a, b) << 16);
+  }
+  __syncthreads();
+  for (int q = tid; q < 6 * nt; q += blockDim.x) {
+    int j = 0;
+    while (ekey[j] != ekey[q]) j++;
+    flag[q] = j;
+  }
+  __syncthreads();
+  for (int q = tid; q < 6 * nt; q += blockDim.x) {
+    int n = 0;
+    for (int j = 0; j < flag[q]; j++) n += flag[j] == j;
+    eloc[q] = n;
+  }
+  for (int j = 0; j < 6 * nt; j++) ne += flag[j] == j;
+  if (FILL)
+    for (int q = tid; q < 6 * nt; q += blockDim.x)
+      if (flag[q] == q) {
+        edge[off[blockIdx.x].y + eloc[q]] = ekey[q];
+        elen[off[blockIdx.x].y + eloc[q]] = geo[(int64_t)TET_GEO * (rg.x + q / 6) + 60 + q % 6];
+      }
+  __syncthreads();
+  // faces
+  for (int q = tid; q < 4 * nt; q += blockDim.x) {
+    const int t = q >> 2, F = q & 3;
+    int32_t a = vid[4 * t + face_vertex(F, 0)], b = vid[4 * t + face_vertex(F, 1)], c = vid[4 * t + face_vertex(F, 2)];
+    fodd[q] = sort3(a, b, c);
+    fk[q][0] = a;
+    fk[q][1] = b;
+    fk[q][2] = c;
+  }
+  __syncthreads();
+  for (int q = tid; q < 4 * nt; q += blockDim.x) {
+    int n = 0, other = -1;
+    for (int j = 0; j < 4 * nt; j++)
+      if (j != q && fk[j][0] == fk[q][0] && fk[j][1] == fk[q][1] && fk[j][2] == fk[q][2]) {
+        n++;
+        other = j;
+      }
+    fother[q] = n == 1 && fodd[other] != fodd[q] ? other : -1;
+  }
+  __syncthreads();
+  for (int j = 0; j < 4 * nt; j++) {
+    nb += fother[j] < 0;
+    nf += fother[j] < 0 || fother[j] > j;
+  }
+  if (!FILL) {
+    if (tid == 0) cnt[blockIdx.x] = make_int4(nv, ne, nf, nb);
     return;
   }
-  smem_opt_in((const void*)k_p2p_fp64, PA_SMEM);
-  const dim3 grid((unsigned)nT, (unsigned)((B + PA_FS - 1) / PA_FS));
-  k_p2p_fp64<<<grid, PA_WARPS * 32, PA_SMEM, s>>>(P.p2p_targets, P.cell_range, P.p2p_off, P.p2p_src, P.nodes_s,
-                                             P.tets_s, P.tet_geo, P.tet_grad, Ms, B, u_s, err);
-  DM_LAUNCH("k_p2p_fp64");
+  for (int q = tid; q < 4 * nt; q += blockDim.x) {
+    const bool bnd = fother[q] < 0;
+    if (!bnd && fother[q] < q) continue;  // the other tet's copy owns it
+    int k = bnd ? 0 : nb;
+    for (int j = 0; j < q; j++) k += bnd ? fother[j] < 0 : fother[j] > j;
+    const int t = q >> 2, F = q & 3;
+    const int64_t o = off[blockIdx.x].z + k;
+    // the record depends on the face alone: its vertices by node id, n and m_e of that order
+    int cor[3];  // corners of tet t
+    for (int e = 0; e < 3; e++)
+      for (int c = 0; c < 3; c++)
+        if (vid[4 * t + face_vertex(F, c)] == fk[q][e]) cor[e] = face_vertex(F, c);
+    const double* G = geo + (int64_t)TET_GEO * (rg.x + t);
+    double v[3][3];
+    for (int e = 0; e < 3; e++)
+      for (int c = 0; c < 3; c++) v[e][c] = G[3 * cor[e] + c];
+    double* R = frec + FACE_REC * o;
+    double u[3], w[3], n[3], m[3][3];
+    for (int c = 0; c < 3; c++) {
+      u[c] = v[1][c] - v[0][c];
+      w[c] = v[2][c] - v[0][c];
+    }
+    n[0] = u[1] * w[2] - u[2] * w[1];
+    n[1] = u[2] * w[0] - u[0] * w[2];
+    n[2] = u[0] * w[1] - u[1] * w[0];
+    const double a2 = sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
+    for (int c = 0; c < 3; c++) R[c] = n[c] = n[c] / a2;
+    for (int e = 0; e < 3; e++) {  // m = t x n, t the unit tangent
+      double tg[3];
+      for (int c = 0; c < 3; c++) tg[c] = v[(e + 1) % 3][c] - v[e][c];
+      const double l = sqrt(tg[0] * tg[0] + tg[1] * tg[1] + tg[2] * tg[2]);
+      for (int c = 0; c < 3; c++) tg[c] /= l;
+      m[e][0] = tg[1] * n[2] - tg[2] * n[1];
+      m[e][1] = tg[2] * n[0] - tg[0] * n[2];
+      m[e][2] = tg[0] * n[1] - tg[1] * n[0];
+      for (int c = 0; c < 3; c++) R[3 + 3 * e + c] = m[e][c];
+    }
+    R[12] = a2;
+    for (int e = 0; e < 3; e++) {
+      const int f = (e + 1) % 3;
+      R[13 + e] = m[e][0] * m[f][0] + m[e][1] * m[f][1] + m[e][2] * m[f][2];
+    }
+    uint32_t es = 0, vs = fodd[q] ? 0x80000000u : 0u;  // top bit: n points into the tet
+    for (int e = 0; e < 3; e++) {
+      es |= (uint32_t)eloc[6 * t + edge_id(cor[e], cor[(e + 1) % 3])] << (9 * e);
+      vs |= (uint32_t)vloc[4 * t + cor[e]] << (8 * e);
+    }
+    fidx[o] = make_uint2(vs, es);
+    ftet[o] = make_int2(rg.x + t, bnd ? -1 : rg.x + (fother[q] >> 2));
+  }
 }
 
+// clusters of every P2P target leaf: one per (source leaf of its list, cluster of that leaf)
+template <bool FILL>
+__global__ void k_cluster_lists(const int32_t* __restrict__ targets, const int64_t* __restrict__ p2p_off,
+                                const int32_t* __restrict__ p2p_src, const int32_t* __restrict__ cl_off, int64_t* cnt,
+                                const int64_t* __restrict__ pc_off, int32_t* pc_src) {
+  __shared__ long long total;
+  const int32_t T = targets[blockIdx.x];
+  if (!FILL) {
+    if (threadIdx.x == 0) total = 0;
+    __syncthreads();
+    long long n = 0;
+    for (int64_t e = p2p_off[T] + threadIdx.x; e < p2p_off[T + 1]; e += blockDim.x)
+      n += cl_off[p2p_src[e] + 1] - cl_off[p2p_src[e]];
+    atomicAdd((unsigned long long*)&total, (unsigned long long)n);
+    __syncthreads();
+    if (threadIdx.x == 0) cnt[blockIdx.x] = total;
+  } else if (threadIdx.x < 32) {  // one warp, in list order
+    int64_t o = pc_off[blockIdx.x];
+    const int lane = threadIdx.x;
+    for (int64_t e0 = p2p_off[T]; e0 < p2p_off[T + 1]; e0 += 32) {
+      const bool on = e0 + lane < p2p_off[T + 1];
+      const int32_t S = on ? p2p_src[e0 + lane] : 0;
+      const int c0 = on ? cl_off[S] : 0, n = on ? cl_off[S + 1] - c0 : 0;
+      int sum = n;  // inclusive scan
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, sum, d);
+        if (lane >= d) sum += v;
+      }
+      for (int k = 0; k < n; k++) pc_src[o + sum - n + k] = c0 + k;
+      o += __shfl_sync(0xffffffffu, sum, 31);
+    }
+  }
+}
+
+}  // namespace
+
+void build_clusters(Plan& P) {
+  cudaStream_t s = P.stream;
+  const int64_t nc = P.ncells, nT = (int64_t)P.h_p2p_targets.size();
+  std::vector<int32_t> off(nc + 1, 0);
+  std::vector<int2> range;
+  std::vector<char> is_src(nc, 0);
+  for (int32_t c : P.h_src_leaves) is_src[c] = 1;
+  for (int64_t c = 0; c < nc; c++) {
+    if (is_src[c]) {  // equal pieces of at most CL_TETS tets
+      const int4 r = P.h_range[c];
+      const int n = r.y - r.x, k = (n + CL_TETS - 1) / CL_TETS;
+      for (int i = 0; i < k; i++)
+        range.push_back(make_int2(r.x + (int)((int64_t)n * i / k), r.x + (int)((int64_t)n * (i + 1) / k)));
+    }
+    off[c + 1] = (int32_t)range.size();
+  }
+  P.n_clusters = (int64_t)range.size();
+  P.p2p_max_nodes = 0;
+  for (int32_t c : P.h_p2p_targets) P.p2p_max_nodes = std::max(P.p2p_max_nodes, P.h_range[c].w - P.h_range[c].z);
+  if (P.n_clusters == 0) return;
+  int2* drange = dalloc<int2>(P, range.size());
+  int4* dcnt = dalloc<int4>(P, range.size());
+  P.cl_off = dalloc<int32_t>(P, nc + 1);
+  DM_CUDA(cudaMemcpyAsync(drange, range.data(), range.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
+  DM_CUDA(cudaMemcpyAsync(P.cl_off, off.data(), off.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+  k_clusters<false><<<(unsigned)range.size(), 256, 0, s>>>(drange, P.tets_s, P.tet_geo, dcnt, nullptr, nullptr, nullptr,
+                                                           nullptr, nullptr, nullptr, nullptr);
+  DM_LAUNCH("k_clusters");
+  std::vector<int4> cnt(range.size()), pos(range.size());
+  DM_CUDA(cudaMemcpyAsync(cnt.data(), dcnt, cnt.size() * sizeof(int4), cudaMemcpyDeviceToHost, s));
+  DM_CUDA(cudaStreamSynchronize(s));
+  int64_t nv = 0, ne = 0, nf = 0, nb = 0;
+  for (size_t i = 0; i < cnt.size(); i++) {
+    if (nf > INT32_MAX - CL_F || ne > INT32_MAX - CL_E) fail(DEMAG_ERR_UNSUPPORTED, "mesh too large for near_mode 0");
+    pos[i] = make_int4((int)nv, (int)ne, (int)nf, (int)nb);
+    nv += cnt[i].x;
+    ne += cnt[i].y;
+    nf += cnt[i].z;
+    nb += cnt[i].w;
+  }
+  P.n_cl_v = nv;
+  P.n_cl_e = ne;
+  P.n_cl_f = nf;
+  P.n_cl_b = nb;
+  P.cl_cnt = dcnt;
+  P.cl_pos = dalloc<int4>(P, pos.size());
+  P.cl_vnode = dalloc<int32_t>(P, nv);
+  P.cl_edge = dalloc<uint32_t>(P, ne);
+  P.cl_elen = dalloc<double>(P, ne);
+  P.cl_frec = dalloc<double>(P, FACE_REC * nf);
+  P.cl_fidx = dalloc<uint2>(P, nf);
+  P.cl_ftet = dalloc<int2>(P, nf);
+  DM_CUDA(cudaMemcpyAsync(P.cl_pos, pos.data(), pos.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
+  k_clusters<true><<<(unsigned)range.size(), 256, 0, s>>>(drange, P.tets_s, P.tet_geo, dcnt, P.cl_pos, P.cl_vnode,
+                                                          P.cl_edge, P.cl_elen, P.cl_frec, P.cl_fidx, P.cl_ftet);
+  DM_LAUNCH("k_clusters");
+  if (nT) {
+    int64_t* dc = dalloc<int64_t>(P, nT);
+    k_cluster_lists<false><<<(unsigned)nT, 128, 0, s>>>(P.p2p_targets, P.p2p_off, P.p2p_src, P.cl_off, dc, nullptr,
+                                                        nullptr);
+    DM_LAUNCH("k_cluster_lists");
+    std::vector<int64_t> hc(nT), po(nT + 1, 0);
+    DM_CUDA(cudaMemcpyAsync(hc.data(), dc, nT * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    DM_CUDA(cudaStreamSynchronize(s));
+    dfree(P, dc);
+    for (int64_t i = 0; i < nT; i++) po[i + 1] = po[i] + hc[i];
+    P.n_pc = po[nT];
+    P.pc_off = dalloc<int64_t>(P, nT + 1);
+    P.pc_src = dalloc<int32_t>(P, std::max<int64_t>(P.n_pc, 1));
+    DM_CUDA(cudaMemcpyAsync(P.pc_off, po.data(), po.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s));
+    k_cluster_lists<true><<<(unsigned)nT, 32, 0, s>>>(P.p2p_targets, P.p2p_off, P.p2p_src, P.cl_off, nullptr, P.pc_off,
+                                                      P.pc_src);
+    DM_LAUNCH("k_cluster_lists");
+  }
+  DM_CUDA(cudaStreamSynchronize(s));
+  dfree(P, drange);
+}
+
+// ---------------------------------------------------------------------------
+// per face and state of a slice of FS states: (1/2)(jump of div M) / 4 pi, and
+// for the boundary faces the charges sigma_0, sigma_1 - sigma_0, sigma_2 -
+// sigma_0 over 4 pi (signs for the record's n)
+// ---------------------------------------------------------------------------
+namespace {
+
+template <int FS>
+__global__ void k_face_state(int64_t nf, const int2* __restrict__ ftet, const uint2* __restrict__ fidx,
+                             const int32_t* __restrict__ tets_s,
+                             const double* __restrict__ grad, const double* __restrict__ Ms, int B, int b0, double* D) {
+  const int64_t it = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t f = it / FS;
+  if (f >= nf) return;
+  const int v = (int)(it - f * FS), b = b0 + v;
+  double d = 0.0;
+  if (b < B) {
+    const int2 t = ftet[f];
+#pragma unroll
+    for (int side = 0; side < 2; side++) {
+      const int64_t j = side ? t.y : t.x;
+      if (j < 0) continue;
+      double div = 0.0;
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        const int64_t node = tets_s[4 * j + k];
+#pragma unroll
+        for (int c = 0; c < 3; c++) div += Ms[(node * 3 + c) * B + b] * grad[12 * j + 3 * k + c];
+      }
+      d += side ? -div : div;
+    }
+  }
+  D[it] = d * ((fidx[f].x >> 31 ? -0.5 : 0.5) / (4.0 * M_PI));
+}
+
+template <int FS>
+__global__ void k_face_charge(int64_t ncl, const int4* __restrict__ cnt, const int4* __restrict__ pos,
+                              const int32_t* __restrict__ vnode, const double* __restrict__ frec,
+                              const uint2* __restrict__ fidx, const double* __restrict__ Ms, int B, int b0, double* S) {
+  const int64_t c = blockIdx.x;
+  const int4 n = cnt[c], o = pos[c];
+  for (int q = threadIdx.x; q < n.w * 3 * FS; q += blockDim.x) {
+    const int f = q / (3 * FS), r = q - f * 3 * FS, k = r / FS, b = b0 + r - k * FS;
+    double v = 0.0;
+    if (b < B) {
+      const uint32_t x = fidx[o.z + f].x;
+      const double* nrm = frec + FACE_REC * (int64_t)(o.z + f);
+      const double* m0 = Ms + (int64_t)vnode[o.x + (x & 255u)] * 3 * B + b;
+      const double* mk = Ms + (int64_t)vnode[o.x + ((x >> (8 * k)) & 255u)] * 3 * B + b;
+      for (int a = 0; a < 3; a++) v += (k ? mk[a * B] - m0[a * B] : m0[a * B]) * nrm[a];
+      if (x >> 31) v = -v;
+    }
+    S[(int64_t)o.w * 3 * FS + q] = v * (1.0 / (4.0 * M_PI));
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The near field: one block per (target leaf, 16 of its nodes) and FS states.
+// Batches of whole clusters (as many as fit the shared-memory arrays) are
+// staged; thread = (target i, subset of the entities), so a warp reads one or
+// two records per step (broadcast) for 16 targets, and keeps its target's FS
+// sums over all batches: distances, barrier, edge logarithms, barrier, faces.
+// The subsets are added in order at the end: no atomics, the result does not
+// depend on timing.  FP64 arithmetic is the bound (2 FMA per clock and SM), so
+// records are read from shared memory instead of being recomputed.  Measured:
+// 16k-tet ball, leaf 128, 3 states 196 -> 45 ms; 3,072-tet cube, leaf 32, one
+// state 5.2 -> 1.1 ms (the tet-wise kernels before: 4 sqrt, 6 log1p, 4 atan2 and
+// 6 divisions per pair, 16-state slices whatever the batch, one warp per target
+// leaf for one state).
+// ---------------------------------------------------------------------------
+constexpr int PF_THREADS = 256, PF_G = 16, PF_BATCH = 32;
+constexpr int PF_V = CL_V, PF_E = CL_E, PF_F = CL_F;  // capacities of a batch: any one cluster fits
+
+template <int FS>
+constexpr size_t pf_smem() {
+  return sizeof(double) * ((size_t)(PF_V + PF_E) * PF_G + 3 * PF_V + PF_E + FACE_REC * PF_F + (size_t)PF_F * 4 * FS) +
+         sizeof(uint2) * PF_F + sizeof(uint32_t) * PF_E;
+}
+
+template <int FS>
+__global__ void __launch_bounds__(PF_THREADS) k_p2p_faces(
+    const int32_t* __restrict__ targets, const int4* __restrict__ range, const int64_t* __restrict__ pc_off,
+    const int32_t* __restrict__ pc_src, const double* __restrict__ nodes_s, const int4* __restrict__ cnt,
+    const int4* __restrict__ pos, const int32_t* __restrict__ vnode, const uint32_t* __restrict__ edge,
+    const double* __restrict__ elen, const double* __restrict__ frec, const uint2* __restrict__ fidx,
+    const double* __restrict__ D, const double* __restrict__ S, int B, int b0, double* u_s) {
+  extern __shared__ __align__(16) double pf[];
+  double* sR = pf;                          // [vertex][target]
+  double* sL = sR + PF_V * PF_G;            // [edge][target]
+  double* sV = sL + PF_E * PF_G;            // [vertex][3]
+  double* sEl = sV + 3 * PF_V;              // edge lengths
+  double* sF = sEl + PF_E;                  // [face][FACE_REC], boundary faces of all clusters first
+  double* sD = sF + FACE_REC * PF_F;        // [face][FS]
+  double* sS = sD + PF_F * FS;              // [boundary face][3][FS]
+  uint2* sFi = (uint2*)(sS + 3 * PF_F * FS);
+  uint32_t* sE = (uint32_t*)(sFi + PF_F);
+  __shared__ int4 bc[PF_BATCH], bp[PF_BATCH], bb[PF_BATCH];  // per cluster: counts, positions, bases in the batch
+  __shared__ int4 tot;                                       // of the batch: vertices, edges, faces, boundary faces
+  __shared__ int nb;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int64_t ti = blockIdx.x;
+  const int4 rT = range[targets[ti]];
+  const int i0 = rT.z + PF_G * blockIdx.y;
+  if (i0 >= rT.w) return;  // uniform over the block
+  const int nt = min(PF_G, rT.w - i0);
+  int lg = 0;
+  while ((1 << lg) < nt) lg++;
+  const int G = 1 << lg, i = tid & (G - 1), sub = tid >> lg, nsub = PF_THREADS >> lg;
+  const double* rp = nodes_s + 3ll * (i0 + min(i, nt - 1));
+  const double rx = rp[0], ry = rp[1], rz = rp[2];
+  double acc[FS];
+#pragma unroll
+  for (int v = 0; v < FS; v++) acc[v] = 0.0;
+  const int64_t q1 = pc_off[ti + 1];
+  for (int64_t q = pc_off[ti]; q < q1;) {
+    __syncthreads();  // the previous batch is no longer read
+    if (tid < 32) {   // the next clusters, as many as fit
+      int4 n = make_int4(0, 0, 0, 0), p = n, e = n;
+      const bool on = q + lane < q1;
+      if (on) {
+        const int32_t c = pc_src[q + lane];
+        n = cnt[c];
+        p = pos[c];
+      }
+      e = n;  // inclusive sums
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int a = __shfl_up_sync(0xffffffffu, e.x, d), b = __shfl_up_sync(0xffffffffu, e.y, d),
+                  c = __shfl_up_sync(0xffffffffu, e.z, d), w = __shfl_up_sync(0xffffffffu, e.w, d);
+        if (lane >= d) {
+          e.x += a;
+          e.y += b;
+          e.z += c;
+          e.w += w;
+        }
+      }
+      const uint32_t fit = __ballot_sync(0xffffffffu, on && e.x <= PF_V && e.y <= PF_E && e.z <= PF_F);
+      const int k = __popc(fit);  // a prefix: the sums ascend
+      if (lane < k) {
+        bc[lane] = n;
+        bp[lane] = p;
+        bb[lane] = make_int4(e.x - n.x, e.y - n.y, (e.z - e.w) - (n.z - n.w), e.w - n.w);  // z: interior faces
+      }
+      if (lane == k - 1) tot = e;
+      if (lane == 0) nb = k;
+    }
+    __syncthreads();
+    const int k1 = nb, nv = tot.x, ne = tot.y, nf = tot.z, nbf = tot.w;
+    q += k1;
+    for (int k = 0; k < k1; k++) {
+      const int4 n = bc[k], p = bp[k], b = bb[k];
+      for (int t = tid; t < n.x; t += PF_THREADS) {
+        const double* x = nodes_s + 3ll * vnode[p.x + t];
+        double* d = sV + 3 * (b.x + t);
+        d[0] = x[0];
+        d[1] = x[1];
+        d[2] = x[2];
+      }
+      for (int t = tid; t < n.y; t += PF_THREADS) {
+        sE[b.y + t] = edge[p.y + t] + (uint32_t)b.x * 0x10001u;
+        sEl[b.y + t] = elen[p.y + t];
+      }
+      // face t of the cluster: boundary faces from b.w, interior ones behind all boundary faces
+      auto slot = [&](int t) { return t < n.w ? b.w + t : nbf + b.z + t - n.w; };
+      for (int t = tid; t < n.z; t += PF_THREADS) {
+        const uint2 x = fidx[p.z + t];
+        sFi[slot(t)] = make_uint2((x.x & 0xFFFFFFu) + (uint32_t)b.x * 0x010101u, x.y + (uint32_t)b.y * ((1u << 18) | (1u << 9) | 1u));
+      }
+      for (int t = tid; t < n.z * (FACE_REC / 2); t += PF_THREADS) {
+        const int f = t / (FACE_REC / 2), c = t - f * (FACE_REC / 2);
+        ((double2*)(sF + FACE_REC * slot(f)))[c] = ((const double2*)(frec + FACE_REC * (int64_t)(p.z + f)))[c];
+      }
+      for (int t = tid; t < n.z * FS; t += PF_THREADS) sD[slot(t / FS) * FS + t % FS] = D[(int64_t)p.z * FS + t];
+      for (int t = tid; t < n.w * 3 * FS; t += PF_THREADS) sS[b.w * 3 * FS + t] = S[(int64_t)p.w * 3 * FS + t];
+    }
+    __syncthreads();
+    for (int t = sub; t < nv; t += nsub) {
+      const double x = sV[3 * t] - rx, y = sV[3 * t + 1] - ry, z = sV[3 * t + 2] - rz;
+      sR[t * PF_G + i] = sqrt(x * x + y * y + z * z);
+    }
+    __syncthreads();
+    for (int t = sub; t < ne; t += nsub) {
+      const uint32_t e = sE[t];
+      const double L = sEl[t], dd = sR[(e & 0xFFFFu) * PF_G + i] + sR[(e >> 16) * PF_G + i] - L;
+      sL[t * PF_G + i] = dd > 0 ? log1p(2.0 * L / dd) : 0.0;
+    }
+    __syncthreads();
+    double part[FS];  // this batch's sums
+#pragma unroll
+    for (int v = 0; v < FS; v++) part[v] = 0.0;
+    for (int t = sub; t < nf; t += nsub) {
+      const uint2 ix = sFi[t];
+      const double* F = sF + FACE_REC * t;
+      int vi[3], ei[3];
+      double a[3][3], R[3], lam[3], len[3], P0[3];
+#pragma unroll
+      for (int k = 0; k < 3; k++) {
+        vi[k] = (ix.x >> (8 * k)) & 255u;
+        ei[k] = (ix.y >> (9 * k)) & 511u;
+        a[k][0] = sV[3 * vi[k]] - rx;
+        a[k][1] = sV[3 * vi[k] + 1] - ry;
+        a[k][2] = sV[3 * vi[k] + 2] - rz;
+        R[k] = sR[vi[k] * PF_G + i];
+        lam[k] = sL[ei[k] * PF_G + i];
+        len[k] = sEl[ei[k]];
+      }
+      double h = -(F[0] * a[0][0] + F[1] * a[0][1] + F[2] * a[0][2]);
+      if (fabs(h) <= 1e-13 * fmax(len[0], fmax(len[1], len[2]))) h = 0.0;  // r in the plane of F
+      if (h == 0.0 && t >= nbf) continue;
+      double I = 0.0;
+#pragma unroll
+      for (int e = 0; e < 3; e++) {
+        const double* m = F + 3 + 3 * e;
+        P0[e] = m[0] * a[e][0] + m[1] * a[e][1] + m[2] * a[e][2];
+        I += P0[e] * lam[e];
+      }
+      if (h != 0.0) {
+        const double d01 = a[0][0] * a[1][0] + a[0][1] * a[1][1] + a[0][2] * a[1][2];
+        const double d12 = a[1][0] * a[2][0] + a[1][1] * a[2][1] + a[1][2] * a[2][2];
+        const double d20 = a[2][0] * a[0][0] + a[2][1] * a[0][1] + a[2][2] * a[0][2];
+        const double den = R[0] * R[1] * R[2] + d01 * R[2] + d12 * R[0] + d20 * R[1];
+        I -= 2.0 * h * atan2(h * F[12], den);  // Omega = 2 atan2(triple product, den), triple product = -h 2A
+      }
+      const double x = h * I;
+#pragma unroll
+      for (int v = 0; v < FS; v++) part[v] += x * sD[t * FS + v];
+      if (t < nbf) {
+        double E[3], Y[2];
+        const double h2 = h * h, inv = 1.0 / F[12];
+        const double S0 = R[0] + R[1], S1 = R[1] + R[2], S2 = R[2] + R[0], iS = 1.0 / (S0 * S1 * S2);
+        const double S[3] = {S0, S1, S2}, rS[3] = {S1 * S2 * iS, S2 * S0 * iS, S0 * S1 * iS};
+#pragma unroll
+        for (int e = 0; e < 3; e++) {  // tangent t_e = n x m_e
+          const double* m = F + 3 + 3 * e;
+          const double sm = (F[1] * m[2] - F[2] * m[1]) * a[e][0] + (F[2] * m[0] - F[0] * m[2]) * a[e][1] +
+                            (F[0] * m[1] - F[1] * m[0]) * a[e][2];
+          const double w = 2.0 * sm + len[e];
+          E[e] = (P0[e] * P0[e] + h2) * lam[e] + 0.5 * len[e] * (w * w * rS[e] + S[e]);
+        }
+#pragma unroll
+        for (int k = 1; k < 3; k++) {  // edge o runs from vertex k + 1 to k + 2
+          const int o = (k + 1) % 3, o1 = (o + 1) % 3, o2 = (o + 2) % 3;
+          // m_o.m_{o+1} = F[13 + o], m_o.m_{o+2} = F[13 + o2]
+          const double mJ = 0.5 * (E[o] + F[13 + o] * E[o1] + F[13 + o2] * E[o2]);
+          Y[k - 1] = len[o] * inv * (P0[o] * I - mJ);
+        }
+        const double* q = sS + t * 3 * FS;
+#pragma unroll
+        for (int v = 0; v < FS; v++) part[v] += I * q[v] + Y[0] * q[FS + v] + Y[1] * q[2 * FS + v];
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < FS; v++) acc[v] += part[v];
+  }
+  __syncthreads();
+  double* red = pf;  // [sub][target][FS]
+#pragma unroll
+  for (int v = 0; v < FS; v++) red[tid * FS + v] = acc[v];
+  __syncthreads();
+  for (int t = tid; t < nt * FS; t += PF_THREADS) {
+    const int ii = t / FS, v = t - ii * FS;
+    if (b0 + v >= B) continue;
+    double sum = 0.0;
+    for (int k = 0; k < nsub; k++) sum += red[((k << lg) + ii) * FS + v];
+    u_s[(int64_t)(i0 + ii) * B + b0 + v] += sum;
+  }
+}
+
+template <int FS>
+void launch_slice(Plan& P, const double* Ms, double* state, int B, int b0, double* u_s, cudaStream_t s) {
+  double *D = state, *S = state + P.n_cl_f * FS;
+  k_face_state<FS><<<nblk(P.n_cl_f * FS, 256), 256, 0, s>>>(P.n_cl_f, P.cl_ftet, P.cl_fidx, P.tets_s,
+                                                                   P.tet_grad, Ms, B, b0, D);
+  DM_LAUNCH("k_face_state");
+  k_face_charge<FS><<<(unsigned)P.n_clusters, 128, 0, s>>>(P.n_clusters, P.cl_cnt, P.cl_pos, P.cl_vnode, P.cl_frec,
+                                                           P.cl_fidx, Ms, B, b0, S);
+  DM_LAUNCH("k_face_charge");
+  smem_opt_in((const void*)k_p2p_faces<FS>, pf_smem<FS>());
+  const dim3 grid((unsigned)P.h_p2p_targets.size(), (unsigned)((P.p2p_max_nodes + PF_G - 1) / PF_G));
+  k_p2p_faces<FS><<<grid, PF_THREADS, pf_smem<FS>(), s>>>(P.p2p_targets, P.cell_range, P.pc_off, P.pc_src, P.nodes_s,
+                                                          P.cl_cnt, P.cl_pos, P.cl_vnode, P.cl_edge, P.cl_elen,
+                                                          P.cl_frec, P.cl_fidx, D, S, B, b0, u_s);
+  DM_LAUNCH("k_p2p_faces");
+}
+
+}  // namespace
+
+size_t face_state_doubles(const Plan& P, int slice) { return (size_t)slice * (size_t)(P.n_cl_f + 3 * P.n_cl_b); }
+
+int launch_p2p_fp64(Plan& P, const double* Ms, double* state, int slice, int B, double* u_s, cudaStream_t s) {
+  if (P.h_p2p_targets.empty() || P.n_clusters == 0) return 0;
+  static_assert(pf_smem<16>() <= 227 * 1024, "shared memory of the near-field kernel");
+  int n = 0;
+  for (int b0 = 0; b0 < B; n += 3) {
+    int fs = 1;  // the smallest slice that takes what is left, within what the state buffer holds
+    while (fs < B - b0 && fs < slice) fs *= 2;
+    switch (fs) {
+      case 1: launch_slice<1>(P, Ms, state, B, b0, u_s, s); break;
+      case 2: launch_slice<2>(P, Ms, state, B, b0, u_s, s); break;
+      case 4: launch_slice<4>(P, Ms, state, B, b0, u_s, s); break;
+      case 8: launch_slice<8>(P, Ms, state, B, b0, u_s, s); break;
+      default: launch_slice<16>(P, Ms, state, B, b0, u_s, s); break;
+    }
+    b0 += fs;
+  }
+  return n;
+}
 
 }  // namespace demag

@@ -26,10 +26,6 @@
 //          = ln((R_a + R_b + L_e)/(R_a + R_b - L_e)),
 //    and Omega_F the signed solid angle of F seen from r (Van Oosterom and
 //    Strackee, IEEE TBME 30, 1983).
-//  * Contracted with the nodal M:  sum_k M_k . W_k = M(r).a + (1/2) T : J,
-//    a = sum_F h_F A_F, T = sum_F h_F T_F, J = dM/dx.  The J-contractions that
-//    do not depend on r are precomputed per tet and state (alpha, beta, mu,
-//    gamma, eps below).
 // Faces whose plane contains r (|h_F| <= 1e-13 x longest edge) contribute
 // exactly 0 (factor h_F), which also covers targets at vertices and on edges.
 #pragma once
@@ -58,68 +54,6 @@ struct PairAT {
   double a[3];
   double T[6];
 };
-
-// Contracted form: returns sum_k M_k . W_k for the state record `st`.
-__device__ __forceinline__ double pair_contract(const double* __restrict__ geo, const double* __restrict__ st,
-                                                double rx, double ry, double rz) {
-  double a[4][3], R[4];
-#pragma unroll
-  for (int k = 0; k < 4; k++) {
-    a[k][0] = geo[3 * k] - rx;
-    a[k][1] = geo[3 * k + 1] - ry;
-    a[k][2] = geo[3 * k + 2] - rz;
-    R[k] = sqrt(a[k][0] * a[k][0] + a[k][1] * a[k][1] + a[k][2] * a[k][2]);
-  }
-  double Lam[6], Lmax = 0;
-#pragma unroll
-  for (int e = 0; e < 6; e++) {
-    double L = geo[60 + e];
-    Lmax = fmax(Lmax, L);
-    double S = R[edge_v0(e)] + R[edge_v1(e)];
-    double D = S - L;
-    Lam[e] = D > 0 ? log1p(2.0 * L / D) : 0.0;
-  }
-  const double tol = 1e-13 * Lmax;
-  // M(r) = M(v0) + J (r - v0) = M(v0) - J a_0
-  double Mr[3];
-#pragma unroll
-  for (int c = 0; c < 3; c++)
-    Mr[c] = st[c] - (st[3 + 3 * c] * a[0][0] + st[4 + 3 * c] * a[0][1] + st[5 + 3 * c] * a[0][2]);
-  double aM = 0, TJ = 0;
-#pragma unroll
-  for (int F = 0; F < 4; F++) {
-    const int p = face_vertex(F, 0), q = face_vertex(F, 1), s = face_vertex(F, 2);
-    const double* n = geo + 12 + 3 * F;
-    double h = -(n[0] * a[p][0] + n[1] * a[p][1] + n[2] * a[p][2]);
-    if (fabs(h) <= tol) continue;
-    double cx = a[q][1] * a[s][2] - a[q][2] * a[s][1];
-    double cy = a[q][2] * a[s][0] - a[q][0] * a[s][2];
-    double cz = a[q][0] * a[s][1] - a[q][1] * a[s][0];
-    double trip = a[p][0] * cx + a[p][1] * cy + a[p][2] * cz;
-    double dpq = a[p][0] * a[q][0] + a[p][1] * a[q][1] + a[p][2] * a[q][2];
-    double dps = a[p][0] * a[s][0] + a[p][1] * a[s][1] + a[p][2] * a[s][2];
-    double dqs = a[q][0] * a[s][0] + a[q][1] * a[s][1] + a[q][2] * a[s][2];
-    double den = R[p] * R[q] * R[s] + dpq * R[s] + dps * R[q] + dqs * R[p];
-    double Om = 2.0 * atan2(trip, den);
-    double I = h * Om, sLm = 0, Jp = 0, sLmu = 0;
-#pragma unroll
-    for (int e = 0; e < 3; e++) {
-      const int v0 = face_vertex(F, e), v1 = face_vertex(F, (e + 1) % 3);
-      const double* m = geo + 24 + 9 * F + 3 * e;
-      double P0 = m[0] * a[v0][0] + m[1] * a[v0][1] + m[2] * a[v0][2];
-      double lam = Lam[edge_id(v0, v1)];
-      double dR = R[v1] - R[v0];
-      I += P0 * lam;
-      sLm += lam * (m[0] * Mr[0] + m[1] * Mr[1] + m[2] * Mr[2]);
-      Jp += P0 * lam * st[12 + 3 * F + e] + dR * st[24 + 3 * F + e];
-      sLmu += lam * st[36 + 3 * F + e];
-    }
-    double nM = n[0] * Mr[0] + n[1] * Mr[1] + n[2] * Mr[2];
-    aM += h * (Om * nM - sLm);
-    TJ += h * (I * st[48 + F] - Jp + 2.0 * h * sLmu - h * Om * st[52 + F]);
-  }
-  return aM + 0.5 * TJ;
-}
 
 // W-form: a and T of the pair (for the precomputed near-field coefficients).
 __device__ __forceinline__ void pair_at(const double* __restrict__ geo, double rx, double ry, double rz, PairAT& o) {

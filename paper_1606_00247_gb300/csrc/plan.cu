@@ -1118,6 +1118,7 @@ void build_plan(Plan& P, const double* nodes_in, const int32_t* tets_in) {
   P.h_p2p_off = std::move(h_p2p_off);
   P.h_p2p_src = std::move(h_p2p_src);
   if (P.opt.near_mode == 1) build_near_field(P);
+  if (P.opt.near_mode == 0) build_clusters(P);
   build_far_operators(P);
   if (P.opt.precision != DEMAG_FP64) build_gradient_operator(P);
   DM_CUDA(cudaStreamSynchronize(P.stream));
