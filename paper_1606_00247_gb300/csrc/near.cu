@@ -256,29 +256,6 @@ __global__ void __launch_bounds__(128) k_near_build(const int32_t* __restrict__ 
 }
 
 
-// u_s[i][b] += sum_col W[col][i] . M[node(col)][.][b]; one block per target leaf
-template <class T>
-__global__ void k_near_apply(const int32_t* __restrict__ targets, const int4* __restrict__ range,
-                             const int64_t* __restrict__ coloff, const int32_t* __restrict__ cols,
-                             const int64_t* __restrict__ woff, const T* __restrict__ W, const T* __restrict__ Ms, int B,
-                             T* u_s) {
-  const int64_t ti = blockIdx.x;
-  const int4 rT = range[targets[ti]];
-  const int nT = rT.w - rT.z;
-  const int64_t c0 = coloff[ti], c1 = coloff[ti + 1];
-  const T* Wt = W + woff[ti];
-  for (int item = threadIdx.x; item < nT * B; item += blockDim.x) {
-    const int i = item / B, b = item - i * B;
-    T acc = 0;
-    for (int64_t c = c0; c < c1; c++) {
-      const T* w = Wt + ((c - c0) * nT + i) * 3;
-      const T* m = Ms + (int64_t)cols[c] * 3 * B + b;
-      acc += w[0] * m[0] + w[1] * m[B] + w[2] * m[2 * B];
-    }
-    u_s[(int64_t)(rT.z + i) * B + b] += acc;
-  }
-}
-
 // FP32 copy in the layout of the mixed apply: [col][target node][4] (x, y, z, 0)
 __global__ void k_pack_w32(const int32_t* __restrict__ targets, const int4* __restrict__ range,
                            const int64_t* __restrict__ coloff, const int64_t* __restrict__ woff,
@@ -1014,12 +991,100 @@ void build_near_field(Plan& P) {
   }
 }
 
+// The stored coefficients applied in FP64: one block of 256 threads per (target
+// leaf, slice of BS <= 16 states).  W of a leaf is contiguous ([col][node][3]), so
+// thread t = g NP + i (node i of a pass of NP nodes, column group g of G = 256 /
+// NP) reads consecutive coefficients for consecutive t and the block sweeps the
+// leaf's W front to back; the NP threads of a column share its M (L1 broadcast).
+// Every thread keeps the sums of its BS states; the column groups are added in a
+// fixed order, so the result does not depend on timing.  One state is bound by
+// the stream of W (24 B per coefficient), sixteen by FP64 arithmetic.  Measured
+// with the thread-per-(node, state) kernel before: 224k-tet ball (2.57 GB of W),
+// one state 5.84 -> 1.06 ms; 29k tets, 16 states 6.29 -> 1.5 ms.
+constexpr int ND_THREADS = 256;
+template <int BS>
+__global__ void __launch_bounds__(ND_THREADS) k_near_apply64(
+    const int32_t* __restrict__ targets, const int4* __restrict__ range, const int64_t* __restrict__ coloff,
+    const int32_t* __restrict__ cols, const int64_t* __restrict__ woff, const double* __restrict__ W,
+    const double* __restrict__ Ms, int B, double* u_s) {
+  __shared__ double red[ND_THREADS * BS];
+  const int64_t ti = blockIdx.x;
+  const int4 rT = range[targets[ti]];
+  const int nT = rT.w - rT.z;
+  const int64_t c0 = coloff[ti];
+  const int ncol = (int)(coloff[ti + 1] - c0);
+  const double* Wt = W + woff[ti];
+  const int b0 = blockIdx.y * BS;
+  const int nlive = min(BS, B - b0);
+  const bool vec = BS >= 2 && nlive == BS && B % 2 == 0;  // M rows of this slice are 16-byte vectors
+  const int t = threadIdx.x;
+  for (int i0 = 0; i0 < nT; i0 += ND_THREADS) {
+    const int NP = min(ND_THREADS, nT - i0), G = ND_THREADS / NP;
+    const int i = t % NP, g = t / NP;
+    double acc[BS];
+#pragma unroll
+    for (int v = 0; v < BS; v++) acc[v] = 0.0;
+    if (g < G) {
+      const double* w = Wt + 3 * (i0 + i);
+#pragma unroll(BS <= 2 ? 4 : 1)
+      for (int c = g; c < ncol; c += G) {
+        const double* wc = w + (int64_t)c * nT * 3;
+        const double wv[3] = {wc[0], wc[1], wc[2]};
+        const double* mp = Ms + (int64_t)cols[c0 + c] * 3 * B + b0;
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+          double m[BS];
+          if (vec) {
+#pragma unroll
+            for (int v = 0; v < BS / 2; v++) {
+              const double2 x = ((const double2*)(mp + (int64_t)k * B))[v];
+              m[2 * v] = x.x;
+              m[2 * v + 1] = x.y;
+            }
+          } else {
+#pragma unroll
+            for (int v = 0; v < BS; v++) m[v] = v < nlive ? mp[(int64_t)k * B + v] : 0.0;
+          }
+#pragma unroll
+          for (int v = 0; v < BS; v++) acc[v] = fma(wv[k], m[v], acc[v]);
+        }
+      }
+    }
+    __syncthreads();  // the previous pass's reduction has been read
+#pragma unroll
+    for (int v = 0; v < BS; v++) red[v * ND_THREADS + t] = acc[v];
+    __syncthreads();
+    for (int q = t; q < NP * BS; q += ND_THREADS) {
+      const int ii = q % NP, v = q / NP;
+      if (v < nlive) {
+        double sum = 0.0;
+        for (int gg = 0; gg < G; gg++) sum += red[v * ND_THREADS + gg * NP + ii];
+        u_s[(int64_t)(rT.z + i0 + ii) * B + b0 + v] += sum;
+      }
+    }
+  }
+}
+
+template <int BS>
+void launch_near64(Plan& P, const double* Ms, int B, double* u_s, cudaStream_t s) {
+  const dim3 grid((unsigned)P.h_p2p_targets.size(), (unsigned)((B + BS - 1) / BS));
+  k_near_apply64<BS><<<grid, ND_THREADS, 0, s>>>(P.p2p_targets, P.cell_range, P.w_coloff, P.w_cols, P.w_off, P.W64, Ms,
+                                                 B, u_s);
+  DM_LAUNCH("k_near_apply64");
+}
+
 void launch_near_apply64(Plan& P, const double* Ms, int B, double* u_s, cudaStream_t s) {
-  const int64_t nT = (int64_t)P.h_p2p_targets.size();
-  if (!nT) return;
-  k_near_apply<double><<<(unsigned)nT, 128, 0, s>>>(P.p2p_targets, P.cell_range, P.w_coloff, P.w_cols, P.w_off, P.W64,
-                                                    Ms, B, u_s);
-  DM_LAUNCH("k_near_apply<double>");
+  if (P.h_p2p_targets.empty()) return;
+  if (B == 1)
+    launch_near64<1>(P, Ms, B, u_s, s);
+  else if (B == 2)
+    launch_near64<2>(P, Ms, B, u_s, s);
+  else if (B <= 4)
+    launch_near64<4>(P, Ms, B, u_s, s);
+  else if (B <= 8)
+    launch_near64<8>(P, Ms, B, u_s, s);
+  else
+    launch_near64<16>(P, Ms, B, u_s, s);
 }
 
 // Small batches: one block of 256 threads per (target leaf, slice of BS <= 8
