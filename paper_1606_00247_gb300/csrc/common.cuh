@@ -33,13 +33,10 @@ constexpr int NF_ROWS = 128;  // target nodes per tile of the tensor-core near f
 
 __host__ __device__ inline int ncoef_of(int p) { return (p + 1) * (p + 2) * (p + 3) / 6; }
 
-// one coefficient of an octree translation: target coefficient += (bit
-// `octant` of neg ? -c : c) * source coefficient k (octant of the child cell)
+// one coefficient of an octree translation (far.cu)
 template <class T>
 struct TEnt {
-  uint16_t k;
-  uint8_t neg;
-  uint8_t pad;
+  uint16_t k;  // M2M: class * nq + moment; L2L: local coefficient of the parent
   T c;
 };
 
@@ -104,6 +101,35 @@ __host__ __device__ inline double h_fold(int a, int b, int c, F&& f) {
     }
   }
   return v;
+}
+
+// SB consecutive values from shared memory, 16 bytes at a time
+template <class T, int SB>
+__device__ __forceinline__ void load_q(const T* q, T (&v)[SB]) {
+  if constexpr (SB * sizeof(T) % 16 == 0) {
+    constexpr int V = 16 / sizeof(T);
+#pragma unroll
+    for (int i = 0; i < SB / V; i++) {
+      if constexpr (sizeof(T) == 4) {
+        const float4 x = ((const float4*)q)[i];
+        v[V * i] = x.x;
+        v[V * i + 1] = x.y;
+        v[V * i + 2] = x.z;
+        v[V * i + 3] = x.w;
+      } else {
+        const double2 x = ((const double2*)q)[i];
+        v[V * i] = x.x;
+        v[V * i + 1] = x.y;
+      }
+    }
+  } else if constexpr (SB == 2) {
+    const float2 x = *(const float2*)q;
+    v[0] = x.x;
+    v[1] = x.y;
+  } else {
+#pragma unroll
+    for (int i = 0; i < SB; i++) v[i] = q[i];
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -256,12 +282,12 @@ struct Plan {
   int g_stride = 0;                 // values per support node of the P2M operator: 3 nq, padded to 4
   void* far_G = nullptr;            // n_sup x g_stride: P2M operator, [moment q][component]
   void* far_h = nullptr;            // nn x nl: the L2P polynomials of every node
-  // octree translations as coefficient lists (TEnt<T>):
-  //   M2M: Qt^P_n += sum over entries e of n: sign_e(octant) c_e Qt^C_{k_e}
-  //   L2L: Lt^C_m += sum over entries e of m: sign_e(octant) c_e Lt^P_{k_e}
-  int32_t* m2m_eoff = nullptr;      // nq + 1
+  // octree translations as coefficient lists (TEnt<T>, far.cu): M2M entry j of
+  // row n at [j][n]; L2L entries of (row, parity class) q in [l2l_cls[q].x, .y)
+  int32_t* m2m_cnt = nullptr;       // nq: entries of every row
   void* m2m_ent = nullptr;
-  int32_t* l2l_eoff = nullptr;      // nl + 1
+  int l2l_nent = 0;
+  int2* l2l_cls = nullptr;          // 8 nl
   void* l2l_ent = nullptr;
   int32_t* par_list = nullptr;      // cells with children, level by level
   std::vector<int64_t> par_start;   // host, nlevels + 1: parents of level l are par_list[par_start[l] ..]

@@ -259,69 +259,206 @@ void launch_p2m_small(Plan& P, int B, const T* Ms, T* Q, cudaStream_t s) {
                                                    Ms, P.nq, B, Q);
 }
 
-// M2M of one level: thread per (cell, n, state); the warp shares (cell, n), so
-// the coefficient list is read as a broadcast and the child moments coalesce
+// Octree translations.  The child centres are at (+-h, +-h, +-h) of the parent's,
+// so a term of index difference j takes the sign prod_a (+-1)^{j_a} of the
+// child's octant o: (-1)^popcount(c & ~o) with c = (j_x, j_y, j_z) mod 2, the
+// term's parity class.  Eight children therefore need every coefficient once:
+//   M2M: T_c = sum_o (-1)^popcount(c & ~o) Qt_o  (Walsh-Hadamard transform over
+//        the octants, 24 additions per moment), Qt^P_n = sum_e c_e T_{class e, k_e};
+//   L2L: S_c = sum of the terms of class c, then the same transform gives the
+//        eight children.
+// At p = 8 ~1,800 products per parent and state instead of ~1,800 per child.
+// Block per (parent, SW states), thread = (row, state); the transformed moments
+// (the parent's coefficients) are staged in shared memory.  Measured against a
+// thread per (parent, row, state) walking all children's terms through L2, one
+// term after another (224k-tet ball): M2M 150 -> 45 us for one state, 777 -> 199
+// us for 256; L2L 87 -> 49 us for one state, 330 -> 267 us for 256.
+constexpr int TR_THREADS = 256;
+
+// x_c = sum_o (-1)^popcount(c & ~o) x_o
 template <class T>
-__global__ void k_m2m(const int32_t* __restrict__ parents, int64_t npar, const int32_t* __restrict__ child0,
-                        const int32_t* __restrict__ nchild, const uint64_t* __restrict__ prefix,
-                        const int32_t* __restrict__ eoff, const TEnt<T>* __restrict__ ent, int nq, int B, T* Q) {
-  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t per = (int64_t)nq * B;
-  if (idx >= npar * per) return;
-  const int64_t P = parents[idx / per];
-  const int rem = (int)(idx % per), n = rem / B, b = rem - n * B;
-  const int nch = nchild[P];
-  const int32_t c0 = child0[P];
-  const int e0 = eoff[n], e1 = eoff[n + 1];
-  T acc = (T)0;
-  for (int k = 0; k < nch; k++) {
-    const int oct = (int)(prefix[c0 + k] & 7ull);
-    const T* Qc = Q + (int64_t)(c0 + k) * per + b;
-    for (int e = e0; e < e1; e++) {
-      const TEnt<T> E = ent[e];
-      const T v = Qc[(int64_t)E.k * B];
-      acc = fma(((E.neg >> oct) & 1) ? -E.c : E.c, v, acc);
-    }
-  }
-  Q[P * per + (int64_t)n * B + b] = acc;
+__device__ __forceinline__ void octant_transform(T (&x)[8]) {
+#pragma unroll
+  for (int d = 1; d < 8; d <<= 1)
+#pragma unroll
+    for (int o = 0; o < 8; o++)
+      if (!(o & d)) {
+        const T lo = x[o], hi = x[o | d];
+        x[o] = hi + lo;
+        x[o | d] = hi - lo;
+      }
 }
 
-// L2L from the parents of one level: thread per (parent, m, state) feeding all
-// children at once (each parent coefficient is loaded once; the octant only
-// flips signs); added to the children's own M2L results
+// x_o = sum_c (-1)^popcount(c & ~o) x_c
 template <class T>
-__global__ void k_l2l(const int32_t* __restrict__ parents, int64_t npar, const int32_t* __restrict__ child0,
-                        const int32_t* __restrict__ nchild, const int4* __restrict__ range,
-                        const uint64_t* __restrict__ prefix, const int32_t* __restrict__ eoff,
-                        const TEnt<T>* __restrict__ ent, int nl, int B, T* L) {
+__device__ __forceinline__ void classes_to_octants(T (&x)[8]) {
+#pragma unroll
+  for (int d = 1; d < 8; d <<= 1)
+#pragma unroll
+    for (int c = 0; c < 8; c++)
+      if (!(c & d)) {
+        const T even = x[c], odd = x[c | d];
+        x[c] = even - odd;  // octant bit 0: the odd terms change sign
+        x[c | d] = even + odd;
+      }
+}
+
+template <class T, int SW>
+__global__ void __launch_bounds__(TR_THREADS) k_m2m(const int32_t* __restrict__ parents,
+                                                    const int32_t* __restrict__ child0,
+                                                    const int32_t* __restrict__ nchild,
+                                                    const uint64_t* __restrict__ prefix,
+                                                    const int32_t* __restrict__ cnt, const TEnt<T>* __restrict__ ent,
+                                                    int nq, int B, T* Q) {
+  extern __shared__ __align__(16) unsigned char tr_smem[];
+  T* sq = (T*)tr_smem;  // [class][moment][state]
+  const int64_t P = parents[blockIdx.x];
+  const int v = threadIdx.x % SW, r0 = threadIdx.x / SW, b = blockIdx.y * SW + v;
+  const int nch = nchild[P];
+  const int32_t c0 = child0[P];
+  int pos[8];  // child of every octant, -1 = none
+#pragma unroll
+  for (int o = 0; o < 8; o++) pos[o] = -1;
+  for (int k = 0; k < nch; k++) {
+    const int o = (int)(prefix[c0 + k] & 7ull);
+#pragma unroll
+    for (int q = 0; q < 8; q++)
+      if (q == o) pos[q] = c0 + k;
+  }
+  for (int n = r0; n < nq; n += TR_THREADS / SW) {
+    T x[8];
+#pragma unroll
+    for (int o = 0; o < 8; o++) x[o] = pos[o] >= 0 && b < B ? Q[((int64_t)pos[o] * nq + n) * B + b] : (T)0;
+    octant_transform(x);
+#pragma unroll
+    for (int o = 0; o < 8; o++) sq[(o * nq + n) * SW + v] = x[o];
+  }
+  __syncthreads();
+  for (int n = r0; n < nq; n += TR_THREADS / SW) {
+    const int ne = cnt[n];
+    T a0 = (T)0, a1 = (T)0;
+    int e = 0;
+#pragma unroll 4
+    for (; e + 1 < ne; e += 2) {
+      const TEnt<T> E = ent[(int64_t)e * nq + n], F = ent[(int64_t)(e + 1) * nq + n];
+      a0 = fma(E.c, sq[E.k * SW + v], a0);
+      a1 = fma(F.c, sq[F.k * SW + v], a1);
+    }
+    if (e < ne) {
+      const TEnt<T> E = ent[(int64_t)e * nq + n];
+      a0 = fma(E.c, sq[E.k * SW + v], a0);
+    }
+    if (b < B) Q[(P * nq + n) * B + b] = a0 + a1;
+  }
+}
+
+// bytes of the parent's coefficients and the class sums, to whole 16 bytes (the
+// staged lists that follow hold 8- and 16-byte items)
+template <class T>
+__host__ __device__ constexpr size_t l2l_smem_base(int nl, int sw) {
+  return (sizeof(T) * 9 * nl * sw + 15) / 16 * 16;
+}
+
+// added to the children's own M2L results
+template <class T, int SW>
+__global__ void __launch_bounds__(TR_THREADS) k_l2l(const int32_t* __restrict__ parents,
+                                                    const int32_t* __restrict__ child0,
+                                                    const int32_t* __restrict__ nchild, const int4* __restrict__ range,
+                                                    const uint64_t* __restrict__ prefix,
+                                                    const int2* __restrict__ cls, const TEnt<T>* __restrict__ ent,
+                                                    int nent, bool staged, int nl, int B, T* L) {
+  extern __shared__ __align__(16) unsigned char tr_smem[];
+  T* sl = (T*)tr_smem;  // [coefficient][state]
+  static_assert(2 * sizeof(TEnt<T>) % 16 == 0, "pairs of entries keep the 16-byte alignment");
+  const int64_t P = parents[blockIdx.x];
+  if (range[P].w == range[P].z) return;  // no target node below this cell
+  const int v = threadIdx.x % SW, r0 = threadIdx.x / SW, b = blockIdx.y * SW + v;
+  const int nch = nchild[P];
+  const int32_t c0 = child0[P];
+  for (int m = r0; m < nl; m += TR_THREADS / SW) sl[m * SW + v] = b < B ? L[(P * nl + m) * B + b] : (T)0;
+  int pos[8];  // child with target nodes of every octant, -1 = none
+#pragma unroll
+  for (int o = 0; o < 8; o++) pos[o] = -1;
+  for (int k = 0; k < nch; k++) {
+    const int o = (int)(prefix[c0 + k] & 7ull);
+    const int4 rg = range[c0 + k];
+#pragma unroll
+    for (int q = 0; q < 8; q++)
+      if (q == o && rg.w > rg.z) pos[q] = c0 + k;
+  }
+  T* sc = sl + nl * SW;  // [row][class][state]: the classes of a row are short chains of their own
+  // the entries too, where they fit (short chains of global loads were what this kernel waited for)
+  const int2* cl = cls;
+  const TEnt<T>* en = ent;
+  if (staged) {
+    TEnt<T>* se = (TEnt<T>*)(tr_smem + l2l_smem_base<T>(nl, SW));
+    int2* scl = (int2*)(se + (nent + 1) / 2 * 2);  // both start on 16 bytes
+    for (int e = threadIdx.x; e < nent; e += TR_THREADS) se[e] = ent[e];
+    for (int q = threadIdx.x; q < 8 * nl; q += TR_THREADS) scl[q] = cls[q];
+    en = se;
+    cl = scl;
+  }
+  __syncthreads();
+  for (int q = r0; q < 8 * nl; q += TR_THREADS / SW) {
+    const int2 range_ = cl[q];
+    T a = (T)0;
+#pragma unroll 2
+    for (int e = range_.x; e < range_.y; e++) {
+      const TEnt<T> E = en[e];
+      a = fma(E.c, sl[E.k * SW + v], a);
+    }
+    sc[q * SW + v] = a;
+  }
+  __syncthreads();
+  for (int m = r0; m < nl; m += TR_THREADS / SW) {
+    T y[8];
+#pragma unroll
+    for (int c = 0; c < 8; c++) y[c] = sc[(8 * m + c) * SW + v];
+    classes_to_octants(y);
+#pragma unroll
+    for (int o = 0; o < 8; o++)
+      if (pos[o] >= 0 && b < B) L[((int64_t)pos[o] * nl + m) * B + b] += y[o];
+  }
+}
+
+// L2L of larger batches: thread per (parent, row, state), the states of a row
+// side by side (whole lines of the children's rows; above 8 states 16-state
+// slices in shared memory were up to 1.7x slower)
+template <class T>
+__global__ void __launch_bounds__(256) k_l2l_rows(const int32_t* __restrict__ parents, int64_t npar,
+                                                  const int32_t* __restrict__ child0,
+                                                  const int32_t* __restrict__ nchild, const int4* __restrict__ range,
+                                                  const uint64_t* __restrict__ prefix, const int2* __restrict__ cls,
+                                                  const TEnt<T>* __restrict__ ent, int nl, int B, T* L) {
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t per = (int64_t)nl * B;
   if (idx >= npar * per) return;
   const int64_t P = parents[idx / per];
-  const int nch = nchild[P];
-  if (range[P].w == range[P].z) return;  // no target node below this cell
+  const int4 rp = range[P];
+  if (rp.w == rp.z) return;  // no target node below this cell
   const int rem = (int)(idx % per), m = rem / B, b = rem - m * B;
-  const int32_t c0 = child0[P];
-  int oct[8];
-  T acc[8];
-#pragma unroll
-  for (int k = 0; k < 8; k++) {
-    oct[k] = k < nch ? (int)(prefix[c0 + k] & 7ull) : 0;
-    acc[k] = (T)0;
-  }
   const T* Lp = L + P * per + b;
-  for (int e = eoff[m], e1 = eoff[m + 1]; e < e1; e++) {
-    const TEnt<T> E = ent[e];
-    const T v = E.c * Lp[(int64_t)E.k * B];
+  T x[8];
 #pragma unroll
-    for (int k = 0; k < 8; k++) acc[k] += ((E.neg >> oct[k]) & 1) ? -v : v;
+  for (int c = 0; c < 8; c++) {
+    const int2 e = cls[8 * m + c];
+    T a = (T)0;
+#pragma unroll 4
+    for (int q = e.x; q < e.y; q++) a = fma(ent[q].c, Lp[(int64_t)ent[q].k * B], a);
+    x[c] = a;
   }
+  classes_to_octants(x);
+  const int nch = nchild[P];
+  const int32_t c0 = child0[P];
+  for (int k = 0; k < nch; k++) {
+    const int4 r = range[c0 + k];
+    if (r.w == r.z) continue;  // only cells with target nodes
+    const int o = (int)(prefix[c0 + k] & 7ull);
+    T y = x[0];
 #pragma unroll
-  for (int k = 0; k < 8; k++)
-    if (k < nch) {
-      const int4 r = range[c0 + k];
-      if (r.w > r.z) L[(int64_t)(c0 + k) * per + (int64_t)m * B + b] += acc[k];  // only cells with target nodes
-    }
+    for (int q = 1; q < 8; q++) y = o == q ? x[q] : y;
+    L[(int64_t)(c0 + k) * per + (int64_t)m * B + b] += y;
+  }
 }
 
 // L2P: block per (leaf holding nodes, 128 states), 256 threads.  The leaf's
@@ -430,10 +567,9 @@ void launch_l2p_small(Plan& P, int B, const T* L, T* u, cudaStream_t s) {
 }
 
 // coefficient lists of the translations on the trace-free coefficients
-// (formulas in the file header), with the sign for the child octant o:
-// d_i = +h if bit i of o is set, else -h.  A fold moves n_x by multiples of
-// two into n_y and n_z, so the sign of a term follows the parities of the
-// folded index difference.
+// (formulas in the file header) for the octant (+h, +h, +h); bit i of an octant
+// is set where d_i = +h.  A fold moves n_x by multiples of two into n_y and
+// n_z, so the parity class of a term is that of the folded index difference.
 template <class T>
 void build_translations(Plan& P) {
   const int p = P.p, nq = P.nq, nl = P.nl;
@@ -446,18 +582,11 @@ void build_translations(Plan& P) {
     if (ja < 0 || jb < 0 || jc < 0) return 0.0;
     return std::pow(h, ja + jb + jc) / (fact(ja) * fact(jb) * fact(jc));
   };
-  auto neg_bits = [](int ja, int jb, int jc) {
-    int bits = 0;
-    for (int o = 0; o < 8; o++) {
-      int odd = ((o & 1) ? 0 : ja) + ((o & 2) ? 0 : jb) + ((o & 4) ? 0 : jc);
-      if (odd & 1) bits |= 1 << o;
-    }
-    return (uint8_t)bits;
-  };
-  std::vector<int32_t> moff(nq + 1), loff(nl + 1);
-  std::vector<TEnt<T>> ment, lent;
+  auto parity = [](int ja, int jb, int jc) { return (ja & 1) | ((jb & 1) << 1) | ((jc & 1) << 2); };
+  std::vector<std::vector<TEnt<T>>> mrow(nq);
+  std::vector<TEnt<T>> lent;
+  std::vector<int2> lcls(8 * nl);
   for (int r = 0; r < nq; r++) {
-    moff[r] = (int32_t)ment.size();
     int ra, rb, rc;
     h_decode(r + 1, ra, rb, rc);
     for (int k = 0; k < nq; k++) {
@@ -465,32 +594,43 @@ void build_translations(Plan& P) {
       h_decode(k + 1, ka, kb, kc);
       const double cf = h_fold(ra, rb, rc, [&](int na, int nb, int nz) { return mono(0.25, na - ka, nb - kb, nz - kc); }) *
                         std::ldexp(1.0, -(ka + kb + kc));
-      if (cf != 0.0) ment.push_back(TEnt<T>{(uint16_t)k, neg_bits(ra + ka, rb + kb, rc + kc), 0, (T)cf});
+      if (cf != 0.0) mrow[r].push_back(TEnt<T>{(uint16_t)(parity(ra + ka, rb + kb, rc + kc) * nq + k), (T)cf});
     }
   }
-  moff[nq] = (int32_t)ment.size();
   for (int m = 0; m < nl; m++) {
-    loff[m] = (int32_t)lent.size();
     int ma, mb, mc;
     h_decode(m, ma, mb, mc);
-    for (int r = 0; r < nl; r++) {  // parent coefficients of degree p are zero
-      int ra, rb, rc;
-      h_decode(r, ra, rb, rc);
-      const int tr = ra + rb + rc;
-      const double cf = h_fold(ra, rb, rc, [&](int ka, int kb, int kz) { return mono(0.5, ka - ma, kb - mb, kz - mc); }) *
-                        std::ldexp(1.0, -tr);
-      if (tr < p && cf != 0.0) lent.push_back(TEnt<T>{(uint16_t)r, neg_bits(ra + ma, rb + mb, rc + mc), 0, (T)cf});
+    for (int cls = 0; cls < 8; cls++) {  // entries by parity class
+      lcls[8 * m + cls].x = (int)lent.size();
+      for (int r = 0; r < nl; r++) {     // parent coefficients of degree p are zero
+        int ra, rb, rc;
+        h_decode(r, ra, rb, rc);
+        if (parity(ra + ma, rb + mb, rc + mc) != cls) continue;
+        const double cf = h_fold(ra, rb, rc, [&](int ka, int kb, int kz) { return mono(0.5, ka - ma, kb - mb, kz - mc); }) *
+                          std::ldexp(1.0, -(ra + rb + rc));
+        if (cf != 0.0) lent.push_back(TEnt<T>{(uint16_t)r, (T)cf});
+      }
+      lcls[8 * m + cls].y = (int)lent.size();
     }
   }
-  loff[nl] = (int32_t)lent.size();
   cudaStream_t s = P.stream;
-  P.m2m_eoff = dalloc<int32_t>(P, nq + 1);
+  size_t width = 1;
+  std::vector<int32_t> mcnt(nq);
+  for (int r = 0; r < nq; r++) {
+    mcnt[r] = (int32_t)mrow[r].size();
+    width = std::max(width, mrow[r].size());
+  }
+  std::vector<TEnt<T>> ment(width * nq, TEnt<T>{0, (T)0});
+  for (int r = 0; r < nq; r++)
+    for (size_t j = 0; j < mrow[r].size(); j++) ment[j * nq + r] = mrow[r][j];
+  P.l2l_nent = (int)lent.size();
+  P.m2m_cnt = dalloc<int32_t>(P, nq);
   P.m2m_ent = dalloc<TEnt<T>>(P, ment.size());
-  P.l2l_eoff = dalloc<int32_t>(P, nl + 1);
+  P.l2l_cls = dalloc<int2>(P, lcls.size());
   P.l2l_ent = dalloc<TEnt<T>>(P, lent.size());
-  DM_CUDA(cudaMemcpyAsync(P.m2m_eoff, moff.data(), moff.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+  DM_CUDA(cudaMemcpyAsync(P.m2m_cnt, mcnt.data(), nq * sizeof(int32_t), cudaMemcpyHostToDevice, s));
   DM_CUDA(cudaMemcpyAsync(P.m2m_ent, ment.data(), ment.size() * sizeof(TEnt<T>), cudaMemcpyHostToDevice, s));
-  DM_CUDA(cudaMemcpyAsync(P.l2l_eoff, loff.data(), loff.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+  DM_CUDA(cudaMemcpyAsync(P.l2l_cls, lcls.data(), lcls.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
   DM_CUDA(cudaMemcpyAsync(P.l2l_ent, lent.data(), lent.size() * sizeof(TEnt<T>), cudaMemcpyHostToDevice, s));
   DM_CUDA(cudaStreamSynchronize(s));
 }
@@ -571,15 +711,48 @@ int launch_p2m(Plan& P, int B, const T* Ms, T* Q, cudaStream_t s) {
   return 1;
 }
 
+namespace {
+
+template <class T, int SW>
+void launch_m2m_level(Plan& P, int64_t pb, int64_t np, int B, T* Q, cudaStream_t s) {
+  const size_t smem = sizeof(T) * SW * 8 * P.nq;
+  smem_opt_in((const void*)k_m2m<T, SW>, smem);
+  k_m2m<T, SW><<<dim3((unsigned)np, (unsigned)((B + SW - 1) / SW)), TR_THREADS, smem, s>>>(
+      P.par_list + pb, P.cell_child0, P.cell_nchild, P.cell_prefix, P.m2m_cnt, (const TEnt<T>*)P.m2m_ent, P.nq, B, Q);
+  DM_LAUNCH("k_m2m");
+}
+
+template <class T, int SW>
+void launch_l2l_level(Plan& P, int64_t pb, int64_t np, int B, T* L, cudaStream_t s) {
+  const size_t base = l2l_smem_base<T>(P.nl, SW);
+  const size_t ents = sizeof(TEnt<T>) * ((P.l2l_nent + 1) / 2 * 2) + sizeof(int2) * 8 * P.nl;
+  const bool staged = base + ents <= 100 * 1024;  // two blocks per SM
+  const size_t smem = base + (staged ? ents : 0);
+  smem_opt_in((const void*)k_l2l<T, SW>, smem);
+  k_l2l<T, SW><<<dim3((unsigned)np, (unsigned)((B + SW - 1) / SW)), TR_THREADS, smem, s>>>(
+      P.par_list + pb, P.cell_child0, P.cell_nchild, P.cell_range, P.cell_prefix, P.l2l_cls,
+      (const TEnt<T>*)P.l2l_ent, P.l2l_nent, staged, P.nl, B, L);
+  DM_LAUNCH("k_l2l");
+}
+
+}  // namespace
+
 template <class T>
 int launch_m2m(Plan& P, int B, T* Q, cudaStream_t s) {
   int n = 0;
   for (int l = P.nlevels - 2; l >= 0; l--) {
     const int64_t pb = P.par_start[l], np = P.par_start[l + 1] - pb;
     if (np == 0) continue;
-    k_m2m<T><<<nblk(np * P.nq * B, 256), 256, 0, s>>>(P.par_list + pb, np, P.cell_child0, P.cell_nchild, P.cell_prefix,
-                                                      P.m2m_eoff, (const TEnt<T>*)P.m2m_ent, P.nq, B, Q);
-    DM_LAUNCH("k_m2m");
+    if (B == 1)
+      launch_m2m_level<T, 1>(P, pb, np, B, Q, s);
+    else if (B == 2)
+      launch_m2m_level<T, 2>(P, pb, np, B, Q, s);
+    else if (B <= 4)
+      launch_m2m_level<T, 4>(P, pb, np, B, Q, s);
+    else if (B <= 8)
+      launch_m2m_level<T, 8>(P, pb, np, B, Q, s);
+    else
+      launch_m2m_level<T, 16>(P, pb, np, B, Q, s);
     n++;
   }
   return n;
@@ -591,9 +764,20 @@ int launch_l2l(Plan& P, int B, T* L, cudaStream_t s) {
   for (int l = 0; l + 1 < P.nlevels; l++) {  // parents at level l, children at l + 1
     const int64_t pb = P.par_start[l], np = P.par_start[l + 1] - pb;
     if (np == 0) continue;
-    k_l2l<T><<<nblk(np * P.nl * B, 256), 256, 0, s>>>(P.par_list + pb, np, P.cell_child0, P.cell_nchild, P.cell_range,
-                                                      P.cell_prefix, P.l2l_eoff, (const TEnt<T>*)P.l2l_ent, P.nl, B, L);
-    DM_LAUNCH("k_l2l");
+    if (B == 1)
+      launch_l2l_level<T, 1>(P, pb, np, B, L, s);
+    else if (B == 2)
+      launch_l2l_level<T, 2>(P, pb, np, B, L, s);
+    else if (B <= 4)
+      launch_l2l_level<T, 4>(P, pb, np, B, L, s);
+    else if (B <= 8)
+      launch_l2l_level<T, 8>(P, pb, np, B, L, s);
+    else {
+      k_l2l_rows<T><<<nblk(np * P.nl * B, 256), 256, 0, s>>>(P.par_list + pb, np, P.cell_child0, P.cell_nchild,
+                                                             P.cell_range, P.cell_prefix, P.l2l_cls,
+                                                             (const TEnt<T>*)P.l2l_ent, P.nl, B, L);
+      DM_LAUNCH("k_l2l_rows");
+    }
     n++;
   }
   return n;

@@ -29,35 +29,6 @@ __device__ __forceinline__ int idx3(int a, int b, int c) {
   return t * (t + 1) * (t + 2) / 6 + j * (j + 1) / 2 + c;
 }
 
-// SB consecutive values from shared memory, 16 bytes at a time
-template <class T, int SB>
-__device__ __forceinline__ void load_q(const T* q, T (&v)[SB]) {
-  if constexpr (SB * sizeof(T) % 16 == 0) {
-    constexpr int V = 16 / sizeof(T);
-#pragma unroll
-    for (int i = 0; i < SB / V; i++) {
-      if constexpr (sizeof(T) == 4) {
-        const float4 x = ((const float4*)q)[i];
-        v[V * i] = x.x;
-        v[V * i + 1] = x.y;
-        v[V * i + 2] = x.z;
-        v[V * i + 3] = x.w;
-      } else {
-        const double2 x = ((const double2*)q)[i];
-        v[V * i] = x.x;
-        v[V * i + 1] = x.y;
-      }
-    }
-  } else if constexpr (SB == 2) {
-    const float2 x = *(const float2*)q;
-    v[0] = x.x;
-    v[1] = x.y;
-  } else {
-#pragma unroll
-    for (int i = 0; i < SB; i++) v[i] = q[i];
-  }
-}
-
 template <class T>
 __global__ void __launch_bounds__(1024) k_m2l_rows(const int32_t* __restrict__ targets,
                                                     const int64_t* __restrict__ m2l_off,
