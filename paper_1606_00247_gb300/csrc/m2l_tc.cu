@@ -452,8 +452,11 @@ __global__ void __launch_bounds__(128) k_m2l_tc_ops(const int4* __restrict__ key
 // when e is not in its list.  Warp 0 lane 0 streams each source's A slices
 // once, plus the K slices of every target that uses it; warp 1 (target 0) and
 // warp 3 (target 1) issue the MMAs into their own 256-column halves of TMEM.
-template <int P, bool BF16, int NT, int LS>
-__global__ void __launch_bounds__(TC_THREADS, NT == 1 ? 2 : 1)
+// PC: promoted 16-column chunks an epilogue thread holds, at most; with one (the
+// default) the kernel takes 48 registers, so that shared memory alone decides
+// how many CTAs share an SM.
+template <int P, bool BF16, int NT, int LS, int PC>
+__global__ void __launch_bounds__(TC_THREADS, NT == 2 ? 1 : (PC == 1 ? 5 : 2))
     k_m2l_tc(const int32_t* __restrict__ gtarget, const int64_t* __restrict__ goff,
              const int32_t* __restrict__ gsrc, const int32_t* __restrict__ gop, const int32_t* __restrict__ level,
              double side, int B, int nsb, const TcRing R, const unsigned char* __restrict__ QP,
@@ -640,9 +643,9 @@ __global__ void __launch_bounds__(TC_THREADS, NT == 1 ? 2 : 1)
     // promotion: the leading columns are summed here in FP32 (round to nearest)
     // and zeroed in TMEM every prom_group sources, so that the accumulator
     // never carries a large running value of the cancelling low-degree terms
-    float tot[64];
+    float tot[16 * PC];
 #pragma unroll
-    for (int i = 0; i < 64; i++) tot[i] = 0.f;
+    for (int i = 0; i < 16 * PC; i++) tot[i] = 0.f;
     const int nprom = (NT == 1 && R.prom_group > 0) ? (int)((e1 - e0 - 1) / R.prom_group) : 0;
     for (int g = 0; g < nprom; g++) {
       if (!mbar_wait(smem_u32(gdone), (uint32_t)(g & 1), abort_flag)) {
@@ -652,7 +655,7 @@ __global__ void __launch_bounds__(TC_THREADS, NT == 1 ? 2 : 1)
       }
       tc_fence_after();
 #pragma unroll
-      for (int c = 0; c < 4; c++) {
+      for (int c = 0; c < PC; c++) {
         if (c < R.prom_chunks) {
           uint32_t r[16];
           const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(16 * c);
@@ -690,7 +693,7 @@ __global__ void __launch_bounds__(TC_THREADS, NT == 1 ? 2 : 1)
             for (int i = 0; i < 16; i++) {
               const int m = c0 + i;
               float v = __uint_as_float(r[i]);
-              if (c0 < 64 && t == 0) v += tot[(c0 < 64 ? c0 : 0) + i];  // promoted part (zero when not promoting)
+              if (c0 < 16 * PC && t == 0) v += tot[(c0 < 16 * PC ? c0 : 0) + i];  // promoted part (zero when not promoting)
               if (m < G.nl) Lt[(int64_t)m * B] = ((h_degree(m) & 1) ? -inv : inv) * v;
             }
           }
@@ -718,19 +721,19 @@ bool split_bf16(const Plan& P) {
 }
 TcLayout layout_of(const Plan& P) { return tc_layout(P.p, split_bf16(P), P.tc_ls); }
 
-template <int PP, bool BF16, int NT, int LS>
+template <int PP, bool BF16, int NT, int LS, int PC>
 void launch_fixed(Plan& P, const TcRing& R, int B, const unsigned char* QP, float* L, int* err, cudaStream_t s) {
   const size_t smem = ring_smem(R);
-  smem_opt_in((const void*)k_m2l_tc<PP, BF16, NT, LS>, smem);
+  smem_opt_in((const void*)k_m2l_tc<PP, BF16, NT, LS, PC>, smem);
   const int nsb = (B + TC_M - 1) / TC_M;
   if (NT == 1) {
     dim3 grid((unsigned)(nsb * P.h_m2l_targets.size()));
-    k_m2l_tc<PP, BF16, NT, LS><<<grid, TC_THREADS, smem, s>>>(P.m2l_targets, P.tc_g1_off, P.m2l_src, P.m2l_op,
+    k_m2l_tc<PP, BF16, NT, LS, PC><<<grid, TC_THREADS, smem, s>>>(P.m2l_targets, P.tc_g1_off, P.m2l_src, P.m2l_op,
                                                               P.cell_level, P.side, B, nsb, R, QP, P.tc_ops, L,
                                                               err);
   } else {
     dim3 grid((unsigned)(nsb * P.tc_n_g2));
-    k_m2l_tc<PP, BF16, NT, LS><<<grid, TC_THREADS, smem, s>>>(P.tc_g2_tgt, P.tc_g2_off, P.tc_g2_src, P.tc_g2_op,
+    k_m2l_tc<PP, BF16, NT, LS, PC><<<grid, TC_THREADS, smem, s>>>(P.tc_g2_tgt, P.tc_g2_off, P.tc_g2_src, P.tc_g2_op,
                                                               P.cell_level, P.side, B, nsb, R, QP, P.tc_ops, L,
                                                               err);
   }
@@ -743,15 +746,18 @@ void launch_fixed(Plan& P, const TcRing& R, int B, const unsigned char* QP, floa
 template <int PP, bool BF16, int LS>
 void launch_ls(Plan& P, const TcRing& R, int B, const unsigned char* QP, float* L, int* err, cudaStream_t s) {
   if constexpr (tc_layout(PP, BF16, LS).tmem_cols <= 256) {
-    if (R.nt == 2) return launch_fixed<PP, BF16, 2, LS>(P, R, B, QP, L, err, s);
+    if (R.nt == 2) return launch_fixed<PP, BF16, 2, LS, 1>(P, R, B, QP, L, err, s);
   }
-  launch_fixed<PP, BF16, 1, LS>(P, R, B, QP, L, err, s);
+  if (R.prom_chunks > 1) return launch_fixed<PP, BF16, 1, LS, 4>(P, R, B, QP, L, err, s);
+  launch_fixed<PP, BF16, 1, LS, 1>(P, R, B, QP, L, err, s);
 }
 
 template <int PP, bool BF16>
 void launch_nt(Plan& P, const TcRing& R, int B, const unsigned char* QP, float* L, int* err, cudaStream_t s) {
   if constexpr (BF16) {
-    if (P.tc_ls == TC_LS_ALL3) return launch_fixed<PP, BF16, 1, TC_LS_ALL3>(P, R, B, QP, L, err, s);
+    if (P.tc_ls == TC_LS_ALL3)
+      return R.prom_chunks > 1 ? launch_fixed<PP, BF16, 1, TC_LS_ALL3, 4>(P, R, B, QP, L, err, s)
+                               : launch_fixed<PP, BF16, 1, TC_LS_ALL3, 1>(P, R, B, QP, L, err, s);
     if (P.tc_ls == tc_split_degree(PP)) return launch_ls<PP, BF16, tc_split_degree(PP)>(P, R, B, QP, L, err, s);
   }
   launch_ls<PP, BF16, TC_LS_ALL2>(P, R, B, QP, L, err, s);
@@ -775,20 +781,39 @@ void launch_main(Plan& P, const TcRing& R, int B, const unsigned char* QP, float
     launch_order<false>(P, R, B, QP, L, err, s);
 }
 
-// ring budgets: ~100 KB lets two CTAs share an SM (when their tensor memory
-// fits), ~200 KB gives one CTA the whole shared memory
-constexpr int TC_BUDGET_2 = 100 * 1024, TC_BUDGET_1 = 200 * 1024;
+// ring budgets that let four, three, two and one CTAs share an SM
+constexpr int TC_BUDGET_4 = 56 * 1024, TC_BUDGET_3 = 72 * 1024, TC_BUDGET_2 = 100 * 1024, TC_BUDGET_1 = 200 * 1024;
 
-// default launch shape (the fastest measured on GB300 for a ball of 224k tets
-// at p = 8): one target per CTA, 2 k-steps per slot, and a ring small enough
-// for two CTAs per SM when their tensor memory fits; nt / kps override it
-void default_ring(const TcLayout& G, int nt, int kps, TcRing& R) {
+// Default launch shape: one target per CTA, the fewest ring steps per source
+// whose two slots fit the budget, cut into equal steps.  A CTA waits for a
+// barrier round trip per step and for its promotions, so the number of CTAs per
+// SM is what counts: 224k-tet ball, p = 8, 256 states, two CTAs per SM 6.7 (two
+// k-steps per slot) and 5.7 ms (five), three CTAs 3.9 ms, four CTAs 3.65 ms (two
+// steps of three); four targets per CTA sharing the moments, two CTAs, 5.3 ms.
+// Three CTAs where the grid does not fill four per SM (473 targets, one state
+// block: 243 against 269 us).  nt / kps override it.
+void default_ring(const Plan& P, const TcLayout& G, int nt, int kps, TcRing& R) {
   if (nt == 0) nt = 1;
-  if (kps == 0) kps = std::min(G.KS, 2);
-  const int budget = (nt == 1 && G.tmem_cols <= 256) ? TC_BUDGET_2 : TC_BUDGET_1;
+  const int64_t work = (int64_t)P.h_m2l_targets.size() * ((P.opt.max_batch + TC_M - 1) / TC_M);
+  int budget = nt == 2 || G.tmem_cols > 256 ? TC_BUDGET_1
+               : P.tc_prom_rows > 16        ? TC_BUDGET_2  // 64 registers of promoted sums
+               : work <= 4 * 152            ? TC_BUDGET_3
+                                            : TC_BUDGET_4;
+  if (kps == 0) {
+    for (kps = G.KS; kps > 1 && !make_ring(G, nt, kps, budget, R); kps--) {
+    }
+    const int steps = (G.KS + kps - 1) / kps;
+    kps = (G.KS + steps - 1) / steps;
+  }
+  kps = std::min(kps, G.KS);
   for (; kps >= 1; kps--)
     if (make_ring(G, nt, kps, budget, R) || make_ring(G, nt, kps, TC_BUDGET_1, R)) return;
   R.nslots = 0;
+}
+
+void set_promotion(const Plan& P, const TcLayout& G, TcRing& R) {
+  R.prom_group = R.nt == 1 ? P.tc_prom_group : 0;
+  R.prom_chunks = R.nt == 1 ? std::min(std::min(4, G.nlp / 16), std::max(1, (P.tc_prom_rows + 15) / 16)) : 0;
 }
 
 // autotune: time every launch shape on the plan's own lists (zero moments,
@@ -809,12 +834,13 @@ void tune_ring(Plan& P, const TcLayout& G) {
   // default) the tuner keeps one target per CTA, whose accuracy it must not trade
   const int nt_max = P.tc_prom_group > 0 ? 1 : 2;
   for (int nt = 1; nt <= nt_max; nt++)
-    for (int budget : {TC_BUDGET_2, TC_BUDGET_1}) {
-      if (budget == TC_BUDGET_2 && (nt == 2 || G.tmem_cols > 256)) continue;  // one CTA per SM anyway
+    for (int budget : {TC_BUDGET_4, TC_BUDGET_3, TC_BUDGET_2, TC_BUDGET_1}) {
+      if (budget < TC_BUDGET_1 && (nt == 2 || G.tmem_cols > 256)) continue;  // one CTA per SM anyway
       for (int kps = 1; kps <= std::min(G.KS, 8); kps++) {
         TcRing R;
         if (!make_ring(G, nt, kps, budget, R)) continue;
         if (ring_smem(R) > 227 * 1024) continue;
+        set_promotion(P, G, R);
         launch_main(P, R, B, qp.p, L.p, err.p, s);  // warm-up
         DM_CUDA(cudaEventRecord(a, s));
         launch_main(P, R, B, qp.p, L.p, err.p, s);
@@ -839,9 +865,8 @@ void tune_ring(Plan& P, const TcLayout& G) {
 
 bool current_ring(const Plan& P, const TcLayout& G, TcRing& R) {
   if (!(P.tc_kps > 0 && make_ring(G, P.tc_nt, P.tc_kps, P.tc_budget, R)))
-    default_ring(G, P.opt.m2l_targets_per_cta, P.opt.m2l_kps, R);
-  R.prom_group = R.nt == 1 ? P.tc_prom_group : 0;
-  R.prom_chunks = std::min(std::min(4, G.nlp / 16), std::max(1, (P.tc_prom_rows + 15) / 16));
+    default_ring(P, G, P.opt.m2l_targets_per_cta, P.opt.m2l_kps, R);
+  set_promotion(P, G, R);
   return R.nslots >= 2;
 }
 
