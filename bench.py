@@ -304,14 +304,7 @@ def _alu_peak(kind, peaks, sm_mhz):
 # version; any other configuration reports null
 NCU_TRAFFIC = {
     # (stage, precision, p, leaf, batch, n_tets): bytes
-    # ball of 559,564 tets, 256 states, leaf 512 (the headline workload): one launch of k_m2l_tc
-    # (22.457 GB read + 0.469 GB written), ncu --metrics
-    # gpu__time_duration.sum,dram__bytes_read.sum,dram__bytes_write.sum on
-    # python bench.py --workload sphere500k --leaf 512 --autotune 1 --steps 1 --warmup 3
-    # --no-cpu-baseline --no-fp64-ref.  The same capture measured k_near_tc at 16.648 GB, but
-    # that kernel has changed since (the M of a column group copied per run of consecutive
-    # node ids), so its traffic is reported as unknown until it is captured again.
-    ("m2l", "bf16x3", 8, 512, 256, 559564): 22.926e9,
+    # none: the M2L and the near field have changed since their captures
 }
 
 

@@ -108,7 +108,8 @@ typedef struct {
                           source's moments in one CTA, 1 or 2; 0 = default
                           (1) or the autotuner's choice                     */
   int m2l_kps;         /* tensor-core M2L: k-steps per shared-memory slot,
-                          1..8; 0 = default (2) or the autotuner's choice.
+                          1..8; 0 = default (by order and grid) or the
+                          autotuner's choice.
                           Every launch shape gives bit-identical results.   */
   int m2l_promote;     /* tensor-core M2L, one target per CTA: every this
                           many sources the leading accumulator rows are
@@ -121,11 +122,12 @@ typedef struct {
   int m2l_promote_rows; /* rows moved (rounded up to 16, at most 64); 0 = 16 */
   int m2l_table_batch; /* TF32 / split BF16: batches B <= this run the M2L in
                           FP32 on CUDA cores, from a per-plan table of the
-                          translation derivatives (p in {4, 6, 8}); larger
+                          translation derivatives; larger
                           batches use the tensor cores, whose tiles hold 128
-                          states.  0 = default (8), < 0 = never.  The FP32
-                          precision always uses the table M2L when there is
-                          one.                                              */
+                          states.  0 = default (8), < 0 = never (FP64 plans:
+                          no table is built).  The FP32 precision and the
+                          orders without a tensor-core M2L use the table
+                          for every batch.                                  */
   int sources;         /* DEMAG_SOURCES_TETS (0): P1 magnetisation on the
                           tetrahedra, exact moments and analytic near field
                           (the paper's method); DEMAG_SOURCES_DIPOLES (1):
@@ -362,7 +364,7 @@ enum {
   DEMAG_STAGE_M2L = 3,
   DEMAG_STAGE_L2L = 4,
   DEMAG_STAGE_L2P = 5,
-  DEMAG_STAGE_NEAR_PREP = 6, /* per-tet records of the FP64 on-the-fly near field, one state */
+  DEMAG_STAGE_NEAR_PREP = 6, /* not used: the integrated near field's face charges count as P2P */
   DEMAG_STAGE_P2P = 7,
   DEMAG_STAGE_H = 8,         /* mass-lumped H and the output layout           */
   DEMAG_N_STAGES = 9

@@ -414,9 +414,10 @@ void launch_near_apply64(Plan& P, const double* Ms, int B, double* u_s, cudaStre
 void launch_near_apply32(Plan& P, const float* Ms, int B, float* u_s, int* err, cudaStream_t s);
 // tensor-core near field (near_tc.cu): used when the plan holds the tiles
 bool near_tc_wanted(const Plan& P);
-// MP: workspace of nf_mp_floats(P, B) floats for M in the layout of the kernel's bulk copies
+// MP: workspace of nf_mp_floats(P, B) floats for M in the layout of the kernel's bulk
+// copies (small batches: for partial sums); returns the kernel launches
 size_t nf_mp_floats(const Plan& P, int B);
-void launch_near_tc(Plan& P, const float* Ms, float* MP, int B, float* u_s, int* err, cudaStream_t s);
+int launch_near_tc(Plan& P, const float* Ms, float* MP, int B, float* u_s, int* err, cudaStream_t s);
 struct M2lKeys {  // distinct translation keys (dl, lattice offset); the key of every pair is P.m2l_op
   bool ok = false;
   std::vector<int4> keys;

@@ -198,8 +198,7 @@ void eval_mixed_ws(Plan& P, Workspace& W, const double* M, int B, double* u, dou
   } else {
     clk.begin(DEMAG_STAGE_P2P);
     if (P.nf_W) {
-      launch_near_tc(P, W.Ms32, W.MP, B, W.u32, W.err, s);
-      clk.launched();
+      clk.launched(launch_near_tc(P, W.Ms32, W.MP, B, W.u32, W.err, s));
     } else if (!P.h_p2p_targets.empty()) {
       launch_near_apply32(P, W.Ms32, B, W.u32, W.err, s);
       clk.launched();

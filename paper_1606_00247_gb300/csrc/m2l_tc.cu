@@ -198,7 +198,7 @@ struct TcRing {
 
 bool make_ring(const TcLayout& G, int nt, int kps, int budget, TcRing& R) {
   if (!G.valid || kps < 1 || kps > G.KS || nt < 1 || nt > 2) return false;
-  if (nt == 2 && (G.tmem_cols > 256 || G.ls == TC_LS_ALL3)) return false;  // two accumulators in 512 columns
+  if (nt == 2 && (G.nq > nq_of(8) || G.ls == TC_LS_ALL3)) return false;  // two targets: orders up to 8, two limbs
   R = TcRing{};
   R.nt = nt;
   R.kps = kps;
@@ -745,7 +745,7 @@ void launch_fixed(Plan& P, const TcRing& R, int B, const unsigned char* QP, floa
 // split BF16 with one target per CTA
 template <int PP, bool BF16, int LS>
 void launch_ls(Plan& P, const TcRing& R, int B, const unsigned char* QP, float* L, int* err, cudaStream_t s) {
-  if constexpr (tc_layout(PP, BF16, LS).tmem_cols <= 256) {
+  if constexpr (PP <= 8) {
     if (R.nt == 2) return launch_fixed<PP, BF16, 2, LS, 1>(P, R, B, QP, L, err, s);
   }
   if (R.prom_chunks > 1) return launch_fixed<PP, BF16, 1, LS, 4>(P, R, B, QP, L, err, s);
@@ -912,7 +912,7 @@ void build_m2l_tc(Plan& P, const M2lKeys& K) {
   DM_CUDA(cudaMemcpyAsync(P.tc_g1_off, g1.data(), (nT + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
   // groups of two consecutive targets, where one may run: the union of their (ascending) lists
   const bool pairs = P.opt.m2l_targets_per_cta == 2 || ((P.opt.autotune & 1) && P.tc_prom_group == 0);
-  if (pairs && G.tmem_cols <= 256) {
+  if (pairs && G.nq <= nq_of(8)) {
     std::vector<int32_t> src(P.n_m2l), op(P.n_m2l);
     DM_CUDA(cudaMemcpyAsync(src.data(), P.m2l_src, src.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     DM_CUDA(cudaMemcpyAsync(op.data(), P.m2l_op, op.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, s));

@@ -43,6 +43,8 @@
 // Every wait is bounded: on expiry the kernel records DEMAG_ERR_TIMEOUT,
 // stops issuing, waits (bounded) for its own copies and MMAs in flight, frees
 // its tensor memory and returns.
+#include <algorithm>
+
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
@@ -387,14 +389,157 @@ __global__ void __launch_bounds__(NF_THREADS, 1)
   if (warp == 2) tmem_dealloc(tmem, NF_TMEM_COLS);
 }
 
+// Batches of at most NFS_MAX states: the tensor-core tile holds 128 states, so a
+// small batch paid for the whole tile (its M, its conversions).  Here the same
+// stored coefficients are streamed by CUDA cores in FP32: W = W_hi + W_lo (exact),
+// M unrounded.  CTA of 256 threads per (tile, part of its column groups): thread =
+// (row, half of a group's 16 columns), six coalesced 16-byte loads per group (hi
+// and lo of three components), M of the group's columns as shared-memory
+// broadcasts for SB states.  A tile is cut into parts so that every SM holds
+// several CTAs; the parts' sums go to `part` and are added in order by
+// k_near_tc_sum, so results do not depend on timing.  Bound by the stream of W
+// (12 B per stored coefficient, 2.5 GB on the 224k-tet ball, 298 tiles).  Measured
+// there against the tensor-core kernel (815 - 830 us up to 128 states): 1 / 4 / 8
+// / 16 states 403 (6.2 TB/s) / 436 / 542 / 842 us; 29k tets (42 tiles, which leave
+// two thirds of the SMs without a tensor-core CTA, 310 us): 46 us for one, 92 us
+// for sixteen states.  Errors against FP64 fall too (u 1.0e-6 -> 3.8e-7, film
+// 2.0e-5 -> 1.1e-5): M is not rounded to 16 bits.
+constexpr int NFS_THREADS = 256;
+constexpr int NFS_SLICE = 16, NFS_MAX = 64;  // states per pass over W, largest batch
+
+// Up to 8 states always; larger batches while their passes of 16 states over the
+// tiles cost less than the tensor-core kernel's waves of one CTA per SM (a pass
+// takes about as long as the tensor cores on a full grid)
+bool small_batch(int64_t ntiles, int B) {
+  const int64_t slices = (B + NFS_SLICE - 1) / NFS_SLICE, waves = (ntiles + 151) / 152;
+  return B <= 8 || (B <= NFS_MAX && 10 * slices * ntiles <= 9 * 152 * waves);
+}
+
+template <int SB>
+__global__ void __launch_bounds__(NFS_THREADS, SB <= 8 ? 4 : 3)
+    k_near_tc_small(const int32_t* __restrict__ order, const int64_t* __restrict__ woff,
+                    const int64_t* __restrict__ coff, const int32_t* __restrict__ ngrp,
+                    const int32_t* __restrict__ npad_t, const int32_t* __restrict__ cols,
+                    const unsigned char* __restrict__ W, const float* __restrict__ Ms, int B, int parts, float* part) {
+  __shared__ __align__(16) float sM[2][48 * SB];  // [half][component][8 columns][state]
+  const int64_t tile = order[blockIdx.x];
+  const int npad = npad_t[tile], ng = ngrp[tile], b0 = blockIdx.z * SB;
+  const int g0 = (int)((int64_t)ng * blockIdx.y / parts), g1 = (int)((int64_t)ng * (blockIdx.y + 1) / parts);
+  const int tid = threadIdx.x, row = tid & 127, half = tid >> 7;
+  const bool on = row < npad;
+  const int kbytes = 64 * npad, limb = 32 * npad;
+  const unsigned char* w = W + woff[tile] + (int64_t)g0 * 3 * kbytes + (row >> 3) * 256 + half * 128 + (row & 7) * 16;
+  const int32_t* ct = cols + coff[tile];
+  // this thread's value(s) of a group's M: q = ((half * 3 + component) * 8 + column) * SB + state
+  constexpr int NM = (48 * SB + NFS_THREADS - 1) / NFS_THREADS;
+  float m[NM];
+  auto load_m = [&](int g) {
+#pragma unroll
+    for (int r = 0; r < NM; r++) {
+      const int q = tid + r * NFS_THREADS, v = q % SB, j = (q / SB) % 8, hc = q / (8 * SB);
+      m[r] = q < 48 * SB && b0 + v < B ? Ms[((int64_t)ct[16 * g + 8 * (hc / 3) + j] * 3 + hc % 3) * B + b0 + v] : 0.f;
+    }
+  };
+  float acc[SB];
+#pragma unroll
+  for (int v = 0; v < SB; v++) acc[v] = 0.f;
+  if (g0 < g1) load_m(g0);
+  for (int g = g0; g < g1; g++, w += 3 * kbytes) {
+    float* buf = sM[(g - g0) & 1];
+    uint4 hi[3], lo[3];
+    if (on)
+#pragma unroll
+      for (int c = 0; c < 3; c++) {
+        hi[c] = __ldcs((const uint4*)(w + c * kbytes));
+        lo[c] = __ldcs((const uint4*)(w + c * kbytes + limb));
+      }
+#pragma unroll
+    for (int r = 0; r < NM; r++)
+      if (tid + r * NFS_THREADS < 48 * SB) buf[tid + r * NFS_THREADS] = m[r];
+    if (g + 1 < g1) load_m(g + 1);
+    __syncthreads();  // this group's M is staged; the buffer of the group before it is free after the next barrier
+    if (on) {
+      const float* mb = buf + half * 24 * SB;
+#pragma unroll
+      for (int c = 0; c < 3; c++) {
+        const uint32_t h4[4] = {hi[c].x, hi[c].y, hi[c].z, hi[c].w}, l4[4] = {lo[c].x, lo[c].y, lo[c].z, lo[c].w};
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+          const uint32_t h = j & 1 ? h4[j >> 1] & 0xffff0000u : h4[j >> 1] << 16;
+          const uint32_t l = j & 1 ? l4[j >> 1] & 0xffff0000u : l4[j >> 1] << 16;
+          const float wv = __uint_as_float(h) + __uint_as_float(l);
+#pragma unroll
+          for (int v = 0; v < SB; v++) acc[v] = fmaf(wv, mb[(c * 8 + j) * SB + v], acc[v]);
+        }
+      }
+    }
+  }
+  __syncthreads();
+  __shared__ float red[128 * SB];
+  if (half == 1)
+#pragma unroll
+    for (int v = 0; v < SB; v++) red[row * SB + v] = acc[v];
+  __syncthreads();
+  if (half == 0 && on) {
+    float* out = part + ((tile * parts + blockIdx.y) * NF_ROWS + row) * B + b0;
+#pragma unroll
+    for (int v = 0; v < SB; v++)
+      if (b0 + v < B) out[v] = acc[v] + red[row * SB + v];
+  }
+}
+
+__global__ void k_near_tc_sum(int64_t n, const int32_t* __restrict__ rownode, const int32_t* __restrict__ ngrp, int B,
+                              int parts, const float* __restrict__ part, float* u) {
+  const int64_t it = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // (tile, row, state)
+  if (it >= n) return;
+  const int64_t r = it / B, tile = r / NF_ROWS;
+  const int b = (int)(it - r * B), node = rownode[r];
+  if (node < 0 || ngrp[tile] == 0) return;
+  const float* p = part + ((tile * parts) * NF_ROWS + r - tile * NF_ROWS) * B + b;
+  float v = 0.f;
+  for (int k = 0; k < parts; k++) v += p[(int64_t)k * NF_ROWS * B];
+  u[(int64_t)node * B + b] += v;
+}
+
+template <int SB>
+void launch_small(Plan& P, const float* Ms, float* part, int B, int parts, float* u_s, cudaStream_t s) {
+  const dim3 grid((unsigned)P.nf_ntiles, (unsigned)parts, (unsigned)((B + SB - 1) / SB));
+  k_near_tc_small<SB><<<grid, NFS_THREADS, 0, s>>>(
+      P.nf_order, P.nf_woff, P.nf_coff, P.nf_ng, P.nf_npad, P.nf_cols, P.nf_W, Ms, B, parts, part);
+  DM_LAUNCH("k_near_tc_small");
+  const int64_t n = P.nf_ntiles * NF_ROWS * B;
+  k_near_tc_sum<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, P.nf_rownode, P.nf_ng, B, parts, part, u_s);
+  DM_LAUNCH("k_near_tc_sum");
+}
+
 }  // namespace
 
 size_t nf_mp_floats(const Plan& P, int B) {
   return P.nf_W ? (size_t)((B + 127) / 128) * (size_t)P.nn * 384 : 0;
 }
 
-void launch_near_tc(Plan& P, const float* Ms, float* MP, int B, float* u_s, int* err, cudaStream_t s) {
-  if (P.nf_ntiles == 0) return;
+int launch_near_tc(Plan& P, const float* Ms, float* MP, int B, float* u_s, int* err, cudaStream_t s) {
+  if (P.nf_ntiles == 0) return 0;
+  if (small_batch(P.nf_ntiles, B) && !(P.debug_flags & 1)) {
+    // parts: ~6 CTAs per SM, at least four column groups each on average, the
+    // sums within MP (whose copy of M this kernel does not use)
+    const int64_t room = (int64_t)nf_mp_floats(P, B) / (P.nf_ntiles * NF_ROWS * B);
+    const int64_t want = std::min<int64_t>((6 * 152 + P.nf_ntiles - 1) / P.nf_ntiles, P.nf_ncols / 64 / P.nf_ntiles);
+    const int parts = (int)std::max<int64_t>(1, std::min(want, room));
+    if (room >= 1) {
+      if (B == 1)
+        launch_small<1>(P, Ms, MP, B, parts, u_s, s);
+      else if (B == 2)
+        launch_small<2>(P, Ms, MP, B, parts, u_s, s);
+      else if (B <= 4)
+        launch_small<4>(P, Ms, MP, B, parts, u_s, s);
+      else if (B <= 8)
+        launch_small<8>(P, Ms, MP, B, parts, u_s, s);
+      else
+        launch_small<16>(P, Ms, MP, B, parts, u_s, s);
+      return 2;
+    }
+  }
   smem_opt_in((const void*)k_near_tc, NF_SMEM);
   const unsigned nsb = (unsigned)((B + 127) / 128);
   k_nf_pack_m<<<dim3((unsigned)P.nn, nsb), 128, 0, s>>>(P.nn, B, Ms, MP);
@@ -411,6 +556,7 @@ void launch_near_tc(Plan& P, const float* Ms, float* MP, int B, float* u_s, int*
   k_near_tc<<<grid, NF_THREADS, NF_SMEM, s>>>(order, P.nf_woff, P.nf_coff, P.nf_ng, P.nf_npad, P.nf_rownode, P.nf_cols,
                                               P.nf_W, MP, P.nf_S, P.nn, B, (int)nsb, u_s, err, P.debug_flags & 1);
   DM_LAUNCH("k_near_tc");
+  return 2;
 }
 
 }  // namespace demag
