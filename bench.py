@@ -217,9 +217,9 @@ def m2l_macs(p):
 
 
 def m2l_split_degree(p):
-    """The library's default split degree of the tensor-core M2L: the products
-    with the second BF16 limb only for terms |m| + |n| <= p - 4 (p - 3 below
-    order 8)."""
+    """The default split degree of an M2L on all multi-indices (m2l_tile_flops):
+    the products with the second BF16 limb only for terms |m| + |n| <= p - 4
+    (p - 3 below order 8)."""
     return p - 4 if p >= 8 else p - 3
 
 

@@ -12,15 +12,16 @@ static inline int nblk(int64_t n, int t) { return (int)((n + t - 1) / t > 0 ? (n
 // input / output layout
 // ---------------------------------------------------------------------------
 // Ms[(i*3+c)*B + b] = M[(b*nn + perm[i])*3 + c]
-// block per (sorted node, 128 states), thread = state: stores coalesce over states
-__global__ void __launch_bounds__(128) k_gather_M(int64_t nn, int B, const int32_t* __restrict__ perm,
+// thread per (sorted node, state), the states of a node side by side: stores coalesce over states
+__global__ void __launch_bounds__(256) k_gather_M(int64_t nn, int B, const int32_t* __restrict__ perm,
                                                   const double* __restrict__ M, double* Ms) {
-  const int64_t i = blockIdx.x;
-  const int b = blockIdx.y * 128 + threadIdx.x;
-  if (b >= B) return;
-  const int64_t g = perm[i];
+  const int64_t it = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (it >= nn * B) return;
+  const int64_t i = it / B;
+  const int b = (int)(it - i * B);
+  const double* src = M + ((int64_t)b * nn + perm[i]) * 3;
 #pragma unroll
-  for (int c = 0; c < 3; c++) Ms[(i * 3 + c) * B + b] = M[((int64_t)b * nn + g) * 3 + c];
+  for (int c = 0; c < 3; c++) Ms[(i * 3 + c) * B + b] = src[c];
 }
 
 // ---------------------------------------------------------------------------
@@ -152,7 +153,7 @@ void eval_fp64_ws(Plan& P, Workspace& W, const double* M, int B, double* u, doub
   const bool dev = eval_io_begin(P, W, M, B, u, H, &Md, &ud, &Hd, s);
   StageClock clk(P, s, profile_ok);
   clk.begin(DEMAG_STAGE_GATHER);
-  k_gather_M<<<dim3((unsigned)P.nn, (unsigned)((B + 127) / 128)), 128, 0, s>>>(P.nn, B, P.node_perm, Md, W.Ms);
+  k_gather_M<<<nblk(P.nn * B, 256), 256, 0, s>>>(P.nn, B, P.node_perm, Md, W.Ms);
   DM_LAUNCH("k_gather_M");
   clk.launched();
   clk.end();
@@ -206,7 +207,7 @@ void near_field_fp64(Plan& P, Workspace& W, int B, StageClock& clk, cudaStream_t
 }
 
 void launch_gather_M(Plan& P, const double* M, int B, double* Ms, cudaStream_t s) {
-  k_gather_M<<<dim3((unsigned)P.nn, (unsigned)((B + 127) / 128)), 128, 0, s>>>(P.nn, B, P.node_perm, M, Ms);
+  k_gather_M<<<nblk(P.nn * B, 256), 256, 0, s>>>(P.nn, B, P.node_perm, M, Ms);
   DM_LAUNCH("k_gather_M");
 }
 

@@ -18,16 +18,17 @@ static inline int nblk(int64_t n, int t) { return (int)((n + t - 1) / t > 0 ? (n
 namespace {
 
 // M (state, original node, component) -> Ms (sorted node, component, state):
-// block per (sorted node, 128 states), thread = state, so the stores coalesce
-// over the states; each thread reads the 24 contiguous bytes of its state's
-// (node, x y z) row
-__global__ void __launch_bounds__(128) k_gather_M32(int64_t nn, int B, const int32_t* __restrict__ perm,
+// thread per (sorted node, state), the states of a node side by side, so the
+// stores coalesce over the states; each thread reads the 24 contiguous bytes of
+// its state's (node, x y z) row.  (A block of 128 threads per node left all but B
+// of them idle: 72 -> 11 us for 126k nodes and two states; 256 states of 36k nodes 109 -> 112 us.)
+__global__ void __launch_bounds__(256) k_gather_M32(int64_t nn, int B, const int32_t* __restrict__ perm,
                                                     const double* __restrict__ M, float* Ms, double* Ms64) {
-  const int64_t i = blockIdx.x;
-  const int b = blockIdx.y * 128 + threadIdx.x;
-  if (b >= B) return;
-  const int64_t g = perm[i];
-  const double* src = M + ((int64_t)b * nn + g) * 3;
+  const int64_t it = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (it >= nn * B) return;
+  const int64_t i = it / B;
+  const int b = (int)(it - i * B);
+  const double* src = M + ((int64_t)b * nn + perm[i]) * 3;
 #pragma unroll
   for (int c = 0; c < 3; c++) {
     const double v = src[c];
@@ -79,6 +80,35 @@ __global__ void __launch_bounds__(256) k_out32(int64_t nn, int B, const int32_t*
       const int bl = q / 96, rr = q - bl * 96;
       if (b0 + bl < B && g0 + rr / 3 < nn) H_out[((int64_t)(b0 + bl) * nn + g0) * 3 + rr] = (double)sh[bl][rr];
     }
+}
+
+// the same for a few states (OUT_SMALL_BATCH): thread per (state, original node),
+// consecutive threads on consecutive nodes, so the stores of u and H coalesce.
+// (The 32-state tiles above are mostly empty then: 64 -> 29 us for 126k
+// nodes and two states.)
+constexpr int OUT_SMALL_BATCH = 8;
+__global__ void __launch_bounds__(256) k_out32_small(int64_t nn, int B, const int32_t* __restrict__ iperm,
+                                                     const int64_t* __restrict__ hoff, const int32_t* __restrict__ hcol,
+                                                     const float4* __restrict__ hw, const float* __restrict__ u32,
+                                                     double* u_out, double* H_out) {
+  const int64_t it = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (it >= nn * B) return;
+  const int b = (int)(it / nn);
+  const int64_t i = iperm[it - (int64_t)b * nn];
+  u_out[it] = (double)u32[i * B + b];
+  if (!H_out) return;
+  float hx = 0.f, hy = 0.f, hz = 0.f;
+#pragma unroll 4
+  for (int64_t e = hoff[i], e1 = hoff[i + 1]; e < e1; e++) {
+    const float4 wv = hw[e];
+    const float uj = u32[(int64_t)hcol[e] * B + b];
+    hx = fmaf(wv.x, uj, hx);
+    hy = fmaf(wv.y, uj, hy);
+    hz = fmaf(wv.z, uj, hz);
+  }
+  H_out[3 * it] = (double)hx;
+  H_out[3 * it + 1] = (double)hy;
+  H_out[3 * it + 2] = (double)hz;
 }
 
 __global__ void k_u32_to_64(int64_t n, const float* __restrict__ a, double* b) {
@@ -159,8 +189,7 @@ void eval_mixed_ws(Plan& P, Workspace& W, const double* M, int B, double* u, dou
   const int nq = P.nq, nl = P.nl;
   StageClock clk(P, s, profile_ok);
   clk.begin(DEMAG_STAGE_GATHER);
-  k_gather_M32<<<dim3((unsigned)P.nn, (unsigned)((B + 127) / 128)), 128, 0, s>>>(P.nn, B, P.node_perm, Md, W.Ms32,
-                                                                                 otf ? W.Ms : nullptr);
+  k_gather_M32<<<nblk(P.nn * B, 256), 256, 0, s>>>(P.nn, B, P.node_perm, Md, W.Ms32, otf ? W.Ms : nullptr);
   DM_LAUNCH("k_gather_M32");
   clk.launched();
   clk.end();
@@ -208,6 +237,9 @@ void eval_mixed_ws(Plan& P, Workspace& W, const double* M, int B, double* u, dou
   clk.begin(DEMAG_STAGE_H);
   if (otf) {
     launch_lumped_H_out(P, B, W.u_s, ud, Hd, s);  // FP64 near field: u in FP64
+  } else if (B <= OUT_SMALL_BATCH) {
+    k_out32_small<<<nblk(P.nn * B, 256), 256, 0, s>>>(P.nn, B, P.node_iperm, P.hg_off, P.hg_col, P.hg_w, W.u32, ud, Hd);
+    DM_LAUNCH("k_out32_small");
   } else {
     k_out32<<<dim3((unsigned)((P.nn + 31) / 32), (unsigned)((B + 31) / 32)), 256, 0, s>>>(
         P.nn, B, P.node_iperm, P.hg_off, P.hg_col, P.hg_w, W.u32, ud, Hd);
