@@ -20,14 +20,31 @@ namespace {
 // M (state, original node, component) -> Ms (sorted node, component, state):
 // thread per (sorted node, state), the states of a node side by side, so the
 // stores coalesce over the states; each thread reads the 24 contiguous bytes of
-// its state's (node, x y z) row.  (A block of 128 threads per node left all but B
-// of them idle: 72 -> 11 us for 126k nodes and two states; 256 states of 36k nodes 109 -> 112 us.)
+// its state's (node, x y z) row.  (A block of 128 threads per node leaves all but B
+// of them idle: 72 -> 11 us for 126k nodes and two states.)
 __global__ void __launch_bounds__(256) k_gather_M32(int64_t nn, int B, const int32_t* __restrict__ perm,
                                                     const double* __restrict__ M, float* Ms, double* Ms64) {
   const int64_t it = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (it >= nn * B) return;
   const int64_t i = it / B;
   const int b = (int)(it - i * B);
+  const double* src = M + ((int64_t)b * nn + perm[i]) * 3;
+#pragma unroll
+  for (int c = 0; c < 3; c++) {
+    const double v = src[c];
+    Ms[(i * 3 + c) * B + b] = (float)v;
+    if (Ms64) Ms64[(i * 3 + c) * B + b] = v;
+  }
+}
+
+// From GATHER_WIDE states on: block per (sorted node, 128 states), thread = state
+// (no division per thread: 256 states of 87k nodes 297 us, 399 with the kernel above)
+constexpr int GATHER_WIDE = 64;
+__global__ void __launch_bounds__(128) k_gather_M32_wide(int64_t nn, int B, const int32_t* __restrict__ perm,
+                                                         const double* __restrict__ M, float* Ms, double* Ms64) {
+  const int64_t i = blockIdx.x;
+  const int b = blockIdx.y * 128 + threadIdx.x;
+  if (b >= B) return;
   const double* src = M + ((int64_t)b * nn + perm[i]) * 3;
 #pragma unroll
   for (int c = 0; c < 3; c++) {
@@ -189,7 +206,11 @@ void eval_mixed_ws(Plan& P, Workspace& W, const double* M, int B, double* u, dou
   const int nq = P.nq, nl = P.nl;
   StageClock clk(P, s, profile_ok);
   clk.begin(DEMAG_STAGE_GATHER);
-  k_gather_M32<<<nblk(P.nn * B, 256), 256, 0, s>>>(P.nn, B, P.node_perm, Md, W.Ms32, otf ? W.Ms : nullptr);
+  if (B >= GATHER_WIDE)
+    k_gather_M32_wide<<<dim3((unsigned)P.nn, (unsigned)((B + 127) / 128)), 128, 0, s>>>(P.nn, B, P.node_perm, Md,
+                                                                                        W.Ms32, otf ? W.Ms : nullptr);
+  else
+    k_gather_M32<<<nblk(P.nn * B, 256), 256, 0, s>>>(P.nn, B, P.node_perm, Md, W.Ms32, otf ? W.Ms : nullptr);
   DM_LAUNCH("k_gather_M32");
   clk.launched();
   clk.end();
