@@ -301,7 +301,6 @@ struct Plan {
   // clusters of source tets of the integrated near field (near_mode 0; p2p.cu):
   // distinct vertices, edges and faces of at most 40 tets of one source leaf
   int64_t n_clusters = 0, n_cl_v = 0, n_cl_e = 0, n_cl_f = 0, n_cl_b = 0;
-  int p2p_max_nodes = 0;            // most target nodes of a P2P target leaf
   int32_t* cl_off = nullptr;        // ncells + 1: clusters of every cell
   int4* cl_cnt = nullptr;           // vertices, edges, faces, boundary faces (which come first)
   int4* cl_pos = nullptr;           // first of each in the arrays below
@@ -314,6 +313,8 @@ struct Plan {
   int64_t n_pc = 0;
   int64_t* pc_off = nullptr;        // per P2P target: its source clusters
   int32_t* pc_src = nullptr;
+  int64_t n_pc_blk = 0;
+  int4* pc_blk = nullptr;           // the near field's blocks: P2P target, first sorted node, nodes, 0
 
   std::vector<DevBuf> bufs;
   int64_t device_bytes = 0;

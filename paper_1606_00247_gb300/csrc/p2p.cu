@@ -30,6 +30,7 @@
 // 0.9 - 7.5e-15 (the tet-wise form 1.2 - 10e-15 batched, 2 - 18e-15 for one
 // state), smooth M with 10 % noise 4.8 - 9.4e-15 (4.8 - 7.4e-15, 8 - 15e-15).
 #include <algorithm>
+#include <utility>
 #include <vector>
 
 #include "common.cuh"
@@ -134,6 +135,8 @@ void build_tet_geometry(Plan& P) {
 // ---------------------------------------------------------------------------
 namespace {
 
+constexpr int PF_G = 16, PF_GMIN = 4;         // target nodes of a near-field block: most, and least of a split leaf
+constexpr double PF_SPLIT = 4.0;
 constexpr int CL_TETS = 40;              // tets per cluster
 constexpr int CL_V = 4 * CL_TETS, CL_E = 6 * CL_TETS, CL_F = 4 * CL_TETS;  // bounds of its parts
 constexpr int FACE_REC = 16;             // doubles per face: n (3), m_e (9), 2 area, m_0.m_1, m_1.m_2, m_2.m_0
@@ -326,6 +329,42 @@ __global__ void k_cluster_lists(const int32_t* __restrict__ targets, const int64
   }
 }
 
+// The near field's blocks, heaviest first: {P2P target, first target node, nodes, 0}.
+// A block's time is its targets times its list, and the lists of an octree's
+// leaves differ several times in length: 16 nodes per block in leaf order left
+// the SMs busy for 48% of the kernel on the 16k-tet ball (708 blocks, the SMs'
+// active cycles 14 to 93 million).  A target leaf whose 16 nodes cost more than
+// 1/PF_SPLIT of the mean share of a resident block takes 8 or 4 at a time: the
+// evaluation 46.4 -> 19.9 ms.  Clusters staged for fewer targets cost little, the
+// FP64 arithmetic is the bound; below 4 targets a warp would read 16 records a step.
+std::vector<int4> face_blocks(const Plan& P, const std::vector<int64_t>& clusters) {
+  const int64_t nT = (int64_t)clusters.size();
+  double total = 0;
+  for (int64_t t = 0; t < nT; t++) {
+    const int4 r = P.h_range[P.h_p2p_targets[t]];
+    total += (double)clusters[t] * (r.w - r.z);
+  }
+  int dev = 0, sms = 0;
+  DM_CUDA(cudaGetDevice(&dev));
+  DM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const double most = total / (2.0 * sms * PF_SPLIT);  // two blocks per SM
+  std::vector<std::pair<double, int4>> q;
+  for (int64_t t = 0; t < nT; t++) {
+    const int4 r = P.h_range[P.h_p2p_targets[t]];
+    int g = PF_G;
+    while (g > PF_GMIN && (double)clusters[t] * g > most) g /= 2;
+    for (int i = r.z; i < r.w; i += g) {
+      const int n = std::min(g, r.w - i);
+      q.emplace_back((double)clusters[t] * n, make_int4((int)t, i, n, 0));
+    }
+  }
+  std::stable_sort(q.begin(), q.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+  std::vector<int4> o;
+  o.reserve(q.size());
+  for (const auto& x : q) o.push_back(x.second);
+  return o;
+}
+
 }  // namespace
 
 void build_clusters(Plan& P) {
@@ -345,8 +384,6 @@ void build_clusters(Plan& P) {
     off[c + 1] = (int32_t)range.size();
   }
   P.n_clusters = (int64_t)range.size();
-  P.p2p_max_nodes = 0;
-  for (int32_t c : P.h_p2p_targets) P.p2p_max_nodes = std::max(P.p2p_max_nodes, P.h_range[c].w - P.h_range[c].z);
   if (P.n_clusters == 0) return;
   int2* drange = dalloc<int2>(P, range.size());
   int4* dcnt = dalloc<int4>(P, range.size());
@@ -401,6 +438,11 @@ void build_clusters(Plan& P) {
     k_cluster_lists<true><<<(unsigned)nT, 32, 0, s>>>(P.p2p_targets, P.p2p_off, P.p2p_src, P.cl_off, nullptr, P.pc_off,
                                                       P.pc_src);
     DM_LAUNCH("k_cluster_lists");
+    const std::vector<int4> blk = face_blocks(P, hc);
+    P.n_pc_blk = (int64_t)blk.size();
+    P.pc_blk = dalloc<int4>(P, std::max<size_t>(blk.size(), 1));
+    DM_CUDA(cudaMemcpyAsync(P.pc_blk, blk.data(), blk.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
+    DM_CUDA(cudaStreamSynchronize(s));  // the host lists end here
   }
   DM_CUDA(cudaStreamSynchronize(s));
   dfree(P, drange);
@@ -463,7 +505,7 @@ __global__ void k_face_charge(int64_t ncl, const int4* __restrict__ cnt, const i
 }
 
 // ---------------------------------------------------------------------------
-// The near field: one block per (target leaf, 16 of its nodes) and FS states.
+// The near field: one block per entry of face_blocks (up to 16 nodes of a target leaf) and FS states.
 // Batches of whole clusters (as many as fit the shared-memory arrays) are
 // staged; thread = (target i, subset of the entities), so a warp reads one or
 // two records per step (broadcast) for 16 targets, and keeps its target's FS
@@ -471,12 +513,13 @@ __global__ void k_face_charge(int64_t ncl, const int4* __restrict__ cnt, const i
 // The subsets are added in order at the end: no atomics, the result does not
 // depend on timing.  FP64 arithmetic is the bound (2 FMA per clock and SM), so
 // records are read from shared memory instead of being recomputed.  Measured:
-// 16k-tet ball, leaf 128, 3 states 196 -> 45 ms; 3,072-tet cube, leaf 32, one
-// state 5.2 -> 1.1 ms (the tet-wise kernels before: 4 sqrt, 6 log1p, 4 atan2 and
-// 6 divisions per pair, 16-state slices whatever the batch, one warp per target
-// leaf for one state).
+// 16k-tet ball, leaf 128, 3 states 196 -> 45 ms with 16 nodes per block in leaf
+// order, and an evaluation 46.4 -> 19.9 ms with face_blocks; 3,072-tet cube, leaf
+// 32, one state 5.2 -> 1.1 ms, an evaluation 1.26 -> 1.06 ms (the tet-wise kernels
+// before: 4 sqrt, 6 log1p, 4 atan2 and 6 divisions per pair, 16-state slices
+// whatever the batch, one warp per target leaf for one state).
 // ---------------------------------------------------------------------------
-constexpr int PF_THREADS = 256, PF_G = 16, PF_BATCH = 32;
+constexpr int PF_THREADS = 256, PF_BATCH = 32;
 constexpr int PF_V = CL_V, PF_E = CL_E, PF_F = CL_F;  // capacities of a batch: any one cluster fits
 
 template <int FS>
@@ -487,8 +530,8 @@ constexpr size_t pf_smem() {
 
 template <int FS>
 __global__ void __launch_bounds__(PF_THREADS) k_p2p_faces(
-    const int32_t* __restrict__ targets, const int4* __restrict__ range, const int64_t* __restrict__ pc_off,
-    const int32_t* __restrict__ pc_src, const double* __restrict__ nodes_s, const int4* __restrict__ cnt,
+    const int4* __restrict__ blk, const int64_t* __restrict__ pc_off, const int32_t* __restrict__ pc_src,
+    const double* __restrict__ nodes_s, const int4* __restrict__ cnt,
     const int4* __restrict__ pos, const int32_t* __restrict__ vnode, const uint32_t* __restrict__ edge,
     const double* __restrict__ elen, const double* __restrict__ frec, const uint2* __restrict__ fidx,
     const double* __restrict__ D, const double* __restrict__ S, int B, int b0, double* u_s) {
@@ -506,11 +549,9 @@ __global__ void __launch_bounds__(PF_THREADS) k_p2p_faces(
   __shared__ int4 tot;                                       // of the batch: vertices, edges, faces, boundary faces
   __shared__ int nb;
   const int tid = threadIdx.x, lane = tid & 31;
-  const int64_t ti = blockIdx.x;
-  const int4 rT = range[targets[ti]];
-  const int i0 = rT.z + PF_G * blockIdx.y;
-  if (i0 >= rT.w) return;  // uniform over the block
-  const int nt = min(PF_G, rT.w - i0);
+  const int4 bk = blk[blockIdx.x];
+  const int64_t ti = bk.x;
+  const int i0 = bk.y, nt = bk.z;
   int lg = 0;
   while ((1 << lg) < nt) lg++;
   const int G = 1 << lg, i = tid & (G - 1), sub = tid >> lg, nsub = PF_THREADS >> lg;
@@ -684,10 +725,10 @@ void launch_slice(Plan& P, const double* Ms, double* state, int B, int b0, doubl
                                                            P.cl_fidx, Ms, B, b0, S);
   DM_LAUNCH("k_face_charge");
   smem_opt_in((const void*)k_p2p_faces<FS>, pf_smem<FS>());
-  const dim3 grid((unsigned)P.h_p2p_targets.size(), (unsigned)((P.p2p_max_nodes + PF_G - 1) / PF_G));
-  k_p2p_faces<FS><<<grid, PF_THREADS, pf_smem<FS>(), s>>>(P.p2p_targets, P.cell_range, P.pc_off, P.pc_src, P.nodes_s,
-                                                          P.cl_cnt, P.cl_pos, P.cl_vnode, P.cl_edge, P.cl_elen,
-                                                          P.cl_frec, P.cl_fidx, D, S, B, b0, u_s);
+  k_p2p_faces<FS><<<(unsigned)P.n_pc_blk, PF_THREADS, pf_smem<FS>(), s>>>(P.pc_blk, P.pc_off, P.pc_src, P.nodes_s,
+                                                                         P.cl_cnt, P.cl_pos, P.cl_vnode, P.cl_edge,
+                                                                         P.cl_elen, P.cl_frec, P.cl_fidx, D, S, B, b0,
+                                                                         u_s);
   DM_LAUNCH("k_p2p_faces");
 }
 
@@ -696,7 +737,7 @@ void launch_slice(Plan& P, const double* Ms, double* state, int B, int b0, doubl
 size_t face_state_doubles(const Plan& P, int slice) { return (size_t)slice * (size_t)(P.n_cl_f + 3 * P.n_cl_b); }
 
 int launch_p2p_fp64(Plan& P, const double* Ms, double* state, int slice, int B, double* u_s, cudaStream_t s) {
-  if (P.h_p2p_targets.empty() || P.n_clusters == 0) return 0;
+  if (P.n_pc_blk == 0 || P.n_clusters == 0) return 0;
   static_assert(pf_smem<16>() <= 227 * 1024, "shared memory of the near-field kernel");
   int n = 0;
   for (int b0 = 0; b0 < B; n += 3) {

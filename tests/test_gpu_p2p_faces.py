@@ -57,3 +57,16 @@ def test_overlapping_tets_are_summed(orc):
     M = inputs.gaussian_unit_m(nodes.shape[0], batch=1, seed=5)
     u = _u(nodes, t, M, p=1, leaf_size=100000)
     assert rel_l2(u[0], orc.direct(nodes, t, M[0])) < 1e-12
+
+
+# blocks of 4, 8 and 16 targets (by the share of the mesh a leaf's 16 nodes are), remainders in all;
+# the stored near field integrates tet by tet, the far field is the same
+@pytest.mark.parametrize("n, leaf", [(18, 20), (24, 32), (30, 32)])
+def test_block_sizes_vs_stored(n, leaf):
+    from paper_1606_00247_gb300.api import Plan
+
+    nodes, tets = inputs.unit_cube(n)
+    M = torch.as_tensor(inputs.gaussian_unit_m(nodes.shape[0], batch=2, seed=n), device="cuda")
+    u = [Plan(nodes, tets, precision="fp64", near_mode=k, theta=0.5, p=3, leaf_size=leaf, max_batch=2)
+         .eval(M)[0].cpu().numpy() for k in (0, 1)]
+    assert rel_l2(u[0], u[1]) < 1e-12
