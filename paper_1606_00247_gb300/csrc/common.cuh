@@ -103,7 +103,7 @@ __host__ __device__ inline double h_fold(int a, int b, int c, F&& f) {
   return v;
 }
 
-// SB consecutive values from shared memory, 16 bytes at a time
+// SB consecutive values, 16 bytes at a time where SB allows (then 16-byte aligned)
 template <class T, int SB>
 __device__ __forceinline__ void load_q(const T* q, T (&v)[SB]) {
   if constexpr (SB * sizeof(T) % 16 == 0) {

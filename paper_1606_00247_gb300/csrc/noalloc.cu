@@ -153,7 +153,7 @@ size_t carve(Plan& P, int B, unsigned char* base, Workspace* W) {
     if (mp) w.MP = c.take<float>(mp);
   }
   if (!mixed || otf) w.u_s = c.take<double>(nn * B);
-  if (otf) {  // the largest slice within the same allowance; one state always fits (16 doubles per tet at most)
+  if (otf) {  // the largest slice within the same allowance; one state always fits (48 doubles per tet at most)
     w.slice = p2p_slice(B);
     while (w.slice > 1 && face_state_doubles(P, w.slice) > nt * NOALLOC_TET_STATE) w.slice /= 2;
     w.state = c.take<double>(face_state_doubles(P, w.slice));

@@ -1,34 +1,44 @@
 // p2p.cu -- near field (Sec. 2.1): per-tet geometry, and the FP64 near field
 // integrated at every evaluation (near_mode 0), by the faces of the source tets.
 //
-// The potential of a tet with affine M is that of its charges,
-//   4 pi u = sum_F int_F (M.n) / R dA - div M int_tet 1 / R dV,
-//   int_tet 1/R dV = -(1/2) sum_F h_F I_F,  I_F = int_F dA / R,  h_F = n_F.(r - a_F)
-// (n_F outward).  M is nodal, so it is continuous, and the face charges of two
-// tets sharing a face cancel exactly: an interior face of a set of tets leaves
-// only (1/2) h_F I_F times the jump of div M.  The source leaves are cut, in
-// their sorted (Morton) order, into clusters of at most CL_TETS tets; a cluster
-// keeps its distinct vertices, edges and faces, and per target
+// The potential of a tet with affine M is a sum over its faces (p2p.cuh),
+//   4 pi u = sum_F h_F (M(r).A_F + (1/2) T_F:J),   h_F = n_F.(r - a_F),  J = dM/dx,
+// M(r) the tet's affine M continued to the target.  A_F and T_F belong to the
+// face, h_F changes sign with the side.  M is nodal, so across a face shared by
+// two tets it is continuous: the difference of the two affine functions is
+// (dM/dn)_jump n.(r' - a), its J difference is of rank one, T_F n = -h_F A_F, and
+// an interior face of a set of tets leaves
+//   h (h j.A - (1/2) h j.A) = (1/2) h^2 j.A_F,   j = jump of dM/dn.
+// The source leaves are cut, in their sorted (Morton) order, into clusters of at
+// most CL_TETS tets; a cluster keeps its distinct vertices, edges and faces, and
+// per target
 //   R_v      once per vertex  (0.5 - 0.7 per tet, 4 in the tet-wise form),
 //   Lam_e    once per edge    (1.8 - 2.2 per tet instead of 6 logarithms),
-//   I_F      once per face    (2.6 - 2.9 per tet instead of 4 solid angles);
-// the cluster's boundary faces also take the charge sigma = n.M,
-//   int_F sigma / R dA = sigma_0 I_F + sum_{k=1,2} (sigma_k - sigma_0) Y_k,
-//   Y_k = int_F lambda_k / R dA = (L_k / 2A) (P0_k I_F - m_k.J)   (edge k opposite vertex k),
-//   J = int_F (q - rho0)/R dA = (1/2) sum_e m_e E_e   (divergence theorem in the plane),
-//   E_e = (P0_e^2 + h^2) Lam_e + s+ R+ - s- R-   (s+- = t_e.(end - r)), the last two
-//       = (L_e / 2) ((s+ + s-)^2 / (R+ + R-) + R+ + R-): no difference of terms in R^2
-// with m_e, t_e, P0_e, Lam_e and Omega_F as in p2p.cuh (I_F = sum_e P0_e Lam_e
-// + h Omega_F).
+//   Omega_F  once per face    (2.6 - 2.9 per tet instead of 4 solid angles).
+// The cluster's boundary faces (one tet in the cluster) take the whole sum.  In
+// the face's frame (t along edge 0, m = t x n, n), with foot (x, y) of r from
+// vertex 0, edge normals m_e = c_e t + d_e m, w_e = P0_e Lam_e, dR_e = R_end -
+// R_start and I = sum_e w_e + h Omega (p2p.cuh has the derivation):
+//   A = (P_t, P_m, Omega),  P_t = -sum c_e Lam_e,  P_m = -sum d_e Lam_e
+//   S_tt = I - sum (w c^2 + dR c d),  S_mm = I - sum (w d^2 - dR c d),
+//   S_tm = -sum (w c d + dR (d^2 - c^2) / 2)     (the in-plane part of T)
+//   4 pi u_F = h [M_0.A + G_t.(x A + (S_tt, S_tm, -h P_t)/2)
+//                       + G_m.(y A + (S_tm, S_mm, -h P_m)/2)] + (1/2) h^2 dM/dn.A
+// M_0 at vertex 0, G the in-plane derivatives of M.
 //
-// Rounding.  Y_k carries an error of eps R, I_F one of eps L (face size L,
-// distance R), so the constant part of sigma goes with I_F.  A face between two
-// clusters is evaluated twice and its charges cancel in the sum: its record is
-// built from its vertices in the order of their node ids, so both evaluations
-// have the same bits and their errors cancel with them.  Against 80-bit
-// arithmetic (theta -> 0; balls of 1k, 4k and 11k tets and a cube): smooth M
-// 0.9 - 7.5e-15 (the tet-wise form 1.2 - 10e-15 batched, 2 - 18e-15 for one
-// state), smooth M with 10 % noise 4.8 - 9.4e-15 (4.8 - 7.4e-15, 8 - 15e-15).
+// Rounding.  The terms are those of the tet-wise form, and so is the error: every
+// one carries the height h, no term is divided by a height of the triangle, and
+// M enters by its derivatives.  (Face charges n.M and jumps of div M need fewer
+// products per state, but int_F (n.M)/R dA carries an error of eps R L per
+// derivative of M where this form has eps h L: 5 to 20 times the error on
+// flattened tets.)  Against 80-bit arithmetic, theta -> 0, smooth M | Gaussian M
+// per node, here (tet-wise kernels for one state / batched in parentheses):
+//   balls of 0.2 - 2k tets (14, means)  3.3e-15 (5.1e-15 / 2.7e-15) | 1.7e-14 (2.6e-14 / 1.4e-14)
+//   film, cells of 6.7:1                3.9e-15 (5.8e-15 / 4.4e-15) | 3.2e-14 (3.4e-14 / 3.3e-14)
+//   film, cells of 20:1                 1.2e-14 (1.5e-14 / 1.1e-14) | 2.2e-13 (3.0e-13 / 2.2e-13)
+//   film, cells of 100:1                1.5e-13 (2.0e-13 / 1.6e-13) | 3.4e-12 (4.0e-12 / 3.5e-12)
+//   ball squeezed to 1:20               1.1e-14 (1.2e-14 / 1.2e-14) | 1.1e-13 (1.2e-13 / 1.0e-13)
+//   ball stretched to 20:1              8.6e-15 (1.1e-14 / 8.7e-15) | 1.3e-13 (1.6e-13 / 1.3e-13)
 #include <algorithm>
 #include <utility>
 #include <vector>
@@ -139,7 +149,7 @@ constexpr int PF_G = 16, PF_GMIN = 4;         // target nodes of a near-field bl
 constexpr double PF_SPLIT = 4.0;
 constexpr int CL_TETS = 40;              // tets per cluster
 constexpr int CL_V = 4 * CL_TETS, CL_E = 6 * CL_TETS, CL_F = 4 * CL_TETS;  // bounds of its parts
-constexpr int FACE_REC = 16;             // doubles per face: n (3), m_e (9), 2 area, m_0.m_1, m_1.m_2, m_2.m_0
+constexpr int FACE_REC = 16;             // doubles per face: n, t, m (9), 2 area, c_1, d_1, c_2, d_2, 1 / length of edge 0, (v2 - v0).t
 static_assert(CL_V <= 256 && CL_E <= 512, "8-bit vertex and 9-bit edge positions");
 
 // sorts, returns 1 for an odd permutation; faces list their vertices counter-clockwise seen from outside
@@ -249,7 +259,7 @@ __global__ void __launch_bounds__(256) k_clusters(const int2* __restrict__ range
     for (int j = 0; j < q; j++) k += bnd ? fother[j] < 0 : fother[j] > j;
     const int t = q >> 2, F = q & 3;
     const int64_t o = off[blockIdx.x].z + k;
-    // the record depends on the face alone: its vertices by node id, n and m_e of that order
+    // the record depends on the face alone: its vertices by node id, the frame of that order
     int cor[3];  // corners of tet t
     for (int e = 0; e < 3; e++)
       for (int c = 0; c < 3; c++)
@@ -259,7 +269,7 @@ __global__ void __launch_bounds__(256) k_clusters(const int2* __restrict__ range
     for (int e = 0; e < 3; e++)
       for (int c = 0; c < 3; c++) v[e][c] = G[3 * cor[e] + c];
     double* R = frec + FACE_REC * o;
-    double u[3], w[3], n[3], m[3][3];
+    double u[3], w[3], n[3], tg[3][3], m[3][3], len0 = 0.0;
     for (int c = 0; c < 3; c++) {
       u[c] = v[1][c] - v[0][c];
       w[c] = v[2][c] - v[0][c];
@@ -268,22 +278,29 @@ __global__ void __launch_bounds__(256) k_clusters(const int2* __restrict__ range
     n[1] = u[2] * w[0] - u[0] * w[2];
     n[2] = u[0] * w[1] - u[1] * w[0];
     const double a2 = sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
-    for (int c = 0; c < 3; c++) R[c] = n[c] = n[c] / a2;
+    for (int c = 0; c < 3; c++) n[c] /= a2;
     for (int e = 0; e < 3; e++) {  // m = t x n, t the unit tangent
-      double tg[3];
-      for (int c = 0; c < 3; c++) tg[c] = v[(e + 1) % 3][c] - v[e][c];
-      const double l = sqrt(tg[0] * tg[0] + tg[1] * tg[1] + tg[2] * tg[2]);
-      for (int c = 0; c < 3; c++) tg[c] /= l;
-      m[e][0] = tg[1] * n[2] - tg[2] * n[1];
-      m[e][1] = tg[2] * n[0] - tg[0] * n[2];
-      m[e][2] = tg[0] * n[1] - tg[1] * n[0];
-      for (int c = 0; c < 3; c++) R[3 + 3 * e + c] = m[e][c];
+      for (int c = 0; c < 3; c++) tg[e][c] = v[(e + 1) % 3][c] - v[e][c];
+      const double l = sqrt(tg[e][0] * tg[e][0] + tg[e][1] * tg[e][1] + tg[e][2] * tg[e][2]);
+      if (e == 0) len0 = l;
+      for (int c = 0; c < 3; c++) tg[e][c] /= l;
+      m[e][0] = tg[e][1] * n[2] - tg[e][2] * n[1];
+      m[e][1] = tg[e][2] * n[0] - tg[e][0] * n[2];
+      m[e][2] = tg[e][0] * n[1] - tg[e][1] * n[0];
     }
-    R[12] = a2;
-    for (int e = 0; e < 3; e++) {
-      const int f = (e + 1) % 3;
-      R[13 + e] = m[e][0] * m[f][0] + m[e][1] * m[f][1] + m[e][2] * m[f][2];
+    auto dot = [](const double* a, const double* b) { return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]; };
+    for (int c = 0; c < 3; c++) {
+      R[c] = n[c];
+      R[3 + c] = tg[0][c];
+      R[6 + c] = m[0][c];
     }
+    R[9] = a2;
+    for (int e = 1; e < 3; e++) {
+      R[8 + 2 * e] = dot(m[e], tg[0]);
+      R[9 + 2 * e] = dot(m[e], m[0]);
+    }
+    R[14] = 1.0 / len0;
+    R[15] = dot(w, tg[0]);
     uint32_t es = 0, vs = fodd[q] ? 0x80000000u : 0u;  // top bit: n points into the tet
     for (int e = 0; e < 3; e++) {
       es |= (uint32_t)eloc[6 * t + edge_id(cor[e], cor[(e + 1) % 3])] << (9 * e);
@@ -334,8 +351,8 @@ __global__ void k_cluster_lists(const int32_t* __restrict__ targets, const int64
 // leaves differ several times in length: 16 nodes per block in leaf order left
 // the SMs busy for 48% of the kernel on the 16k-tet ball (708 blocks, the SMs'
 // active cycles 14 to 93 million).  A target leaf whose 16 nodes cost more than
-// 1/PF_SPLIT of the mean share of a resident block takes 8 or 4 at a time: the
-// evaluation 46.4 -> 19.9 ms.  Clusters staged for fewer targets cost little, the
+// 1/PF_SPLIT of the mean share of a resident block takes 8 or 4 at a time: an
+// evaluation of three states 46.4 -> 19.9 ms (the kernel of that time).  Clusters staged for fewer targets cost little, the
 // FP64 arithmetic is the bound; below 4 targets a warp would read 16 records a step.
 std::vector<int4> face_blocks(const Plan& P, const std::vector<int64_t>& clusters) {
   const int64_t nT = (int64_t)clusters.size();
@@ -449,87 +466,123 @@ void build_clusters(Plan& P) {
 }
 
 // ---------------------------------------------------------------------------
-// per face and state of a slice of FS states: (1/2)(jump of div M) / 4 pi, and
-// for the boundary faces the charges sigma_0, sigma_1 - sigma_0, sigma_2 -
-// sigma_0 over 4 pi (signs for the record's n)
+// per face and state of a slice of FS states, over 4 pi, in the face's frame,
+// signs for the record's n: half the jump of dM/dn (half of dM/dn on a boundary
+// face), [face][3][FS]; for the boundary faces M_0, G_t, G_m, [face][9][FS]
 // ---------------------------------------------------------------------------
 namespace {
 
 template <int FS>
 __global__ void k_face_state(int64_t nf, const int2* __restrict__ ftet, const uint2* __restrict__ fidx,
-                             const int32_t* __restrict__ tets_s,
+                             const double* __restrict__ frec, const int32_t* __restrict__ tets_s,
                              const double* __restrict__ grad, const double* __restrict__ Ms, int B, int b0, double* D) {
   const int64_t it = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t f = it / FS;
   if (f >= nf) return;
   const int v = (int)(it - f * FS), b = b0 + v;
-  double d = 0.0;
+  const double* R = frec + FACE_REC * f;
+  double j[3] = {0.0, 0.0, 0.0};
   if (b < B) {
     const int2 t = ftet[f];
 #pragma unroll
     for (int side = 0; side < 2; side++) {
-      const int64_t j = side ? t.y : t.x;
-      if (j < 0) continue;
-      double div = 0.0;
+      const int64_t e = side ? t.y : t.x;
+      if (e < 0) continue;
+      double dn[3] = {0.0, 0.0, 0.0};
 #pragma unroll
       for (int k = 0; k < 4; k++) {
-        const int64_t node = tets_s[4 * j + k];
+        const int64_t node = tets_s[4 * e + k];
+        const double* g = grad + 12 * e + 3 * k;
+        const double gn = g[0] * R[0] + g[1] * R[1] + g[2] * R[2];
 #pragma unroll
-        for (int c = 0; c < 3; c++) div += Ms[(node * 3 + c) * B + b] * grad[12 * j + 3 * k + c];
+        for (int c = 0; c < 3; c++) dn[c] += Ms[(node * 3 + c) * B + b] * gn;
       }
-      d += side ? -div : div;
+#pragma unroll
+      for (int c = 0; c < 3; c++) j[c] += side ? -dn[c] : dn[c];
     }
   }
-  D[it] = d * ((fidx[f].x >> 31 ? -0.5 : 0.5) / (4.0 * M_PI));
+  const double sg = (fidx[f].x >> 31 ? -0.5 : 0.5) / (4.0 * M_PI);
+#pragma unroll
+  for (int x = 0; x < 3; x++) {  // frame (t, m, n) = records 3, 6, 0
+    const double* e = R + (x == 0 ? 3 : x == 1 ? 6 : 0);
+    D[(3 * f + x) * FS + v] = sg * (j[0] * e[0] + j[1] * e[1] + j[2] * e[2]);
+  }
 }
 
 template <int FS>
-__global__ void k_face_charge(int64_t ncl, const int4* __restrict__ cnt, const int4* __restrict__ pos,
+__global__ void k_face_affine(const int4* __restrict__ cnt, const int4* __restrict__ pos,
                               const int32_t* __restrict__ vnode, const double* __restrict__ frec,
                               const uint2* __restrict__ fidx, const double* __restrict__ Ms, int B, int b0, double* S) {
   const int64_t c = blockIdx.x;
   const int4 n = cnt[c], o = pos[c];
-  for (int q = threadIdx.x; q < n.w * 3 * FS; q += blockDim.x) {
-    const int f = q / (3 * FS), r = q - f * 3 * FS, k = r / FS, b = b0 + r - k * FS;
-    double v = 0.0;
+  for (int q = threadIdx.x; q < n.w * FS; q += blockDim.x) {
+    const int f = q / FS, v = q - f * FS, b = b0 + v;
+    const uint32_t x = fidx[o.z + f].x;
+    const double* R = frec + FACE_REC * (int64_t)(o.z + f);
+    double M0[3] = {0.0, 0.0, 0.0}, Gt[3] = {0.0, 0.0, 0.0}, Gm[3] = {0.0, 0.0, 0.0};
     if (b < B) {
-      const uint32_t x = fidx[o.z + f].x;
-      const double* nrm = frec + FACE_REC * (int64_t)(o.z + f);
-      const double* m0 = Ms + (int64_t)vnode[o.x + (x & 255u)] * 3 * B + b;
-      const double* mk = Ms + (int64_t)vnode[o.x + ((x >> (8 * k)) & 255u)] * 3 * B + b;
-      for (int a = 0; a < 3; a++) v += (k ? mk[a * B] - m0[a * B] : m0[a * B]) * nrm[a];
-      if (x >> 31) v = -v;
+      const double il = R[14], ih = -1.0 / (R[9] * il);  // vertex 2 lies at (R[15], -height)
+#pragma unroll
+      for (int a = 0; a < 3; a++) {
+        double m[3];
+#pragma unroll
+        for (int k = 0; k < 3; k++) m[k] = Ms[((int64_t)vnode[o.x + ((x >> (8 * k)) & 255u)] * 3 + a) * B + b];
+        M0[a] = m[0];
+        Gt[a] = (m[1] - m[0]) * il;
+        Gm[a] = ((m[2] - m[0]) - Gt[a] * R[15]) * ih;
+      }
     }
-    S[(int64_t)o.w * 3 * FS + q] = v * (1.0 / (4.0 * M_PI));
+    const double sg = (x >> 31 ? -1.0 : 1.0) / (4.0 * M_PI);
+    double* s = S + (9ll * (o.w + f)) * FS + v;
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      const double* e = R + (k == 0 ? 3 : k == 1 ? 6 : 0);
+      s[k * FS] = sg * (M0[0] * e[0] + M0[1] * e[1] + M0[2] * e[2]);
+      s[(3 + k) * FS] = sg * (Gt[0] * e[0] + Gt[1] * e[1] + Gt[2] * e[2]);
+      s[(6 + k) * FS] = sg * (Gm[0] * e[0] + Gm[1] * e[1] + Gm[2] * e[2]);
+    }
   }
 }
 
 // ---------------------------------------------------------------------------
-// The near field: one block per entry of face_blocks (up to 16 nodes of a target leaf) and FS states.
-// Batches of whole clusters (as many as fit the shared-memory arrays) are
-// staged; thread = (target i, subset of the entities), so a warp reads one or
-// two records per step (broadcast) for 16 targets, and keeps its target's FS
-// sums over all batches: distances, barrier, edge logarithms, barrier, faces.
-// The subsets are added in order at the end: no atomics, the result does not
-// depend on timing.  FP64 arithmetic is the bound (2 FMA per clock and SM), so
-// records are read from shared memory instead of being recomputed.  Measured:
-// 16k-tet ball, leaf 128, 3 states 196 -> 45 ms with 16 nodes per block in leaf
-// order, and an evaluation 46.4 -> 19.9 ms with face_blocks; 3,072-tet cube, leaf
-// 32, one state 5.2 -> 1.1 ms, an evaluation 1.26 -> 1.06 ms (the tet-wise kernels
-// before: 4 sqrt, 6 log1p, 4 atan2 and 6 divisions per pair, 16-state slices
-// whatever the batch, one warp per target leaf for one state).
+// The near field: one block per entry of face_blocks (up to 16 nodes of a target
+// leaf) and FS states.  Batches of whole clusters (as many as fit the
+// shared-memory arrays) are staged; thread = (target i, subset of the entities),
+// so a warp reads one or two records per step (broadcast) for 16 targets, and
+// keeps its target's FS sums over all batches: distances, barrier, edge
+// logarithms, barrier, faces.  The per-state values of a face are read once per
+// block, so they come straight from global memory, and any FS leaves room for two
+// blocks per SM.  The subsets are added in order at the end: no atomics, the
+// result does not depend on timing.  FP64 arithmetic is the bound (2 FMA per
+// clock and SM), so records are read from shared memory instead of being
+// recomputed.  Near-field stage, against the tet-wise kernels before (4 sqrt, 6
+// log1p, 4 atan2 and 6 divisions per pair): 3,072-tet cube, leaf 32, one state 5.2
+// -> 0.77 ms; 16k-tet ball, leaf 128, 3 states 196 -> 17.8 ms, 16 states 26.8 ms.
+// With face charges in the sum instead (less accurate on flattened tets, two
+// divisions per boundary face) 0.91, 18.8 and 27.0 ms.
 // ---------------------------------------------------------------------------
 constexpr int PF_THREADS = 256, PF_BATCH = 32;
 constexpr int PF_V = CL_V, PF_E = CL_E, PF_F = CL_F;  // capacities of a batch: any one cluster fits
 
+constexpr size_t PF_SMEM = sizeof(double) * ((size_t)(PF_V + PF_E) * PF_G + 3 * PF_V + PF_E + FACE_REC * PF_F) +
+                           sizeof(uint2) * PF_F + sizeof(int2) * PF_F + sizeof(uint32_t) * PF_E;
+static_assert(PF_SMEM <= 227 * 1024 && PF_SMEM >= sizeof(double) * PF_THREADS * P2P_SLICE, "arrays, final sums");
+
+// s[v] += f sum_k x_k q[k][v]
 template <int FS>
-constexpr size_t pf_smem() {
-  return sizeof(double) * ((size_t)(PF_V + PF_E) * PF_G + 3 * PF_V + PF_E + FACE_REC * PF_F + (size_t)PF_F * 4 * FS) +
-         sizeof(uint2) * PF_F + sizeof(uint32_t) * PF_E;
+__device__ __forceinline__ void add(double (&s)[FS], double f, const double (&x)[3], const double* __restrict__ q) {
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    const double w = f * x[k];
+    double y[FS];
+    load_q<double, FS>(q + k * FS, y);
+#pragma unroll
+    for (int v = 0; v < FS; v++) s[v] += w * y[v];
+  }
 }
 
 template <int FS>
-__global__ void __launch_bounds__(PF_THREADS) k_p2p_faces(
+__global__ void __launch_bounds__(PF_THREADS, 2) k_p2p_faces(
     const int4* __restrict__ blk, const int64_t* __restrict__ pc_off, const int32_t* __restrict__ pc_src,
     const double* __restrict__ nodes_s, const int4* __restrict__ cnt,
     const int4* __restrict__ pos, const int32_t* __restrict__ vnode, const uint32_t* __restrict__ edge,
@@ -541,10 +594,9 @@ __global__ void __launch_bounds__(PF_THREADS) k_p2p_faces(
   double* sV = sL + PF_E * PF_G;            // [vertex][3]
   double* sEl = sV + 3 * PF_V;              // edge lengths
   double* sF = sEl + PF_E;                  // [face][FACE_REC], boundary faces of all clusters first
-  double* sD = sF + FACE_REC * PF_F;        // [face][FS]
-  double* sS = sD + PF_F * FS;              // [boundary face][3][FS]
-  uint2* sFi = (uint2*)(sS + 3 * PF_F * FS);
-  uint32_t* sE = (uint32_t*)(sFi + PF_F);
+  uint2* sFi = (uint2*)(sF + FACE_REC * PF_F);
+  int2* sId = (int2*)(sFi + PF_F);          // face's rows of D and (boundary faces) S
+  uint32_t* sE = (uint32_t*)(sId + PF_F);
   __shared__ int4 bc[PF_BATCH], bp[PF_BATCH], bb[PF_BATCH];  // per cluster: counts, positions, bases in the batch
   __shared__ int4 tot;                                       // of the batch: vertices, edges, faces, boundary faces
   __shared__ int nb;
@@ -614,13 +666,12 @@ __global__ void __launch_bounds__(PF_THREADS) k_p2p_faces(
       for (int t = tid; t < n.z; t += PF_THREADS) {
         const uint2 x = fidx[p.z + t];
         sFi[slot(t)] = make_uint2((x.x & 0xFFFFFFu) + (uint32_t)b.x * 0x010101u, x.y + (uint32_t)b.y * ((1u << 18) | (1u << 9) | 1u));
+        sId[slot(t)] = make_int2(p.z + t, p.w + t);
       }
       for (int t = tid; t < n.z * (FACE_REC / 2); t += PF_THREADS) {
         const int f = t / (FACE_REC / 2), c = t - f * (FACE_REC / 2);
         ((double2*)(sF + FACE_REC * slot(f)))[c] = ((const double2*)(frec + FACE_REC * (int64_t)(p.z + f)))[c];
       }
-      for (int t = tid; t < n.z * FS; t += PF_THREADS) sD[slot(t / FS) * FS + t % FS] = D[(int64_t)p.z * FS + t];
-      for (int t = tid; t < n.w * 3 * FS; t += PF_THREADS) sS[b.w * 3 * FS + t] = S[(int64_t)p.w * 3 * FS + t];
     }
     __syncthreads();
     for (int t = sub; t < nv; t += nsub) {
@@ -640,62 +691,45 @@ __global__ void __launch_bounds__(PF_THREADS) k_p2p_faces(
     for (int t = sub; t < nf; t += nsub) {
       const uint2 ix = sFi[t];
       const double* F = sF + FACE_REC * t;
-      int vi[3], ei[3];
-      double a[3][3], R[3], lam[3], len[3], P0[3];
+      const int2 id = sId[t];
+      double a[3][3], R[3], lam[3], longest = 0.0, len0 = 0.0;
 #pragma unroll
       for (int k = 0; k < 3; k++) {
-        vi[k] = (ix.x >> (8 * k)) & 255u;
-        ei[k] = (ix.y >> (9 * k)) & 511u;
-        a[k][0] = sV[3 * vi[k]] - rx;
-        a[k][1] = sV[3 * vi[k] + 1] - ry;
-        a[k][2] = sV[3 * vi[k] + 2] - rz;
-        R[k] = sR[vi[k] * PF_G + i];
-        lam[k] = sL[ei[k] * PF_G + i];
-        len[k] = sEl[ei[k]];
+        const int vi = (ix.x >> (8 * k)) & 255u, ei = (ix.y >> (9 * k)) & 511u;
+        a[k][0] = sV[3 * vi] - rx;
+        a[k][1] = sV[3 * vi + 1] - ry;
+        a[k][2] = sV[3 * vi + 2] - rz;
+        R[k] = sR[vi * PF_G + i];
+        lam[k] = sL[ei * PF_G + i];
+        if (k == 0) len0 = sEl[ei];
+        longest = fmax(longest, sEl[ei]);
       }
-      double h = -(F[0] * a[0][0] + F[1] * a[0][1] + F[2] * a[0][2]);
-      if (fabs(h) <= 1e-13 * fmax(len[0], fmax(len[1], len[2]))) h = 0.0;  // r in the plane of F
-      if (h == 0.0 && t >= nbf) continue;
-      double I = 0.0;
-#pragma unroll
-      for (int e = 0; e < 3; e++) {
-        const double* m = F + 3 + 3 * e;
-        P0[e] = m[0] * a[e][0] + m[1] * a[e][1] + m[2] * a[e][2];
-        I += P0[e] * lam[e];
-      }
-      if (h != 0.0) {
-        const double d01 = a[0][0] * a[1][0] + a[0][1] * a[1][1] + a[0][2] * a[1][2];
-        const double d12 = a[1][0] * a[2][0] + a[1][1] * a[2][1] + a[1][2] * a[2][2];
-        const double d20 = a[2][0] * a[0][0] + a[2][1] * a[0][1] + a[2][2] * a[0][2];
-        const double den = R[0] * R[1] * R[2] + d01 * R[2] + d12 * R[0] + d20 * R[1];
-        I -= 2.0 * h * atan2(h * F[12], den);  // Omega = 2 atan2(triple product, den), triple product = -h 2A
-      }
-      const double x = h * I;
-#pragma unroll
-      for (int v = 0; v < FS; v++) part[v] += x * sD[t * FS + v];
+      const double h = -(F[0] * a[0][0] + F[1] * a[0][1] + F[2] * a[0][2]);
+      if (fabs(h) <= 1e-13 * longest) continue;  // r in the plane of F
+      const double d01 = a[0][0] * a[1][0] + a[0][1] * a[1][1] + a[0][2] * a[1][2];
+      const double d12 = a[1][0] * a[2][0] + a[1][1] * a[2][1] + a[1][2] * a[2][2];
+      const double d20 = a[2][0] * a[0][0] + a[2][1] * a[0][1] + a[2][2] * a[0][2];
+      const double den = R[0] * R[1] * R[2] + d01 * R[2] + d12 * R[0] + d20 * R[1];
+      const double Om = -2.0 * atan2(h * F[9], den);  // 2 atan2(triple product, den), triple product = -h 2A
+      const double c1 = F[10], d1 = F[11], c2 = F[12], d2 = F[13];
+      const double A[3] = {-(c1 * lam[1] + c2 * lam[2]), -(lam[0] + d1 * lam[1] + d2 * lam[2]), Om};
+      add<FS>(part, h * h, A, D + 3ll * FS * id.x);
       if (t < nbf) {
-        double E[3], Y[2];
-        const double h2 = h * h, inv = 1.0 / F[12];
-        const double S0 = R[0] + R[1], S1 = R[1] + R[2], S2 = R[2] + R[0], iS = 1.0 / (S0 * S1 * S2);
-        const double S[3] = {S0, S1, S2}, rS[3] = {S1 * S2 * iS, S2 * S0 * iS, S0 * S1 * iS};
-#pragma unroll
-        for (int e = 0; e < 3; e++) {  // tangent t_e = n x m_e
-          const double* m = F + 3 + 3 * e;
-          const double sm = (F[1] * m[2] - F[2] * m[1]) * a[e][0] + (F[2] * m[0] - F[0] * m[2]) * a[e][1] +
-                            (F[0] * m[1] - F[1] * m[0]) * a[e][2];
-          const double w = 2.0 * sm + len[e];
-          E[e] = (P0[e] * P0[e] + h2) * lam[e] + 0.5 * len[e] * (w * w * rS[e] + S[e]);
-        }
-#pragma unroll
-        for (int k = 1; k < 3; k++) {  // edge o runs from vertex k + 1 to k + 2
-          const int o = (k + 1) % 3, o1 = (o + 1) % 3, o2 = (o + 2) % 3;
-          // m_o.m_{o+1} = F[13 + o], m_o.m_{o+2} = F[13 + o2]
-          const double mJ = 0.5 * (E[o] + F[13 + o] * E[o1] + F[13 + o2] * E[o2]);
-          Y[k - 1] = len[o] * inv * (P0[o] * I - mJ);
-        }
-        const double* q = sS + t * 3 * FS;
-#pragma unroll
-        for (int v = 0; v < FS; v++) part[v] += I * q[v] + Y[0] * q[FS + v] + Y[1] * q[2 * FS + v];
+        const double x = -(F[3] * a[0][0] + F[4] * a[0][1] + F[5] * a[0][2]);
+        const double y = -(F[6] * a[0][0] + F[7] * a[0][1] + F[8] * a[0][2]);
+        const double w0 = -y * lam[0], w1 = (c1 * (len0 - x) - d1 * y) * lam[1], w2 = -(c2 * x + d2 * y) * lam[2];
+        const double dR0 = R[1] - R[0], dR1 = R[2] - R[1], dR2 = R[0] - R[2];
+        const double z = c1 * d1 * dR1 + c2 * d2 * dR2, I = w0 + w1 + w2 + h * Om;
+        const double Stt = I - (w1 * c1 * c1 + w2 * c2 * c2) - z;
+        const double Smm = I - (w0 + w1 * d1 * d1 + w2 * d2 * d2) + z;
+        const double Stm = -(w1 * c1 * d1 + w2 * c2 * d2) -
+                           0.5 * (dR0 + (d1 * d1 - c1 * c1) * dR1 + (d2 * d2 - c2 * c2) * dR2);
+        const double kt[3] = {x * A[0] + 0.5 * Stt, x * A[1] + 0.5 * Stm, x * Om - 0.5 * h * A[0]};
+        const double km[3] = {y * A[0] + 0.5 * Stm, y * A[1] + 0.5 * Smm, y * Om - 0.5 * h * A[1]};
+        const double* q = S + 9ll * FS * id.y;
+        add<FS>(part, h, A, q);
+        add<FS>(part, h, kt, q + 3 * FS);
+        add<FS>(part, h, km, q + 6 * FS);
       }
     }
 #pragma unroll
@@ -717,28 +751,26 @@ __global__ void __launch_bounds__(PF_THREADS) k_p2p_faces(
 
 template <int FS>
 void launch_slice(Plan& P, const double* Ms, double* state, int B, int b0, double* u_s, cudaStream_t s) {
-  double *D = state, *S = state + P.n_cl_f * FS;
-  k_face_state<FS><<<nblk(P.n_cl_f * FS, 256), 256, 0, s>>>(P.n_cl_f, P.cl_ftet, P.cl_fidx, P.tets_s,
-                                                                   P.tet_grad, Ms, B, b0, D);
+  double *D = state, *S = state + 3 * P.n_cl_f * FS;
+  k_face_state<FS><<<nblk(P.n_cl_f * FS, 256), 256, 0, s>>>(P.n_cl_f, P.cl_ftet, P.cl_fidx, P.cl_frec, P.tets_s,
+                                                            P.tet_grad, Ms, B, b0, D);
   DM_LAUNCH("k_face_state");
-  k_face_charge<FS><<<(unsigned)P.n_clusters, 128, 0, s>>>(P.n_clusters, P.cl_cnt, P.cl_pos, P.cl_vnode, P.cl_frec,
-                                                           P.cl_fidx, Ms, B, b0, S);
-  DM_LAUNCH("k_face_charge");
-  smem_opt_in((const void*)k_p2p_faces<FS>, pf_smem<FS>());
-  k_p2p_faces<FS><<<(unsigned)P.n_pc_blk, PF_THREADS, pf_smem<FS>(), s>>>(P.pc_blk, P.pc_off, P.pc_src, P.nodes_s,
-                                                                         P.cl_cnt, P.cl_pos, P.cl_vnode, P.cl_edge,
-                                                                         P.cl_elen, P.cl_frec, P.cl_fidx, D, S, B, b0,
-                                                                         u_s);
+  k_face_affine<FS><<<(unsigned)P.n_clusters, 128, 0, s>>>(P.cl_cnt, P.cl_pos, P.cl_vnode, P.cl_frec, P.cl_fidx, Ms, B,
+                                                           b0, S);
+  DM_LAUNCH("k_face_affine");
+  smem_opt_in((const void*)k_p2p_faces<FS>, PF_SMEM);
+  k_p2p_faces<FS><<<(unsigned)P.n_pc_blk, PF_THREADS, PF_SMEM, s>>>(P.pc_blk, P.pc_off, P.pc_src, P.nodes_s, P.cl_cnt,
+                                                                    P.cl_pos, P.cl_vnode, P.cl_edge, P.cl_elen,
+                                                                    P.cl_frec, P.cl_fidx, D, S, B, b0, u_s);
   DM_LAUNCH("k_p2p_faces");
 }
 
 }  // namespace
 
-size_t face_state_doubles(const Plan& P, int slice) { return (size_t)slice * (size_t)(P.n_cl_f + 3 * P.n_cl_b); }
+size_t face_state_doubles(const Plan& P, int slice) { return (size_t)slice * (size_t)(3 * P.n_cl_f + 9 * P.n_cl_b); }
 
 int launch_p2p_fp64(Plan& P, const double* Ms, double* state, int slice, int B, double* u_s, cudaStream_t s) {
   if (P.n_pc_blk == 0 || P.n_clusters == 0) return 0;
-  static_assert(pf_smem<16>() <= 227 * 1024, "shared memory of the near-field kernel");
   int n = 0;
   for (int b0 = 0; b0 < B; n += 3) {
     int fs = 1;  // the smallest slice that takes what is left, within what the state buffer holds

@@ -1,7 +1,8 @@
 """The integrated FP64 near field by faces of tet clusters (near_mode 0): the
-charges of a face shared by two tets of a cluster are left out, its div M jump
-is kept.  theta -> 0 makes every interaction near field, so u is the oracle's
-direct sum (tet by tet, no sharing); 1e-12 as in test_gpu_p2p_fp64."""
+affine functions of the two tets sharing a face differ by the jump of dM/dn alone,
+a boundary face of a cluster takes the whole sum.  theta -> 0 makes every interaction
+near field, so u is the oracle's direct sum (tet by tet, no sharing); 1e-12 as in
+test_gpu_p2p_fp64."""
 import numpy as np
 import pytest
 import torch
@@ -47,7 +48,7 @@ def test_single_tet_and_flat_cells(orc):
 
 def test_overlapping_tets_are_summed(orc):
     """A tet listed three times, and one laid over its neighbour on the same side of their
-    face: the faces these share are no interior faces and keep their charges."""
+    face: the faces these share are no interior faces."""
     nodes, tets = inputs.sphere(h=0.45)
     a = tets[0]
     centre = nodes[tets[:, :]].mean(1)[0]
@@ -70,3 +71,29 @@ def test_block_sizes_vs_stored(n, leaf):
     u = [Plan(nodes, tets, precision="fp64", near_mode=k, theta=0.5, p=3, leaf_size=leaf, max_batch=2)
          .eval(M)[0].cpu().numpy() for k in (0, 1)]
     assert rel_l2(u[0], u[1]) < 1e-12
+
+
+def _film(ratio):  # cells of 333 x 333 and 333 / ratio
+    return inputs.thin_film(6, 3, 2, size=(2000.0, 1000.0, 2.0 * 1000.0 / (3.0 * ratio)))
+
+
+# Flattened and stretched tets, smooth M: no term of the face form is divided by a height of a triangle,
+# so it is as accurate as the tet by tet form.  `stored`: the error of the stored coefficients (that form)
+# against 80-bit arithmetic for these meshes and this M; the bar is four times that, as both results carry
+# an error of its own.  (Face charges n.M instead: 1.2e-14, 3.7e-14, 4.9e-13, 1.6e-14 and 5.4e-14.)
+@pytest.mark.parametrize("mesh, stored", [
+    (lambda: _film(6.67), 1.65e-15), (lambda: _film(20.0), 3.97e-15), (lambda: _film(100.0), 1.72e-14),
+    (lambda: inputs.sphere(h=0.3, scale=(1.0, 1.0, 0.05)), 3.17e-15),
+    (lambda: inputs.sphere(h=0.3, scale=(1.0, 1.0, 20.0)), 3.63e-15)], ids=["film7", "film20", "film100", "disc", "needle"])
+def test_flattened_tets_smooth_m(mesh, stored):
+    from paper_1606_00247_gb300.api import Plan
+
+    nodes, tets = mesh()
+    r = np.random.default_rng(3)
+    x = (nodes - nodes.mean(0)) / np.ptp(nodes, axis=0).max()
+    M = sum(r.standard_normal(3) * np.cos(x @ (6.0 * r.standard_normal(3)) + 6.3 * r.random())[:, None] for _ in range(4))
+    M = torch.as_tensor((M / np.linalg.norm(M, axis=1, keepdims=True))[None], device="cuda")
+    for leaf in (4, 64):
+        u = [Plan(nodes, tets, precision="fp64", near_mode=k, theta=1e-9, p=1, leaf_size=leaf).eval(M)[0].cpu().numpy()
+             for k in (0, 1)]
+        assert rel_l2(u[0], u[1]) < 4.0 * stored
