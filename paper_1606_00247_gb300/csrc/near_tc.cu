@@ -391,19 +391,23 @@ __global__ void __launch_bounds__(NF_THREADS, 1)
 
 // Batches of at most NFS_MAX states: the tensor-core tile holds 128 states, so a
 // small batch paid for the whole tile (its M, its conversions).  Here the same
-// stored coefficients are streamed by CUDA cores in FP32: W = W_hi + W_lo (exact),
-// M unrounded.  CTA of 256 threads per (tile, part of its column groups): thread =
-// (row, half of a group's 16 columns), six coalesced 16-byte loads per group (hi
-// and lo of three components), M of the group's columns as shared-memory
-// broadcasts for SB states.  A tile is cut into parts so that every SM holds
-// several CTAs; the parts' sums go to `part` and are added in order by
-// k_near_tc_sum, so results do not depend on timing.  Bound by the stream of W
-// (12 B per stored coefficient, 2.5 GB on the 224k-tet ball, 298 tiles).  Measured
-// there against the tensor-core kernel (815 - 830 us up to 128 states): 1 / 4 / 8
-// / 16 states 403 (6.2 TB/s) / 436 / 542 / 842 us; 29k tets (42 tiles, which leave
-// two thirds of the SMs without a tensor-core CTA, 310 us): 46 us for one, 92 us
-// for sixteen states.  Errors against FP64 fall too (u 1.0e-6 -> 3.8e-7, film
-// 2.0e-5 -> 1.1e-5): M is not rounded to 16 bits.
+// product is streamed by CUDA cores in FP32: W = W_hi + W_lo (exact) times M - Mbar,
+// not rounded to 16 bits, and S_i . Mbar added by k_near_tc_sum (file header: W
+// itself holds 16 bits only).  Mbar is the mean over 32 columns of the tile: the
+// first column alone makes M - Mbar of a random M larger than M itself.  CTA of
+// 256 threads per (tile, part of its column groups): thread = (row, half of a
+// group's 16 columns), six coalesced 16-byte loads per group (hi and lo of three
+// components), M - Mbar of the group's columns as shared-memory broadcasts for SB
+// states.  A tile is cut into parts so that every SM holds several CTAs; the parts'
+// sums go to `part` and are added in order by k_near_tc_sum, so results do not
+// depend on timing.  Bound by the stream of W (12 B per stored coefficient, 2.5 GB
+// on the 224k-tet ball, 298 tiles).  Measured there against the tensor-core kernel
+// (815 - 830 us up to 128 states): 1 / 4 / 8 / 16 states 407 (6.2 TB/s) / 436 / 565
+// / 832 us; 29k tets (42 tiles, which leave two thirds of the SMs without a
+// tensor-core CTA, 310 us): 47 us for one, 95 us for sixteen states.  Errors of
+// u of an evaluation against FP64 (7 states, ball of 22k tets, p = 8), tensor-core
+// kernel / full M instead of M - Mbar / here: uniform M 5.5e-07 / 3.2e-07 / 1.7e-07, 1 % noise 5.5e-07 / 3.0e-07 / 1.5e-07,
+// long waves with 10 % noise 1.7e-06 / 5.2e-07 / 5.1e-07, random 6.9e-06 / 2.4e-06 / 2.4e-06.
 constexpr int NFS_THREADS = 256;
 constexpr int NFS_SLICE = 16, NFS_MAX = 64;  // states per pass over W, largest batch
 
@@ -420,8 +424,10 @@ __global__ void __launch_bounds__(NFS_THREADS, SB <= 8 ? 4 : 3)
     k_near_tc_small(const int32_t* __restrict__ order, const int64_t* __restrict__ woff,
                     const int64_t* __restrict__ coff, const int32_t* __restrict__ ngrp,
                     const int32_t* __restrict__ npad_t, const int32_t* __restrict__ cols,
-                    const unsigned char* __restrict__ W, const float* __restrict__ Ms, int B, int parts, float* part) {
-  __shared__ __align__(16) float sM[2][48 * SB];  // [half][component][8 columns][state]
+                    const unsigned char* __restrict__ W, const float* __restrict__ Ms, int B, int parts, float* part,
+                    float* mbar) {
+  __shared__ __align__(16) float sM[2][48 * SB];  // M - Mbar: [half][component][8 columns][state]
+  __shared__ float sMbar[3 * SB];                 // Mbar: [component][state]
   const int64_t tile = order[blockIdx.x];
   const int npad = npad_t[tile], ng = ngrp[tile], b0 = blockIdx.z * SB;
   const int g0 = (int)((int64_t)ng * blockIdx.y / parts), g1 = (int)((int64_t)ng * (blockIdx.y + 1) / parts);
@@ -444,6 +450,24 @@ __global__ void __launch_bounds__(NFS_THREADS, SB <= 8 ? 4 : 3)
 #pragma unroll
   for (int v = 0; v < SB; v++) acc[v] = 0.f;
   if (g0 < g1) load_m(g0);
+  if (g0 < g1 && tid < 96) {  // Mbar: warp = component, lane = (one of 32 / SB columns, state), summed as a binary
+    const int c = tid >> 5, v = tid % SB, b = b0 + v;  // tree: exact where all columns hold the same M
+    float s[SB];
+#pragma unroll
+    for (int j = 0; j < SB; j++)
+      s[j] = b < B ? Ms[((int64_t)ct[ng * ((tid & 31) / SB + j * (32 / SB)) / 2] * 3 + c) * B + b] : 0.f;
+#pragma unroll
+    for (int o = SB / 2; o > 0; o >>= 1)
+#pragma unroll
+      for (int j = 0; j < o; j++) s[j] += s[j + o];
+#pragma unroll
+    for (int o = SB; o < 32; o <<= 1) s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+    if ((tid & 31) < SB) {
+      sMbar[c * SB + v] = s[0] * (1.f / 32);
+      if (g0 == 0 && b < B) mbar[(tile * 3 + c) * B + b] = s[0] * (1.f / 32);
+    }
+  }
+  __syncthreads();
   for (int g = g0; g < g1; g++, w += 3 * kbytes) {
     float* buf = sM[(g - g0) & 1];
     uint4 hi[3], lo[3];
@@ -454,8 +478,10 @@ __global__ void __launch_bounds__(NFS_THREADS, SB <= 8 ? 4 : 3)
         lo[c] = __ldcs((const uint4*)(w + c * kbytes + limb));
       }
 #pragma unroll
-    for (int r = 0; r < NM; r++)
-      if (tid + r * NFS_THREADS < 48 * SB) buf[tid + r * NFS_THREADS] = m[r];
+    for (int r = 0; r < NM; r++) {
+      const int q = tid + r * NFS_THREADS;
+      if (q < 48 * SB) buf[q] = m[r] - sMbar[(q / (8 * SB)) % 3 * SB + q % SB];
+    }
     if (g + 1 < g1) load_m(g + 1);
     __syncthreads();  // this group's M is staged; the buffer of the group before it is free after the next barrier
     if (on) {
@@ -488,8 +514,9 @@ __global__ void __launch_bounds__(NFS_THREADS, SB <= 8 ? 4 : 3)
   }
 }
 
-__global__ void k_near_tc_sum(int64_t n, const int32_t* __restrict__ rownode, const int32_t* __restrict__ ngrp, int B,
-                              int parts, const float* __restrict__ part, float* u) {
+__global__ void k_near_tc_sum(int64_t n, const int32_t* __restrict__ rownode, const int32_t* __restrict__ ngrp,
+                              const float* __restrict__ S, int B, int parts, const float* __restrict__ part,
+                              const float* __restrict__ mbar, float* u) {
   const int64_t it = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // (tile, row, state)
   if (it >= n) return;
   const int64_t r = it / B, tile = r / NF_ROWS;
@@ -498,17 +525,20 @@ __global__ void k_near_tc_sum(int64_t n, const int32_t* __restrict__ rownode, co
   const float* p = part + ((tile * parts) * NF_ROWS + r - tile * NF_ROWS) * B + b;
   float v = 0.f;
   for (int k = 0; k < parts; k++) v += p[(int64_t)k * NF_ROWS * B];
-  u[(int64_t)node * B + b] += v;
+  const float* mb = mbar + tile * 3 * B + b;
+  const float* Si = S + 3ll * node;
+  u[(int64_t)node * B + b] += v + (Si[0] * mb[0] + Si[1] * mb[B] + Si[2] * mb[2 * B]);
 }
 
 template <int SB>
 void launch_small(Plan& P, const float* Ms, float* part, int B, int parts, float* u_s, cudaStream_t s) {
   const dim3 grid((unsigned)P.nf_ntiles, (unsigned)parts, (unsigned)((B + SB - 1) / SB));
+  float* mbar = part + P.nf_ntiles * parts * NF_ROWS * B;
   k_near_tc_small<SB><<<grid, NFS_THREADS, 0, s>>>(
-      P.nf_order, P.nf_woff, P.nf_coff, P.nf_ng, P.nf_npad, P.nf_cols, P.nf_W, Ms, B, parts, part);
+      P.nf_order, P.nf_woff, P.nf_coff, P.nf_ng, P.nf_npad, P.nf_cols, P.nf_W, Ms, B, parts, part, mbar);
   DM_LAUNCH("k_near_tc_small");
   const int64_t n = P.nf_ntiles * NF_ROWS * B;
-  k_near_tc_sum<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, P.nf_rownode, P.nf_ng, B, parts, part, u_s);
+  k_near_tc_sum<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, P.nf_rownode, P.nf_ng, P.nf_S, B, parts, part, mbar, u_s);
   DM_LAUNCH("k_near_tc_sum");
 }
 
@@ -522,8 +552,8 @@ int launch_near_tc(Plan& P, const float* Ms, float* MP, int B, float* u_s, int* 
   if (P.nf_ntiles == 0) return 0;
   if (small_batch(P.nf_ntiles, B) && !(P.debug_flags & 1)) {
     // parts: ~6 CTAs per SM, at least four column groups each on average, the
-    // sums within MP (whose copy of M this kernel does not use)
-    const int64_t room = (int64_t)nf_mp_floats(P, B) / (P.nf_ntiles * NF_ROWS * B);
+    // sums and Mbar within MP (whose copy of M this kernel does not use)
+    const int64_t room = ((int64_t)nf_mp_floats(P, B) / (P.nf_ntiles * B) - 3) / NF_ROWS;
     const int64_t want = std::min<int64_t>((6 * 152 + P.nf_ntiles - 1) / P.nf_ntiles, P.nf_ncols / 64 / P.nf_ntiles);
     const int parts = (int)std::max<int64_t>(1, std::min(want, room));
     if (room >= 1) {
