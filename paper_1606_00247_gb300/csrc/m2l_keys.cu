@@ -160,16 +160,16 @@ M2lKeys build_m2l_keys(Plan& P) {
     if (hw == 0) {
       size_t b1 = 0, b2 = 0;
       const int bits = 6 + 3 * KEY_OFF_BITS;
-      DM_CUDA(cub::DeviceRadixSort::SortKeys(nullptr, b1, keys.p, sorted.p, (int)n, 0, bits, s));
+      DM_CUDA(cub::DeviceRadixSort::SortKeys(nullptr, b1, keys.p, sorted.p, n, 0, bits, s));
       {
         Buf<unsigned char> tmp(b1);
-        DM_CUDA(cub::DeviceRadixSort::SortKeys(tmp.p, b1, keys.p, sorted.p, (int)n, 0, bits, s));
+        DM_CUDA(cub::DeviceRadixSort::SortKeys(tmp.p, b1, keys.p, sorted.p, n, 0, bits, s));
         DM_CUDA(cudaStreamSynchronize(s));
       }
       Buf<uint64_t> uniq(n);
-      DM_CUDA(cub::DeviceSelect::Unique(nullptr, b2, sorted.p, uniq.p, nu.p, (int)n, s));
+      DM_CUDA(cub::DeviceSelect::Unique(nullptr, b2, sorted.p, uniq.p, nu.p, n, s));
       Buf<unsigned char> tmp(b2);
-      DM_CUDA(cub::DeviceSelect::Unique(tmp.p, b2, sorted.p, uniq.p, nu.p, (int)n, s));
+      DM_CUDA(cub::DeviceSelect::Unique(tmp.p, b2, sorted.p, uniq.p, nu.p, n, s));
       int h_nu = 0;
       DM_CUDA(cudaMemcpyAsync(&h_nu, nu.p, sizeof h_nu, cudaMemcpyDeviceToHost, s));
       DM_CUDA(cudaStreamSynchronize(s));

@@ -951,9 +951,9 @@ void build_plan(Plan& P, const double* nodes_in, const int32_t* tets_in) {
       int32_t* src = which == 0 ? P.m2l_src : P.p2p_src;
       if (n > 0) {
         size_t b = 0;
-        cub::DeviceRadixSort::SortKeys(nullptr, b, in, sorted.p, (int)n, 0, 64, s);
+        cub::DeviceRadixSort::SortKeys(nullptr, b, in, sorted.p, n, 0, 64, s);
         ct.need(b);
-        DM_CUDA(cub::DeviceRadixSort::SortKeys(ct.p, b, in, sorted.p, (int)n, 0, 64, s));
+        DM_CUDA(cub::DeviceRadixSort::SortKeys(ct.p, b, in, sorted.p, n, 0, 64, s));
       }
       k_csr_offsets<<<nblk(std::max<int64_t>(nc + 1, n), 256), 256, 0, s>>>(sorted.p, n, nc, off, src);
       DM_LAUNCH("k_csr_offsets");
