@@ -190,17 +190,14 @@ class Auditor {
         cudaGetLastError();
         fail(DEMAG_ERR_OUT_OF_MEMORY, "plan audit buffers");
       }
-      if (dout_) {
-        DM_CUDA(cudaMemcpyAsync(d, dout_, sizeof(AuditOut) * cap_, cudaMemcpyDeviceToDevice, s_));
-        DM_CUDA(cudaStreamSynchronize(s_));
-        cudaFree(dout_);
-      }
+      const std::vector<AuditOut> init(nc, AuditOut{0ull, ULLONG_MAX});
+      DM_CUDA(cudaMemcpyAsync(d, init.data(), sizeof(AuditOut) * nc, cudaMemcpyHostToDevice, s_));
+      if (dout_) DM_CUDA(cudaMemcpyAsync(d, dout_, sizeof(AuditOut) * cap_, cudaMemcpyDeviceToDevice, s_));
+      DM_CUDA(cudaStreamSynchronize(s_));
+      if (dout_) cudaFree(dout_);
       dout_ = d;
       cap_ = nc;
     }
-    const AuditOut init{0ull, ULLONG_MAX};
-    DM_CUDA(cudaMemcpyAsync(dout_ + k, &init, sizeof init, cudaMemcpyHostToDevice, s_));
-    DM_CUDA(cudaStreamSynchronize(s_));  // init is a host temporary
     return dout_ + k;
   }
 

@@ -94,10 +94,10 @@ template <class F>
 __host__ __device__ inline double h_fold(int a, int b, int c, F&& f) {
   double v = 0.0;
   for (int i = 0; 2 * i <= b; i++) {
-    double w = (i & 1) ? -1.0 : 1.0;  // (-1)^(i+l) C(i+l, i)
+    int w = (i & 1) ? -1 : 1;  // (-1)^(i+l) C(i+l, i)
     for (int l = 0; 2 * l <= c; l++) {
       v += w * f(a + 2 * (i + l), b - 2 * i, c - 2 * l);
-      w *= -(double)(i + l + 1) / (double)(l + 1);
+      w = -(w * (i + l + 1)) / (l + 1);  // exact
     }
   }
   return v;

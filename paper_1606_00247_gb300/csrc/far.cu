@@ -58,28 +58,35 @@ __global__ void k_p2m_op(const int32_t* __restrict__ leaves, const int32_t* __re
   }
 }
 
-// L2P polynomials h_m(z/s) of every node at its leaf, rows of nl values
+// L2P polynomials h_m(z/s) of every node at its leaf, rows of nl values: block per
+// NODE_H nodes, whose scaled monomials z^e/e! are formed once
+constexpr int NODE_H = 16;
 template <class T>
-__global__ void k_node_h(int64_t nn, const int32_t* __restrict__ node_leaf, const int32_t* __restrict__ level,
-                         const double* __restrict__ nodes_s, const double* __restrict__ centre, double side, int nl,
-                         T* h) {
-  const int64_t it = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t i = it / nl;
-  if (i >= nn) return;
-  const int m = (int)(it - i * nl);
-  const int32_t c = node_leaf[i];
-  const double inv_s = 1.0 / ldexp(side, -level[c]);
-  double z[3];
-  for (int x = 0; x < 3; x++) z[x] = (nodes_s[3 * i + x] - centre[3 * c + x]) * inv_s;
-  int a, b, g;
-  h_decode(m, a, b, g);
-  h[it] = (T)h_fold(a, b, g, [&](int na, int nb, int nz) {
-    const int e[3] = {na, nb, nz};
+__global__ void __launch_bounds__(256) k_node_h(int64_t nn, const int32_t* __restrict__ node_leaf,
+                                                const int32_t* __restrict__ level, const double* __restrict__ nodes_s,
+                                                const double* __restrict__ centre, double side, int p, int nl, T* h) {
+  __shared__ double s[NODE_H][3][MAX_P];  // degrees below p
+  const int64_t i0 = blockIdx.x * (int64_t)NODE_H;
+  const int nb = (int)min((int64_t)NODE_H, nn - i0);
+  if (threadIdx.x < 3 * nb) {
+    const int k = threadIdx.x / 3, x = threadIdx.x - 3 * k;
+    const int64_t i = i0 + k;
+    const int32_t c = node_leaf[i];
+    const double z = (nodes_s[3 * i + x] - centre[3 * c + x]) * (1.0 / ldexp(side, -level[c]));
     double v = 1.0;
-    for (int x = 0; x < 3; x++)
-      for (int k = 1; k <= e[x]; k++) v = v * z[x] / k;
-    return v;
-  });
+    for (int e = 0; e < p; e++) {
+      s[k][x][e] = v;
+      v = v * z / (e + 1);
+    }
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < nb * nl; q += blockDim.x) {
+    const int k = q / nl, m = q - k * nl;
+    int a, b, g;
+    h_decode(m, a, b, g);
+    h[i0 * nl + q] =
+        (T)h_fold(a, b, g, [&](int na, int nb_, int nz) { return s[k][0][na] * s[k][1][nb_] * s[k][2][nz]; });
+  }
 }
 
 // P2M: one block per (source leaf, NN moments, 128 SPT states), 128 threads,
@@ -573,14 +580,11 @@ void launch_l2p_small(Plan& P, int B, const T* L, T* u, cudaStream_t s) {
 template <class T>
 void build_translations(Plan& P) {
   const int p = P.p, nq = P.nq, nl = P.nl;
-  auto fact = [](int n) {
-    double f = 1;
-    for (int i = 2; i <= n; i++) f *= i;
-    return f;
-  };
-  auto mono = [&](double h, int ja, int jb, int jc) {  // s_j(h, h, h), 0 below the index range
+  double fact[MAX_P + 1] = {1.0};
+  for (int i = 1; i <= MAX_P; i++) fact[i] = i * fact[i - 1];
+  auto mono = [&](int e, int ja, int jb, int jc) {  // s_j(h, h, h) at h = 2^e, 0 below the index range
     if (ja < 0 || jb < 0 || jc < 0) return 0.0;
-    return std::pow(h, ja + jb + jc) / (fact(ja) * fact(jb) * fact(jc));
+    return std::ldexp(1.0, e * (ja + jb + jc)) / (fact[ja] * fact[jb] * fact[jc]);
   };
   auto parity = [](int ja, int jb, int jc) { return (ja & 1) | ((jb & 1) << 1) | ((jc & 1) << 2); };
   std::vector<std::vector<TEnt<T>>> mrow(nq);
@@ -592,7 +596,7 @@ void build_translations(Plan& P) {
     for (int k = 0; k < nq; k++) {
       int ka, kb, kc;
       h_decode(k + 1, ka, kb, kc);
-      const double cf = h_fold(ra, rb, rc, [&](int na, int nb, int nz) { return mono(0.25, na - ka, nb - kb, nz - kc); }) *
+      const double cf = h_fold(ra, rb, rc, [&](int na, int nb, int nz) { return mono(-2, na - ka, nb - kb, nz - kc); }) *
                         std::ldexp(1.0, -(ka + kb + kc));
       if (cf != 0.0) mrow[r].push_back(TEnt<T>{(uint16_t)(parity(ra + ka, rb + kb, rc + kc) * nq + k), (T)cf});
     }
@@ -606,7 +610,7 @@ void build_translations(Plan& P) {
         int ra, rb, rc;
         h_decode(r, ra, rb, rc);
         if (parity(ra + ma, rb + mb, rc + mc) != cls) continue;
-        const double cf = h_fold(ra, rb, rc, [&](int ka, int kb, int kz) { return mono(0.5, ka - ma, kb - mb, kz - mc); }) *
+        const double cf = h_fold(ra, rb, rc, [&](int ka, int kb, int kz) { return mono(-1, ka - ma, kb - mb, kz - mc); }) *
                           std::ldexp(1.0, -(ra + rb + rc));
         if (cf != 0.0) lent.push_back(TEnt<T>{(uint16_t)r, (T)cf});
       }
@@ -667,8 +671,8 @@ void build_operators(Plan& P) {
                                                                 P.nc1, P.nq, P.g_stride, G);
     DM_LAUNCH("k_p2m_op");
   }
-  k_node_h<T><<<nblk(P.nn * P.nl, 256), 256, 0, s>>>(P.nn, P.node_leaf, P.cell_level, P.nodes_s, P.cell_centre, P.side,
-                                                     P.nl, h);
+  k_node_h<T><<<nblk(P.nn, NODE_H), 256, 0, s>>>(P.nn, P.node_leaf, P.cell_level, P.nodes_s, P.cell_centre, P.side, P.p,
+                                                 P.nl, h);
   DM_LAUNCH("k_node_h");
 }
 

@@ -147,36 +147,35 @@ M2lKeys build_m2l_keys(Plan& P) {
   const int64_t n = P.n_m2l;
   std::vector<uint64_t> hk;
   {
-    Buf<uint64_t> keys(n), sorted(n);
-    Buf<unsigned long long> wide(1);
-    Buf<int> nu(1);
-    DM_CUDA(cudaMemsetAsync(wide.p, 0, sizeof(unsigned long long), s));
+    // one allocation: keys, sorted and distinct keys, two counters, sort workspace
+    struct Counters {
+      unsigned long long wide;  // offsets beyond the packing
+      long long nu;             // distinct keys
+    };
+    const int bits = 6 + 3 * KEY_OFF_BITS;
+    size_t b1 = 0, b2 = 0;
+    uint64_t* none = nullptr;
+    DM_CUDA(cub::DeviceRadixSort::SortKeys(nullptr, b1, none, none, n, 0, bits, s));
+    DM_CUDA(cub::DeviceSelect::Unique(nullptr, b2, none, none, (long long*)nullptr, n, s));
+    const size_t list = ((size_t)n * sizeof(uint64_t) + 255) / 256 * 256;
+    Buf<unsigned char> buf(3 * list + 256 + std::max(b1, b2));
+    uint64_t *keys = (uint64_t*)buf.p, *sorted = (uint64_t*)(buf.p + list), *uniq = (uint64_t*)(buf.p + 2 * list);
+    Counters* cnt = (Counters*)(buf.p + 3 * list);
+    unsigned char* tmp = buf.p + 3 * list + 256;
+    DM_CUDA(cudaMemsetAsync(cnt, 0, sizeof(Counters), s));
     k_pair_keys<<<(unsigned)P.h_m2l_targets.size(), 128, 0, s>>>(P.m2l_targets, P.m2l_off, P.m2l_src, P.cell_prefix,
-                                                                 P.cell_level, keys.p, wide.p);
+                                                                 P.cell_level, keys, &cnt->wide);
     DM_LAUNCH("k_pair_keys");
-    unsigned long long hw = 0;
-    DM_CUDA(cudaMemcpyAsync(&hw, wide.p, sizeof hw, cudaMemcpyDeviceToHost, s));
+    DM_CUDA(cub::DeviceRadixSort::SortKeys(tmp, b1, keys, sorted, n, 0, bits, s));
+    DM_CUDA(cub::DeviceSelect::Unique(tmp, b2, sorted, uniq, &cnt->nu, n, s));
+    Counters h{};
+    DM_CUDA(cudaMemcpyAsync(&h, cnt, sizeof h, cudaMemcpyDeviceToHost, s));
     DM_CUDA(cudaStreamSynchronize(s));
-    if (hw == 0) {
-      size_t b1 = 0, b2 = 0;
-      const int bits = 6 + 3 * KEY_OFF_BITS;
-      DM_CUDA(cub::DeviceRadixSort::SortKeys(nullptr, b1, keys.p, sorted.p, n, 0, bits, s));
-      {
-        Buf<unsigned char> tmp(b1);
-        DM_CUDA(cub::DeviceRadixSort::SortKeys(tmp.p, b1, keys.p, sorted.p, n, 0, bits, s));
-        DM_CUDA(cudaStreamSynchronize(s));
-      }
-      Buf<uint64_t> uniq(n);
-      DM_CUDA(cub::DeviceSelect::Unique(nullptr, b2, sorted.p, uniq.p, nu.p, n, s));
-      Buf<unsigned char> tmp(b2);
-      DM_CUDA(cub::DeviceSelect::Unique(tmp.p, b2, sorted.p, uniq.p, nu.p, n, s));
-      int h_nu = 0;
-      DM_CUDA(cudaMemcpyAsync(&h_nu, nu.p, sizeof h_nu, cudaMemcpyDeviceToHost, s));
-      DM_CUDA(cudaStreamSynchronize(s));
-      hk.resize(h_nu);
-      DM_CUDA(cudaMemcpyAsync(hk.data(), uniq.p, h_nu * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+    if (h.wide == 0) {
+      hk.resize(h.nu);
+      DM_CUDA(cudaMemcpyAsync(hk.data(), uniq, h.nu * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
       P.m2l_op = dalloc<int32_t>(P, n);
-      k_key_index<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, keys.p, uniq.p, h_nu, P.m2l_op);
+      k_key_index<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, keys, uniq, (int)h.nu, P.m2l_op);
       DM_LAUNCH("k_key_index");
       DM_CUDA(cudaStreamSynchronize(s));
     }
