@@ -3,8 +3,9 @@
 // Every list that an evaluation kernel follows into another array (node and
 // tet permutations, cell links and ranges, the CSR interaction lists of
 // Sec. 3.3, support nodes, near-field columns and tile rows, M2L operator
-// indices and groups, gradient-operator columns) is written once, while the
-// plan is built, and only read afterwards.  Checking each entry once here is
+// indices and groups, gradient-operator columns, the parts of the integrated near
+// field's clusters, translation entries) is written once, while the plan is built,
+// and only read afterwards.  Checking each entry once here is
 // therefore the same guarantee as a bounds check at every read, at no cost to
 // an evaluation, and without a device assert (which would end the context).
 // Each list's count is first checked against the size of the allocation it
@@ -71,19 +72,103 @@ __global__ void k_audit_children(const int32_t* __restrict__ child0, const int32
   }
 }
 
-// a device scratch array freed on scope exit
-struct Scratch32 {
-  int32_t* p = nullptr;
-  explicit Scratch32(int64_t n) {
-    if (cudaMalloc(&p, sizeof(int32_t) * (size_t)std::max<int64_t>(n, 1)) != cudaSuccess) {
+// blocks of the integrated near field: a target, 1 .. PF_G of its leaf's nodes
+__global__ void k_audit_blocks(const int4* __restrict__ blk, int64_t n, const int32_t* __restrict__ targets, int64_t nT,
+                               const int4* __restrict__ range, AuditOut* o) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int4 b = blk[i];
+    bool ok = b.x >= 0 && b.x < nT && b.z >= 1 && b.z <= PF_G;
+    if (ok) {
+      const int4 r = range[targets[b.x]];
+      ok = b.y >= r.z && (int64_t)b.y + b.z <= r.w;
+    }
+    if (!ok) audit_fail(o, i);
+  }
+}
+
+// clusters: 1 .. CL_V vertices, CL_E edges, CL_F faces, boundary faces among them, each part inside its array
+__global__ void k_audit_clusters(const int4* __restrict__ cnt, const int4* __restrict__ pos, int64_t n, int64_t nv,
+                                 int64_t ne, int64_t nf, int64_t nb, AuditOut* o) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int4 c = cnt[i], p = pos[i];
+    const bool ok = c.x >= 1 && c.x <= CL_V && c.y >= 1 && c.y <= CL_E && c.z >= 1 && c.z <= CL_F && c.w >= 0 &&
+                    c.w <= c.z && p.x >= 0 && (int64_t)p.x + c.x <= nv && p.y >= 0 && (int64_t)p.y + c.y <= ne &&
+                    p.z >= 0 && (int64_t)p.z + c.z <= nf && p.w >= 0 && (int64_t)p.w + c.w <= nb;
+    if (!ok) audit_fail(o, i);
+  }
+}
+
+// packed positions of a cluster's edges (two vertices) and faces (three vertices, three edges) below its
+// counts; the failing position is that of the edge or face.  One block per cluster (checked before).
+__global__ void k_audit_cluster_edges(const int4* __restrict__ cnt, const int4* __restrict__ pos,
+                                      const uint32_t* __restrict__ edge, int64_t ne, AuditOut* o) {
+  const int4 c = cnt[blockIdx.x], p = pos[blockIdx.x];
+  for (int t = threadIdx.x; t < c.y && t < CL_E; t += blockDim.x) {
+    const int64_t q = (int64_t)p.y + t;
+    if (q < 0 || q >= ne) continue;  // reported by k_audit_clusters
+    if ((int)(edge[q] & 0xFFFFu) >= c.x || (int)(edge[q] >> 16) >= c.x) audit_fail(o, q);
+  }
+}
+__global__ void k_audit_cluster_faces(const int4* __restrict__ cnt, const int4* __restrict__ pos,
+                                      const uint2* __restrict__ fidx, int64_t nf, AuditOut* o) {
+  const int4 c = cnt[blockIdx.x], p = pos[blockIdx.x];
+  for (int t = threadIdx.x; t < c.z && t < CL_F; t += blockDim.x) {
+    const int64_t q = (int64_t)p.z + t;
+    if (q < 0 || q >= nf) continue;
+    bool ok = true;
+    for (int k = 0; k < 3; k++)
+      ok = ok && (int)((fidx[q].x >> (8 * k)) & 255u) < c.x && (int)((fidx[q].y >> (9 * k)) & 511u) < c.y;
+    if (!ok) audit_fail(o, q);
+  }
+}
+
+// entries of an octree translation: position below hi
+template <class T>
+__global__ void k_audit_entries(const TEnt<T>* __restrict__ ent, int64_t n, int hi, AuditOut* o) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    if (ent[i].k >= hi) audit_fail(o, i);
+}
+
+// items of the table M2L: table positions up to the zero at nc, the chunk's moments within the padded block
+__global__ void k_audit_items(const TabItem* __restrict__ it, int64_t n, int nc, int nchunk, AuditOut* o) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    bool ok = it[i].chunk >= 0 && it[i].chunk < nchunk;
+    for (int k = 0; k < TAB_TR * TAB_TC; k++) ok = ok && it[i].idx[k] <= nc;
+    if (!ok) audit_fail(o, i);
+  }
+}
+
+// ranges [x, y) within [0, hi]
+__global__ void k_audit_spans(const int2* __restrict__ r, int64_t n, int hi, AuditOut* o) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    if (!(0 <= r[i].x && r[i].x <= r[i].y && r[i].y <= hi)) audit_fail(o, i);
+}
+
+// a scratch copy of a device list with one entry replaced, freed on scope exit (test hook)
+template <class T>
+struct Planted {
+  T* p = nullptr;
+  Planted(const T* list, int64_t n, int64_t at, T value, cudaStream_t s) {
+    if (cudaMalloc(&p, sizeof(T) * (size_t)n) != cudaSuccess) {
       cudaGetLastError();
       fail(DEMAG_ERR_OUT_OF_MEMORY, "plan audit scratch");
     }
+    DM_CUDA(cudaMemcpyAsync(p, list, sizeof(T) * n, cudaMemcpyDeviceToDevice, s));
+    DM_CUDA(cudaMemcpyAsync(p + at, &value, sizeof value, cudaMemcpyHostToDevice, s));
+    DM_CUDA(cudaStreamSynchronize(s));
   }
-  ~Scratch32() {
+  Planted(const Planted&) = delete;
+  ~Planted() {
     if (p) cudaFree(p);
   }
 };
+
+template <class T>
+T entry(const T* list, int64_t at) {
+  T v{};
+  DM_CUDA(cudaMemcpy(&v, list + at, sizeof v, cudaMemcpyDeviceToHost));
+  return v;
+}
 
 struct Check {
   std::string name;
@@ -116,6 +201,43 @@ class Auditor {
     k_audit_children<<<grid(n), 256, 0, s_>>>(child0, nchild, n, out(name));
     DM_LAUNCH("k_audit_children");
   }
+  void blocks(const char* name, const int4* blk, int64_t n) {
+    if (!begin(name, blk, n, 0, n * (int64_t)sizeof(int4))) return;
+    k_audit_blocks<<<grid(n), 256, 0, s_>>>(blk, n, P_.p2p_targets, (int64_t)P_.h_p2p_targets.size(), P_.cell_range,
+                                            out(name));
+    DM_LAUNCH("k_audit_blocks");
+  }
+  void clusters(const char* name, const int4* cnt, const int4* pos, int64_t n) {
+    if (!begin(name, cnt, n, 0, n * (int64_t)sizeof(int4))) return;
+    k_audit_clusters<<<grid(n), 256, 0, s_>>>(cnt, pos, n, P_.n_cl_v, P_.n_cl_e, P_.n_cl_f, P_.n_cl_b, out(name));
+    DM_LAUNCH("k_audit_clusters");
+  }
+  void cluster_edges(const char* name, const uint32_t* edge, int64_t n) {
+    if (!begin(name, edge, n, 0, n * (int64_t)sizeof(uint32_t))) return;
+    k_audit_cluster_edges<<<(unsigned)P_.n_clusters, 128, 0, s_>>>(P_.cl_cnt, P_.cl_pos, edge, n, out(name));
+    DM_LAUNCH("k_audit_cluster_edges");
+  }
+  void cluster_faces(const char* name, const uint2* fidx, int64_t n) {
+    if (!begin(name, fidx, n, 0, n * (int64_t)sizeof(uint2))) return;
+    k_audit_cluster_faces<<<(unsigned)P_.n_clusters, 128, 0, s_>>>(P_.cl_cnt, P_.cl_pos, fidx, n, out(name));
+    DM_LAUNCH("k_audit_cluster_faces");
+  }
+  template <class T>
+  void entries(const char* name, const TEnt<T>* ent, int64_t n, int hi) {
+    if (!begin(name, ent, n, 0, n * (int64_t)sizeof(TEnt<T>))) return;
+    k_audit_entries<T><<<grid(n), 256, 0, s_>>>(ent, n, hi, out(name));
+    DM_LAUNCH("k_audit_entries");
+  }
+  void items(const char* name, const TabItem* it, int64_t n) {
+    if (!begin(name, it, n, 0, n * (int64_t)sizeof(TabItem))) return;
+    k_audit_items<<<grid(n), 256, 0, s_>>>(it, n, P_.nc, (P_.nq + TAB_TC - 1) / TAB_TC, out(name));
+    DM_LAUNCH("k_audit_items");
+  }
+  void spans(const char* name, const int2* r, int64_t n, int hi) {
+    if (!begin(name, r, n, 0, n * (int64_t)sizeof(int2))) return;
+    k_audit_spans<<<grid(n), 256, 0, s_>>>(r, n, hi, out(name));
+    DM_LAUNCH("k_audit_spans");
+  }
   // the last of n + 1 device offsets (the length of the list they index)
   int64_t last(const int64_t* off, int64_t n) {
     int64_t v = 0;
@@ -125,15 +247,17 @@ class Auditor {
     return v;
   }
 
-  void finish() {
+  // the first failed check ("": none); ends this auditor's checks
+  std::string report() {
+    std::string msg;
     if (!checks_.empty()) {
       std::vector<AuditOut> h(checks_.size());
       DM_CUDA(cudaMemcpyAsync(h.data(), dout_, sizeof(AuditOut) * h.size(), cudaMemcpyDeviceToHost, s_));
       DM_CUDA(cudaStreamSynchronize(s_));
-      for (size_t k = 0; k < h.size(); k++) {
+      for (size_t k = 0; k < h.size() && msg.empty(); k++) {
         if (h[k].bad == 0) continue;
         const Check& c = checks_[k];
-        std::string msg = "plan audit: " + c.name + "[" + std::to_string(h[k].first) + "]";
+        msg = "plan audit: " + c.name + "[" + std::to_string(h[k].first) + "]";
         if (c.esize == 4 || c.esize == 8) {
           int64_t v = 0;
           int32_t v32 = 0;
@@ -142,15 +266,15 @@ class Auditor {
           msg += " = " + std::to_string(c.esize == 4 ? (int64_t)v32 : v);
         }
         msg += " out of range (" + std::to_string(h[k].bad) + " entries)";
-        release();
-        fail(DEMAG_ERR_INTERNAL, msg);
       }
     }
-    if (!error_.empty()) {
-      release();
-      fail(DEMAG_ERR_INTERNAL, error_);
-    }
+    if (msg.empty()) msg = error_;
     release();
+    return msg;
+  }
+  void finish() {
+    const std::string msg = report();
+    if (!msg.empty()) fail(DEMAG_ERR_INTERNAL, msg);
   }
   ~Auditor() { release(); }
 
@@ -205,6 +329,8 @@ class Auditor {
     if (dout_) cudaFree(dout_);
     dout_ = nullptr;
     cap_ = 0;
+    checks_.clear();
+    error_.clear();
   }
 
   Plan& P_;
@@ -214,6 +340,58 @@ class Auditor {
   size_t cap_ = 0;
   std::string error_;
 };
+
+template <class T>
+void audit_translations(Plan& P, Auditor& A) {
+  A.entries("m2m_ent", (const TEnt<T>*)P.m2m_ent, (int64_t)P.m2m_width * P.nq, 8 * P.nq);
+  A.entries("l2l_ent", (const TEnt<T>*)P.l2l_ent, P.l2l_nent, P.nl);
+}
+
+// test hook: lists of every kind as scratch copies with one entry out of range (read by the audit only, the
+// plan's own lists are untouched); the reports of all of them
+std::string planted(Plan& P, Auditor& A) {
+  std::string all = A.report();
+  cudaStream_t s = P.stream;
+  auto add = [&] {
+    const std::string m = A.report();
+    all += (all.empty() || m.empty() ? "" : "; ") + m;
+  };
+  if (P.n_clusters > 0 && P.n_pc_blk > 0) {
+    const int64_t c = P.n_clusters - 1;
+    const int4 cnt = entry(P.cl_cnt, c), pos = entry(P.cl_pos, c);
+    Planted<int4> n(P.cl_cnt, P.n_clusters, c, make_int4(cnt.x, cnt.y, CL_F + 1, cnt.w), s);
+    A.clusters("cl_cnt (planted copy)", n.p, P.cl_pos, P.n_clusters);
+    add();
+    Planted<uint32_t> e(P.cl_edge, P.n_cl_e, pos.y, entry(P.cl_edge, pos.y) | (uint32_t)cnt.x << 16, s);
+    A.cluster_edges("cl_edge (planted copy)", e.p, P.n_cl_e);
+    add();
+    Planted<uint2> f(P.cl_fidx, P.n_cl_f, pos.z, make_uint2(entry(P.cl_fidx, pos.z).x, 511u << 18), s);
+    A.cluster_faces("cl_fidx (planted copy)", f.p, P.n_cl_f);
+    add();
+    const int4 b = entry(P.pc_blk, P.n_pc_blk - 1);
+    Planted<int4> k(P.pc_blk, P.n_pc_blk, P.n_pc_blk - 1, make_int4(b.x, b.y, PF_G + 1, 0), s);
+    A.blocks("pc_blk (planted copy)", k.p, P.n_pc_blk);
+    add();
+  }
+  if (P.l2l_nent > 0) {
+    Planted<int2> r(P.l2l_cls, 8 * P.nl, 0, make_int2(0, P.l2l_nent + 1), s);
+    A.spans("l2l_cls (planted copy)", r.p, 8 * P.nl, P.l2l_nent);
+    add();
+  }
+  if (P.m2l_tab_nitems > 0) {
+    TabItem it = entry(P.m2l_tab_items, 0);
+    it.idx[0] = (uint16_t)(P.nc + 1);
+    Planted<TabItem> t(P.m2l_tab_items, P.m2l_tab_nitems, 0, it, s);
+    A.items("m2l_tab_items (planted copy)", t.p, P.m2l_tab_nitems);
+    add();
+  }
+  if (P.n_m2l > 0) {
+    Planted<int32_t> m(P.m2l_src, P.n_m2l, P.n_m2l - 1, (int32_t)P.ncells, s);
+    A.values("m2l_src (planted copy)", m.p, P.n_m2l, 0, P.ncells);
+    add();
+  }
+  return all;
+}
 
 }  // namespace
 
@@ -268,6 +446,10 @@ void audit_plan(Plan& P, bool plant) {
     A.values("cl_off", P.cl_off, nc + 1, 0, P.n_clusters + 1);
     A.values("cl_vnode", P.cl_vnode, P.n_cl_v, 0, nn);
     A.values("cl_ftet", (const int32_t*)P.cl_ftet, 2 * P.n_cl_f, -1, nt);
+    A.clusters("cl_cnt", P.cl_cnt, P.cl_pos, P.n_clusters);
+    A.cluster_edges("cl_edge", P.cl_edge, P.n_cl_e);
+    A.cluster_faces("cl_fidx", P.cl_fidx, P.n_cl_f);
+    A.blocks("pc_blk", P.pc_blk, P.n_pc_blk);
     if (P.pc_off) {
       A.offsets("pc_off", P.pc_off, nT, 0, P.n_pc, 0, P.n_pc);
       A.values("pc_src", P.pc_src, P.n_pc, 0, P.n_clusters);
@@ -275,8 +457,15 @@ void audit_plan(Plan& P, bool plant) {
   }
   // far field: parent lists, M2L operator indices
   A.values("par_list", P.par_list, P.par_start.empty() ? 0 : P.par_start.back(), 0, nc);
+  A.values("m2m_cnt", P.m2m_cnt, P.nq, 0, P.m2m_width + 1);
+  A.spans("l2l_cls", P.l2l_cls, 8 * P.nl, P.l2l_nent);
+  if (P.opt.precision == DEMAG_FP64)
+    audit_translations<double>(P, A);
+  else
+    audit_translations<float>(P, A);
   if (P.m2l_op) A.values("m2l_op", P.m2l_op, P.n_m2l, 0, P.n_m2l_keys);
   if (P.m2l_tab_opdl) A.values("m2l_tab_opdl", P.m2l_tab_opdl, P.n_m2l, 0, P.n_m2l_keys, 0x00ffffff);
+  A.items("m2l_tab_items", P.m2l_tab_items, P.m2l_tab_nitems);
   // mixed path: gradient operator, M2L groups
   if (P.opt.precision != DEMAG_FP64) {
     A.values("node_iperm", P.node_iperm, nn, 0, nn);
@@ -293,16 +482,9 @@ void audit_plan(Plan& P, bool plant) {
       A.values("tc_g2_op", P.tc_g2_op, 2 * ne, -1, P.n_m2l_keys);
     }
   }
-  // test hook: a scratch copy of the M2L source list with its last entry set
-  // to n_cells (read by this audit only; the plan's own list is untouched)
-  if (plant && P.n_m2l > 0) {
-    Scratch32 bad(P.n_m2l);
-    DM_CUDA(cudaMemcpyAsync(bad.p, P.m2l_src, sizeof(int32_t) * P.n_m2l, cudaMemcpyDeviceToDevice, P.stream));
-    const int32_t v = (int32_t)nc;
-    DM_CUDA(cudaMemcpyAsync(bad.p + P.n_m2l - 1, &v, sizeof v, cudaMemcpyHostToDevice, P.stream));
-    DM_CUDA(cudaStreamSynchronize(P.stream));
-    A.values("m2l_src (planted copy)", bad.p, P.n_m2l, 0, nc);
-    A.finish();  // before the copy is freed
+  if (plant) {
+    const std::string found = planted(P, A);
+    if (!found.empty()) fail(DEMAG_ERR_INTERNAL, found);
     return;
   }
   A.finish();

@@ -40,6 +40,14 @@ struct TEnt {
   T c;
 };
 
+// one item of the table-driven M2L (m2l32.cu): TAB_TR rows m times TAB_TC moments n
+constexpr int TAB_TR = 4, TAB_TC = 8;
+struct TabItem {  // 80 bytes
+  uint16_t idx[TAB_TR * TAB_TC];  // table position of b_{m+n} for row r, moment j (nc, a zero, where there is no term)
+  uint8_t deg[TAB_TC];            // |n|
+  int32_t chunk, pad;             // moments TAB_TC chunk ..
+};
+
 // Graded multi-index order: total degree t ascending; within t, n_x descending,
 // then n_z ascending.  Index of (a,b,c):
 //   t(t+1)(t+2)/6 + (b+c)(b+c+1)/2 + c,  t = a+b+c.
@@ -142,8 +150,11 @@ __device__ __forceinline__ void load_q(const T* q, T (&v)[SB]) {
 // faces have the fixed counter-clockwise vertex orders below.
 // ---------------------------------------------------------------------------
 constexpr int TET_GEO = 66;
-// states per slice of the integrated near field (at most)
-constexpr int P2P_SLICE = 16;
+// integrated near field (p2p.cu): states per slice and target nodes per block (at
+// most); tets per cluster, and the bounds of a cluster's vertices, edges and faces
+constexpr int P2P_SLICE = 16, PF_G = 16;
+constexpr int CL_TETS = 40;
+constexpr int CL_V = 4 * CL_TETS, CL_E = 6 * CL_TETS, CL_F = 4 * CL_TETS;
 
 // ---------------------------------------------------------------------------
 // the plan
@@ -265,7 +276,8 @@ struct Plan {
   int32_t* m2l_op = nullptr;        // n_m2l
   int64_t n_m2l_keys = 0;           // distinct translation keys (m2l_keys.cu)
   void* m2l_tab = nullptr;          // b_k(v) per key for the CUDA-core M2L (FP64 plans: doubles, else floats)
-  void* m2l_tab_items = nullptr;    // its work items (per order)
+  TabItem* m2l_tab_items = nullptr; // its work items (per order)
+  int m2l_tab_nitems = 0;
   int32_t* m2l_tab_opdl = nullptr;  // n_m2l: key index | (level difference & 255) << 24
   int tc_nt = 1, tc_kps = 0, tc_budget = 0;  // M2L launch shape: targets per CTA, k-steps per slot, ring bytes
   int tc_ls = 0;                    // split BF16 limb scheme of the tensor-core M2L (m2l_tc.cu)
@@ -284,6 +296,7 @@ struct Plan {
   void* far_h = nullptr;            // nn x nl: the L2P polynomials of every node
   // octree translations as coefficient lists (TEnt<T>, far.cu): M2M entry j of
   // row n at [j][n]; L2L entries of (row, parity class) q in [l2l_cls[q].x, .y)
+  int m2m_width = 0;                // most entries of a row
   int32_t* m2m_cnt = nullptr;       // nq: entries of every row
   void* m2m_ent = nullptr;
   int l2l_nent = 0;

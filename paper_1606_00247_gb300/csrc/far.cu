@@ -627,6 +627,7 @@ void build_translations(Plan& P) {
   std::vector<TEnt<T>> ment(width * nq, TEnt<T>{0, (T)0});
   for (int r = 0; r < nq; r++)
     for (size_t j = 0; j < mrow[r].size(); j++) ment[j * nq + r] = mrow[r][j];
+  P.m2m_width = (int)width;
   P.l2l_nent = (int)lent.size();
   P.m2m_cnt = dalloc<int32_t>(P, nq);
   P.m2m_ent = dalloc<TEnt<T>>(P, ment.size());

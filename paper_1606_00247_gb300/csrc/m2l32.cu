@@ -176,7 +176,7 @@ template void launch_m2l_rows<double>(Plan&, int, const double*, double*, cudaSt
 // order at the end, so results do not depend on timing.
 namespace tab {
 
-constexpr int TR = 4, TC = 8, THREADS = 256, WARPS = THREADS / 32;
+constexpr int TR = TAB_TR, TC = TAB_TC, THREADS = 256, WARPS = THREADS / 32;
 constexpr int MAX_CHUNKS = (MAX_P + 1) * (MAX_P + 1) / TC + 1;
 constexpr int KS_MAX = 32;  // sources per step, at most KS_MAX / WARPS per staging warp
 
@@ -184,12 +184,6 @@ struct Shape {
   int ks, kg;                    // sources per step, source subgroups
   int nchunk, nitems;
   int16_t off[MAX_CHUNKS + 1];   // first item of every chunk: row group g is item off[c] + g
-};
-
-struct Item {  // 80 bytes
-  uint16_t idx[TR * TC];  // table position of b_{m+n} for row r, moment j (the zero slot where there is no term)
-  uint8_t deg[TC];        // |n|
-  int32_t chunk, pad;
 };
 
 // items of order p: chunk c of row group g exists when the group's lowest row takes moments of it
@@ -243,7 +237,7 @@ __global__ void __launch_bounds__(THREADS, 2) k_m2l_tab(const int32_t* __restric
                                                      const int64_t* __restrict__ m2l_off,
                                                      const int32_t* __restrict__ m2l_src,
                                                      const int32_t* __restrict__ m2l_opdl, const T* __restrict__ tab,
-                                                     const Item* __restrict__ items, const Shape S, const int32_t* __restrict__ level, double side,
+                                                     const TabItem* __restrict__ items, const Shape S, const int32_t* __restrict__ level, double side,
                                                      int p, int nc, int B, const T* __restrict__ Q, T* L) {
   extern __shared__ __align__(16) unsigned char tab_smem[];
   T* sm = (T*)tab_smem;
@@ -265,7 +259,7 @@ __global__ void __launch_bounds__(THREADS, 2) k_m2l_tab(const int32_t* __restric
   // this thread's item
   const int k0 = tid / S.nitems;
   const bool has = k0 < S.kg;
-  const Item* it = items + (tid - k0 * S.nitems);
+  const TabItem* it = items + (tid - k0 * S.nitems);
   const int c = it->chunk;
   // table positions; FP64 (bound by its arithmetic, short of registers) keeps two per word
   constexpr int IP = sizeof(T) == 8 ? 2 : 1;
@@ -405,7 +399,7 @@ void launch_sb(Plan& P, int B, const T* Q, T* L, cudaStream_t s) {
   smem_opt_in((const void*)k_m2l_tab<T, SB>, smem);
   const dim3 grid((unsigned)P.h_m2l_targets.size(), (unsigned)((B + SB - 1) / SB));
   k_m2l_tab<T, SB><<<grid, THREADS, smem, s>>>(P.m2l_targets, P.m2l_off, P.m2l_src, P.m2l_tab_opdl,
-                                               (const T*)P.m2l_tab, (const Item*)P.m2l_tab_items, S,
+                                               (const T*)P.m2l_tab, P.m2l_tab_items, S,
                                                P.cell_level, P.side, P.p, P.nc, B, Q, L);
   DM_LAUNCH("k_m2l_tab");
 }
@@ -454,10 +448,10 @@ void build_m2l_tab(Plan& P, const M2lKeys& K) {
   const size_t nk = K.keys.size();
   const bool fp64 = P.opt.precision == DEMAG_FP64;
   const tab::Shape S = tab::shape(P.p, fp64 ? 8 : 4);
-  std::vector<tab::Item> items(S.nitems);
+  std::vector<TabItem> items(S.nitems);
   for (int c = 0; c < S.nchunk; c++)
     for (int i = S.off[c]; i < S.off[c + 1]; i++) {
-      tab::Item& it = items[i];
+      TabItem& it = items[i];
       it.chunk = c;
       it.pad = 0;
       for (int j = 0; j < tab::TC; j++) {
@@ -474,8 +468,9 @@ void build_m2l_tab(Plan& P, const M2lKeys& K) {
         }
       }
     }
-  P.m2l_tab_items = dalloc<tab::Item>(P, items.size());
-  DM_CUDA(cudaMemcpyAsync(P.m2l_tab_items, items.data(), items.size() * sizeof(tab::Item), cudaMemcpyHostToDevice, s));
+  P.m2l_tab_nitems = S.nitems;
+  P.m2l_tab_items = dalloc<TabItem>(P, items.size());
+  DM_CUDA(cudaMemcpyAsync(P.m2l_tab_items, items.data(), items.size() * sizeof(TabItem), cudaMemcpyHostToDevice, s));
   P.m2l_tab_opdl = dalloc<int32_t>(P, P.n_m2l);
   P.m2l_tab = dalloc<unsigned char>(P, nk * (size_t)tab::row_len(P.nc) * (fp64 ? sizeof(double) : sizeof(float)));
   int4* dkeys = nullptr;

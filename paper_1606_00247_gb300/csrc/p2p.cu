@@ -145,10 +145,8 @@ void build_tet_geometry(Plan& P) {
 // ---------------------------------------------------------------------------
 namespace {
 
-constexpr int PF_G = 16, PF_GMIN = 4;         // target nodes of a near-field block: most, and least of a split leaf
+constexpr int PF_GMIN = 4;               // target nodes of a block of a split leaf, at least
 constexpr double PF_SPLIT = 4.0;
-constexpr int CL_TETS = 40;              // tets per cluster
-constexpr int CL_V = 4 * CL_TETS, CL_E = 6 * CL_TETS, CL_F = 4 * CL_TETS;  // bounds of its parts
 constexpr int FACE_REC = 16;             // doubles per face: n, t, m (9), 2 area, c_1, d_1, c_2, d_2, 1 / length of edge 0, (v2 - v0).t
 static_assert(CL_V <= 256 && CL_E <= 512, "8-bit vertex and 9-bit edge positions");
 

@@ -59,3 +59,22 @@ def test_audit_reports_an_index_out_of_range_and_the_plan_stays_usable():
     u1, H1 = pl.eval(M)
     assert torch.equal(u0, u1) and torch.equal(H0, H1)
     assert _lib.demag_plan_debug(pl.handle, 4) == _lib.DEMAG_ERR_INVALID_ARG
+
+
+def test_audit_covers_the_integrated_near_field_and_the_translations():
+    """One entry of each list of the clusters, their blocks and the translations out of range."""
+    from paper_1606_00247_gb300 import _lib
+
+    nodes, tets = inputs.sphere(h=0.2)
+    pl = _plan(nodes, tets, p=4, leaf_size=16, precision="fp64", near_mode=0)
+    M = torch.as_tensor(inputs.gaussian_unit_m(nodes.shape[0], batch=1, seed=504), device="cuda")
+    u0, _ = pl.eval(M)
+    assert _lib.demag_plan_audit(pl.handle) == _lib.DEMAG_OK
+    assert _lib.demag_plan_debug(pl.handle, 2) == _lib.DEMAG_OK
+    assert _lib.demag_plan_audit(pl.handle) == _lib.DEMAG_ERR_INTERNAL
+    msg = _lib.demag_last_error()
+    for name in ("cl_cnt", "cl_edge", "cl_fidx", "pc_blk", "l2l_cls", "m2l_tab_items", "m2l_src"):
+        assert f"plan audit: {name} (planted copy)[" in msg, (name, msg)
+    assert msg.count("(1 entries)") == 7
+    assert _lib.demag_plan_debug(pl.handle, 0) == _lib.DEMAG_OK
+    assert torch.equal(pl.eval(M)[0], u0)
