@@ -390,7 +390,8 @@ typedef struct {
   int64_t n_m2l_ops;     /* distinct M2L translation keys (level difference,
                             lattice offset) tabulated for the tensor-core and
                             table-driven M2L of the mixed path (0: none)    */
-  int m2l_kps;           /* tensor-core M2L ring: k-steps per slot          */
+  int m2l_kps;           /* tensor-core M2L ring (of max_batch states unless
+                            tuned): k-steps per slot                    */
   int m2l_ring_bytes;    /* tensor-core M2L ring: shared memory per CTA     */
   int m2l_targets_per_cta; /* tensor-core M2L: target cells sharing each
                             source's moments in one CTA (1 or 2)            */

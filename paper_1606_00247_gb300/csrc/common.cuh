@@ -279,7 +279,9 @@ struct Plan {
   TabItem* m2l_tab_items = nullptr; // its work items (per order)
   int m2l_tab_nitems = 0;
   int32_t* m2l_tab_opdl = nullptr;  // n_m2l: key index | (level difference & 255) << 24
-  int tc_nt = 1, tc_kps = 0, tc_budget = 0;  // M2L launch shape: targets per CTA, k-steps per slot, ring bytes
+  // M2L launch shape of max_batch states: targets per CTA, k-steps per slot, ring bytes; tuned: of every batch
+  int tc_nt = 1, tc_kps = 0, tc_budget = 0;
+  bool tc_tuned = false;
   int tc_ls = 0;                    // split BF16 limb scheme of the tensor-core M2L (m2l_tc.cu)
   int tc_prom_group = 0, tc_prom_rows = 16;  // accumulator promotion: sources per group (0 = off), rows
   int64_t* tc_g1_off = nullptr;     // one-target groups: list offsets in target order

@@ -790,11 +790,11 @@ constexpr int TC_BUDGET_4 = 56 * 1024, TC_BUDGET_3 = 72 * 1024, TC_BUDGET_2 = 10
 // SM is what counts: 224k-tet ball, p = 8, 256 states, two CTAs per SM 6.7 (two
 // k-steps per slot) and 5.7 ms (five), three CTAs 3.9 ms, four CTAs 3.65 ms (two
 // steps of three); four targets per CTA sharing the moments, two CTAs, 5.3 ms.
-// Three CTAs where the grid does not fill four per SM (473 targets, one state
-// block: 243 against 269 us).  nt / kps override it.
-void default_ring(const Plan& P, const TcLayout& G, int nt, int kps, TcRing& R) {
+// Three CTAs where the grid of the evaluated batch does not fill four per SM (473
+// targets, one state block: 243 against 269 us).  nt / kps override it.
+void default_ring(const Plan& P, const TcLayout& G, int B, int nt, int kps, TcRing& R) {
   if (nt == 0) nt = 1;
-  const int64_t work = (int64_t)P.h_m2l_targets.size() * ((P.opt.max_batch + TC_M - 1) / TC_M);
+  const int64_t work = (int64_t)P.h_m2l_targets.size() * ((B + TC_M - 1) / TC_M);
   int budget = nt == 2 || G.tmem_cols > 256 ? TC_BUDGET_1
                : P.tc_prom_rows > 16        ? TC_BUDGET_2  // 64 registers of promoted sums
                : work <= 4 * 152            ? TC_BUDGET_3
@@ -863,9 +863,10 @@ void tune_ring(Plan& P, const TcLayout& G) {
   if (h_err) fail(DEMAG_ERR_TIMEOUT, "tensor-core M2L timed out while tuning");
 }
 
-bool current_ring(const Plan& P, const TcLayout& G, TcRing& R) {
-  if (!(P.tc_kps > 0 && make_ring(G, P.tc_nt, P.tc_kps, P.tc_budget, R)))
-    default_ring(P, G, P.opt.m2l_targets_per_cta, P.opt.m2l_kps, R);
+// the tuned shape, or the default one for a batch of B states
+bool current_ring(const Plan& P, const TcLayout& G, int B, TcRing& R) {
+  if (!(P.tc_tuned && make_ring(G, P.tc_nt, P.tc_kps, P.tc_budget, R)))
+    default_ring(P, G, B, P.opt.m2l_targets_per_cta, P.opt.m2l_kps, R);
   set_promotion(P, G, R);
   return R.nslots >= 2;
 }
@@ -960,9 +961,10 @@ void build_m2l_tc(Plan& P, const M2lKeys& K) {
     } else {
       tune_ring(P, G);
     }
+    P.tc_tuned = P.tc_kps > 0;
   }
   TcRing R;
-  if (!current_ring(P, G, R)) fail(DEMAG_ERR_UNSUPPORTED, "no ring shape fits the tensor-core M2L");
+  if (!current_ring(P, G, P.opt.max_batch, R)) fail(DEMAG_ERR_UNSUPPORTED, "no ring shape fits the tensor-core M2L");
   P.tc_nt = R.nt;
   P.tc_kps = R.kps;
   P.tc_budget = R.nslots * R.slot_bytes;
@@ -981,7 +983,7 @@ bool launch_m2l_tc(Plan& P, int B, const float* Q, unsigned char* QP, float* L, 
   if (!tc_enabled(P) || QP == nullptr) return false;
   const TcLayout G = layout_of(P);
   TcRing R;
-  if (!current_ring(P, G, R)) return false;
+  if (!current_ring(P, G, B, R)) return false;
   const int nsb = (B + TC_M - 1) / TC_M;
   const dim3 grid((unsigned)P.ncells, (unsigned)nsb);
   if (G.bf16)
