@@ -196,6 +196,7 @@ static demag_plan_s* new_plan(const demag_options& o, int64_t n_nodes, int64_t n
     P->nn = n_nodes;
     P->nt = n_tets;
     DM_CUDA(cudaGetDevice(&P->device));
+    DM_CUDA(cudaDeviceGetAttribute(&P->sms, cudaDevAttrMultiProcessorCount, P->device));
     DM_CUDA(cudaStreamCreateWithFlags(&P->stream, cudaStreamNonBlocking));
     build_plan(*P, nodes, tets);
   } catch (...) {

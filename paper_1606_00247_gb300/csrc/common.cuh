@@ -169,6 +169,7 @@ struct DevBuf {
 
 struct Plan {
   int device = 0;
+  int sms = 0;                    // streaming multiprocessors of the device
   cudaStream_t stream = nullptr;  // plan-build stream
   demag_options opt{};
   int p = 4, nc = 35, nc1 = 20;   // order, ncoef(p), ncoef(p-1)

@@ -797,7 +797,7 @@ void default_ring(const Plan& P, const TcLayout& G, int B, int nt, int kps, TcRi
   const int64_t work = (int64_t)P.h_m2l_targets.size() * ((B + TC_M - 1) / TC_M);
   int budget = nt == 2 || G.tmem_cols > 256 ? TC_BUDGET_1
                : P.tc_prom_rows > 16        ? TC_BUDGET_2  // 64 registers of promoted sums
-               : work <= 4 * 152            ? TC_BUDGET_3
+               : work <= 4 * P.sms          ? TC_BUDGET_3
                                             : TC_BUDGET_4;
   if (kps == 0) {
     for (kps = G.KS; kps > 1 && !make_ring(G, nt, kps, budget, R); kps--) {

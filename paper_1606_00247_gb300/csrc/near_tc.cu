@@ -414,9 +414,9 @@ constexpr int NFS_SLICE = 16, NFS_MAX = 64;  // states per pass over W, largest 
 // Up to 8 states always; larger batches while their passes of 16 states over the
 // tiles cost less than the tensor-core kernel's waves of one CTA per SM (a pass
 // takes about as long as the tensor cores on a full grid)
-bool small_batch(int64_t ntiles, int B) {
-  const int64_t slices = (B + NFS_SLICE - 1) / NFS_SLICE, waves = (ntiles + 151) / 152;
-  return B <= 8 || (B <= NFS_MAX && 10 * slices * ntiles <= 9 * 152 * waves);
+bool small_batch(int64_t ntiles, int B, int sms) {
+  const int64_t slices = (B + NFS_SLICE - 1) / NFS_SLICE, waves = (ntiles + sms - 1) / sms;
+  return B <= 8 || (B <= NFS_MAX && 10 * slices * ntiles <= 9 * sms * waves);
 }
 
 template <int SB>
@@ -550,11 +550,11 @@ size_t nf_mp_floats(const Plan& P, int B) {
 
 int launch_near_tc(Plan& P, const float* Ms, float* MP, int B, float* u_s, int* err, cudaStream_t s) {
   if (P.nf_ntiles == 0) return 0;
-  if (small_batch(P.nf_ntiles, B) && !(P.debug_flags & 1)) {
+  if (small_batch(P.nf_ntiles, B, P.sms) && !(P.debug_flags & 1)) {
     // parts: ~6 CTAs per SM, at least four column groups each on average, the
     // sums and Mbar within MP (whose copy of M this kernel does not use)
     const int64_t room = ((int64_t)nf_mp_floats(P, B) / (P.nf_ntiles * B) - 3) / NF_ROWS;
-    const int64_t want = std::min<int64_t>((6 * 152 + P.nf_ntiles - 1) / P.nf_ntiles, P.nf_ncols / 64 / P.nf_ntiles);
+    const int64_t want = std::min<int64_t>((6 * P.sms + P.nf_ntiles - 1) / P.nf_ntiles, P.nf_ncols / 64 / P.nf_ntiles);
     const int parts = (int)std::max<int64_t>(1, std::min(want, room));
     if (room >= 1) {
       if (B == 1)
@@ -580,9 +580,7 @@ int launch_near_tc(Plan& P, const float* Ms, float* MP, int B, float* u_s, int* 
   // the M of neighbouring columns from L2 (on GB300 the first is faster on the
   // 224k-tet ball at 128 states, ~2 waves; the second on the 559k-tet ball at
   // 256 states, ~10 waves)
-  int nsm = 152;
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, P.device);
-  const int32_t* order = (int64_t)grid.x < 4ll * nsm ? P.nf_order : nullptr;
+  const int32_t* order = (int64_t)grid.x < 4ll * P.sms ? P.nf_order : nullptr;
   k_near_tc<<<grid, NF_THREADS, NF_SMEM, s>>>(order, P.nf_woff, P.nf_coff, P.nf_ng, P.nf_npad, P.nf_rownode, P.nf_cols,
                                               P.nf_W, MP, P.nf_S, P.nn, B, (int)nsb, u_s, err, P.debug_flags & 1);
   DM_LAUNCH("k_near_tc");

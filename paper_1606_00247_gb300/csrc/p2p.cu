@@ -359,10 +359,7 @@ std::vector<int4> face_blocks(const Plan& P, const std::vector<int64_t>& cluster
     const int4 r = P.h_range[P.h_p2p_targets[t]];
     total += (double)clusters[t] * (r.w - r.z);
   }
-  int dev = 0, sms = 0;
-  DM_CUDA(cudaGetDevice(&dev));
-  DM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const double most = total / (2.0 * sms * PF_SPLIT);  // two blocks per SM
+  const double most = total / (2.0 * P.sms * PF_SPLIT);  // two blocks per SM
   std::vector<std::pair<double, int4>> q;
   for (int64_t t = 0; t < nT; t++) {
     const int4 r = P.h_range[P.h_p2p_targets[t]];
