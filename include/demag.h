@@ -143,15 +143,19 @@ typedef struct {
                           nodes; exact patch moments and analytic patch near
                           field; the same u as the tets up to the FMM
                           truncation; needs near_mode = 1                  */
-  int near_tc;         /* DEMAG_MIXED_BF16X3 with near_mode = 1: 0
-                          (default) applies the stored near-field
-                          coefficients (Sec. 3.4) on the tensor cores --
-                          tiles of up to 128 target nodes over the union of
-                          their source columns, coefficients and M in two
-                          BF16 limbs (16 significant bits; up to ~1e-5
-                          relative error per product), three MMAs per
-                          k-step, FP32 accumulation; < 0: FP32 CUDA cores,
-                          as in the other mixed precisions (BF16X6 always) */
+  int near_tc;         /* DEMAG_MIXED_BF16X3 with near_mode = 1: > 0
+                          applies the stored near-field coefficients
+                          (Sec. 3.4) on the tensor cores -- tiles of up to
+                          128 target nodes over the union of their source
+                          columns, coefficients and M in two BF16 limbs
+                          (16 significant bits; up to ~1e-5 relative error
+                          per product), three MMAs per k-step, FP32
+                          accumulation; 0 (default): batches of at most 8
+                          states (up to 64 where few tiles leave SMs idle)
+                          apply the same tiles on CUDA cores, M in FP32,
+                          larger ones on the tensor cores; < 0: FP32
+                          coefficients on CUDA cores, as in the other mixed
+                          precisions (BF16X6 always)                        */
   int graph;           /* 1: demag_eval with device pointers (and profile =
                           0) runs the first call with a given (M, u, H,
                           batch, workspace) directly, records it as a CUDA
@@ -328,17 +332,19 @@ demag_status demag_llg_rk4(demag_plan plan, double* m, int batch, double Ms, dou
 demag_status demag_plan_destroy(demag_plan plan);
 
 /* Test hooks (the paper has no counterpart).
- * flags bit 0, the error path of the bounded device waits: the tensor-core near field (DEMAG_MIXED_BF16X3,
- * near_mode = 1) issues none of its coefficient copies, so its MMA issuer's
- * bounded wait for them expires (after about a second) with no copy and no MMA
+ * flags bit 0, the error path of the bounded device waits: the tensor-core
+ * near field (DEMAG_MIXED_BF16X3, near_mode = 1, near_tc > 0 or a batch that it
+ * takes) issues none of its coefficient copies, so its MMA issuer's bounded wait
+ * for them expires (after about a second) with no copy and no MMA
  * in flight; the kernel records DEMAG_ERR_TIMEOUT, frees its tensor memory and
  * returns.  demag_eval then returns DEMAG_ERR_TIMEOUT for host pointers, and
  * demag_eval_status reports it for device pointers; the plan and the CUDA
  * context stay usable.
  * flags bit 1, the error path of the plan audit: demag_plan_audit also audits
- * a scratch copy of the M2L source list whose last entry is set to n_cells
- * (only the audit reads the copy; the plan's own lists are untouched), so it
- * returns DEMAG_ERR_INTERNAL naming that entry.
+ * scratch copies of lists of each kind with one entry out of range, among them
+ * the M2L source list with its last entry set to n_cells (only the audit reads
+ * the copies; the plan's own lists are untouched), so it returns
+ * DEMAG_ERR_INTERNAL naming those entries.
  * flags = 0 restores normal behaviour.
  * Errors: DEMAG_ERR_INVALID_ARG (NULL plan, unknown flag bits). */
 demag_status demag_plan_debug(demag_plan plan, int flags);

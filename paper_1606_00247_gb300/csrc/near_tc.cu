@@ -550,7 +550,7 @@ size_t nf_mp_floats(const Plan& P, int B) {
 
 int launch_near_tc(Plan& P, const float* Ms, float* MP, int B, float* u_s, int* err, cudaStream_t s) {
   if (P.nf_ntiles == 0) return 0;
-  if (small_batch(P.nf_ntiles, B, P.sms) && !(P.debug_flags & 1)) {
+  if (P.opt.near_tc == 0 && small_batch(P.nf_ntiles, B, P.sms)) {
     // parts: ~6 CTAs per SM, at least four column groups each on average, the
     // sums and Mbar within MP (whose copy of M this kernel does not use)
     const int64_t room = ((int64_t)nf_mp_floats(P, B) / (P.nf_ntiles * B) - 3) / NF_ROWS;

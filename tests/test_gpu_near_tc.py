@@ -5,7 +5,8 @@ The stored near-field coefficients (Sec. 3.4) are applied per tile of up to
 With theta -> 0 every interaction is near field, so the evaluation is the
 near-field kernel alone: it is held against the oracle's direct sum and
 against the FP64 path of the library, at batches that fill one or two
-128-state blocks per CTA, partly or exactly.  The plan build adds the
+128-state blocks per CTA, partly or exactly (near_tc = 1 keeps small batches
+on the tensor cores; with the default 0 the same tiles go to CUDA cores there).  The plan build adds the
 per-tet contributions to the coefficients as exact integer sums, so two
 builds give the same bits.
 """
@@ -33,8 +34,8 @@ def _plan(nodes, tets, **kw):
     return Plan(nodes, tets, **kw)
 
 
-@pytest.mark.parametrize("B", [1, 3, 128, 160, 256])
-def test_near_tc_theta_zero_vs_fp64_and_direct(orc, B):
+@pytest.mark.parametrize("B, near_tc", [(1, 1), (3, 1), (3, 0), (128, 0), (160, 0), (256, 0)])
+def test_near_tc_theta_zero_vs_fp64_and_direct(orc, B, near_tc):
     """Every pair in the near field: the split-BF16 tensor-core product against
     the FP64 coefficients applied in FP64, per state, and state 0 against the
     oracle's direct sum.  Two BF16 limbs keep 16 significant bits of each
@@ -43,7 +44,7 @@ def test_near_tc_theta_zero_vs_fp64_and_direct(orc, B):
     nodes, tets = inputs.sphere(h=0.2)
     M = inputs.gaussian_unit_m(nodes.shape[0], batch=B, seed=300 + B)
     kw = dict(p=2, leaf_size=32, theta=1e-9, near_mode=1, max_batch=B)
-    ptc = _plan(nodes, tets, precision="bf16x3", **kw)
+    ptc = _plan(nodes, tets, precision="bf16x3", near_tc=near_tc, **kw)
     st = ptc.stats()
     assert st["n_near_tiles"] > 0 and st["n_m2l"] == 0
     u, H = ptc.eval(M)
@@ -74,7 +75,8 @@ def test_near_tc_vs_cuda_core_near_field():
     assert per_state(Ha.cpu().numpy(), H64.cpu().numpy()) < 1e-4
 
 
-def test_near_tc_split_tiles_of_a_large_leaf(orc):
+@pytest.mark.parametrize("near_tc", [1, 0])
+def test_near_tc_split_tiles_of_a_large_leaf(orc, near_tc):
     """Leaves with more than 128 target nodes get tiles of their own (128 rows
     each, the leaf's columns in every one)."""
     nodes, tets = inputs.sphere(h=0.13)
@@ -84,7 +86,7 @@ def test_near_tc_split_tiles_of_a_large_leaf(orc):
     nodes_per_leaf = ex["cell_ranges"][:, 3] - ex["cell_ranges"][:, 2]
     assert nodes_per_leaf[leaf].max() > 128
     M = inputs.gaussian_unit_m(nodes.shape[0], batch=2, seed=402)
-    ptc = _plan(nodes, tets, precision="bf16x3", **kw)
+    ptc = _plan(nodes, tets, precision="bf16x3", near_tc=near_tc, **kw)
     u, H = ptc.eval(M)
     u64, H64 = _plan(nodes, tets, precision="fp64", **kw).eval(M)
     assert per_state(u.cpu().numpy(), u64.cpu().numpy()) < 3e-5
@@ -104,19 +106,20 @@ def test_plan_build_is_deterministic(prec):
     assert torch.equal(ua, ub) and torch.equal(Ha, Hb)
 
 
-def test_near_tc_dipole_sources(orc):
+@pytest.mark.parametrize("near_tc", [1, 0])
+def test_near_tc_dipole_sources(orc, near_tc):
     """The point-dipole comparison model through the tensor-core near field:
     theta -> 0 against the direct dipole sum."""
     nodes, tets = inputs.sphere(h=0.2)
     M = inputs.gaussian_unit_m(nodes.shape[0], batch=2, seed=404)
     kw = dict(p=2, leaf_size=32, theta=1e-9, near_mode=1, max_batch=2, sources="dipoles")
-    u, _ = _plan(nodes, tets, precision="bf16x3", **kw).eval(M)
+    u, _ = _plan(nodes, tets, precision="bf16x3", near_tc=near_tc, **kw).eval(M)
     ref = orc.dipole_direct(nodes, tets, M[0])
     assert rel_l2(u[0].cpu().numpy(), ref) < 3e-5
 
 
-@pytest.mark.parametrize("B", [2, 160])
-def test_near_tc_repeated_evaluations_are_identical(B):
+@pytest.mark.parametrize("B, near_tc", [(2, 1), (2, 0), (160, 0)])
+def test_near_tc_repeated_evaluations_are_identical(B, near_tc):
     """One plan evaluated five times: every evaluation gives the same bits and
     no device wait expires.  The state warps take part in every column group,
     so each waits for every use of each shared-memory stage in order (a
@@ -134,7 +137,7 @@ def test_near_tc_repeated_evaluations_are_identical(B):
         nodes, tets = inputs.sphere(h=0.06)
         M = inputs.smoothed_unit_m(tets, nodes.shape[0], batch=B, seed=405)
         kw = dict(p=6, leaf_size=64)
-    pl = _plan(nodes, tets, theta=0.5, near_mode=1, max_batch=B, precision="bf16x3", **kw)
+    pl = _plan(nodes, tets, theta=0.5, near_mode=1, max_batch=B, precision="bf16x3", near_tc=near_tc, **kw)
     assert pl.stats()["n_near_tiles"] > 0
     Md = torch.as_tensor(M, device="cuda")
     u0, H0 = pl.eval(Md)

@@ -21,7 +21,7 @@ def test_expired_wait_is_reported_and_the_plan_recovers():
     nodes, tets = inputs.sphere(h=0.2)
     B = 4
     M = torch.as_tensor(inputs.gaussian_unit_m(nodes.shape[0], batch=B, seed=501), device="cuda")
-    plan = Plan(nodes, tets, p=6, leaf_size=32, max_batch=B, precision="bf16x3", near_mode=1)
+    plan = Plan(nodes, tets, p=6, leaf_size=32, max_batch=B, precision="bf16x3", near_mode=1, near_tc=1)
     assert plan.stats()["n_near_tiles"] > 0
     u_ok, H_ok = plan.eval(M)
     torch.cuda.synchronize()

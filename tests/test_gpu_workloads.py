@@ -60,15 +60,15 @@ def test_film_full_size(orc):
     assert np.linalg.norm(g - ref[sel]) / np.linalg.norm(ref[sel]) < 1e-10
     # split BF16 (promotion on by default) vs FP64, per state; and without promotion
     errs = {}
-    for promote in (0, -1):  # tensor-core M2L forced at this batch of 2
+    for promote in (0, -1):  # tensor-core M2L and near field forced at this batch of 2
         pl = Plan(nodes, tets, p=8, leaf_size=128, theta=0.5, precision="bf16x3", near_mode=1, max_batch=2,
-                  m2l_promote=promote, m2l_table_batch=-1)
+                  m2l_promote=promote, m2l_table_batch=-1, near_tc=1)
         u, H = pl.eval(Md)
         errs[promote] = max(max(rel(u[k], u64[k]), rel(H[k], H64[k])) for k in range(2))
         del pl
     assert errs[0] <= 1e-4, errs
     assert errs[0] < errs[-1] / 3, errs  # promotion is what brings the film under the bar
-    # default at a batch of 2: the table-driven FP32 M2L on CUDA cores
+    # default at a batch of 2: the table-driven FP32 M2L and the tiles of the near field on CUDA cores
     pl = Plan(nodes, tets, p=8, leaf_size=128, theta=0.5, precision="bf16x3", near_mode=1, max_batch=2)
     u, H = pl.eval(Md)
     err = max(max(rel(u[k], u64[k]), rel(H[k], H64[k])) for k in range(2))
@@ -82,11 +82,13 @@ def test_ball_uniform_m_tensor_core():
     M = torch.as_tensor(np.stack([inputs.uniform_m(nodes.shape[0], d) for d in ((0, 0, 1), (1, 0, 0))]),
                         device="cuda")
     u64, H64 = Plan(nodes, tets, p=8, leaf_size=128, theta=0.5, near_mode=1, max_batch=2).eval(M)
-    for prec, bar, tb in (("bf16x3", 1e-5, -1), ("bf16x6", 1e-5, -1), ("fp32", 1e-5, 0)):
+    # tensor cores in the M2L and the near field forced at this batch of 2; both defaults (CUDA cores); the others
+    for prec, bar, tb, ntc in (("bf16x3", 1e-5, -1, 1), ("bf16x3", 1e-5, 0, 0), ("bf16x6", 1e-5, -1, 0),
+                               ("fp32", 1e-5, 0, 0)):
         u, H = Plan(nodes, tets, p=8, leaf_size=128, theta=0.5, precision=prec, near_mode=1, max_batch=2,
-                    m2l_table_batch=tb).eval(M)
+                    m2l_table_batch=tb, near_tc=ntc).eval(M)
         for k in range(2):
-            assert rel(u[k], u64[k]) <= bar and rel(H[k], H64[k]) <= bar, (prec, k)
+            assert rel(u[k], u64[k]) <= bar and rel(H[k], H64[k]) <= bar, (prec, tb, k)
 
 
 def test_ball500k_256_states():
