@@ -3,6 +3,7 @@ parallel, then a shared-library link.  No cmake, no torch extension machinery.""
 from __future__ import annotations
 
 import concurrent.futures as cf
+import hashlib
 import os
 import shutil
 import subprocess
@@ -33,17 +34,31 @@ def _deps():
     return hdrs
 
 
+def source_hash(csrc: str = CSRC) -> int:
+    """64 bits of the kernel and host sources: part of the tuner cache's key."""
+    h = hashlib.sha256()
+    for f in sorted(os.listdir(csrc)):
+        if f.endswith((".cu", ".cuh")):
+            with open(os.path.join(csrc, f), "rb") as src:
+                h.update(f.encode() + b"\0" + src.read())
+    return int.from_bytes(h.digest()[:8], "little")
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
     nvcc = _nvcc()
     hdr_t = max(os.path.getmtime(h) for h in _deps())
+    all_t = max(os.path.getmtime(os.path.join(CSRC, s)) for s in SOURCES)
     objs, jobs = [], []
     for src in SOURCES:
         s = os.path.join(CSRC, src)
         o = os.path.join(BUILD, src.replace(".cu", ".o"))
         objs.append(o)
-        if force or not os.path.exists(o) or os.path.getmtime(o) < max(os.path.getmtime(s), hdr_t):
-            jobs.append([nvcc, *ARCH, *FLAGS, "-c", s, "-o", o])
+        keyed = src == "api.cu"  # holds the hash of all sources
+        t = max(all_t if keyed else os.path.getmtime(s), hdr_t)
+        if force or not os.path.exists(o) or os.path.getmtime(o) < t:
+            extra = [f"-DDEMAG_SOURCE_HASH={source_hash():#x}ull"] if keyed else []
+            jobs.append([nvcc, *ARCH, *FLAGS, *extra, "-c", s, "-o", o])
     if jobs:
         with cf.ThreadPoolExecutor(max_workers=len(jobs)) as ex:
             res = list(ex.map(lambda c: subprocess.run(c, capture_output=True, text=True), jobs))

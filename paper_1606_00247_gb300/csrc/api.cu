@@ -359,13 +359,17 @@ static int tune_p(const demag_options& o, int64_t n_nodes, int64_t n_tets, const
 // Tuner cache.  The tuners choose by timing, which costs up to ~50 s of plan
 // time on a ball of half a million tets.  With the environment variable
 // DEMAG_TUNE_CACHE naming a file, a tuned plan's choices are appended to it
-// under a key that hashes the mesh, the options and the device, and a later
+// under a key that hashes the mesh, the options, the device and the sources that
+// this library was built from (the choices are those of its kernels), and a later
 // demag_plan_create with the same key builds the plan from them without timing.
 // Every candidate plan is built deterministically, so the plan built from the
 // cached choices is the one the tuners kept.  Lines that do not parse, carry
 // another format version or hold values out of range are skipped; the last
 // valid line of a key wins.
 constexpr int TUNE_CACHE_VERSION = 1;
+#ifndef DEMAG_SOURCE_HASH  // given by the build (build.py)
+#define DEMAG_SOURCE_HASH 0
+#endif
 
 static const char* tune_cache_path() {
   const char* p = std::getenv("DEMAG_TUNE_CACHE");
@@ -408,6 +412,7 @@ static uint64_t tune_key(const demag_options& o, int64_t n_nodes, int64_t n_tets
                          const int32_t* tets) {
   Fnv1a f;
   f.word(TUNE_CACHE_VERSION);
+  f.word((uint64_t)DEMAG_SOURCE_HASH);
   int dev = 0;
   DM_CUDA(cudaGetDevice(&dev));
   cudaDeviceProp prop{};

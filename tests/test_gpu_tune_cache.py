@@ -1,12 +1,13 @@
 """Tuner cache (environment variable DEMAG_TUNE_CACHE).
 
 A tuned plan's choices (p, leaf size, M2L launch shape) are appended to the
-file under a key that hashes the mesh, the options and the device; a second
-plan of the same mesh and options is built from them without timing and is the
-same plan (identical statistics, bit-identical results).  A different theta or
-a moved node is another key; lines that do not parse or hold values out of
-range are skipped, the last valid line of a key wins, and a file that cannot
-be written leaves a warning but not a failure.
+file under a key that hashes the mesh, the options, the device and the library's
+sources (another build's choices are not reused); a second plan of the same mesh
+and options is built from them without timing and is the same plan (identical
+statistics, bit-identical results).  A different theta or a moved node is another
+key; lines that do not parse or hold values out of range are skipped, the last
+valid line of a key wins, and a file that cannot be written leaves a warning but
+not a failure.
 """
 import pytest
 import torch
@@ -85,6 +86,38 @@ def test_cache_lines_are_validated_and_the_last_valid_one_wins(tmp_path, monkeyp
     ub, Hb = b.eval(M)
     uc, Hc = _plan(nodes, tets, **dict(kw, p=p_other, leaf_size=leaf_other, autotune=0)).eval(M)
     assert torch.equal(ub, uc) and torch.equal(Hb, Hc)
+
+
+def _fnv(words):
+    h = 1469598103934665603
+    for w in words:
+        h = ((h ^ (int(w) & (2**64 - 1))) * 1099511628211) & (2**64 - 1)
+    return h
+
+
+def _bytes(b):
+    pad = b + b"\0" * (-len(b) % 8)
+    return [int.from_bytes(pad[i:i + 8], "little") for i in range(0, len(pad), 8)] + [len(b)]
+
+
+def test_key_holds_the_hash_of_the_sources(tmp_path, monkeypatch):
+    """The key of an entry, formed here again: choices timed with other kernels are not found."""
+    import importlib
+    import struct
+
+    build = importlib.import_module("paper_1606_00247_gb300.build")
+
+    path = tmp_path / "tune.txt"
+    monkeypatch.setenv("DEMAG_TUNE_CACHE", str(path))
+    nodes, tets = inputs.sphere(h=0.4)
+    _plan(nodes, tets, p=4, leaf_size=32, theta=0.5, near_mode=1, precision="fp32", autotune=2)
+    (e,) = _entries(path)
+    prop = torch.cuda.get_device_properties(0)
+    opts = [4, 32, 1, 1, 1, 2] + [0] * 8  # p, leaf, precision fp32, near mode, batch, autotune, the other options
+    words = [1, build.source_hash(), *_bytes(prop.name.encode()), prop.multi_processor_count,
+             100 * prop.major + prop.minor, *opts, struct.unpack("<Q", struct.pack("<d", 0.5))[0], len(nodes), len(tets),
+             *_bytes(nodes.astype("<f8").tobytes()), *_bytes(tets.astype("<i4").tobytes())]
+    assert int(e[2], 16) == _fnv(words)
 
 
 def test_no_tuning_no_cache_and_unwritable_cache(tmp_path, monkeypatch):
