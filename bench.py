@@ -193,34 +193,36 @@ def live_peaks():
     return peaks
 
 
-# FP64 operations of the integrated near field per (target node, source tet)
-# pair in the tet-wise form of the method (p2p.cuh: a and T of the pair once,
-# then every state): pair 1457 = 12 + 20 + 24 + 1, then 4 faces x (h 5, triple
-# product 14, 3 dots 15, denominator 8, Om and I 2, 3 edges x 69, a 12, T 87);
-# 44 per state; for one state 470 (the contracted form).  sqrt, log1p, divisions
-# and atan2 are not counted.  The kernel (p2p.cu) shares distances, logarithms
-# and solid angles between the tets of a cluster and executes fewer.
-P2P_AT_MIN_B = 2
-P2P_PAIR_FLOPS, P2P_STATE_FLOPS, P2P_PERSTATE_FLOPS = 1457, 44, 470
-
-
-def p2p_fp64_flops(B):
-    """FP64 flops of one (target node, source tet) pair for a batch of B states."""
-    return P2P_PERSTATE_FLOPS * B if B < P2P_AT_MIN_B else P2P_PAIR_FLOPS + P2P_STATE_FLOPS * B
+# FP64 operations of the integrated near field (k_p2p_faces, p2p.cu) per target
+# and part of a cluster, counted from the source (a multiply-add is two); sqrt,
+# log1p, divisions and atan2 are not counted:
+#  vertex 8 (3 subtractions, norm 5), edge 3;
+#  face 50 + 6 per state: 9 subtractions, h 5, 3 dots 15, denominator 8, solid
+#  angle 2, A 7, h^2 1, weights 3, and 3 multiply-adds per state;
+#  boundary face 93 + 18 per state besides: foot 10, w_e 10, dR 3, z 5, I 4, S 32,
+#  vectors 20, weights 9, and 9 multiply-adds per state.
+def p2p_fp64_flops(stats, B):
+    """FP64 flops per (target node, source tet) pair for a batch of B states, from
+    the mean number of a tet's cluster parts; slices of at most 16 states repeat
+    all but the per-state part."""
+    nt = stats["n_tets"]
+    v, e, f, b = (stats[k] / nt for k in ("cluster_vertices", "cluster_edges", "cluster_faces",
+                                          "cluster_boundary_faces"))
+    return -(-B // 16) * (8 * v + 3 * e + 50 * f + 93 * b) + B * (6 * f + 18 * b)
 
 
 def m2l_macs(p):
-    """Multiply-adds of one M2L pair for one state: #{(n, m): |n| + |m| <= p} = C(p+6, 6)."""
+    """Multiply-adds of one M2L pair for one state on all multi-indices (the form of
+    Sec. 2.3): #{(n, m): |n| + |m| <= p} = C(p+6, 6)."""
     from math import comb
 
     return comb(p + 6, 6)
 
 
-def m2l_split_degree(p):
-    """The default split degree of an M2L on all multi-indices (m2l_tile_flops):
-    the products with the second BF16 limb only for terms |m| + |n| <= p - 4
-    (p - 3 below order 8)."""
-    return p - 4 if p >= 8 else p - 3
+def m2l_products(p):
+    """Multiply-adds of one M2L pair for one state on the trace-free indices:
+    (2 |m| + 1) rows m of every degree below p, (p - |m| + 1)^2 - 1 moments each."""
+    return sum((2 * t + 1) * ((p - t + 1) ** 2 - 1) for t in range(p))
 
 
 def m2l_issued_flops(p, precision, split_all=False):
@@ -243,29 +245,6 @@ def m2l_issued_flops(p, precision, split_all=False):
         total += rows * kw
         if precision == "bf16x3":
             rows2 = rows if split_all else min(pad(rows_of(sd if ks == 0 else sd - d), 16), rows)
-            total += 2 * rows2 * kw
-    return 2.0 * total
-
-
-def m2l_tile_flops(p, precision, split_all=False):
-    """The same for an M2L on all C(p+3, 3) multi-indices: every k-step
-    (16 BF16 or 8 TF32 values of n) is one M = 128 MMA over the rows m still
-    needed at that k-step (rows of degree t need |n| < C(p - t + 3, 3)),
-    padded to 16.  Split BF16 adds the hi x lo and lo x hi MMAs over the rows
-    whose terms take the second limb (degree <= split degree - the k-step's
-    lowest |n|; every row with split_all)."""
-    cnc = lambda t: 0 if t < 0 else (t + 1) * (t + 2) * (t + 3) // 6
-    pad = lambda x, m: (x + m - 1) // m * m
-    deg = lambda m: next(t for t in range(p + 1) if cnc(t) > m)
-    kw = 16 if precision == "bf16x3" else 8
-    sd = m2l_split_degree(p)
-    total = 0
-    for ks in range(pad(cnc(p), kw) // kw):
-        rows = pad(max([cnc(t) for t in range(p + 1) if cnc(p - t) > ks * kw] or [0]), 16)
-        total += rows * kw
-        if precision == "bf16x3":
-            r = sd - deg(ks * kw)
-            rows2 = rows if split_all else min(pad(cnc(r), 16) if r >= 0 else 0, rows)
             total += 2 * rows2 * kw
     return 2.0 * total
 
@@ -299,15 +278,6 @@ def _alu_peak(kind, peaks, sm_mhz):
                                            + (" / 64 (FP64)" if kind == "fp64" else ""))
 
 
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of a
-# kernel, from one ncu capture on GB300 of this exact configuration and kernel
-# version; any other configuration reports null
-NCU_TRAFFIC = {
-    # (stage, precision, p, leaf, batch, n_tets): bytes
-    # none: the M2L and the near field have changed since their captures
-}
-
-
 def m2l_on_tensor_cores(precision, B, table_batch):
     """The tensor-core precisions run the FP32 table M2L on CUDA cores up to
     m2l_table_batch states (0: the library default of 8; < 0: never)."""
@@ -330,10 +300,11 @@ def stage_roofline(stage, stats, steps_profiled, precision, peaks, sm_mhz, tenso
     launches_per_eval = launches / max(1, steps_profiled)
     B, p, nn = stats["_batch"], stats["p"], stats["n_nodes"]
     out = {"kernel": stage, "ms_per_step": ms / max(1, steps_profiled), "launches_per_step": launches_per_eval}
-    key = (stage, precision, p, stats["leaf_size"], B, stats["n_tets"])
     kind = "fp64" if precision == "fp64" else "fp32"
     if stage == "m2l":
-        work = 2.0 * stats["n_m2l"] * m2l_macs(p) * B / launches_per_eval
+        # flops of the trace-free form that runs; method_tflops: those of all multi-indices in the same time
+        work = 2.0 * stats["n_m2l"] * m2l_products(p) * B / launches_per_eval
+        out["method_tflops"] = 2.0 * stats["n_m2l"] * m2l_macs(p) * B / launches_per_eval / per_launch_s / 1e12
         if precision in ("tf32", "bf16x3") and tensor_m2l:
             # tcgen05 M2L timed inside a long step: the sustained measured BF16 rate is
             # the denominator (TF32: x the nominal TF32/BF16 ratio 1.1 / 2.25 PFLOP/s)
@@ -347,29 +318,32 @@ def stage_roofline(stage, stats, steps_profiled, precision, peaks, sm_mhz, tenso
                           / launches_per_eval)
             achieved = work / per_launch_s / 1e12
             out.update({"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                        "frac": achieved / peak, "traffic": NCU_TRAFFIC.get(key),
+                        "frac": achieved / peak, "traffic": None,
                         "executed_tflops": tile_flops / per_launch_s / 1e12,
                         "peak_source": src,
-                        "note": "achieved counts the method's 2*C(p+6,6) flops per pair per state (all multi-indices); "
-                                "the M2L runs on the trace-free ones, executed_tflops "
-                                "counts the padded per-k-step row prefixes issued to the tensor pipe "
+                        "note": f"achieved counts the {2 * m2l_products(p)} flops per pair and state of the trace-free "
+                                f"form, method_tflops the {2 * m2l_macs(p)} of all multi-indices, executed_tflops "
+                                "the padded per-k-step row prefixes issued to the tensor pipe "
                                 + ("(hi x hi everywhere, hi x lo and lo x hi on the rows whose terms take the "
                                    "second limb)" if precision == "bf16x3" else "(1 TF32 MMA per tile)")})
             return out
         achieved = work / per_launch_s / 1e12
         peak, src = _alu_peak(kind, peaks, sm_mhz)
         out.update({"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                    "traffic": NCU_TRAFFIC.get(key), "peak_source": src,
-                    "note": f"the method's 2*C(p+6,6) flops per pair per state (all multi-indices), {kind} CUDA cores"})
+                    "traffic": None, "peak_source": src,
+                    "note": f"achieved counts the {2 * m2l_products(p)} flops per pair and state of the trace-free form, "
+                            f"method_tflops the {2 * m2l_macs(p)} of all multi-indices; {kind} CUDA cores"})
         return out
     if stage == "p2p" and stats["near_mode"] == 0:
-        work = stats["n_p2p_pairs"] * p2p_fp64_flops(B) / launches_per_eval
+        per_pair = p2p_fp64_flops(stats, B)
+        work = stats["n_p2p_pairs"] * per_pair / launches_per_eval
         achieved = work / per_launch_s / 1e12
         peak, src = _alu_peak("fp64", peaks, sm_mhz)
         out.update({"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                    "traffic": NCU_TRAFFIC.get(key), "peak_source": src,
-                    "note": (f"FP64 pipe, {p2p_fp64_flops(B)} FP64 flops per (node, tet) pair for {B} states "
-                             "(pair geometry once per pair from 2 states on); transcendentals not counted")})
+                    "traffic": None, "peak_source": src,
+                    "note": (f"FP64 pipe, {per_pair:.0f} FP64 flops per (node, tet) pair for {B} states: distances, "
+                             "edges and faces of the clusters of source tets; square roots, logarithms, divisions "
+                             "and arctangents are not counted")})
         return out
     if stage == "p2p":
         # stored near field: every (target node, source node) coefficient triple read once per
@@ -383,7 +357,7 @@ def stage_roofline(stage, stats, steps_profiled, precision, peaks, sm_mhz, tenso
         peak = peaks.get("hbm_gbs", 6800.0)
         flops = 2.0 * 3 * pairs * B / launches_per_eval
         out.update({"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                    "traffic": NCU_TRAFFIC.get(key), "algorithmic_bytes": alg,
+                    "traffic": None, "algorithmic_bytes": alg,
                     "stored_bytes": stats.get("near_bytes"),
                     "peak_source": "measured copy bandwidth (MEASURED_PEAKS.json)" if "hbm_gbs" in peaks
                                    else "fallback 6800 GB/s",

@@ -409,6 +409,9 @@ typedef struct {
   int tune_source;       /* 0: autotune = 0; 1: the tuners timed their
                             candidates; 2: their choices were read from the
                             DEMAG_TUNE_CACHE file                           */
+  /* integrated near field: parts of all clusters of source tets (0: none)  */
+  int64_t cluster_vertices, cluster_edges, cluster_faces;
+  int64_t cluster_boundary_faces; /* faces with one tet in their cluster    */
 } demag_stats;
 
 demag_status demag_plan_stats(demag_plan plan, demag_stats* out);

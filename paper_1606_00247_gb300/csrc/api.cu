@@ -720,6 +720,10 @@ demag_status demag_plan_stats(demag_plan plan, demag_stats* o) {
   o->n_near_tiles = plan->nf_ntiles;
   o->near_tile_cols = plan->nf_ncols;
   o->tune_source = plan->tune_source;
+  o->cluster_vertices = plan->n_cl_v;
+  o->cluster_edges = plan->n_cl_e;
+  o->cluster_faces = plan->n_cl_f;
+  o->cluster_boundary_faces = plan->n_cl_b;
   o->near_bytes = plan->nf_W ? plan->nf_wbytes
                              : (plan->W32 ? plan->n_wentries / 3 * 16
                                           : (plan->W64 ? plan->n_wentries * 8 : 0));

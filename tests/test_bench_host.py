@@ -28,14 +28,35 @@ def test_m2l_path_choice():
 
 def test_m2l_counts():
     assert bench.m2l_macs(8) == 3003 and bench.m2l_macs(4) == 210  # C(p + 6, 6)
-    # split BF16, p = 8: k-step row prefixes 176, 64, 48, 32 and seven of 16, K = 16
-    rows = [176, 64, 48, 32] + [16] * 7
-    assert bench.m2l_tile_flops(8, "bf16x3", split_all=True) == 2.0 * sum(r * 16 for r in rows) * 3
-    # default split degree p - 4 = 4: the second-limb rows are those of degree <= 4 - (lowest |n| of
-    # the k-step) -- 35 (pad 48), 4 (16), 1 (16) for k-steps 0-2 (lowest |n| 0, 3, 4), none after
-    rows2 = [48, 16, 16] + [0] * 8
-    assert bench.m2l_tile_flops(8, "bf16x3") == 2.0 * 16 * (sum(rows) + 2 * sum(rows2))
-    assert bench.m2l_split_degree(8) == 4 and bench.m2l_split_degree(6) == 3
+    # trace-free: nl rows m, nq(p - |m|) moments each, counted one by one
+    for p in (1, 4, 8):
+        deg = [t for t in range(p + 1) for _ in range(2 * t + 1)]
+        assert bench.m2l_products(p) == sum(m + n <= p for m in deg for n in deg if m < p and n > 0)
+    assert bench.m2l_products(8) == 1284
+    # split BF16, p = 8: k-steps of 16 moments with lowest degrees 1, 4, 5, 7, 8; rows of degree <= 8 - d
+    # are 64, 25, 16, 4, 1, padded to 16
+    rows = [64, 32, 16, 16, 16]
+    assert bench.m2l_issued_flops(8, "bf16x3", split_all=True) == 2.0 * sum(r * 16 for r in rows) * 3
+    # default split degree p - 4 = 4: second-limb rows of degree <= 4 in the first k-step (25, pad 32),
+    # <= 4 - d in the others (1, pad 16, for d = 4; none after)
+    assert bench.m2l_issued_flops(8, "bf16x3") == 2.0 * 16 * (sum(rows) + 2 * (32 + 16))
+
+
+def test_executed_fp64_work_stays_below_the_peak():
+    """The integrated near field and the FP64 M2L counted as they run, at measured times: an operation
+    that the kernels do not execute would put the fraction above 1."""
+    stats = {"stage_ms": {"m2l": 1.0, "p2p": 17.8}, "stage_launches": {"m2l": 1, "p2p": 3}, "_batch": 3, "p": 8,
+             "n_m2l": 870000, "near_mode": 0, "n_p2p_pairs": 17.4e6, "leaf_size": 128, "n_tets": 16000, "n_nodes": 3000,
+             "cluster_vertices": 9600, "cluster_edges": 32000, "cluster_faces": 44000, "cluster_boundary_faces": 16000}
+    peaks = {"fp64_fma_measured": 1.058}
+    r = bench.stage_roofline("p2p", stats, 1, "fp64", peaks, 2070.0)
+    per_pair = 8 * 0.6 + 3 * 2 + 50 * 2.75 + 93 + 3 * (6 * 2.75 + 18)
+    assert abs(bench.p2p_fp64_flops(stats, 3) - per_pair) < 1e-9 and 0.2 < r["frac"] < 1.0
+    assert abs(r["achieved"] - 17.4e6 * per_pair / 17.8e-3 / 1e12) < 1e-9
+    stats["stage_ms"]["m2l"] = 2.55  # the 224k-tet ball, one state
+    stats["_batch"] = 1
+    m = bench.stage_roofline("m2l", stats, 1, "fp64", peaks, 2070.0, tensor_m2l=False)
+    assert 0.5 < m["frac"] < 1.0 and abs(m["method_tflops"] / m["achieved"] - 3003 / 1284) < 1e-12
 
 
 def test_roofline_record_tensor_and_alu():
@@ -45,7 +66,7 @@ def test_roofline_record_tensor_and_alu():
     peaks = {"bf16_tflops_sustained": 1744.5, "hbm_gbs": 6689.8}
     r = bench.roofline_for(stats, 10, "bf16x3", peaks, 2070.0, tensor_m2l=True)
     assert r["kernel"] == "m2l" and r["bound"] == "tensor" and r["peak"] == 1744.5
-    achieved = 2.0 * 866523 * 3003 * 128 / 8e-3 / 1e12
+    achieved = 2.0 * 866523 * 1284 * 128 / 8e-3 / 1e12
     assert abs(r["achieved"] - achieved) < 1e-9 * achieved and abs(r["frac"] - achieved / 1744.5) < 1e-12
     r2 = bench.roofline_for(stats, 10, "bf16x3", peaks, 2070.0, tensor_m2l=False)
     assert r2["bound"] == "alu" and abs(r2["peak"] - 152 * 128 * 2 * 2070e6 / 1e12) < 1e-9
