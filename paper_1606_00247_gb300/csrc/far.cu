@@ -247,8 +247,15 @@ __global__ void __launch_bounds__(P2MS_THREADS) k_p2m_small(const int32_t* __res
   }
 }
 
-// batches up to this take the small-batch P2M and L2P (slices of 8 states)
-constexpr int FAR_SMALL_BATCH = 32;
+// Largest batches of the small-batch P2M and L2P (slices of 8 states), whose time
+// grows with the slices; the tiles cost the same up to 128 states.  P2M, leaves of 43
+// support nodes on average (224k-tet ball, leaf 128), p = 8: 32 states 162 against 239
+// us, 48 equal; leaves of 13 (leaf 64): 16 states 234 / 288 us and 24 states 352 / 292
+// at p = 6, 16 states 183 / 167 at p = 4.  L2P, 24 and 32 states: p = 8 41 / 45 and 53
+// / 45 us; leaf 64, p = 6 59 / 98 and 87 / 98, p = 4 45 / 55 and 55 / 56; 29k tets, p
+// = 8 12 / 16 and 14 / 16.
+inline int p2m_small_batch(const Plan& P) { return P.n_sup >= 25 * (int64_t)P.h_src_leaves.size() ? 32 : 16; }
+constexpr int L2P_SMALL_BATCH = 32;
 
 template <int SPT, int NN>
 void launch_p2m_tile(Plan& P, int B, const float* Ms, float* Q, cudaStream_t s) {
@@ -702,7 +709,7 @@ int launch_p2m(Plan& P, int B, const T* Ms, T* Q, cudaStream_t s) {
     launch_p2m_small<T, 2>(P, B, Ms, Q, s);
   else if (B <= 4)
     launch_p2m_small<T, 4>(P, B, Ms, Q, s);
-  else if (B <= FAR_SMALL_BATCH || std::is_same<T, double>::value)
+  else if (B <= p2m_small_batch(P) || std::is_same<T, double>::value)
     launch_p2m_small<T, 8>(P, B, Ms, Q, s);
   else if constexpr (std::is_same<T, float>::value) {
     if (P.nq <= 24)
@@ -797,7 +804,7 @@ int launch_l2p(Plan& P, int B, const T* L, T* u, cudaStream_t s) {
     launch_l2p_small<T, 2>(P, B, L, u, s);
   else if (B <= 4)
     launch_l2p_small<T, 4>(P, B, L, u, s);
-  else if (B <= FAR_SMALL_BATCH || std::is_same<T, double>::value)
+  else if (B <= L2P_SMALL_BATCH || std::is_same<T, double>::value)
     launch_l2p_small<T, 8>(P, B, L, u, s);
   else if constexpr (std::is_same<T, float>::value) {
     const size_t smem = sizeof(float) * (size_t)P.nl * (128 + L2P_NCH);

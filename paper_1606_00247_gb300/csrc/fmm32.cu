@@ -38,7 +38,9 @@ __global__ void __launch_bounds__(256) k_gather_M32(int64_t nn, int B, const int
 }
 
 // From GATHER_WIDE states on: block per (sorted node, 128 states), thread = state
-// (no division per thread: 256 states of 87k nodes 297 us, 399 with the kernel above)
+// (no division per thread).  Against the kernel above, 36k nodes: 48 states 32 / 30 us,
+// 64 to 160 states equal (37 us at 64), 256 states 110 / 113; 87k nodes, 256 states 309 /
+// 399.
 constexpr int GATHER_WIDE = 64;
 __global__ void __launch_bounds__(128) k_gather_M32_wide(int64_t nn, int B, const int32_t* __restrict__ perm,
                                                          const double* __restrict__ M, float* Ms, double* Ms64) {

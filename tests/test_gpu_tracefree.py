@@ -35,9 +35,9 @@ def orc():
     return oracle
 
 
-# every order (the moment tile of the P2M holds 24, 48 or 80 moments, p = 12 takes three tiles; the
-# table M2L ends at p = 10), batches on both sides of the small-batch kernels (32) and of one and two
-# states per thread (128), odd ones included.  FP32: sums of 1e3 rounded terms, ~1e-6 of the largest.
+# every order (the moment tile of the P2M holds 24, 48 or 80 moments, p = 12 takes three tiles), batches
+# on both sides of the small-batch kernels (16 in the P2M of these small leaves, 32 in the L2P) and of one
+# and two states per thread (128), odd ones included.  FP32: sums of 1e3 rounded terms, ~1e-6 of the largest.
 @pytest.mark.parametrize("B", [1, 32, 33, 129])
 @pytest.mark.parametrize("p", [1, 2, 4, 5, 6, 7, 8, 10, 11, 12])
 def test_fp32_vs_oracle(orc, p, B):
