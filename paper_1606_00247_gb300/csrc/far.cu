@@ -248,13 +248,18 @@ __global__ void __launch_bounds__(P2MS_THREADS) k_p2m_small(const int32_t* __res
 }
 
 // Largest batches of the small-batch P2M and L2P (slices of 8 states), whose time
-// grows with the slices; the tiles cost the same up to 128 states.  P2M, leaves of 43
-// support nodes on average (224k-tet ball, leaf 128), p = 8: 32 states 162 against 239
-// us, 48 equal; leaves of 13 (leaf 64): 16 states 234 / 288 us and 24 states 352 / 292
-// at p = 6, 16 states 183 / 167 at p = 4.  L2P, 24 and 32 states: p = 8 41 / 45 and 53
-// / 45 us; leaf 64, p = 6 59 / 98 and 87 / 98, p = 4 45 / 55 and 55 / 56; 29k tets, p
-// = 8 12 / 16 and 14 / 16.
-inline int p2m_small_batch(const Plan& P) { return P.n_sup >= 25 * (int64_t)P.h_src_leaves.size() ? 32 : 16; }
+// grows with the slices; the tiles cost the same up to 128 states.  P2M, small
+// against tiles: 2,360 leaves (68k-tet ball, leaf 128) p = 8 32 states 81 / 123 us, p =
+// 6 63 / 82, p = 4 24 states 46 / 51 and 32 states 55 / 50; 2,571 leaves (224k tets) p =
+// 8 162 / 239, p = 6 115 / 155; 16,941 leaves of 13 tets, where a slice costs most, p =
+// 8 24 states 391 / 481 and 32 states 520 / 489, p = 6 16 states 234 / 288 and 24 states
+// 352 / 292, p = 4 8 states 95 / 165 and 16 states 183 / 167.  L2P, 24 and 32 states: p =
+// 8 41 / 45 and 53 / 45 us; leaf 64, p = 6 59 / 98 and 87 / 98, p = 4 45 / 55 and 55 /
+// 56; 29k tets, p = 8 12 / 16 and 14 / 16.
+inline int p2m_small_batch(const Plan& P) {
+  const bool many = P.h_src_leaves.size() > 8192;
+  return P.nq <= 24 ? (many ? 8 : 24) : P.nq <= 48 ? (many ? 16 : 32) : (many ? 24 : 32);
+}
 constexpr int L2P_SMALL_BATCH = 32;
 
 template <int SPT, int NN>

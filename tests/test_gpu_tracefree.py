@@ -36,8 +36,8 @@ def orc():
 
 
 # every order (the moment tile of the P2M holds 24, 48 or 80 moments, p = 12 takes three tiles), batches
-# on both sides of the small-batch kernels (16 in the P2M of these small leaves, 32 in the L2P) and of one
-# and two states per thread (128), odd ones included.  FP32: sums of 1e3 rounded terms, ~1e-6 of the largest.
+# on both sides of the small-batch kernels (P2M 24 up to p = 4, else 32; L2P 32) and of one and two states
+# per thread (128), odd ones included.  FP32: sums of 1e3 rounded terms, ~1e-6 of the largest.
 @pytest.mark.parametrize("B", [1, 32, 33, 129])
 @pytest.mark.parametrize("p", [1, 2, 4, 5, 6, 7, 8, 10, 11, 12])
 def test_fp32_vs_oracle(orc, p, B):
