@@ -370,7 +370,7 @@ enum {
   DEMAG_STAGE_M2L = 3,
   DEMAG_STAGE_L2L = 4,
   DEMAG_STAGE_L2P = 5,
-  DEMAG_STAGE_NEAR_PREP = 6, /* not used: the integrated near field's face charges count as P2P */
+  DEMAG_STAGE_NEAR_PREP = 6, /* not used: the integrated near field's per-face values count as P2P */
   DEMAG_STAGE_P2P = 7,
   DEMAG_STAGE_H = 8,         /* mass-lumped H and the output layout           */
   DEMAG_N_STAGES = 9

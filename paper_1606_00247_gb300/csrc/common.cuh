@@ -385,7 +385,7 @@ T* dalloc(Plan& P, size_t n) {
 void dfree_all(Plan& P);
 void dfree(Plan& P, void* ptr);  // one plan buffer, before the plan is destroyed
 
-// stages (defined in plan.cu / fmm.cu / p2p.cu / eval.cu)
+// plan construction (plan.cu), FP64 evaluation and workspace (fmm.cu)
 void build_plan(Plan& P, const double* nodes, const int32_t* tets);
 // opt a kernel in to `bytes` of dynamic shared memory on the current device
 // (set once per kernel, device and size; thread-safe)

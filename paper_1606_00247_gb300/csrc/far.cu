@@ -4,7 +4,7 @@
 //
 // With s the side of a cell, the stored coefficients are
 //   Qt_n = Qhat_n / s^|n|      Lt_m = L_m s^|m|
-// (Qhat_n = Q_n/n!, L_m = d^m u, see fmm.cu), kept in the trace-free form of
+// (Qhat_n = Q_n/n!, Q_n the moments of Sec. 2.2, L_m = d^m u), kept in the trace-free form of
 // common.cuh (nq = (p+1)^2 - 1 moments, nl = p^2 local coefficients: 80 and 64
 // instead of 165 at p = 8).  All of them are O(1) whatever the mesh scale, so
 // FP32 neither overflows nor underflows, and the octree translations become

@@ -8,7 +8,7 @@
 // accumulated over all sources S of T in tensor memory (M = 128 states = TMEM
 // lanes, N = rows m, K = n).  n and m run over the trace-free indices of
 // common.cuh (80 moments, 64 local coefficients at p = 8): 9 MMAs, 28 KB of
-// moments and 5.6 KB of operator per pair and 128 states, where the 165 full
+// moments and 6.1 KB of operator per pair and 128 states, where the 165 full
 // multi-indices took 17 MMAs, 56 KB and 16.4 KB.
 //
 // Translation operators.  Expansion centres are octree box centres, so
