@@ -134,7 +134,7 @@ size_t admission_bytes(const Plan& P, int B) {
 
 size_t carve(Plan& P, int B, unsigned char* base, Workspace* W) {
   Carver c{base};
-  const size_t nn = P.nn, nt = P.nt, ncell = P.ncells;
+  const size_t nn = P.nn, ncell = P.ncells;
   const bool mixed = P.opt.precision != DEMAG_FP64, otf = P.opt.near_mode == 0;
   Workspace w;
   w.B = B;
@@ -153,9 +153,10 @@ size_t carve(Plan& P, int B, unsigned char* base, Workspace* W) {
     if (mp) w.MP = c.take<float>(mp);
   }
   if (!mixed || otf) w.u_s = c.take<double>(nn * B);
-  if (otf) {  // the largest slice within the same allowance; one state always fits (48 doubles per tet at most)
+  if (otf) {  // the largest slice that leaves room for the flag; one state takes at most 48 doubles per tet
+    auto end = [&](int slice) { return (c.used + 511) / 256 * 256 + sizeof(double) * face_state_doubles(P, slice) + 512; };
     w.slice = p2p_slice(B);
-    while (w.slice > 1 && face_state_doubles(P, w.slice) > nt * NOALLOC_TET_STATE) w.slice /= 2;
+    while (w.slice > 1 && end(w.slice) > (size_t)DEMAG_NOALLOC_SCRATCH_BYTES) w.slice /= 2;
     w.state = c.take<double>(face_state_doubles(P, w.slice));
   }
   w.err = c.take<int>(1);

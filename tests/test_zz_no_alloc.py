@@ -79,6 +79,25 @@ def test_noalloc_first_call_allocates_nothing(precision, near_mode, B):
     assert float(torch.linalg.norm(H - H_ref) / torch.linalg.norm(H_ref)) <= tol
 
 
+def test_noalloc_slices_of_the_integrated_near_field():
+    """The per-face values of 16 states (75 MB) do not fit the scratch area: slices of 8 states."""
+    from paper_1606_00247_gb300 import _lib
+    from paper_1606_00247_gb300.api import Plan
+
+    nodes, tets = inputs.sphere(h=0.1)
+    B = 16
+    plan = Plan(nodes, tets, p=4, leaf_size=128, max_batch=B, near_mode=0)
+    st = plan.stats()
+    assert 8 * B * (3 * st["cluster_faces"] + 9 * st["cluster_boundary_faces"]) > 64 * 2**20
+    M = torch.as_tensor(inputs.gaussian_unit_m(nodes.shape[0], seed=13, batch=B), device="cuda")
+    u_ref, H_ref = plan.eval(M)
+    u, H = torch.full_like(u_ref, float("nan")), torch.full_like(H_ref, float("nan"))
+    assert _call_noalloc(plan, M, u, H) == _lib.DEMAG_OK, _lib.demag_last_error()
+    torch.cuda.synchronize()
+    assert float(torch.linalg.norm(u - u_ref) / torch.linalg.norm(u_ref)) <= 1e-12
+    assert float(torch.linalg.norm(H - H_ref) / torch.linalg.norm(H_ref)) <= 1e-12
+
+
 def test_noalloc_rejects_oversized_scratch_and_host_pointers():
     from paper_1606_00247_gb300 import _lib
     from paper_1606_00247_gb300.api import Plan
