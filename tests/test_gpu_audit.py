@@ -4,9 +4,9 @@ demag_plan_create audits every plan before returning it, so every plan of the
 suite passes through it; here it is run again on plans of each kind (FP64 on
 the fly, stored FP64, FP32, split BF16 with both tensor-core stages, two-target
 M2L groups, point dipoles and vertex patches), and its error path is taken by
-auditing a scratch copy of the M2L source list with one entry out of range
-(demag_plan_debug bit 1): only the audit kernel reads that copy, so nothing
-follows the bad index, and the plan's own lists stay as they were."""
+auditing scratch copies of lists of each kind with one entry out of range
+(demag_plan_debug bit 1): only the audit kernels read the copies, so nothing
+follows a bad index, and the plan's own lists stay as they were."""
 import pytest
 import torch
 
